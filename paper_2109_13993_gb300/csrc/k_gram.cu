@@ -1,106 +1,121 @@
 // k_gram.cu -- CalculateCovMat (Algorithm 3): Sigma = Xn Xn^T / (n-1)
 // of the normalised rows, the covariance the closed forms of Sec. III-E start
-// from.  SIMT version: 64 x 64 output tiles of the upper triangle, K-chunks of
-// 32 samples staged in shared memory; FP32 products with FP32 chunk sums
-// folded into Kahan-compensated FP32 totals (mixed path), or FP64 throughout.
-// The diagonal is exactly 1 (normalised rows).
-#include <type_traits>
+// from.  The FP64 path's version, and the mixed path's for the small problems of a batch.  The
+// diagonal is exactly 1 (normalised rows).
+#include <algorithm>
 
 #include "common.cuh"
 #include "launch.h"
 
 namespace lingam {
 
-constexpr int kGT = 64;   // output tile
-constexpr int kGK = 32;   // samples per chunk
+// ------------------------------------------------------------------ FP64
+// 32 x 32 tiles of the upper triangle times splits of the sample axis, so that the whole GPU works
+// also on few variables; a thread has 2 x 2 elements, and chunks of 32 samples of the tile's rows and
+// columns are staged in shared memory, the next chunk loaded into registers meanwhile.  Bound by the
+// FP64 rate (1.7 FMAs a clock and SM), so small tiles cost nothing: their operand reads hide behind
+// it, and less of the triangle is padding.  A covariance call at p = 300, n = 5000 took 5.87 ms
+// with 64 x 64 tiles and no split (15 CTAs), 0.89 ms now (0.47 ms of it the FMAs at that rate).  The splits' partial tiles are added in split order by a second kernel.
+constexpr int kGT = 32;        // output tile
+constexpr int kGK = 32;        // samples per chunk
+constexpr int kGSplitCtas = 608;   // CTAs wanted: four per SM, so that the last round is short
 
-template <class T>
-__global__ void __launch_bounds__(256) k_gram(Fit f) {
-    __shared__ __align__(16) T As[kGK][kGT + 4];
-    __shared__ __align__(16) T Bs[kGK][kGT + 4];
-    const int p = f.p, ld = f.ld, tid = threadIdx.x;
-    // blockIdx.x -> (bi, bj) with bi <= bj
-    const int nt = (p + kGT - 1) / kGT;
-    int rem = blockIdx.x, bi = 0;
-    while (rem >= nt - bi) {
-        rem -= nt - bi;
+__device__ __forceinline__ void gram_tile(int tile, int nt, int& bi, int& bj) {
+    bi = 0;
+    while (tile >= nt - bi) {
+        tile -= nt - bi;
         ++bi;
     }
-    const int bj = bi + rem;
-    const int i0 = bi * kGT, j0 = bj * kGT;
-    const T* xt = static_cast<const T*>(f.xt);
-    const int ty = tid >> 4, tx = tid & 15;
+    bj = bi + tile;
+}
+__device__ __forceinline__ void gram_store(const Fit& f, int i, int j, double s) {
+    const int p = f.p;
+    if (i >= p || j >= p || i > j) return;
+    const double v = i == j ? 1.0 : s * (1.0 / double(f.n - 1));
+    f.sig[size_t(i) * p + j] = v;
+    f.sig[size_t(j) * p + i] = v;
+    f.sig0[size_t(i) * p + j] = v;
+    f.sig0[size_t(j) * p + i] = v;
+}
 
-    T sum[4][4], comp[4][4];
+__global__ void __launch_bounds__(256) k_gram(Fit f, double* __restrict__ partial, int nt, int nsplit) {
+    __shared__ double As[kGT][kGK + 1], Bs[kGT][kGK + 1];
+    const int p = f.p, ld = f.ld, tid = threadIdx.x;
+    const int tile = blockIdx.x / nsplit, split = blockIdx.x - tile * nsplit;
+    int bi, bj;
+    gram_tile(tile, nt, bi, bj);
+    const int nch = ld / kGK, c0 = int((long long)split * nch / nsplit), c1 = int((long long)(split + 1) * nch / nsplit);
+    const double* xt = static_cast<const double*>(f.xt);
+    const int lane = tid & 31, w = tid >> 5;   // warp w stages rows w, w + 8, ...
+    const int ty = tid >> 4, tx = tid & 15;
+    double ra[4], rb[4];
+    auto load = [&](int c) {
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            sum[a][b] = T(0);
-            comp[a][b] = T(0);
+        for (int q = 0; q < 4; ++q) {
+            const int i = bi * kGT + w + 8 * q, j = bj * kGT + w + 8 * q;
+            ra[q] = i < p ? xt[size_t(i) * ld + c * kGK + lane] : 0.0;
+            rb[q] = j < p ? xt[size_t(j) * ld + c * kGK + lane] : 0.0;
         }
-    for (int k0 = 0; k0 < ld; k0 += kGK) {
-        // stage: 64 rows x 32 samples of each operand, transposed to [k][row]
-        for (int e = tid; e < kGT * kGK; e += 256) {
-            const int rr = e / kGK, kk = e % kGK;
-            const int gi = i0 + rr, gj = j0 + rr;
-            As[kk][rr] = gi < p ? xt[size_t(gi) * ld + k0 + kk] : T(0);
-            Bs[kk][rr] = gj < p ? xt[size_t(gj) * ld + k0 + kk] : T(0);
+    };
+    double acc[2][2] = {};
+    if (c0 < c1) load(c0);
+    for (int c = c0; c < c1; ++c) {
+        __syncthreads();   // the previous chunk is consumed
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            As[w + 8 * q][lane] = ra[q];
+            Bs[w + 8 * q][lane] = rb[q];
         }
         __syncthreads();
-        T acc[4][4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
+        if (c + 1 < c1) load(c + 1);
 #pragma unroll 8
-        for (int kk = 0; kk < kGK; ++kk) {
-            T av[4], bv[4];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) av[a] = As[kk][ty * 4 + a];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) bv[b] = Bs[kk][tx * 4 + b];
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
+        for (int k = 0; k < kGK; ++k) {
+            const double a0 = As[ty][k], a1 = As[ty + 16][k], b0 = Bs[tx][k], b1 = Bs[tx + 16][k];
+            acc[0][0] = fma(a0, b0, acc[0][0]);
+            acc[0][1] = fma(a0, b1, acc[0][1]);
+            acc[1][0] = fma(a1, b0, acc[1][0]);
+            acc[1][1] = fma(a1, b1, acc[1][1]);
         }
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                if constexpr (std::is_same<T, float>::value) {   // Kahan step
-                    const float y = acc[a][b] - comp[a][b];
-                    const float t = sum[a][b] + y;
-                    comp[a][b] = (t - sum[a][b]) - y;
-                    sum[a][b] = t;
-                } else {
-                    sum[a][b] += acc[a][b];
-                }
-            }
-        __syncthreads();
     }
-    const double scale = 1.0 / double(f.n - 1);
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const int i = i0 + ty * 4 + a, j = j0 + tx * 4 + b;
-            if (i < p && j < p && i <= j) {
-                const double v = (i == j) ? 1.0 : double(sum[a][b]) * scale;
-                f.sig[size_t(i) * p + j] = v;
-                f.sig[size_t(j) * p + i] = v;
-                f.sig0[size_t(i) * p + j] = v;
-                f.sig0[size_t(j) * p + i] = v;
-            }
+        for (int b = 0; b < 2; ++b) {
+            const int i = ty + 16 * a, j = tx + 16 * b;
+            if (nsplit > 1) partial[(size_t(blockIdx.x) * kGT + i) * kGT + j] = acc[a][b];
+            else gram_store(f, bi * kGT + i, bj * kGT + j, acc[a][b]);
         }
 }
 
-cudaError_t launch_gram(const Fit& f, cudaStream_t st) {
-    const int nt = (f.p + kGT - 1) / kGT;
-    const int grid = nt * (nt + 1) / 2;
-    if (f.precision == LINGAM_MIXED) k_gram<float><<<grid, 256, 0, st>>>(f);
-    else k_gram<double><<<grid, 256, 0, st>>>(f);
+__global__ void __launch_bounds__(256) k_gram_reduce(Fit f, const double* __restrict__ partial, int nt, int nsplit) {
+    int bi, bj;
+    gram_tile(blockIdx.x, nt, bi, bj);
+    const int e = blockIdx.y * 256 + threadIdx.x, i = e / kGT, j = e % kGT;
+    const double* src = partial + size_t(blockIdx.x) * nsplit * kGT * kGT + e;
+    double s = 0.0;
+    int k = 0;
+    for (; k + 8 <= nsplit; k += 8) {   // split order, eight loads in flight
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = src[size_t(k + q) * kGT * kGT];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) s += v[q];
+    }
+    for (; k < nsplit; ++k) s += src[size_t(k) * kGT * kGT];
+    gram_store(f, bi * kGT + i, bj * kGT + j, s);
+}
+
+// (the partial tiles take at most 608 x 8 KB, or nothing: they fit the FP64 path's partial-moment
+// region, at least 64 KB per tile of 32 variables and 32 samples, up to 320 of them)
+cudaError_t launch_gram(const Fit& f, size_t partial_bytes, cudaStream_t st) {
+    const int nt = (f.p + kGT - 1) / kGT, ntri = nt * (nt + 1) / 2;
+    const int room = int(std::min<size_t>(partial_bytes / (size_t(ntri) * kGT * kGT * sizeof(double)), 1 << 20));
+    const int nsplit = std::max(1, std::min(std::min(kGSplitCtas / ntri, f.ld / kGK), room));
+    double* partial = static_cast<double*>(f.partials);
+    k_gram<<<ntri * nsplit, 256, 0, st>>>(f, partial, nt, nsplit);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || nsplit == 1) return e;
+    k_gram_reduce<<<dim3(ntri, kGT * kGT / 256), 256, 0, st>>>(f, partial, nt, nsplit);
     return cudaGetLastError();
 }
 

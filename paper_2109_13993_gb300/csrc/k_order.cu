@@ -1,0 +1,1682 @@
+// k_order.cu -- the ordering loop (Algorithm 3: ParaFindRoot, UpdateData, UpdateCovMat) of one
+// problem, or of many at once, in one persistent cooperative launch.
+//
+// A problem is worked on by a group of CTAs: one lane of control, the group's rank 0 (the
+// "controller"), and the workers (the other CTAs; in groups below kDedicated CTAs rank 0 works
+// too).  A single fit's group is the whole grid; a batch's problems get groups sized by their
+// work, and small ones queue for groups of one.  Groups never wait for each other.
+//
+// Which pairs are compared.  As in the tile kernels, a wave completes up to kMaxCols candidates
+// (the columns) against every variable that was not a column yet (the rows), and the lowest
+// complete score bounds the root's score exactly (threshold, Sec. III-B).  Two things keep the
+// waves few and narrow:
+//   - every variable remembers the partner that contributed most to its score (its killer).  The
+//     first wave of an iteration also compares each row with its killer, which alone nearly
+//     always puts the row's partial score above the bound: one pair instead of a column;
+//   - candidates are taken in the order of their last known score without the contribution of
+//     the variable just removed, so that the children of the removed root come first.
+// Neither changes the root: a partial score is a lower bound of the score whatever pairs it holds.
+// Pairs evaluated, of all pairs: p = 300, n = 5000 graphs with one causal order 83 % -> 5-8 %, the
+// paper's sparse / dense generator at p = 200 51 / 62 % -> 9-13 / 12-16 %, with 1.0-1.4 waves per
+// iteration instead of 1.6-3.2.
+//
+// One hand-over per wave.  The first wave of an iteration removes the previous root on the way:
+// a worker reads the old rows, forms (x_w - Sigma[w,root] x_root) / sqrt(1 - Sigma[w,root]^2) of
+// the rows, columns and killers it needs in registers and shared memory, and writes the rows it
+// owns to the other of two copies; the pair coefficients come from the old covariance the same
+// way, and the covariance downdate itself (Eq. CovUpdate, FP64, upper triangle) goes to its other
+// copy.  So no barrier separates removal and comparison: the workers arrive once per wave, the
+// controller merges, decides and publishes the next wave in one word.
+//
+// Work split of a wave: nseg segments of the sample axis times W / nseg row groups; a worker
+// stages its segment of the columns (and of the root) in shared memory and streams its rows from
+// L2.  A warp takes blocks of samples of one row against four columns (lanes across the
+// samples, coalesced), closes a block with one lg2 per residual and lane, adds the lanes in a
+// fixed tree and the blocks in float-float, so that a sum does not depend on how the blocks were
+// spread over warps and CTAs (beyond 2^-48).
+#include <algorithm>
+#include <queue>
+#include <type_traits>
+#include <utility>
+#include <vector>
+
+#include "common.cuh"
+#include "launch.h"
+#include "pair_math.cuh"
+
+namespace lingam {
+
+constexpr int kMaxCols = 16;     // columns of a wave at most (four quads)
+// Samples of a block: FP32 32 per lane, one lg2 per residual; FP64 8 per lane (a block against four
+// columns then takes about 25 us of a SM's FP64 pipe, so that small fits still spread over the GPU).
+template <class T>
+__host__ __device__ constexpr int blk() { return sizeof(T) == 4 ? 1024 : 256; }
+constexpr int kRowBatch = 32;    // rows of a worker between two CTA barriers
+constexpr int kDedicated = 8;    // groups of this many CTAs or more have a controller that does not work
+
+extern __shared__ __align__(128) unsigned char smem_order[];
+
+template <class T>
+struct OrderTraits;
+template <>
+struct OrderTraits<float> {
+    using V = float4;                      // consecutive samples of a lane
+    using Sum = float2;                    // float-float sum
+    static constexpr int VN = 4;
+};
+template <>
+struct OrderTraits<double> {
+    using V = double2;
+    using Sum = double;
+    static constexpr int VN = 2;
+};
+
+// A row of the current wave (rows 0 .. ncol - 1 are its columns).
+struct __align__(16) RowEnt {
+    int var;       // variable
+    float off;     // its 32-sample log-cosh offset (FP32 path)
+    int kvar;      // its killer (-1: none)
+    float koff;    // the killer's offset
+};
+static_assert(sizeof(RowEnt) == 16, "one 16-byte load");
+
+__device__ __forceinline__ RowEnt load_row(const RowEnt* t) {
+    const int4 v = __ldcg(reinterpret_cast<const int4*>(t));
+    return RowEnt{v.x, __int_as_float(v.y), v.z, __int_as_float(v.w)};
+}
+
+// The wave word: sequence number (bits 51-63), done (50), removal (49), killers (48), columns
+// (42-46), rows (24-41), segments (0-15).
+__device__ __forceinline__ unsigned long long pack_order_wave(unsigned seq, int done, int removal, int kill, int ncol,
+                                                              int nrow, int nseg) {
+    return (static_cast<unsigned long long>(seq & 0x1fffu) << 51) | (static_cast<unsigned long long>(done) << 50) |
+           (static_cast<unsigned long long>(removal) << 49) | (static_cast<unsigned long long>(kill) << 48) |
+           (static_cast<unsigned long long>(ncol) << 42) | (static_cast<unsigned long long>(nrow) << 24) |
+           static_cast<unsigned long long>(nseg);
+}
+struct OrderWave {
+    int done, removal, kill, ncol, nrow, nseg;
+};
+__device__ __forceinline__ OrderWave unpack_order_wave(unsigned long long w) {
+    return {int((w >> 50) & 1), int((w >> 49) & 1), int((w >> 48) & 1), int((w >> 42) & 31), int((w >> 24) & 0x3ffff),
+            int(w & 0xffff)};
+}
+
+// ------------------------------------------------------------------ sums
+__device__ __forceinline__ float2 sum_of(float v) { return make_float2(v, 0.f); }
+__device__ __forceinline__ double sum_of(double v) { return v; }
+__device__ __forceinline__ float2 sum_add(float2 a, float2 b) { return ff_add(a, b); }
+__device__ __forceinline__ double sum_add(double a, double b) { return a + b; }
+__device__ __forceinline__ float sum_val(float2 a) { return a.x + a.y; }
+__device__ __forceinline__ double sum_val(double a) { return a; }
+__device__ __forceinline__ float2 shfl_xor_sum(float2 v, int o) {
+    return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+}
+__device__ __forceinline__ double shfl_xor_sum(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+
+// The 32 lanes' sums of N values (a power of two up to 16), in a fixed tree; lane l ends with the
+// total of value lane_value<N>(l).
+template <int N, class T>
+__device__ __forceinline__ T lane_totals(T (&v)[N]) {
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int h = N / 2; h >= 1; h >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const T keep = up ? v[i + h] : v[i], send = up ? v[i] : v[i + h];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+        o >>= 1;
+    }
+    T s = v[0];
+    for (; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+template <int N>
+__device__ __forceinline__ int lane_value() {
+    const int lane = threadIdx.x & 31;
+    int idx = 0, o = 16;
+#pragma unroll
+    for (int h = N / 2; h >= 1; h >>= 1) {
+        idx += (lane & o) ? h : 0;
+        o >>= 1;
+    }
+    return idx;
+}
+
+// ------------------------------------------------------------------ sample blocks
+__device__ __forceinline__ float4 reduce_root(float4 a, float4 r, float c, float inv) {
+    return make_float4(fmaf(-c, r.x, a.x) * inv, fmaf(-c, r.y, a.y) * inv, fmaf(-c, r.z, a.z) * inv,
+                       fmaf(-c, r.w, a.w) * inv);
+}
+__device__ __forceinline__ double2 reduce_root(double2 a, double2 r, double c, double inv) {
+    return make_double2(fma(-c, r.x, a.x) * inv, fma(-c, r.y, a.y) * inv);
+}
+__device__ __forceinline__ float4 zero_of(float4) { return make_float4(0.f, 0.f, 0.f, 0.f); }
+__device__ __forceinline__ double2 zero_of(double2) { return make_double2(0.0, 0.0); }
+
+// Moments of one residual over a lane's samples of a block.
+struct AccD {
+    double A, P, G;
+};
+template <class T>
+struct AccOf;
+template <>
+struct AccOf<float> {
+    using Acc = Acc2;
+};
+template <>
+struct AccOf<double> {
+    using Acc = AccD;
+};
+__device__ __forceinline__ void acc_start(Acc2& a) { acc_init(a); }
+__device__ __forceinline__ void acc_start(AccD& a) {
+    a.A = 0.0;
+    a.P = 1.0;
+    a.G = 0.0;
+}
+// FP64 exponentials.  DFMA runs at 1.7 lanes a clock and SM on this part, so the operations of an
+// exponential are counted: e^{-c w}, w >= 0, by the table-driven method (Tang, "Table-driven
+// implementation of the exponential function in IEEE floating-point arithmetic", ACM TOMS 1989):
+// c w = -k ln2 / 256 + c r with k the nearest integer (<= 0), e^{-c w} = 2^{k/256} e^{-c r}, the
+// table 2^{j/256} in shared memory and a polynomial of degree 4 in r (|c r| <= ln2 / 512: its error is
+// below 2^-54).  Eight FP64 operations, against about sixty of the library's exp().  The argument is
+// reduced with one constant: an absolute error below 2^-53 c w e^{-c w}, and the terms are summed.
+constexpr int kExpTab = 256;
+__device__ __forceinline__ double exp_neg(double w, const double c, const double* tab) {
+    const double kln2 = 0.69314718055994530942;
+    const double magic = 6755399441055744.0;   // 1.5 2^52: rounds to an integer in the low word
+    const double t = fma(w, -c * (kExpTab / kln2), magic);
+    const int k = __double2loint(t);
+    const double r = fma(t - magic, kln2 / kExpTab / c, w);
+    double h = fma(r, c * c * c * c / 24.0, -c * c * c / 6.0);
+    h = fma(r, h, c * c / 2.0);
+    h = fma(r, h, -c);
+    h = r * h;
+    const double e = tab[k & (kExpTab - 1)];
+    // times 2^(k >> 8) in the exponent field; zero below about e^-700 (c w >= 700)
+    const int big = __double2hiint(w) >= (c > 1.0 ? 0x4075e000 : 0x4095e000);   // 350, 1400
+    const double s = __hiloint2double(big ? 0 : __double2hiint(e) + (k >> 8) * (1 << 20), big ? 0 : __double2loint(e));
+    return fma(s, h, s);
+}
+__device__ __forceinline__ void acc_one(AccD& s, double u, const double* tab) {
+    const double a = fabs(u);
+    s.P = fma(s.P, exp_neg(a, 2.0, tab), s.P);
+    s.A += a;
+    s.G = fma(u, exp_neg(u * u, 0.5, tab), s.G);
+}
+// Both residuals of a pair: s x_i - sr x_j and s x_j - sr x_i.
+__device__ __forceinline__ void acc_pair(Acc2& aa, Acc2& ab, float4 xi, float4 xj, float s, float sr, const double*) {
+    acc_pair4(aa, ab, xi, xj, make_float2(s, s), make_float2(-sr, -sr));
+}
+__device__ __forceinline__ void acc_pair(AccD& aa, AccD& ab, double2 xi, double2 xj, double s, double sr,
+                                         const double* tab) {
+    acc_one(aa, fma(s, xi.x, -sr * xj.x), tab);
+    acc_one(ab, fma(s, xj.x, -sr * xi.x), tab);
+    acc_one(aa, fma(s, xi.y, -sr * xj.y), tab);
+    acc_one(ab, fma(s, xj.y, -sr * xi.y), tab);
+}
+// The variable itself (its own moments).
+__device__ __forceinline__ void acc_self(Acc2& a, float4 x, const double*) {
+    const float2 k = make_float2(kScale, kScale);
+    acc2_add(a, __fmul2_rn(k, make_float2(x.x, x.y)));
+    acc2_add(a, __fmul2_rn(k, make_float2(x.z, x.w)));
+}
+__device__ __forceinline__ void acc_self(AccD& a, double2 x, const double* tab) {
+    acc_one(a, x.x, tab);
+    acc_one(a, x.y, tab);
+}
+// Closes a warp's block: per residual i the lanes' centred log-cosh sum and their sum of u e^{-u^2/2}
+// (FP32: of u' = kScale u), totals 2 i and 2 i + 1 in lane order (lane_value<2 N>).  off is the offset
+// of 32 samples and part the lane's share of them; its low mantissa bits are zero (var_offset), so
+// that the product is exact.  FP32: one lg2 per residual and lane.  FP64: the lanes' products are
+// multiplied first (at most 2^256 for 8 samples a lane) and each log is taken once per warp.
+template <int N>
+__device__ __forceinline__ float close_block(const Acc2 (&a)[N], const float (&off)[N], float part) {
+    float v[2 * N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        v[2 * i] = fmaf(float(kLn2), lg2_approx(a[i].P.x * a[i].P.y), fmaf(a[i].A.x + a[i].A.y, kInvScale / -kC3, off[i] * part));
+        v[2 * i + 1] = a[i].G.x + a[i].G.y;
+    }
+    return lane_totals<2 * N>(v);
+}
+template <int N>
+__device__ __forceinline__ double close_block(const AccD (&a)[N], const double (&off)[N], double part) {
+    double v[2 * N], pr[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        v[2 * i] = fma(off[i], part, a[i].A);
+        v[2 * i + 1] = a[i].G;
+        pr[i] = a[i].P;
+    }
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int h = N / 2; h >= 1; h >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const double keep = up ? pr[i + h] : pr[i], send = up ? pr[i] : pr[i + h];
+            pr[i] = keep * __shfl_xor_sync(0xffffffffu, send, o);
+        }
+        o >>= 1;
+    }
+    const int odd = o;   // this bit of the lane tells a total's kind: 0 the log-cosh sum, else the other
+    double q = pr[0];
+    for (; o > 0; o >>= 1) q *= __shfl_xor_sync(0xffffffffu, q, o);
+    const double lg = log(q);
+    return lane_totals<2 * N>(v) + ((lane & odd) ? 0.0 : lg);
+}
+__device__ __forceinline__ float pair_scale(double om, float) { return kScale / sqrtf(float(om)); }
+__device__ __forceinline__ double pair_scale(double om, double) { return 1.0 / sqrt(om); }
+// The 32-sample offset of the log-cosh sums: the variable's (FP32), beta's (FP64).
+__device__ __forceinline__ float pair_offset(float off, float) { return off; }
+__device__ __forceinline__ double pair_offset(float, double) { return -double(kSub) * (kLn2 + kBeta); }
+
+// One block of one row against four columns: the 16 sums (per pair the row's residual's two, then
+// the column's two) in lane order.  m of the SPB steps of 32 V's; xg the old row at this lane, rs
+// the staged root, cs the staged columns (cstr elements apart), all at this lane's first sample.
+// The row's next two steps are loaded while two are evaluated.
+template <class T, class V>
+__device__ __forceinline__ T quad_block(const V* __restrict__ xg, const V* rs, const T* cs, int cstr, int m, T c, T inv,
+                                        const T* sc, T off_r, const T* offc, T part, const double* tab) {
+    typename AccOf<T>::Acc acc[8];
+    T s[4], sr[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        s[q] = sc[2 * q];
+        sr[q] = sc[2 * q + 1];
+        acc_start(acc[2 * q]);
+        acc_start(acc[2 * q + 1]);
+    }
+    auto step = [&](V a, int k) {
+        const V u = reduce_root(a, rs[32 * k], c, inv);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const V w = *(reinterpret_cast<const V*>(cs + q * cstr) + 32 * k);
+            acc_pair(acc[2 * q], acc[2 * q + 1], u, w, s[q], sr[q], tab);
+        }
+    };
+    V n0 = __ldcg(xg), n1 = n0;
+    if (m > 1) n1 = __ldcg(xg + 32);
+#pragma unroll 1
+    for (int k = 0; k < m; k += 2) {
+        const V a0 = n0, a1 = n1;
+        if (k + 2 < m) n0 = __ldcg(xg + 32 * (k + 2));
+        if (k + 3 < m) n1 = __ldcg(xg + 32 * (k + 3));
+        step(a0, k);
+        if (k + 1 < m) step(a1, k + 1);
+    }
+    T off[8];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        off[2 * q] = off_r;
+        off[2 * q + 1] = offc[q];
+    }
+    return close_block<8>(acc, off, part);
+}
+
+// One block of one row on its own: the row without the root is written to its new copy with its
+// moments, and compared with its killer.  Eight sums: the killer pair's four, the row's two, 0, 0.
+template <class T, class V>
+__device__ __forceinline__ T single_block(const V* __restrict__ xg, const V* __restrict__ kg, const V* rs,
+                                          V* __restrict__ out, int m, T c, T inv, T kc, T kinv, T s, T sr, T off_r,
+                                          T off_k, T part, const double* tab) {
+    typename AccOf<T>::Acc acc[4];   // the row's and the killer's residual, the row, nothing
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc_start(acc[q]);
+    V n0 = __ldcg(xg), n1 = n0, k0 = n0, k1 = n0;
+    if (m > 1) n1 = __ldcg(xg + 32);
+    if (kg) {
+        k0 = __ldcg(kg);
+        if (m > 1) k1 = __ldcg(kg + 32);
+    }
+    auto step = [&](V a, V b, int k) {
+        const V r = rs[32 * k];
+        const V u = reduce_root(a, r, c, inv);
+        out[32 * k] = u;
+        acc_self(acc[2], u, tab);
+        if (kg) acc_pair(acc[0], acc[1], u, reduce_root(b, r, kc, kinv), s, sr, tab);
+    };
+#pragma unroll 1
+    for (int k = 0; k < m; k += 2) {
+        const V a0 = n0, a1 = n1, b0 = k0, b1 = k1;
+        if (k + 2 < m) {
+            n0 = __ldcg(xg + 32 * (k + 2));
+            if (kg) k0 = __ldcg(kg + 32 * (k + 2));
+        }
+        if (k + 3 < m) {
+            n1 = __ldcg(xg + 32 * (k + 3));
+            if (kg) k1 = __ldcg(kg + 32 * (k + 3));
+        }
+        step(a0, b0, k);
+        if (k + 1 < m) step(a1, b1, k + 1);
+    }
+    const T off[4] = {off_r, off_k, off_r, T(0)};
+    return close_block<4>(acc, off, part);
+}
+
+// ------------------------------------------------------------------ the group and its memory
+struct Group {
+    int rank, size;      // this CTA's rank in the group, CTAs of the group
+    int W, wk;           // workers, this CTA's worker index (-1: the controller of a large group)
+    unsigned work;       // offset of the work area in shared memory
+    unsigned cap;        // bytes of the work area
+    unsigned tab;        // offset of the table 2^{j/256} (FP64)
+};
+
+// Controller state per variable slot (shared memory).
+constexpr size_t kSlotBytes = 16 + 8 + 4 * 11;
+// A worker's tables before the staged rows: the batch's rows and the columns, the pairs'
+// coefficients, the warps' sums, and the rows' and columns' coefficients and offsets.
+template <class T>
+__host__ __device__ constexpr size_t order_fixed_bytes(int nw) {
+    return size_t(kRowBatch + kMaxCols) * sizeof(RowEnt) + size_t(kRowBatch) * (kMaxCols + 1) * 2 * sizeof(T) +
+           (size_t(kRowBatch) * (kMaxCols / 4 + 1) + nw) * 16 * 8 +
+           size_t(2 * kRowBatch + kMaxCols) * 3 * sizeof(double) +                       // S[root][v], D, new D
+           (size_t(kRowBatch) * 6 + size_t(kMaxCols) * 4) * sizeof(T);
+}
+// Columns a wave may have with a work area of `cap` bytes and nrow rows: one block of the root and
+// of the columns must fit beside the fixed tables, and the controller's I table (one T per row and
+// column or killer) into ctl_cap bytes.
+template <class T>
+__host__ __device__ inline int order_max_cols(size_t cap, int nw, int nrow, size_t ctl_cap) {
+    for (int c = kMaxCols; c >= 4; c -= 4)
+        if (order_fixed_bytes<T>(nw) + size_t(c + 1) * blk<T>() * sizeof(T) <= cap && size_t(c + 1) * nrow * sizeof(T) <= ctl_cap)
+            return c;
+    return 0;
+}
+__host__ __device__ inline size_t order_state_bytes(int p) { return (size_t(p) * kSlotBytes + 127) / 128 * 128; }
+
+// Estimated SM clocks of a wave with nseg segments of the sample axis.  A worker evaluates its rows'
+// pairs at about 6 pair-samples a clock (FP64: one in 14 clocks), stages its columns at about 40
+// bytes a clock, and the controller reads every segment's sums (32 bytes a pair) at about 30.
+template <class T>
+__device__ __forceinline__ float seg_cost(int nseg, int nrow, int ncol, int W, int nblk, int extra) {
+    constexpr bool f32 = sizeof(T) == 4;
+    const int groups = W / nseg;
+    const int rows = (nrow + groups - 1) / groups, blks = (nblk + nseg - 1) / nseg;
+    const int quads = (ncol + 3) / 4;
+    const float unit = (f32 ? 4.f / 6.f : 4.f * 14.f) * blk<T>();   // a block against four columns, at the SM's rate
+    const float lone = f32 ? 6.f * unit : unit;                    // and by one warp alone
+    const float work = fmaxf(float(rows) * blks * (quads * unit + extra * 0.5f * unit), lone);
+    const float stage = float(blks) * (ncol + 1) * (blk<T>() * sizeof(T) / 40.f);
+    const float merge = float(nseg) * nrow * (ncol + extra) * (32.f / 30.f);
+    return work + stage + merge;
+}
+
+// ------------------------------------------------------------------ a worker's part of a wave
+
+// 1 / sqrt(x) in FP64 from the FP32 value y0 (relative error e0 below 2^-21) by one step of fourth
+// order: with h = 1 - x y0^2, 1/sqrt(1 - h) = 1 + h/2 + 3 h^2/8 + O(h^3), h^3 below 2^-60.
+__device__ __forceinline__ double rsqrt_fast(double x) {
+    const double y = double(rsqrtf(float(x)));
+    const double h = fma(-x, y * y, 1.0);
+    return fma(y * h, fma(h, 0.375, 0.5), y);
+}
+
+// The removal's coefficients of variable v: S the covariance of the un-normalised remaining rows and
+// D their scales (row = residual times D, so Sigma[v][w] = S[v][w] D[v] D[w]); with rho = S[v][root]
+// D[v] D[root], the normalised row loses rho times the root's and is scaled by 1 / sqrt(1 - rho^2).
+struct Removal {
+    double rho, inv;
+};
+
+template <class T, int NT>
+__device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const Group g, const T* __restrict__ xold,
+                                         T* __restrict__ xnew, const double* __restrict__ sold, double* __restrict__ snew,
+                                         const double* __restrict__ dold, double* __restrict__ dnew) {
+    using V = typename OrderTraits<T>::V;
+    using Sum = typename OrderTraits<T>::Sum;
+    constexpr int VN = OrderTraits<T>::VN, NW = NT / 32, STEP = 32 * VN, SPB = blk<T>() / STEP;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int p = f.p, ld = f.ld, nst = ld / STEP, nblk = (nst + SPB - 1) / SPB;
+    const int ncol = wv.ncol, nrow = wv.nrow, nseg = wv.nseg, nq = (ncol + 3) / 4;
+    const bool rm = wv.removal != 0;
+    const int has_k = wv.removal;             // the rows' own blocks (new copy, moments, killer)
+    const int ntypes = nq + has_k, RECN = 16 * nq + 8 * has_k, np = ncol + has_k;
+    const RowEnt* tab = static_cast<const RowEnt*>(f.rowtab);
+    Sum* rec = static_cast<Sum*>(f.rec);
+    // shared memory
+    unsigned char* work = smem_order + g.work;
+    RowEnt* s_row = reinterpret_cast<RowEnt*>(work);
+    RowEnt* s_col = s_row + kRowBatch;
+    T* s_sc = reinterpret_cast<T*>(s_col + kMaxCols);                       // [row][kMaxCols + 1][2]
+    Sum* s_f = reinterpret_cast<Sum*>(s_sc + kRowBatch * (kMaxCols + 1) * 2);
+    // per item (row j: j; its killer: kRowBatch + j; column c: 2 kRowBatch + c): S[root][v], new D
+    double* s_sr = reinterpret_cast<double*>(s_f + (size_t(kRowBatch) * (kMaxCols / 4 + 1) + NW) * 16);
+    double* s_dn = s_sr + 2 * kRowBatch + kMaxCols;
+    T* s_rc = reinterpret_cast<T*>(s_dn + 2 * (2 * kRowBatch + kMaxCols));   // [row][4]: rho, inv, killer's
+    T* s_cc = s_rc + kRowBatch * 4;                                         // [column][2]: rho, inv
+    T* s_offr = s_cc + kMaxCols * 2;                                        // [row][2]: offset, killer's
+    T* s_offc = s_offr + kRowBatch * 2;                                     // [column]
+    T* s_root = reinterpret_cast<T*>(work + order_fixed_bytes<T>(NW));
+    const double* etab = reinterpret_cast<const double*>(smem_order + g.tab);
+    const int bp = min(nblk, int((g.cap - order_fixed_bytes<T>(NW)) / (size_t(4 * nq + 1) * blk<T>() * sizeof(T))));
+    const int cstr = bp * blk<T>();
+    T* s_cols = s_root + cstr;
+
+    const int ngr = g.W / nseg, grp = g.wk / nseg, seg = g.wk - grp * nseg;
+    const int b0 = seg * nblk / nseg, b1 = (seg + 1) * nblk / nseg;
+    const int nr = grp < ngr && grp < nrow ? (nrow - 1 - grp) / ngr + 1 : 0;
+    const int root = rm ? __ldcg(&f.ctl->rm_root) : -1;
+    const double droot = rm ? __ldcg(dold + root) : 0.0;
+    const V* xroot = reinterpret_cast<const V*>(xold + size_t(rm ? root : 0) * ld);
+    for (int bs = b0; bs < b1 && nr > 0; bs += bp) {
+        const int nb = min(bp, b1 - bs);
+        for (int r0 = 0; r0 < nr; r0 += kRowBatch) {
+            const int nrb = min(kRowBatch, nr - r0);
+            if (tid < nrb) {
+                const RowEnt e = load_row(tab + grp + (r0 + tid) * ngr);
+                s_row[tid] = e;
+                s_offr[2 * tid] = pair_offset(e.off, T());
+                s_offr[2 * tid + 1] = pair_offset(e.koff, T());
+            } else if (tid >= 64 && tid < 64 + kMaxCols && r0 == 0 && bs == b0) {
+                const int c = tid - 64;
+                RowEnt e = {-1, 0.f, -1, 0.f};
+                if (c < ncol) e = load_row(tab + c);
+                s_col[c] = e;
+                s_offc[c] = pair_offset(e.off, T());
+            }
+            __syncthreads();   // the tables are there; the previous batch's sums were read
+            // everything that depends on the tables alone is loaded before the coefficients are
+            // formed: this thread's covariance elements and its first samples of root and columns
+            const int base = bs * SPB * 32, nv = min(nb * SPB, nst - bs * SPB) * 32;
+            const bool stage = r0 == 0;
+            V pr = zero_of(V()), px[4];
+            if (stage && tid < nv) {
+                if (rm) pr = __ldcg(xroot + base + tid);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (q < ncol) px[q] = __ldcg(reinterpret_cast<const V*>(xold + size_t(s_col[q].var) * ld) + base + tid);
+            }
+            // the pairs: row j against column c (c == ncol: its killer)
+            constexpr int PU = (kRowBatch * (kMaxCols + 1) + NT - 1) / NT;
+            double pc[PU];
+            int pu[PU];   // the pair's row and item, or -1
+#pragma unroll
+            for (int q = 0; q < PU; ++q) {
+                const int u = tid + q * NT, j = u / np, c = u - j * np, e = grp + (r0 + j) * ngr;
+                pu[q] = -1;
+                if (u < nrb * np) {
+                    const bool kill = c == ncol;
+                    const int vi = s_row[j].var, vj = kill ? s_row[j].kvar : s_col[c].var;
+                    if (vj >= 0 && (kill || (f.reuse ? e >= ncol || c < e : e != c)) &&
+                        LINGAM_INBOUNDS(f.ctl, vi >= 0 && vi < p && vj < p)) {
+                        pu[q] = j | (kill ? kMaxCols : c) << 8;
+                        pc[q] = __ldcg(sold + size_t(min(vi, vj)) * p + max(vi, vj));
+                    }
+                }
+            }
+            // the rows', killers' and columns' removal coefficients (FP64)
+            if (tid < 2 * kRowBatch + kMaxCols) {
+                const int k = tid;
+                int v = -1;
+                if (k < kRowBatch) v = k < nrb ? s_row[k].var : -1;
+                else if (k < 2 * kRowBatch) v = k - kRowBatch < nrb && has_k ? s_row[k - kRowBatch].kvar : -1;
+                else v = s_col[k - 2 * kRowBatch].var;
+                double sr = 0.0, d = 0.0, rho = 0.0, inv = 1.0;
+                if (v >= 0) {
+                    d = __ldcg(dold + v);
+                    if (rm) {
+                        sr = __ldcg(sold + size_t(min(v, root)) * p + max(v, root));
+                        rho = sr * (d * droot);
+                        double om = fma(-rho, rho, 1.0);
+                        if (!(om > degenerate_om(sizeof(T) == 4))) {
+                            set_status(f.ctl, LINGAM_EDEGENERATE);
+                            om = 1.0;
+                        }
+                        inv = rsqrt_fast(om);
+                        d *= inv;
+                        if (k < kRowBatch && bs == 0) dnew[v] = d;   // (one worker per row: the first segment's)
+                    }
+                }
+                s_sr[k] = sr;
+                s_dn[k] = d;
+                T* rc = k < kRowBatch ? s_rc + 4 * k : k < 2 * kRowBatch ? s_rc + 4 * (k - kRowBatch) + 2 : s_cc + 2 * (k - 2 * kRowBatch);
+                rc[0] = T(rho);
+                rc[1] = T(inv);
+            }
+            __syncthreads();
+            const double dr2 = droot * droot;   // 1 / S[root][root]
+#pragma unroll
+            for (int q = 0; q < PU; ++q)
+                if (pu[q] >= 0) {
+                    const int j = pu[q] & 0xff, c = pu[q] >> 8, it = c == kMaxCols ? kRowBatch + j : 2 * kRowBatch + c;
+                    double cv = pc[q];
+                    if (rm) cv = fma(-s_sr[j] * dr2, s_sr[it], cv);
+                    double rho = cv * (s_dn[j] * s_dn[it]);
+                    double om = fma(-rho, rho, 1.0);
+                    constexpr bool f32 = sizeof(T) == 4;
+                    if (!((f32 ? double(float(om)) : om) > (f32 ? double(float(degenerate_om(true))) : degenerate_om(false)))) {
+                        set_status(f.ctl, LINGAM_EDEGENERATE);
+                        rho = 0.0;
+                        om = 1.0;
+                    }
+                    const T s = pair_scale(om, T());
+                    T* sc = s_sc + (j * (kMaxCols + 1) + c) * 2;
+                    sc[0] = s;
+                    sc[1] = s * T(rho);
+                }
+            if (stage) {
+                // the segment of the root and of the columns, without the root
+                for (int t = tid; t < nv; t += NT) {
+                    const bool first = t == tid;
+                    const V r = first ? pr : rm ? __ldcg(xroot + base + t) : zero_of(V());
+                    reinterpret_cast<V*>(s_root)[t] = r;
+#pragma unroll 1
+                    for (int c0 = 0; c0 < ncol; c0 += 4) {
+                        V x[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            if (first && c0 == 0) x[q] = px[q];
+                            else if (c0 + q < ncol)
+                                x[q] = __ldcg(reinterpret_cast<const V*>(xold + size_t(s_col[c0 + q].var) * ld) + base + t);
+                        }
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (c0 + q < ncol)
+                                reinterpret_cast<V*>(s_cols + size_t(c0 + q) * cstr)[t] =
+                                    reduce_root(x[q], r, s_cc[2 * (c0 + q)], s_cc[2 * (c0 + q) + 1]);
+                    }
+                }
+            }
+            __syncthreads();
+            // the blocks of all rows, in the order (row, quad or own, block), spread over the
+            // warps by cost (a quad 4, an own block 2)
+            const int qcost = 4 * nq * nb, rcost = qcost + 2 * has_k * nb, total = nrb * rcost;
+            {
+                const int lo = wid * total / NW, hi = (wid + 1) * total / NW;
+                int j = lo / rcost, u;
+                {
+                    const int rem = lo - j * rcost;
+                    u = rem <= qcost ? (rem + 3) / 4 : nq * nb + (rem - qcost + 1) / 2;
+                    if (u >= ntypes * nb) {
+                        u = 0;
+                        ++j;
+                    }
+                }
+                int gcur = -1;
+                Sum acc = sum_of(T(0));
+                auto flush = [&]() {
+                    if (gcur < 0) return;
+                    const bool own = gcur % ntypes == nq;
+                    const int idx = own ? lane_value<8>() : lane_value<16>();
+                    if ((lane & (own ? 3 : 1)) == 0) s_f[(gcur + wid) * 16 + idx] = acc;
+                };
+                while (j < nrb) {
+                    const int start = j * rcost + (u < nq * nb ? 4 * u : qcost + 2 * (u - nq * nb));
+                    if (start >= hi) break;
+                    const int t = u / nb, b = u - t * nb;
+                    const int gi = j * ntypes + t;
+                    if (gi != gcur) {
+                        flush();
+                        gcur = gi;
+                        acc = sum_of(T(0));
+                    }
+                    const int st0 = (bs + b) * SPB, m = min(SPB, nst - st0);
+                    const T part = T(m) * T(1.0 / (SPB == 8 ? 8 : 16));   // of 32 samples a lane
+                    const RowEnt ri = s_row[j];
+                    const T c = s_rc[4 * j], inv = s_rc[4 * j + 1], off_r = s_offr[2 * j];
+                    const V* xg = reinterpret_cast<const V*>(xold + size_t(ri.var) * ld) + st0 * 32 + lane;
+                    const V* rs = reinterpret_cast<const V*>(s_root) + b * SPB * 32 + lane;
+                    T tot;
+                    if (t < nq) {
+                        const T* cs = s_cols + (4 * t) * cstr + (b * SPB * 32 + lane) * VN;
+                        tot = quad_block<T, V>(xg, rs, cs, cstr, m, c, inv, s_sc + (j * (kMaxCols + 1) + 4 * t) * 2,
+                                                    off_r, s_offc + 4 * t, part, etab);
+                    } else {
+                        const V* kg = ri.kvar >= 0
+                                          ? reinterpret_cast<const V*>(xold + size_t(ri.kvar) * ld) + st0 * 32 + lane
+                                          : nullptr;
+                        V* out = reinterpret_cast<V*>(xnew + size_t(ri.var) * ld) + st0 * 32 + lane;
+                        const T* sk = s_sc + (j * (kMaxCols + 1) + kMaxCols) * 2;
+                        tot = single_block<T, V>(xg, kg, rs, out, m, c, inv, s_rc[4 * j + 2], s_rc[4 * j + 3], sk[0],
+                                                      sk[1], off_r, s_offr[2 * j + 1], part, etab);
+                    }
+                    acc = sum_add(acc, sum_of(tot));
+                    if (++u == ntypes * nb) {
+                        u = 0;
+                        ++j;
+                    }
+                }
+                flush();
+            }
+            __syncthreads();
+            // the warps' sums of each (row, quad or own) in warp order, to the wave's records
+            for (int x = tid; x < nrb * RECN; x += NT) {
+                const int j = x / RECN, v = x - j * RECN;
+                const int t = min(v >> 4, nq), val = v - 16 * t;
+                const int step = t < nq ? 4 : 2;
+                const int s0 = j * rcost + (t < nq ? 4 * t * nb : qcost), s1 = s0 + step * (nb - 1);
+                const int w0 = ((s0 + 1) * NW + total - 1) / total - 1, w1 = ((s1 + 1) * NW + total - 1) / total - 1;
+                const int gi = j * ntypes + t;
+                Sum s = s_f[(gi + w0) * 16 + val];
+                for (int w = w0 + 1; w <= w1; ++w) {
+                    // (a warp whose share of the costs holds no block's start has no sum)
+                    const int lo = w * total / NW, hi = (w + 1) * total / NW;
+                    const int first = s0 + (lo - s0 + step - 1) / step * step;
+                    if (first < hi) s = sum_add(s, s_f[(gi + w) * 16 + val]);
+                }
+                const int e = grp + (r0 + j) * ngr;
+                const size_t at = (size_t(seg) * nrow + e) * RECN + v;
+                if (LINGAM_INBOUNDS(f.ctl, (at + 1) * sizeof(Sum) <= f.rec_bytes))
+                    rec[at] = bs == b0 ? s : sum_add(rec[at], s);
+            }
+        }
+    }
+    // UpdateCovMat (Eq. CovUpdate) on S, FP64, upper triangle by variable index, into the other copy:
+    // S[w][j] - S[w][root] S[j][root] / S[root][root] for this worker's rows w of the remaining
+    // variables and every j > w (of a removed j the element is never read again).  Eight elements of a
+    // thread in flight.
+    if (rm) {
+        const double dr2 = droot * droot;
+        const int mine = g.wk < nrow ? (nrow - 1 - g.wk) / g.W + 1 : 0;
+        constexpr int CB = 8;
+        for (int i0 = 0; i0 < mine * p; i0 += CB * NT) {
+            int at_w[CB], at_j[CB];
+#pragma unroll
+            for (int q = 0; q < CB; ++q) {
+                const int i = i0 + q * NT + tid, row = i / p;
+                at_j[q] = i - row * p;
+                at_w[q] = row < mine ? __ldcg(&tab[g.wk + row * g.W].var) : p;
+            }
+            double a[CB], b[CB], c[CB];
+#pragma unroll
+            for (int q = 0; q < CB; ++q) {
+                const int w = at_w[q], j = at_j[q];
+                if (j > w) {
+                    a[q] = __ldcg(sold + size_t(w) * p + j);
+                    b[q] = __ldcg(sold + size_t(min(w, root)) * p + max(w, root));
+                    c[q] = __ldcg(sold + size_t(min(j, root)) * p + max(j, root));
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < CB; ++q)
+                if (at_j[q] > at_w[q]) snew[size_t(at_w[q]) * p + at_j[q]] = fma(-b[q] * dr2, c[q], a[q]);
+        }
+    }
+}
+
+// ------------------------------------------------------------------ the controller
+// Scores: float-float sums of FP32 contributions, or FP64.
+__device__ __forceinline__ double score_out(float2 a) { return double(a.x) + double(a.y); }
+__device__ __forceinline__ double score_out(double a) { return a; }
+__device__ __forceinline__ float score_float(float2 a) { return a.x; }
+__device__ __forceinline__ float score_float(double a) { return float(a); }
+// Scores are >= 0 (or +inf): 64-bit integers in their order.
+__device__ __forceinline__ long long score_key(float2 a) {
+    const unsigned lo = __float_as_uint(a.y);
+    const unsigned l = (lo & 0x80000000u) ? ~lo : (lo | 0x80000000u);
+    return static_cast<long long>((static_cast<unsigned long long>(__float_as_uint(a.x)) << 32) | l);
+}
+__device__ __forceinline__ long long score_key(double a) { return __double_as_longlong(a); }
+constexpr long long kMaxScore = 0x7fffffffffffffffll;
+__device__ __forceinline__ float2 score_of_key(long long k, float2) {
+    const unsigned l = unsigned(static_cast<unsigned long long>(k) & 0xffffffffu);
+    return make_float2(__uint_as_float(unsigned(static_cast<unsigned long long>(k) >> 32)),
+                       __uint_as_float((l & 0x80000000u) ? (l & 0x7fffffffu) : ~l));
+}
+__device__ __forceinline__ double score_of_key(long long k, double) { return __longlong_as_double(k); }
+// Adds the square of a contribution.
+__device__ __forceinline__ void add_square(float2& s, float m) {
+    FF t;
+    t.hi = s.x;
+    t.lo = s.y;
+    t.add_sq(m);
+    s = make_float2(t.hi, t.lo);
+}
+__device__ __forceinline__ void add_square(double& s, double m) { s = fma(m, m, s); }
+
+// Order-preserving bits of a float.
+__device__ __forceinline__ unsigned key_bits(float x) {
+    const unsigned b = __float_as_uint(x);
+    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+constexpr unsigned kNoKey = 0xffffffffu;
+
+struct OrderShared {
+    unsigned long long word;
+    int ok, nseg, npick, root;
+    int qnext;
+    long long col[kMaxCols];      // the wave's complete scores (keys)
+    unsigned ckey[16 * kMaxCols];
+    int cslot[16 * kMaxCols];
+    int pick[kMaxCols];
+    long long lred[16];
+    int ired[16], nkill[16];
+    long long rootpt;
+};
+
+// Four sums of one record, and their sum over the segments first, first + step, ... (four segments'
+// loads in flight).
+__device__ __forceinline__ void load4(float2 (&v)[4], const float2* p) {
+    const float4 a = __ldcg(reinterpret_cast<const float4*>(p)), b = __ldcg(reinterpret_cast<const float4*>(p) + 1);
+    v[0] = make_float2(a.x, a.y);
+    v[1] = make_float2(a.z, a.w);
+    v[2] = make_float2(b.x, b.y);
+    v[3] = make_float2(b.z, b.w);
+}
+__device__ __forceinline__ void load4(double (&v)[4], const double* p) {
+    const double2 a = __ldcg(reinterpret_cast<const double2*>(p)), b = __ldcg(reinterpret_cast<const double2*>(p) + 1);
+    v[0] = a.x;
+    v[1] = a.y;
+    v[2] = b.x;
+    v[3] = b.y;
+}
+template <class Sum>
+__device__ __forceinline__ void sum_segments(Sum (&s)[4], const Sum* p, size_t stride, int nseg, int first, int step) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] = Sum();
+    int i = first;
+    for (; i + 3 * step < nseg; i += 4 * step) {
+        Sum v[4][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) load4(v[q], p + size_t(i + q * step) * stride);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) s[k] = sum_add(s[k], v[q][k]);
+    }
+    for (; i < nseg; i += step) {
+        Sum v[4];
+        load4(v, p + size_t(i) * stride);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s[k] = sum_add(s[k], v[k]);
+    }
+}
+
+// The 32-sample offset of a variable from its 2 (m - beta).
+__device__ __forceinline__ float stat_offset(float y) {
+    return var_offset(-float(kSub) * (float(kLn2 + kBeta) + 0.5f * y));
+}
+
+// Slots 0 .. r - 1 hold the remaining variables: first those that were columns in this iteration's
+// earlier waves (a of them), then the current wave's columns, then the others; so the current
+// wave's rows are the slots a .. r - 1.  Every thread holds the same r, a, it, best, ...
+template <class T, int NT>
+struct Controller {
+    using Sum = typename OrderTraits<T>::Sum;
+    static constexpr bool f32 = std::is_same<T, float>::value;
+    static constexpr int NW = NT / 32;
+    const Fit& f;
+    const Group& g;
+    OrderShared& sh;
+    // per slot
+    float4* st;       // {corr, 2 (m - beta), g, offset} (FP32), or {H(x) - H(nu)} as a double (FP64)
+    Sum* part;        // score so far; complete for columns
+    float* kc;        // the killer pair's contribution of this iteration
+    float* kv0;       // the two largest known contributions, and their partners
+    float* kv1;
+    float* key;       // the next iteration's candidate order
+    int* keval;       // the killer that was compared (-1: none)
+    int* kp0;
+    int* kp1;
+    int* var;
+    int* slot;        // slot of each variable
+    int* fl;          // kNoRoot
+    int* row;         // candidate keys of a selection
+    T* I;             // the wave's pair measures
+    size_t icap;
+    int r, a, it, iters, cmax, want;
+    bool gmode, prunes;
+    long long best;   // key of the iteration's lowest complete score
+    int bestv;
+    long long pairs;
+    double gamma;
+
+    __device__ __forceinline__ Controller(const Fit& f_, const Group& g_, OrderShared& sh_, size_t smem_bytes, int iters_)
+        : f(f_), g(g_), sh(sh_) {
+        const int p = f.p;
+        st = reinterpret_cast<float4*>(smem_order);
+        part = reinterpret_cast<Sum*>(st + p);
+        kc = reinterpret_cast<float*>(part + p);
+        kv0 = kc + p;
+        kv1 = kv0 + p;
+        key = kv1 + p;
+        keval = reinterpret_cast<int*>(key + p);
+        kp0 = keval + p;
+        kp1 = kp0 + p;
+        var = kp1 + p;
+        slot = var + p;
+        fl = slot + p;
+        row = fl + p;
+        const size_t state = order_state_bytes(p);
+        I = reinterpret_cast<T*>(smem_order + state);
+        icap = smem_bytes - state;
+        iters = iters_;
+        prunes = f.prune && f.reuse;
+        gmode = f.gamma0 > 0.0 && prunes;
+        want = kMaxCols;
+        cmax = order_max_cols<T>(g.cap, NW, p, icap);
+        r = p;
+        a = it = 0;
+        new_iteration();
+    }
+    __device__ __forceinline__ void new_iteration() {
+        best = kMaxScore;
+        bestv = -1;
+        pairs = 0;
+        gamma = f.gamma0;
+    }
+
+    // The slot of a wave's row (without pair reuse the rows are all variables, the columns first).
+    __device__ __forceinline__ int row_slot(int e) const { return a + e < r ? a + e : a + e - r; }
+    // Exchanges two slots (one warp; a lane per array).
+    __device__ __forceinline__ void swap_slots(int x, int y) {
+        if (x == y) return;
+        const int lane = threadIdx.x & 31;
+        const int vx = var[x], vy = var[y];
+        __syncwarp();
+        if (lane == 0) {
+            const float4 t = st[x];
+            st[x] = st[y];
+            st[y] = t;
+        } else if (lane == 1) {
+            const Sum t = part[x];
+            part[x] = part[y];
+            part[y] = t;
+        } else if (lane < 11) {   // the 4-byte arrays kc .. var but slot, and fl, lie one after another
+            int* q = reinterpret_cast<int*>(kc) + size_t(lane < 10 ? lane - 2 : 9) * f.p;
+            const int t = q[x];
+            q[x] = q[y];
+            q[y] = t;
+        } else if (lane == 11) {
+            slot[vx] = y;
+        } else if (lane == 12) {
+            slot[vy] = x;
+        }
+        __syncwarp();
+    }
+
+    // The `n` slots of [lo, hi) of lowest key (row[k]: the key's bits, kNoKey not a candidate), lowest
+    // first, to the positions lo, lo + 1, ...; sh.npick of them.  Each warp takes its lowest by warp
+    // minima, the first warp the lowest of those.  All threads.
+    __device__ __forceinline__ void select_lowest(int lo, int hi, int n) {
+        const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+        __syncthreads();
+        for (int i = 0; i < n; ++i) {
+            unsigned b = kNoKey;
+            int at = -1;
+            for (int k = lo + tid; k < hi; k += NT) {
+                const unsigned v = unsigned(row[k]);
+                if (v < b) {
+                    b = v;
+                    at = k;
+                }
+            }
+            const unsigned m = __reduce_min_sync(0xffffffffu, b);
+            if (m == kNoKey) {
+                for (int q = i + lane; q < n; q += 32) sh.ckey[wid * kMaxCols + q] = kNoKey;
+                break;
+            }
+            const int src = __ffs(__ballot_sync(0xffffffffu, b == m)) - 1;
+            if (lane == src) {
+                row[at] = int(kNoKey);
+                sh.ckey[wid * kMaxCols + i] = m;
+                sh.cslot[wid * kMaxCols + i] = var[at];
+            }
+            __syncwarp();
+        }
+        __syncthreads();
+        if (wid == 0) {
+            int pos = 0, got = 0;
+            for (; got < n; ++got) {   // lane w walks the ascending list of warp w
+                const unsigned v = lane < NW && pos < n ? sh.ckey[lane * kMaxCols + pos] : kNoKey;
+                const unsigned m = __reduce_min_sync(0xffffffffu, v);
+                if (m == kNoKey) break;
+                const int src = __ffs(__ballot_sync(0xffffffffu, v == m)) - 1;
+                int c = lane == src ? sh.cslot[lane * kMaxCols + pos] : 0;
+                if (lane == src) ++pos;
+                c = __shfl_sync(0xffffffffu, c, src);
+                swap_slots(lo + got, slot[c]);
+            }
+            if (lane == 0) sh.npick = got;
+        }
+        __syncthreads();
+    }
+
+    // The wave's rows (and the segments, by the last warp).
+    __device__ __forceinline__ void write_wave(bool removal, bool kill, int ncol, OrderWave& wv) {
+        const int tid = threadIdx.x, nrow = f.reuse ? r - a : r;
+        RowEnt* tab = static_cast<RowEnt*>(f.rowtab);
+        if (tid < NT - 32) {
+            for (int i = tid; i < nrow; i += NT - 32) {
+                const int k = row_slot(i);
+                RowEnt e = {var[k], st[k].w, -1, 0.f};
+                if (kill) {
+                    int kv = -1;
+                    if (k >= ncol && !(fl[k] & kNoRoot) && kv0[k] > 0.f) {
+                        kv = kp0[k];
+                        if (kv >= 0 && slot[kv] < ncol) kv = -1;   // a column: compared anyway
+                    }
+                    keval[k] = kv;
+                    if (kv >= 0) {
+                        e.kvar = kv;
+                        e.koff = st[slot[kv]].w;
+                    }
+                } else if (a == 0) {
+                    keval[k] = -1;
+                }
+                if (a == 0) kc[k] = 0.f;
+                if (LINGAM_INBOUNDS(f.ctl, i < f.p && e.var < f.p)) tab[i] = e;
+            }
+        } else {
+            const int lane = tid & 31, has_k = removal ? 1 : 0;
+            const int nblk = (f.ld + blk<T>() - 1) / blk<T>();
+            const unsigned recb = (16 * ((ncol + 3) / 4) + 8 * has_k) * 8u * unsigned(nrow);
+            const int room = int(min(f.rec_bytes, 0xffffffffull)) < 0 ? int(0xffffffffu / recb) : int(unsigned(f.rec_bytes) / recb);
+            int most = min(min(nblk, g.W), room);
+            if (f.split_n > 0) most = min(most, f.split_n);
+            float b = INFINITY;
+            int at = 1;
+            for (int n = 1 + lane; n <= most; n += 32) {
+                const float c = seg_cost<T>(n, nrow, ncol, g.W, nblk, has_k);
+                if (c < b) {
+                    b = c;
+                    at = n;
+                }
+            }
+            const unsigned m = __reduce_min_sync(0xffffffffu, __float_as_uint(b));
+            at = __reduce_min_sync(0xffffffffu, __float_as_uint(b) == m ? at : 0x7fffffff);
+            if (lane == 0) sh.nseg = at;
+        }
+        __syncthreads();
+        wv = OrderWave{0, removal ? 1 : 0, kill ? 1 : 0, ncol, nrow, sh.nseg};
+    }
+
+    // Iteration 0: every variable, most non-Gaussian first, nothing known of the pairs.
+    __device__ __forceinline__ bool start() {
+        for (int v = threadIdx.x; v < f.p; v += NT) {
+            var[v] = v;
+            slot[v] = v;
+            part[v] = Sum();
+            kc[v] = kv0[v] = kv1[v] = 0.f;
+            keval[v] = kp0[v] = kp1[v] = -1;
+            fl[v] = f.prior && __ldcg(f.anc_cnt + v) > 0 ? kNoRoot : 0;
+            const double h = __ldcg(f.hx + v);
+            if constexpr (f32) {
+                st[v] = __ldcg(f.vstat + v);
+            } else {
+                st[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+                *reinterpret_cast<double*>(&st[v]) = h;
+            }
+            key[v] = float(h);
+            f.dscale[0][v] = 1.0;
+        }
+        __syncthreads();
+        if (r > 1) return true;
+        last_variable();
+        return false;
+    }
+
+    // Algorithm 2: a single remaining variable is the root.
+    __device__ __forceinline__ void last_variable() {
+        if (threadIdx.x == 0) {
+            f.order[it] = var[0];
+            f.rep_root_score[it] = 0.0;
+            f.rep_margin[it] = INFINITY;
+            f.rep_pairs[it] = 0;
+        }
+        if (f.want_scores)
+            for (int v = threadIdx.x; v < f.p; v += NT) f.rep_scores[size_t(it) * f.p + v] = v == var[0] ? 0.0 : NAN;
+    }
+
+    // The first wave of iteration it: columns of lowest key, killers of the others.
+    __device__ __forceinline__ void plan(bool removal, OrderWave& wv) {
+        if (f.want_scores)
+            for (int v = threadIdx.x; v < f.p; v += NT) f.rep_scores[size_t(it) * f.p + v] = NAN;
+        for (int k = threadIdx.x; k < r; k += NT) row[k] = int((fl[k] & kNoRoot) ? kNoKey : key_bits(key[k]));
+        int c = min(want, cmax);
+        if (r - c <= 2 && r <= cmax) c = r;   // one or two rows left over: columns as well
+        select_lowest(0, r, min(c, r));
+        write_wave(removal, removal && prunes && !gmode, sh.npick, wv);
+    }
+
+    // The score so far, or more where the killer's pair is not part of it yet.
+    __device__ __forceinline__ Sum lower_bound(int k, int an) const {
+        Sum lb = part[k];
+        const int ke = keval[k];
+        if (ke >= 0 && slot[ke] >= an) lb = sum_add(lb, sum_of(T(kc[k])));
+        return lb;
+    }
+
+    // One pair's measure from its four sums: row slot k against slot j.
+    __device__ __forceinline__ T measure(const Sum (&v)[4], int k, int j) const {
+        T x;
+        if constexpr (f32) {
+            x = pair_measure_f(sum_val(v[0]), sum_val(v[1]), sum_val(v[2]), sum_val(v[3]), st[k], st[j], __frcp_rn(float(f.n)));
+        } else {
+            const double pad = double(f.ld - f.n) * kBeta;
+            const double ha = hterm_inv(v[0] + pad, v[1], f.inv_n), hb = hterm_inv(v[2] + pad, v[3], f.inv_n);
+            x = (*reinterpret_cast<const double*>(&st[j]) - *reinterpret_cast<const double*>(&st[k])) + (ha - hb);
+        }
+        if (!isfinite(x)) set_status(f.ctl, LINGAM_EDEGENERATE);
+        return x;
+    }
+
+    // After a wave: scores, threshold, and the next wave (or the root and the next iteration's
+    // first wave).  wv: the wave, then the next one (done: the fit is over).
+    __device__ __forceinline__ void finish_wave(OrderWave& wv) {
+        const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+        const int ncol = wv.ncol, nrow = wv.nrow, nseg = wv.nseg, nq = (ncol + 3) / 4, has_k = wv.removal;
+        const int RECN = 16 * nq + 8 * has_k, np = ncol + has_k;
+        const Sum* rec = static_cast<const Sum*>(f.rec);
+        const size_t stride = size_t(nrow) * RECN;
+        const int split = nseg >= 8 ? 8 : 1;   // lanes of one sum over the segments
+        const int sl = tid & (split - 1);
+        // 1. the sums of this thread's first pair are loaded while the rows' own statistics (removal:
+        //    of the new rows) are formed.  Pairs: row e against column c, and its killer (c = ncol)
+        const int units = nrow * np;
+        auto pair_of_unit = [&](int u, int& e, int& c, int& kj) {
+            e = u / np;
+            c = u - e * np;
+            kj = -1;
+            if (u >= units) return;
+            if (c < ncol) {
+                if (f.reuse ? e >= ncol || c < e : e != c) kj = a + c;
+            } else {
+                const int kv = keval[a + e];
+                if (kv >= 0) kj = slot[kv];
+            }
+        };
+        int e0, c0, kj0;
+        pair_of_unit(tid / split, e0, c0, kj0);
+        Sum v0[4] = {Sum(), Sum(), Sum(), Sum()};
+        if (kj0 >= 0) sum_segments<Sum>(v0, rec + size_t(e0) * RECN + (c0 < ncol ? 4 * c0 : 16 * nq), stride, nseg, sl, split);
+        if (has_k) {
+            for (int u0 = 0; u0 < nrow * split; u0 += NT) {
+                const int e = (u0 + tid) / split;
+                Sum v[4] = {Sum(), Sum(), Sum(), Sum()};
+                if (e < nrow) sum_segments<Sum>(v, rec + size_t(e) * RECN + 16 * nq + 4, stride, nseg, sl, split);
+                for (int o = split >> 1; o > 0; o >>= 1) {
+                    v[0] = sum_add(v[0], shfl_xor_sum(v[0], o));
+                    v[1] = sum_add(v[1], shfl_xor_sum(v[1], o));
+                }
+                if (e < nrow && sl == 0) {
+                    const int k = a + e;
+                    if constexpr (f32) {
+                        // T is centred by the old offset -32 (ln 2 + m0) over the padded row
+                        const float inv_n = __frcp_rn(float(f.n));
+                        const float Ts = sum_val(v[0]), off = st[k].w;
+                        const float m0 = -off * (1.f / kSub) - float(kLn2);
+                        const float y = 2.f * ((m0 - float(kBeta)) + fmaf(float(f.ld - f.n), m0, Ts) * inv_n);
+                        st[k] = make_float4(-Ts * inv_n, y, sum_val(v[1]) * (kInvScale * inv_n), off);
+                    } else {
+                        *reinterpret_cast<double*>(&st[k]) =
+                            hterm_inv(sum_val(v[0]) + double(f.ld - f.n) * kBeta, sum_val(v[1]), f.inv_n);
+                    }
+                }
+            }
+            __syncthreads();
+        }
+        // 2. I of every pair
+        for (int u0 = 0; u0 < units * split; u0 += NT) {
+            int e = e0, c = c0, kj = kj0;
+            const int u = (u0 + tid) / split;
+            if (u0 > 0) {
+                pair_of_unit(u, e, c, kj);
+                if (kj >= 0)
+                    sum_segments<Sum>(v0, rec + size_t(e) * RECN + (c < ncol ? 4 * c : 16 * nq), stride, nseg, sl, split);
+            }
+            for (int o = split >> 1; o > 0; o >>= 1) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v0[k] = sum_add(v0[k], shfl_xor_sum(v0[k], o));
+            }
+            if (u < units && sl == 0) I[u] = kj >= 0 ? measure(v0, row_slot(e), kj) : T(0);
+        }
+        __syncthreads();
+        // 3. rows: contributions min(0, I)^2 of the columns, of the killer, and the killers to come
+        int nk = 0;   // pairs besides the columns' (distinct ones: a pair may be both's killer, and a
+                      // later wave may compare a killer pair again)
+        for (int e = tid; e < nrow && f.reuse; e += NT) {
+            const int k = a + e, ke = keval[k];
+            if (ke >= 0) {
+                const int sk = slot[ke];
+                if (keval[sk] != var[k] || var[k] < ke)
+                    nk += has_k ? 1 : (sk >= a && (k < a + ncol || sk < a + ncol)) ? -1 : 0;
+            }
+            const T* Ir = I + e * np;
+            const int cm = min(e, ncol);
+            Sum acc = Sum();
+            float top = 0.f;
+            int topc = -1;
+            int p0 = kp0[k], p1 = kp1[k];
+            float w0 = kv0[k], w1 = kv1[k];
+            if (has_k && ke >= 0) {
+                const float m = fminf(float(Ir[ncol]), 0.f);
+                w0 = m * m;   // keval is kp0
+                kc[k] = w0;
+            }
+            for (int c = 0; c < cm; ++c) {
+                const T m = Ir[c] < T(0) ? Ir[c] : T(0);
+                add_square(acc, m);
+                const float ctr = float(m) * float(m);
+                const int vc = var[a + c];
+                if (vc == p0) {
+                    w0 = ctr;
+                } else if (vc == p1) {
+                    w1 = ctr;
+                } else if (ctr > top) {
+                    top = ctr;
+                    topc = vc;
+                }
+            }
+            if (w1 > w0) {
+                const float tv = w0;
+                w0 = w1;
+                w1 = tv;
+                const int tp = p0;
+                p0 = p1;
+                p1 = tp;
+            }
+            if (top > w0) {
+                w1 = w0;
+                p1 = p0;
+                w0 = top;
+                p0 = topc;
+            } else if (top > w1) {
+                w1 = top;
+                p1 = topc;
+            }
+            kp0[k] = p0;
+            kp1[k] = p1;
+            kv0[k] = w0;
+            kv1[k] = w1;
+            part[k] = sum_add(part[k], acc);
+        }
+        nk = __reduce_add_sync(0xffffffffu, nk);
+        if (lane == 0) sh.nkill[wid] = nk;
+        __syncthreads();
+        // 4. columns: max(0, I)^2 over the rows below them, a warp per column
+        for (int c = wid; c < ncol; c += NW) {
+            Sum acc = Sum();
+            unsigned top = 0;
+            int tope = -1;
+            for (int e = (f.reuse ? c + 1 : 0) + lane; e < nrow; e += 32) {
+                const T x = I[e * np + c];   // (0 for the column itself)
+                const T m = x > T(0) ? x : T(0);
+                add_square(acc, m);
+                const float ctr = float(m) * float(m);
+                if (__float_as_uint(ctr) > top) {
+                    top = __float_as_uint(ctr);
+                    tope = e;
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc = sum_add(acc, shfl_xor_sum(acc, o));
+            const unsigned m = __reduce_max_sync(0xffffffffu, top);
+            const unsigned who = __ballot_sync(0xffffffffu, top == m && tope >= 0);
+            if (lane == (who ? __ffs(who) - 1 : 0)) {
+                const int k = a + c;
+                const Sum sc = sum_add(part[k], acc);
+                part[k] = sc;
+                sh.col[c] = score_key(sc);
+                if (f.want_scores) f.rep_scores[size_t(it) * f.p + var[k]] = score_out(sc);
+                const float tv = __uint_as_float(m);
+                if (who && tv > kv0[k]) {
+                    const int v = var[row_slot(tope)];
+                    if (v != kp0[k]) {
+                        kp1[k] = kp0[k];
+                        kv1[k] = kv0[k];
+                        kp0[k] = v;
+                    }
+                    kv0[k] = tv;
+                }
+            }
+        }
+        __syncthreads();
+        // 5. lowest complete score of the iteration (lowest variable index on ties); every thread
+        for (int c = 0; c < ncol; ++c) {
+            const long long kk = sh.col[c];
+            const int vc = var[a + c];
+            if (bestv < 0 || kk < best || (kk == best && vc < bestv)) {
+                best = kk;
+                bestv = vc;
+            }
+        }
+        pairs += f.reuse ? (long long)ncol * (ncol - 1) / 2 + (long long)ncol * (nrow - ncol) : (long long)ncol * (nrow - 1);
+        for (int w = 0; w < NW; ++w) pairs += sh.nkill[w];
+        ++waves;
+        const int an = a + ncol;   // columned so far
+        // 6. threshold: the live candidates of the others
+        int live;
+        for (int pass = 0;; ++pass) {
+            const long long thr = gmode ? score_key(sum_from(gamma)) : best;
+            int n = 0;
+            for (int k = an + tid; k < r; k += NT) {
+                const Sum lb = gmode ? part[k] : lower_bound(k, an);
+                const bool on = !(fl[k] & kNoRoot) && !(prunes && score_key(lb) > thr);
+                n += on ? 1 : 0;
+                row[k] = int(on ? key_bits(score_float(lb)) : kNoKey);
+            }
+            live = __syncthreads_or(n);
+            // the paper's schedule: nothing can go on and nothing finished at or below gamma: raise
+            // gamma by factors gamma_c until the lowest score that may be the root's is at or below it
+            if (!gmode || live || best <= thr || pass > 0) break;
+            long long km = best;
+            for (int k = an + tid; k < r; k += NT)
+                if (!(fl[k] & kNoRoot)) km = min(km, score_key(part[k]));
+            km = block_min(km);
+            const double target = score_out(score_of_key(km, Sum()));
+            int n2 = 0;
+            while (gamma < target && n2 < 4096) {   // gamma_c > 1 and target finite: a few steps
+                gamma *= f.gamma_c;
+                ++n2;
+            }
+            if (!(score_key(sum_from(gamma)) >= km)) gamma = target;
+            gsteps += n2;
+        }
+        if (live) {
+            a = an;
+            cmax = order_max_cols<T>(g.cap, NW, f.reuse ? r - a : r, icap);
+            select_lowest(a, r, min(cmax, r - a));
+            write_wave(false, false, sh.npick, wv);
+            return;
+        }
+        // 7. the root, its margin, and the next iteration's candidate order
+        const int root = f.has_forced ? f.forced[it] : bestv;
+        const int rs = slot[root];
+        long long second = kMaxScore;
+        int need = 0;
+        for (int k = tid; k < r; k += NT) {
+            const Sum lb = k < an ? part[k] : lower_bound(k, an);
+            const int v = var[k];
+            if (v != bestv && !(fl[k] & kNoRoot)) second = min(second, score_key(lb));
+            // a column whose strongest pair alone would not have excluded it
+            if (k < an && score_key(sum_of(T(kv0[k]))) <= best) ++need;
+            // without the root's contribution, where this iteration's last wave compared the two
+            float ctr = 0.f;
+            if (rs >= a && rs < an && k >= a && k != rs) {
+                const int c = rs - a, e = k - a;
+                const float x = e > c ? fminf(float(I[e * np + c]), 0.f) : fmaxf(float(I[c * np + e]), 0.f);
+                ctr = x * x;
+            } else if (rs >= an && keval[k] == root) {
+                ctr = kc[k];
+            }
+            key[k] = fmaxf(score_float(lb) - ctr, 0.f);
+            if (k == rs) sh.rootpt = score_key(part[k]);
+            if (kp0[k] == root) {
+                kp0[k] = kp1[k];
+                kv0[k] = kv1[k];
+                kp1[k] = -1;
+                kv1[k] = 0.f;
+            } else if (kp1[k] == root) {
+                kp1[k] = -1;
+                kv1[k] = 0.f;
+            }
+            if (f.prior && f.prior[size_t(v) * f.p + root] == 1) {   // root was a known ancestor
+                const int left = f.anc_cnt[v] - 1;
+                f.anc_cnt[v] = left;
+                if (left == 0) fl[k] &= ~kNoRoot;
+            }
+            if constexpr (f32) st[k].w = stat_offset(st[k].y);
+            if (k >= an) part[k] = Sum();   // (the columns' are read below)
+        }
+        {
+            // the lowest other score and the count, one barrier for both
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) second = min(second, __shfl_xor_sync(0xffffffffu, second, o));
+            need = __reduce_add_sync(0xffffffffu, need);
+            if (lane == 0) {
+                sh.lred[wid] = second;
+                sh.ired[wid] = need;
+            }
+            __syncthreads();
+            need = 0;
+            for (int w = 0; w < NW; ++w) need += sh.ired[w];
+            for (int k = tid; k < an; k += NT) part[k] = Sum();
+        }
+        if (tid == 0) {
+            for (int w = 0; w < NW; ++w) second = min(second, sh.lred[w]);
+            f.order[it] = root;
+            const double bs = score_out(score_of_key(best, Sum()));
+            f.rep_root_score[it] = root == bestv ? bs : score_out(score_of_key(sh.rootpt, Sum()));
+            f.rep_margin[it] = (second == kMaxScore ? double(INFINITY) : score_out(score_of_key(second, Sum()))) - bs;
+            f.rep_pairs[it] = pairs;
+            f.ctl->rm_root = root;
+        }
+        total += pairs;
+        ++it;
+        if (it >= iters) {
+            wv.done = 1;
+            return;
+        }
+        if (tid < 32) swap_slots(rs, r - 1);   // the root leaves
+        __syncthreads();
+        r -= 1;
+        a = 0;
+        new_iteration();
+        if (r == 1) {
+            last_variable();
+            wv.done = 1;
+            return;
+        }
+        cmax = order_max_cols<T>(g.cap, NW, r, icap);
+        want = prunes && !gmode ? (need + 4) / 4 * 4 : kMaxCols;
+        plan(true, wv);
+    }
+
+    int waves = 0;
+    long long total = 0, gsteps = 0;
+
+    __device__ __forceinline__ static Sum sum_from(double x) {
+        if constexpr (f32) {
+            const float hi = float(x);
+            return make_float2(hi, isfinite(hi) ? float(x - double(hi)) : 0.f);
+        } else {
+            return x;
+        }
+    }
+    __device__ __forceinline__ long long block_min(long long v) {
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
+        __syncthreads();
+        if (lane == 0) sh.lred[wid] = v;
+        __syncthreads();
+        for (int w = 0; w < NW; ++w) v = min(v, sh.lred[w]);
+        __syncthreads();
+        return v;
+    }
+};
+
+// ------------------------------------------------------------------ hand-overs (bounded waits)
+__device__ __forceinline__ bool give_up(Ctl* ctl, Ctl* top, unsigned long long& t0, unsigned long long tmo) {
+    if (*reinterpret_cast<volatile int*>(&top->abort)) return true;
+    const unsigned long long now = global_ns();
+    if (t0 == 0) {
+        t0 = now;
+    } else if (now - t0 > tmo) {
+        set_status(ctl, LINGAM_ETIMEOUT);
+        set_status(top, LINGAM_ETIMEOUT);
+        top->abort = 1;
+        return true;
+    }
+    return false;
+}
+// Wait until the group's workers have arrived `target` times; false: gave up (recorded).
+__device__ __forceinline__ bool wait_arrivals(Ctl* ctl, Ctl* top, unsigned target, unsigned long long tmo, OrderShared& sh) {
+    if (threadIdx.x == 0) {
+        int ok = 1;
+        unsigned long long t0 = 0;
+        while (int(ld_acquire(&ctl->bar_count) - target) < 0)
+            if (give_up(ctl, top, t0, tmo)) {
+                ok = 0;
+                break;
+            }
+        sh.ok = ok;
+    }
+    __syncthreads();
+    return sh.ok != 0;
+}
+// Wait for wave word `seq` of the group's controller.
+__device__ __forceinline__ bool wait_order_wave(Ctl* ctl, Ctl* top, unsigned seq, unsigned long long tmo, OrderShared& sh,
+                                                OrderWave& wv) {
+    if (threadIdx.x == 0) {
+        int ok = 1;
+        unsigned long long w = 0, t0 = 0;
+        for (;;) {
+            w = ld_acquire64(&ctl->wave_word);
+            if (unsigned(w >> 51) == (seq & 0x1fffu)) break;
+            if (give_up(ctl, top, t0, tmo)) {
+                ok = 0;
+                break;
+            }
+        }
+        sh.word = w;
+        sh.ok = ok;
+    }
+    __syncthreads();
+    wv = unpack_order_wave(sh.word);
+    return sh.ok != 0;
+}
+
+// ------------------------------------------------------------------ one problem by one group
+// Returns false when the launch is to end (a wait ran out here or elsewhere).
+template <class T, int NT>
+__device__ __forceinline__ bool run_problem(const Fit& f, Ctl* top, int rank, int size, int iters, unsigned smem_bytes,
+                                            OrderShared& sh) {
+    Group g;
+    g.rank = rank;
+    g.size = size;
+    const bool dedicated = size >= kDedicated;
+    g.W = dedicated ? size - 1 : size;
+    g.wk = dedicated ? rank - 1 : rank;
+    g.work = dedicated ? 0u : unsigned(order_state_bytes(f.p));
+    g.cap = smem_bytes - g.work;
+    g.tab = smem_bytes;
+    const unsigned long long tmo = *reinterpret_cast<volatile unsigned long long*>(&top->timeout_ns);
+    T* xb[2] = {static_cast<T*>(f.xt), static_cast<T*>(f.xalt)};
+    double* sb[2] = {f.sig, f.sigalt};
+    int cur = 0;   // the copy before the next removal
+    if (rank != 0) {
+        for (unsigned seq = 1;; ++seq) {
+            OrderWave wv;
+            if (!wait_order_wave(f.ctl, top, seq, tmo, sh, wv)) return false;
+            if (wv.done) {
+                return true;
+            }
+            worker_wave<T, NT>(f, wv, g, xb[cur], xb[cur ^ 1], sb[cur], sb[cur ^ 1], f.dscale[cur], f.dscale[cur ^ 1]);
+            if (wv.removal) cur ^= 1;
+            __syncthreads();
+            if (threadIdx.x == 0) atom_add_release(&f.ctl->bar_count, 1u);
+        }
+    }
+    // the controller
+    Controller<T, NT> c(f, g, sh, smem_bytes, iters);
+    OrderWave wv{1, 0, 0, 0, 0, 0};
+    if (threadIdx.x == 0) sh.ok = *reinterpret_cast<volatile int*>(&f.ctl->status) == 0;
+    __syncthreads();
+    if (sh.ok != 0 && c.start()) c.plan(false, wv);
+    const bool timed = f.timing && threadIdx.x == 0;
+    unsigned long long tit = timed ? global_ns() : 0, tph = tit;
+    unsigned arrivals = 0;
+    for (unsigned seq = 1;; ++seq) {
+        __syncthreads();   // the row table is written
+        if (threadIdx.x == 0 && size > 1)
+            st_release64(&f.ctl->wave_word, pack_order_wave(seq, wv.done, wv.removal, wv.kill, wv.ncol, wv.nrow, wv.nseg));
+        if (wv.done) break;
+        if (timed) {
+            const unsigned long long t = global_ns();
+            f.ctl->phase_ns[1] += t - tph;
+            tph = t;
+        }
+        if (!dedicated) {
+            worker_wave<T, NT>(f, wv, g, xb[cur], xb[cur ^ 1], sb[cur], sb[cur ^ 1], f.dscale[cur], f.dscale[cur ^ 1]);
+            __syncthreads();
+        }
+        if (wv.removal) cur ^= 1;
+        arrivals += unsigned(size - 1);
+        if (size > 1 && !wait_arrivals(f.ctl, top, arrivals, tmo, sh)) return false;
+        if (timed) {
+            const unsigned long long t = global_ns();
+            f.ctl->phase_ns[0] += t - tph;
+            tph = t;
+        }
+        // a failure recorded by a worker ends the fit (the others of a batch go on); read now, looked
+        // at after the wave's work
+        int bad = 0;
+        if (threadIdx.x == 0) bad = *reinterpret_cast<volatile int*>(&f.ctl->status);
+        const int before = c.it;
+        c.finish_wave(wv);
+        if (__syncthreads_or(bad)) wv = OrderWave{1, 0, 0, 0, 0, 0};
+        if (timed && c.it != before) {
+            const unsigned long long t = global_ns();
+            f.prev[before] = double(t - tit) * 1e-6;
+            tit = t;
+        }
+    }
+    if (threadIdx.x == 0) {
+        f.ctl->waves = c.waves;
+        f.ctl->tile_pairs = c.total;
+        f.ctl->gsteps = c.gsteps;
+    }
+    return true;
+}
+
+// ------------------------------------------------------------------ the kernel
+// one problem (fits == nullptr): every CTA of the grid is the group of `one`.  Many: assign[cta] =
+// {problem, rank, group size} of this CTA's first problem (problem -1: none), then the problems of
+// queue[0 .. nqueue) one after another, each by a single CTA.
+template <class T, int NT>
+__global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2)
+    k_order(const __grid_constant__ Fit one, int iters, const Fit* __restrict__ fits, const int4* __restrict__ assign,
+            const int* __restrict__ queue, int nqueue, unsigned* qhead, Ctl* top, unsigned smem_bytes) {
+    __shared__ OrderShared sh;
+    __shared__ Fit s_fit;
+    if (*reinterpret_cast<volatile int*>(&top->status) != 0) return;
+    if constexpr (sizeof(T) == 8) {   // the exponentials' table, behind everything else
+        smem_bytes -= kExpTab * sizeof(double);
+        double* tab = reinterpret_cast<double*>(smem_order + smem_bytes);
+        for (int j = threadIdx.x; j < kExpTab; j += NT) tab[j] = exp2(double(j) / kExpTab);
+    }
+    int d = 0, rank = blockIdx.x, size = gridDim.x;
+    if (fits) {
+        const int4 as = assign[blockIdx.x];
+        d = as.x;
+        rank = as.y;
+        size = as.z;
+    }
+    for (;;) {
+        if (d >= 0) {
+            __syncthreads();
+            if (threadIdx.x == 0) s_fit = fits ? fits[d] : one;
+            __syncthreads();
+            if (!run_problem<T, NT>(s_fit, top, rank, size, fits ? s_fit.p : iters, smem_bytes, sh)) return;
+        }
+        if (!fits) return;
+        __syncthreads();
+        if (threadIdx.x == 0) sh.qnext = int(atomicAdd(qhead, 1u));
+        __syncthreads();
+        const int q = sh.qnext;
+        if (q >= nqueue) return;
+        d = queue[q];
+        rank = 0;
+        size = 1;
+    }
+}
+
+// ------------------------------------------------------------------ host side
+constexpr size_t kOrderSmem512 = 220 * 1024;
+constexpr size_t kOrderSmem256 = 108 * 1024;
+
+// Largest p whose controller state and I table (four columns) fit.
+template <class T>
+static bool order_fits_smem(long long p, size_t smem, bool dedicated, int nw) {
+    const size_t state = order_state_bytes(int(p));
+    if (state >= smem) return false;
+    return order_max_cols<T>(smem - (dedicated ? 0 : state), nw, int(p), smem - state) >= 4;
+}
+
+bool order_supported(const Fit& f, bool batch) {
+    const bool f32 = f.precision == LINGAM_MIXED;
+    if (f.p > 4096 || f.ld / 256 > 0xffff) return false;
+    if (f.rec_bytes < size_t(f.p) * (16 * (kMaxCols / 4) + 8) * 8) return false;   // one segment of a full wave
+    const size_t smem = (batch ? kOrderSmem256 : kOrderSmem512) - (f32 ? 0 : kExpTab * sizeof(double));
+    // (a single fit's group is below kDedicated CTAs only when p is small)
+    return f32 ? order_fits_smem<float>(f.p, smem, !batch && f.p >= 64, batch ? 8 : 16)
+               : order_fits_smem<double>(f.p, smem, !batch && f.p >= 64, batch ? 8 : 16);
+}
+
+template <class T, int NT>
+static cudaError_t launch_order_t(const Fit& f, int iters, const Fit* fits, const int4* assign, const int* queue, int nqueue,
+                                  unsigned* qhead, Ctl* top, int grid, cudaStream_t st) {
+    const void* fn = reinterpret_cast<const void*>(k_order<T, NT>);
+    unsigned smem = unsigned(NT == 512 ? kOrderSmem512 : kOrderSmem256);
+    cudaError_t e = ensure_smem_attr(fn, smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;   // all CTAs co-resident: they wait for each other
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_order<T, NT>, f, iters, fits, assign, queue, nqueue, qhead, top, smem);
+}
+
+// CTAs of a single fit: enough for four warps' blocks each (a row against a quad, and the row's own;
+// FP64: for one block) in the first wave, the whole GPU at most.
+int order_grid(const Fit& f, int nsm) {
+    const bool f32 = f.precision == LINGAM_MIXED;
+    const int b = f32 ? blk<float>() : blk<double>();
+    const long long units = (long long)f.p * ((f.ld + b - 1) / b) * 2;
+    return int(std::max(1ll, std::min((long long)nsm, 1 + (f32 ? (units + 3) / 4 : units))));
+}
+
+cudaError_t launch_order(const Fit& f, int iters, int nsm, cudaStream_t st) {
+    const int grid = order_grid(f, nsm);
+    return f.precision == LINGAM_MIXED ? launch_order_t<float, 512>(f, iters, nullptr, nullptr, nullptr, 0, nullptr, f.ctl, grid, st)
+                                       : launch_order_t<double, 512>(f, iters, nullptr, nullptr, nullptr, 0, nullptr, f.ctl, grid, st);
+}
+
+// Clocks (estimate) of a problem on g CTAs of 256 threads: 3 pair-samples a clock and CTA (FP64:
+// 1/40 of that), about 7 pairs per row and iteration, and the hand-over of a wave.
+static double batch_clocks(const Fit& f, int g) {
+    const double p = f.p, rate = f.precision == LINGAM_MIXED ? 3.0 : 0.075;
+    const double work = 3.5 * p * p * f.ld / rate;
+    const int W = g >= kDedicated ? g - 1 : g;
+    return work / W + p * (g > 1 ? 16000.0 : 8000.0);
+}
+
+// Groups of a batch: with fewer problems than CTA slots every problem has a group, and the slots
+// left go one by one to the problem that would take longest; with more, problems of more than
+// twice a slot's share of the work get groups of their own, and the others queue, longest first,
+// for single CTAs.
+void order_batch_plan(const Fit* fits, int count, int nsm, std::vector<int4>& assign, std::vector<int>& queue) {
+    const int slots = std::min(2 * nsm, kOrderSlots);
+    std::vector<int> g(static_cast<size_t>(count), 1), big;
+    queue.clear();
+    if (count <= slots) {
+        std::priority_queue<std::pair<double, int>> longest;
+        for (int d = 0; d < count; ++d) longest.push({batch_clocks(fits[d], 1), d});
+        for (int left = slots - count; left > 0 && !longest.empty(); --left) {
+            const int d = longest.top().second;
+            longest.pop();
+            ++g[size_t(d)];
+            const long long most = (long long)fits[d].p * ((fits[d].ld + 1023) / 1024);   // rows x blocks
+            if (g[size_t(d)] < most) longest.push({batch_clocks(fits[d], g[size_t(d)]), d});
+        }
+        for (int d = 0; d < count; ++d) big.push_back(d);
+    } else {
+        double total = 0.0;
+        std::vector<std::pair<double, int>> by;
+        for (int d = 0; d < count; ++d) {
+            by.push_back({batch_clocks(fits[d], 1), d});
+            total += by.back().first;
+        }
+        std::sort(by.begin(), by.end(), [](const auto& a, const auto& b) { return a.first > b.first || (a.first == b.first && a.second < b.second); });
+        int left = slots - 1;   // one slot at least for the queue
+        for (const auto& b : by) {
+            const int want = int(std::min(double(slots), b.first / (total / slots)));
+            if (want >= 2 && want <= left) {
+                g[size_t(b.second)] = want;
+                left -= want;
+                big.push_back(b.second);
+            } else {
+                queue.push_back(b.second);
+            }
+        }
+    }
+    assign.clear();
+    for (int d : big)
+        for (int k = 0; k < g[size_t(d)]; ++k) assign.push_back(make_int4(d, k, g[size_t(d)], 0));
+    while (int(assign.size()) < slots && !queue.empty()) assign.push_back(make_int4(-1, 0, 0, 0));
+}
+
+cudaError_t launch_order_batch(const Fit* fits_dev, int precision, const int4* assign, int grid, const int* queue, int nqueue,
+                               unsigned* qhead, Ctl* bctl, cudaStream_t st) {
+    const Fit none = {};
+    return precision == LINGAM_MIXED
+               ? launch_order_t<float, 256>(none, 0, fits_dev, assign, queue, nqueue, qhead, bctl, grid, st)
+               : launch_order_t<double, 256>(none, 0, fits_dev, assign, queue, nqueue, qhead, bctl, grid, st);
+}
+
+}  // namespace lingam

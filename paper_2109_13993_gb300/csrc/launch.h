@@ -18,8 +18,9 @@ cudaError_t launch_standardize(const Fit& f, const void* x, int input_dtype, cud
 // rows of `count` problems (rowoff[d] = first global row of problem d, `rows` in all).
 cudaError_t launch_standardize_batch(const Fit* fits, const SrcDesc* src, const int* rowoff, int count, int rows,
                                      int precision, int input_dtype, cudaStream_t st);
-// Sigma = Xn Xn^T / (n-1) of the normalised rows (CalculateCovMat, Algorithm 3); sig0 = sig.
-cudaError_t launch_gram(const Fit& f, cudaStream_t st);
+// FP64 path: Sigma = Xn Xn^T / (n-1) of the normalised rows (CalculateCovMat, Algorithm 3); sig0 = sig.
+// partial_bytes: what f.partials holds.
+cudaError_t launch_gram(const Fit& f, size_t partial_bytes, cudaStream_t st);
 // The same product on the tensor cores (mixed path): the rows are split into exact
 // TF32 digits (three p x ld float planes and p exponents in `digits`), tcgen05 MMAs
 // over 128 x 128 tiles of the upper triangle with the sample axis split over CTAs,

@@ -67,6 +67,7 @@ struct Layout {
         off_rows, off_cols, off_order, off_forced, off_prior, off_anc, off_scratch, off_rowsum, off_colsum, off_partials, off_invroot,
         off_tilecnt, off_rs, off_rm, off_rp, off_rsc, off_cmat, off_rmat, off_rinv, off_bout, off_ctl, off_ibuf;
     int ld, maxtiles, maxsplit, esz, nslots;
+    size_t partial_bytes;
 };
 
 static int chunk_of(int precision) { return precision == LINGAM_MIXED ? kChunk : kChunk64; }
@@ -120,8 +121,8 @@ static Layout make_layout(long long p, long long n, int precision, int input_dty
     // (the Gram's split partial tiles use the same region before the first iteration)
     L.nslots = int(size_t(L.maxtiles) + std::min(size_t(kMaxGrid), units));
     const size_t pair_partials = size_t(L.nslots) * kPairThreads * 16 * L.esz;
-    L.off_partials =
-        take(std::max(pair_partials, precision == LINGAM_MIXED ? gram_tc_partial_bytes(p, L.ld) : size_t(0)));
+    L.partial_bytes = std::max(pair_partials, precision == LINGAM_MIXED ? gram_tc_partial_bytes(p, L.ld) : size_t(0));
+    L.off_partials = take(L.partial_bytes);
     L.off_invroot = take(P * 8);
     L.off_tilecnt = take(size_t(L.maxtiles) * 4);
     L.off_ibuf = take(size_t(L.maxtiles) * 64 * kTJ * L.esz);
@@ -392,7 +393,7 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
             }
             launches += 4;
         } else {
-            if (launch_gram(f, st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
+            if (launch_gram(f, L.partial_bytes, st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
             launches += 2;
         }
         if (cudaEventRecord(ev[2], st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
@@ -703,7 +704,7 @@ static cudaError_t enqueue_batch(char* ws, const BatchLayout& BL, const std::vec
         cudaStream_t sk = nfork > 0 ? fs->s[j++ % nfork] : st;
         e = o.precision == LINGAM_MIXED
                 ? launch_gram_tc(fits[size_t(k)], ws + BL.region[size_t(k)] + Ls[size_t(k)].off_xin, fits[size_t(k)].partials, sk)
-                : launch_gram(fits[size_t(k)], sk);
+                : launch_gram(fits[size_t(k)], Ls[size_t(k)].partial_bytes, sk);
     }
     for (int i = 0; i < nfork; ++i) {
         const cudaError_t ej = cudaEventRecord(fs->join[i], fs->s[i]) == cudaSuccess
