@@ -44,9 +44,10 @@
  *     line per call on stderr (entry point, sizes, status); LINGAM_FAULT=<step>
  *     makes the named step of every call report a failed launch (host-side
  *     fault injection for testing: standardize, covariance, iteration:<k>,
- *     bfit, batch); LINGAM_NARROW=<rows> sets the fewest rows for which a wave
- *     of 16 columns or fewer of a 64 x 32 single fit runs on 128 x 16 tiles
- *     (default 256; 0 turns these narrow waves off, a switch for measurement).
+ *     bfit, batch); LINGAM_NARROW=<rows> makes single fits run on the tile
+ *     kernels and sets the fewest rows for which a wave of 16 columns or fewer of
+ *     a 64 x 32 fit runs on 128 x 16 tiles (256 without it; 0 turns these narrow
+ *     waves off), a switch for measurement.
  */
 #ifndef LINGAM_H
 #define LINGAM_H
@@ -79,18 +80,19 @@ typedef struct {
     int input_dtype;         /* element type of X: LINGAM_F32 or LINGAM_F64 */
     int prune;               /* 1 = threshold pruning (Sec. III-B), 0 = compare every pair */
     int reuse;               /* 1 = one evaluation per unordered pair (Sec. III-A), 0 = every ordered pair */
-    int tile_i, tile_j;      /* pair-tile shape of the mixed path, rows x columns: 64 x 32, 32 x 32 or
-                                64 x 16, and for batch calls only 32 x 16 and 1 x 1 (one pair per warp)
-                                (a zero in one takes 64 rows or 32 columns); both 0 = the autotuner's
-                                table (lingam_tile_rows/_cols, lingam_batch_tile_rows/_cols).  The FP64
-                                path uses 32 x 32. */
-    int split_n;             /* single fits: split of the sample axis.  0 (default) = stream-K over
-                                (tile, 32-sample group) units: a wave's units are spread over the whole
-                                grid, so a tile's samples are cut into as many CTA segments as it takes
-                                to fill every SM.  s > 0 = at most ntiles * s CTAs work on a wave, so a
-                                tile is cut into about s segments (s = 1: one CTA per tile while a wave
-                                has fewer tiles than SMs).  Results move by FP32 rounding only (the
-                                partial moments of a tile are summed over its segments in fixed order).
+    int tile_i, tile_j;      /* both 0 (default): single fits run the ordering kernel (no tiles; p up to
+                                about 2000), batch calls as lingam_fit_batch says.  Else the pair-tile
+                                shape of the tile kernels on the mixed path, rows x columns: 64 x 32,
+                                32 x 32 or 64 x 16, and for batch calls only 32 x 16, and 1 x 1 (the
+                                ordering kernel) (a zero in one takes 64 rows or 32 columns).  The FP64
+                                path's tiles are 32 x 32.  Larger problems run the tile kernels with the
+                                autotuner's shape (lingam_tile_rows/_cols, lingam_batch_tile_rows/_cols). */
+    int split_n;             /* single fits: split of the sample axis.  0 (default) = as the kernel
+                                chooses (the ordering kernel the number of segments that takes the
+                                shortest estimated time; the tile kernels spread a wave's (tile, 32-sample
+                                group) units over the whole grid).  s > 0 = at most s segments (s = 1: one
+                                CTA per row group or tile).  Results move by FP32 rounding only (the
+                                partial moments are summed over the segments in fixed order).
                                 Ignored by the batch entry points. */
     double timeout_s;        /* bound on any device-side wait; <= 0 means 10 s */
     void* stream;            /* cudaStream_t to run on; NULL = the legacy default stream */
@@ -99,9 +101,10 @@ typedef struct {
                                 those of the current iteration.  Used for iteration-by-iteration checks. */
     int max_iters;           /* 0 = all p iterations; else stop after this many (order[k] = -1 beyond,
                                 B is then not computed).  Used to time a bounded prefix of a run. */
-    int timing;              /* 1 = also time every iteration's launch (report t_pair_ms and
-                                t_pair_iter_ms; one CUDA event recorded after each launch) and
-                                run the device phase timers (t_compute_ms ...); 0 for production */
+    int timing;              /* 1 = also time the ordering launch and its iterations (report t_pair_ms and
+                                t_pair_iter_ms; tile kernels: every iteration's launch, one CUDA event
+                                recorded after each) and run the device phase timers (t_compute_ms ...);
+                                0 for production */
     const signed char* prior; /* NULL, or a p x p HOST matrix of prior knowledge (the paper notes
                                 that DirectLiNGAM accepts prior knowledge, Sec. II-C; read as known
                                 ancestors): prior[i*p + j] = 1 says X_j is known to be an ancestor
@@ -132,7 +135,7 @@ typedef struct {
     double* root_score;          /* [p] score S of the root chosen at iteration k */
     double* margin_lb;           /* [p] lower bound of (second lowest score - root score) at iteration k;
                                     +inf when a single variable is left */
-    long long* pairs_evaluated;  /* [p] pair evaluations at iteration k (unordered pairs when reuse = 1) */
+    long long* pairs_evaluated;  /* [p] pairs evaluated at iteration k (distinct unordered pairs when reuse = 1) */
     double* scores;              /* [p*p] scores[k*p + v]: S_v at iteration k if v was compared with every
                                     other remaining variable at that iteration; NaN if v was already
                                     ordered or was pruned before completing */
@@ -142,14 +145,17 @@ typedef struct {
     long long pairs_unpruned;    /* sum over iterations of r(r-1)/2 (r(r-1) when reuse = 0) */
     double t_pair_ms;            /* device time of the pair-comparison launches (opts.timing = 1), else 0 */
     long long kernel_launches;   /* kernels this call launched */
-    double* t_pair_iter_ms;      /* NULL or a HOST array [p]: with opts.timing = 1, the time of the
-                                    launch of iteration k, between the stream events recorded after
-                                    launch k - 1 (before the first launch) and after launch k */
+    double* t_pair_iter_ms;      /* NULL or a HOST array [p]: with opts.timing = 1, the time of
+                                    iteration k by CTA 0's global timer (tile kernels: of its launch,
+                                    between the stream events recorded after launch k - 1, or before
+                                    the first launch, and after launch k) */
     /* With opts.timing = 1 (single fits): device wall time (CTA 0's global timer, summed
-       over all iterations) of CTA 0's own pair-compute phases of the waves, of the rest of
-       each wave as CTA 0 sees it (the wait for the slower CTAs' tiles, the merge and the
-       finalisation, up to the wave's published result), and of CTA 0's part of the
-       removals (UpdateData, UpdateCovMat).  0 otherwise. */
+       over all iterations).  Ordering kernel: from each wave's publication until its sums are
+       there (pair comparison and removal, which are one phase; t_remove_ms stays 0), and CTA
+       0's merge and decision up to the next publication.  Tile kernels: CTA 0's own
+       pair-compute phases of the waves, the rest of each wave as CTA 0 sees it (the wait for
+       the slower CTAs' tiles, the merge and the finalisation, up to the wave's published
+       result), and CTA 0's part of the removals (UpdateData, UpdateCovMat).  0 otherwise. */
     double t_compute_ms, t_merge_ms, t_remove_ms;
     long long threshold_updates; /* opts.gamma0 > 0: times the threshold was multiplied by gamma_c,
                                     summed over the iterations (each one a kernel launch and a
@@ -157,7 +163,8 @@ typedef struct {
     long long waves;             /* pair waves run over the fit (single fits) */
     long long tile_pairs;        /* pairs the waves' tiles computed: tiles x rows x columns, row
                                     padding, unused columns and the duplicate half of the
-                                    columns' own block included (pairs_total are the useful ones) */
+                                    columns' own block included (pairs_total are the useful ones,
+                                    and all there are in the ordering kernel) */
     long long empty_col_pairs;   /* of tile_pairs: those in column slots a wave left empty */
     long long pad_row_pairs;     /* of tile_pairs: those of the padding rows of a wave's last tile */
 } lingam_report;
@@ -207,15 +214,16 @@ int lingam_covariance(const void* X, long long p, long long n, double* Sigma, vo
 
 /*
  * Pair-tile autotuner (the paper has no counterpart: its GPU design has one tile shape).
- * The mixed path evaluates pairs in tiles of rows x columns variables: 64 x 32 (512
- * threads), 32 x 32 or 64 x 16 (256 threads, two CTAs per SM).  The columns of a tile are
+ * The tile kernels evaluate pairs in tiles of rows x columns variables: 64 x 32 (512
+ * threads), 32 x 32 or 64 x 16 (256 threads, two CTAs per SM).  Single fits with the default
+ * options do not use them (lingam_opts.tile_i), larger ones than the ordering kernel takes do.  The columns of a tile are
  * the candidates a wave completes, so 16-column tiles prune more finely (fewer pairs, more
  * waves).  Which shape is faster depends on p, n and the data.  The library keeps a
  * process-wide table of the choice per size bucket (ceil(log2 p), ceil(log2 n)); a
  * bucket never measured uses 64 x 32.
  *
- * lingam_tile_rows, lingam_tile_cols -- the shape lingam_fit uses for a p x n problem
- *                       when opts->tile_i and opts->tile_j are 0.
+ * lingam_tile_rows, lingam_tile_cols -- the shape lingam_fit's tile kernels use for a p x n
+ *                       problem when opts->tile_i and opts->tile_j are 0.
  * lingam_autotune    -- measures the ordering of X (as lingam_fit with opts, B not
  *                       fitted) once with each shape, records the fastest for X's size
  *                       bucket and returns it in *tile_rows, *tile_cols; ms[0..2] (if
@@ -226,19 +234,18 @@ int lingam_covariance(const void* X, long long p, long long n, double* Sigma, vo
  *                       lingam_fit_bootstrap use on the mixed path for a batch whose
  *                       largest problem has maxp variables and maxn samples, when
  *                       opts->tile_i and opts->tile_j are 0.  Batches have a table of their
- *                       own (bucket of the largest p and n); a bucket never measured uses
- *                       the pair mode, 1 x 1, when maxp <= 128 (it was the fastest shape on
- *                       every measured batch of small problems), else 32 x 32.  With
- *                       opts->reuse = 0 the pair mode runs as 64 x 16.
+ *                       own (bucket of the largest p and n); a bucket never measured runs the
+ *                       ordering kernel (1 x 1) where it takes every problem of the call (p up to
+ *                       about 800), else, and as these functions report it, 1 x 1 when maxp <= 128
+ *                       and 32 x 32 tiles beyond.  With opts->reuse = 0, 1 x 1 runs as 64 x 16.
  * lingam_autotune_batch -- measures lingam_fit_batch on the caller's count datasets (as
  *                       lingam_fit_batch with opts on the mixed path, B not fitted) with
  *                       each shape: a warm-up call, the call that captures the graph, and
  *                       the timed third call (host wall time of the synchronous call).
  *                       Batches have two more shapes for many small problems: 32 x 16
- *                       tiles (128 threads, three CTAs per SM, 64-sample chunks), and the
- *                       pair mode, 1 x 1, in which every pair a wave needs is evaluated
- *                       whole by one warp (no tile, so no pair slot is computed in vain;
- *                       waves of up to 16 columns).  Records the fastest for the bucket of
+ *                       tiles (128 threads, three CTAs per SM, 64-sample chunks), and 1 x 1, the
+ *                       ordering kernel (groups of CTAs per problem, none waiting for another's).
+ *                       Records the fastest for the bucket of
  *                       the batch's largest p and n, returns it in *tile_rows, *tile_cols,
  *                       and ms[0..4] (if not NULL) receive the times with 64 x 32, 32 x 32,
  *                       64 x 16, 32 x 16 and 1 x 1.  Costs fifteen batch calls; the
@@ -285,17 +292,19 @@ size_t lingam_workspace_size_batch(int count, const long long* p, const long lon
  * status, else LINGAM_OK.  A dataset that turns out degenerate does not stop the
  * others; a timeout stops all of them.
  *
- * All problems run in one persistent cooperative launch per 512 problems, in
- * lockstep over iterations: each wave's pair tiles of all problems are partitioned
- * over the whole GPU together.  The device work of a call is captured into a CUDA
+ * All problems run in one persistent cooperative launch per 512 problems.  In the ordering
+ * kernel every problem has a group of CTAs sized by its work (small ones of a large batch
+ * queue for single CTAs); on tiles they advance in lockstep over iterations, each wave's pair
+ * tiles of all problems partitioned over the whole GPU together.  The device work of a call is captured into a CUDA
  * graph on the second call with the same workspace and problem shapes (and options),
  * and replayed by every later such call; calls on the legacy default stream (NULL)
  * run without a graph.  opts->forced_order and opts->prior must be NULL, and
  * opts->max_iters and opts->gamma0 0; opts->split_n is ignored.  Pair tiles: on the
  * mixed path opts->tile_i x opts->tile_j for every problem of the call (64 x 32, 32 x 32,
- * 64 x 16, 32 x 16, or 1 x 1: one pair per warp, which needs opts->reuse = 1 and otherwise
- * runs 64 x 16), or, with both 0, the batch autotuner's shape for the largest p and n
- * (lingam_batch_tile_rows/_cols); 32 x 32 on the FP64 path.
+ * 64 x 16, 32 x 16, or 1 x 1: the ordering kernel, which needs opts->reuse = 1 and p up to
+ * about 800 and otherwise runs as 64 x 16), or, with both 0, what the batch autotuner measured
+ * for the largest p and n, else the ordering kernel where it takes the call (see
+ * lingam_batch_tile_rows/_cols); on the FP64 path the ordering kernel, else 32 x 32.
  */
 int lingam_fit_batch(int count, const void* const* X, const long long* p, const long long* n, int* const* order,
                      double* const* B, void* workspace, const lingam_opts* opts, int* status,

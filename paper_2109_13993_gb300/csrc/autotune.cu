@@ -45,17 +45,21 @@ void autotune_record(long long p, long long n, TileShape shape) {
     g_tune[bucket(p, n)] = shape;
 }
 
-// Batch calls: a table of its own, keyed by the batch's largest p and n.  Default: 32 x 32
-// tiles, which a batch of many small problems pads least once r < 32.
+// Batch calls: a table of its own, keyed by the batch's largest p and n.
 static std::map<std::pair<int, int>, TileShape> g_tune_batch;
 
 TileShape autotune_batch_shape(long long maxp, long long maxn) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune_batch.find(bucket(maxp, maxn));
     if (it != g_tune_batch.end()) return it->second;
-    // never measured: the pair-per-warp mode up to 128 variables (it wins over every tile
-    // shape on the measured batches of small problems), else 32 x 32
+    // never measured: 1 x 1 up to 128 variables, else 32 x 32 tiles (for a batch that the ordering
+    // kernel does not take: an untuned batch runs it whatever the size where it can)
     return maxp <= 128 ? TileShape{1, 1} : TileShape{32, 32};
+}
+
+bool autotune_batch_measured(long long maxp, long long maxn) {
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    return g_tune_batch.count(bucket(maxp, maxn)) != 0;
 }
 
 void autotune_batch_record(long long maxp, long long maxn, TileShape shape) {

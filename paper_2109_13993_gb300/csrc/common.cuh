@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cstdint>
+#include <cstring>
 #include <cuda_runtime.h>
 
 #include "lingam.h"
@@ -177,6 +178,13 @@ struct Fit {
                          // schedule (Sec. III-B/C): threshold gamma0, times gamma_c while no variable
                          // can finish below it
     double gamma_c;
+    // the ordering kernel (k_order.cu)
+    void* xalt;          // [p x ld] the other copy of the rows (each removal writes the one it does not read)
+    double* sigalt;      // [p x p] the other copy of the covariance (upper triangle)
+    void* rec;           // sums of the current wave, per segment, row and column (8-byte values)
+    unsigned long long rec_bytes;
+    void* rowtab;        // [p] rows of the current wave (RowEnt)
+    double* dscale[2];   // [p] by variable, two copies: the normalised row is the residual times this
 };
 
 // ---------------------------------------------------------------------------
@@ -305,14 +313,28 @@ __host__ __device__ __forceinline__ float hterm_f(float lcc, float g, float inv_
     return -float(kK1) * a * a - float(kK2) * b * b;
 }
 
+// A group offset with its three lowest mantissa bits cleared, so that the part of it that belongs
+// to k / 8 of a group is exact.
+__host__ __device__ inline float var_offset(float x) {
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(__float_as_uint(x) & ~7u);
+#else
+    unsigned b;
+    std::memcpy(&b, &x, sizeof(b));
+    b &= ~7u;
+    std::memcpy(&x, &b, sizeof(b));
+    return x;
+#endif
+}
+
 // Statistics of one normalised row that the FP32 pair path needs, from the row's FP64
 // moment sums L = sum_t (log cosh u_t - beta) and Gs = sum_t u_t exp(-u_t^2/2) over its n
 // samples (row length ld with zero padding):
-//   .w  the offset -kSub (ln 2 + m) of a 32-sample group, in FP32, m = mean log cosh.  The
+//   .w  the offset -kSub (ln 2 + m) of a 32-sample group (var_offset), m = mean log cosh.  The
 //       pair kernel centres a residual's log-cosh group sums by its variable's own mean
 //       (instead of beta), so that the FP32 sums stay small also for strongly
 //       non-Gaussian variables;
-//   .x  corr = (m (ld - n) - (ld / kSub) eps) / n, eps = the FP32 rounding of .w: for a
+//   .x  corr = (m (ld - n) - (ld / kSub) eps) / n, eps = the rounding of .w: for a
 //       residual whose centred sum over the padded row is T, its mean log cosh exceeds m by
 //       delta = T / n + corr exactly (padding samples have log cosh 0);
 //   .y  2 (m - beta) and .z  the mean of u exp(-u^2/2), with which the entropy difference of
@@ -321,7 +343,7 @@ __host__ __device__ __forceinline__ float hterm_f(float lcc, float g, float inv_
 __host__ __device__ inline float4 var_stats(double L, double Gs, int n, int ld) {
     const double m = kBeta + L / double(n);
     const double g = Gs / double(n);
-    const float off = float(-double(kSub) * (kLn2 + m));
+    const float off = var_offset(float(-double(kSub) * (kLn2 + m)));
     const double eps = double(off) + double(kSub) * (kLn2 + m);
     const double corr = (m * double(ld - n) - double(ld / kSub) * eps) / double(n);
     return make_float4(float(corr), float(2.0 * (m - kBeta)), float(g), off);
@@ -336,7 +358,7 @@ __host__ __device__ __forceinline__ double hterm_inv(double lcc, double g, doubl
 __host__ __device__ inline float4 var_stats_inv(double L, double Gs, int n, int ld, double inv_n) {
     const double m = kBeta + L * inv_n;
     const double g = Gs * inv_n;
-    const float off = float(-double(kSub) * (kLn2 + m));
+    const float off = var_offset(float(-double(kSub) * (kLn2 + m)));
     const double eps = double(off) + double(kSub) * (kLn2 + m);
     const double corr = (m * double(ld - n) - double(ld / kSub) * eps) * inv_n;
     return make_float4(float(corr), float(2.0 * (m - kBeta)), float(g), off);

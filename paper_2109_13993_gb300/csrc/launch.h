@@ -1,6 +1,8 @@
 // launch.h -- host-side launchers of the CUDA kernels (internal to the library).
 #pragma once
 
+#include <vector>
+
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -42,6 +44,19 @@ size_t gram_tc_partial_bytes(long long p, int ld);
 cudaError_t launch_iteration(const Fit& f, int it, int grid, cudaStream_t st);
 // Largest co-resident grid of the iteration kernel (one CTA per SM).
 int iteration_grid(const Fit& f, int nsm);
+// The ordering kernel (k_order.cu): all iterations in one persistent cooperative launch, with
+// killer pairs.  order_supported: whether it takes a problem (pair reuse on; the state of its
+// variables in shared memory, p up to about 2300 for a single fit; batch: 256-thread CTAs, two per
+// SM, p up to about 1200).
+bool order_supported(const Fit& f, bool batch);
+int order_grid(const Fit& f, int nsm);
+cudaError_t launch_order(const Fit& f, int iters, int nsm, cudaStream_t st);
+// Batches: the CTAs' first problems (assign, one entry per CTA of the grid) and the queue of the
+// others, planned on the host; then the launch of the table.
+constexpr int kOrderSlots = 320;
+void order_batch_plan(const Fit* fits, int count, int nsm, std::vector<int4>& assign, std::vector<int>& queue);
+cudaError_t launch_order_batch(const Fit* fits_dev, int precision, const int4* assign, int grid, const int* queue, int nqueue,
+                               unsigned* qhead, Ctl* bctl, cudaStream_t st);
 // The ordering of up to 512 problems (a Fit table in device memory, each with its own
 // control block) in one persistent cooperative launch, all iterations, in lockstep;
 // bctl carries the launch's barrier, abort flag and timeout.  The mixed path's pair tiles
@@ -69,6 +84,7 @@ void autotune_record(long long p, long long n, TileShape shape);
 void autotune_clear();
 // The same for batch calls, keyed by the batch's largest p and largest n.
 TileShape autotune_batch_shape(long long maxp, long long maxn);
+bool autotune_batch_measured(long long maxp, long long maxn);
 void autotune_batch_record(long long maxp, long long maxn, TileShape shape);
 
 }  // namespace lingam

@@ -68,6 +68,7 @@ struct Layout {
         off_tilecnt, off_rs, off_rm, off_rp, off_rsc, off_cmat, off_rmat, off_rinv, off_bout, off_ctl, off_ibuf;
     int ld, maxtiles, maxsplit, esz, nslots;
     size_t partial_bytes;
+    bool alt_in_xin;   // the ordering kernel's second copy of the rows: the input copy's region, else behind the sums
 };
 
 static int chunk_of(int precision) { return precision == LINGAM_MIXED ? kChunk : kChunk64; }
@@ -90,7 +91,19 @@ static Layout make_layout(long long p, long long n, int precision, int input_dty
     // the host-input copy is dead once the rows are normalised; the mixed path's
     // tensor-core Gram reuses it for the digit planes of its operands
     const size_t split_bytes = precision == LINGAM_MIXED ? gram_tc_digit_bytes(p, L.ld) : 0;
-    L.off_xin = take(std::max(P * size_t(n) * in_esz, split_bytes));
+    // one partial-moment slot per (tile, CTA) segment; slot index tile + CTA, and a wave never
+    // uses more CTAs than it has (tile, 32-sample group) units
+    const size_t units = size_t(L.maxtiles) * size_t(L.ld / kSub);
+    // (the Gram's split partial tiles use the same region before the first iteration, and the
+    // ordering kernel's sums instead of the tile kernels' partial moments)
+    L.nslots = int(size_t(L.maxtiles) + std::min(size_t(kMaxGrid), units));
+    const size_t pair_partials = size_t(L.nslots) * kPairThreads * 16 * L.esz;
+    L.partial_bytes = std::max(pair_partials, precision == LINGAM_MIXED ? gram_tc_partial_bytes(p, L.ld) : size_t(0));
+    // The ordering kernel's second copy of the rows: over the digit planes on the mixed path; on the
+    // FP64 path the second half of the partial-moment region, or the input copy's where it is larger
+    const size_t copy_bytes = P * size_t(L.ld) * L.esz;
+    L.alt_in_xin = precision == LINGAM_MIXED || copy_bytes > L.partial_bytes / 2;
+    L.off_xin = take(std::max(std::max(P * size_t(n) * in_esz, split_bytes), L.alt_in_xin ? copy_bytes : size_t(0)));
     L.off_xt = take(P * size_t(L.ld) * L.esz);
     L.off_mu = take(P * 8);
     L.off_sd = take(P * 8);
@@ -115,13 +128,6 @@ static Layout make_layout(long long p, long long n, int precision, int input_dty
     L.off_scratch = take(P * 4);
     L.off_rowsum = take(P * 8);
     L.off_colsum = take(size_t(L.maxtiles) * (kPairThreads / 64) * kTJ * 8);   // per (tile, merge item)
-    // one partial-moment slot per (tile, CTA) segment; slot index tile + CTA, and a wave never
-    // uses more CTAs than it has (tile, 32-sample group) units
-    const size_t units = size_t(L.maxtiles) * size_t(L.ld / kSub);
-    // (the Gram's split partial tiles use the same region before the first iteration)
-    L.nslots = int(size_t(L.maxtiles) + std::min(size_t(kMaxGrid), units));
-    const size_t pair_partials = size_t(L.nslots) * kPairThreads * 16 * L.esz;
-    L.partial_bytes = std::max(pair_partials, precision == LINGAM_MIXED ? gram_tc_partial_bytes(p, L.ld) : size_t(0));
     L.off_partials = take(L.partial_bytes);
     L.off_invroot = take(P * 8);
     L.off_tilecnt = take(size_t(L.maxtiles) * 4);
@@ -211,6 +217,13 @@ static EventPool* event_pool(int dev) {
 // Narrow waves: waves of <= 16 columns and at least this many rows run on 128 x 16 tiles
 // (LINGAM_NARROW=<rows> overrides the default; 0 turns them off, a switch for measuring them).
 constexpr int kNarrowMinRows = 256;
+static bool narrow_set() {
+    static const bool v = [] {
+        const char* e = std::getenv("LINGAM_NARROW");
+        return e && *e;
+    }();
+    return v;
+}
 static int narrow_min_rows() {
     static const int v = [] {
         const char* e = std::getenv("LINGAM_NARROW");
@@ -264,6 +277,15 @@ static Fit make_fit(char* base, const Layout& L, int p, int n, const lingam_opts
     f.rinv = reinterpret_cast<double*>(base + L.off_rinv);
     f.bout = reinterpret_cast<double*>(base + L.off_bout);
     f.ctl = reinterpret_cast<Ctl*>(base + L.off_ctl);
+    // the ordering kernel's buffers lie over what it does not use: see make_layout; the row table
+    // and the rows' scales (32 bytes a variable) over the I buffer (at least 256)
+    f.rec = f.partials;
+    f.rec_bytes = L.alt_in_xin ? L.partial_bytes : L.partial_bytes / 2 / kAlign * kAlign;
+    f.xalt = L.alt_in_xin ? base + L.off_xin : base + L.off_partials + f.rec_bytes;
+    f.sigalt = f.cmat;
+    f.rowtab = f.ibuf;
+    f.dscale[0] = reinterpret_cast<double*>(static_cast<char*>(f.ibuf) + size_t(p) * 16);
+    f.dscale[1] = f.dscale[0] + p;
     f.maxtiles = L.maxtiles;
     f.maxsplit = L.maxsplit;
     f.nslots = L.nslots;
@@ -297,6 +319,12 @@ static bool check_prior(const signed char* prior, int p, std::vector<int>& anc) 
             if (i != j && prior[size_t(i) * p + j] == 1 && --left[size_t(i)] == 0) queue.push_back(i);
     }
     return int(queue.size()) == p;
+}
+
+// Single fits run the ordering kernel (k_order.cu) unless an option asks for the tile kernels
+// (an explicit tile shape, LINGAM_NARROW) or the problem is too large for it.
+static bool use_order_kernel(const Fit& f, const lingam_opts& o) {
+    return o.tile_i == 0 && o.tile_j == 0 && !narrow_set() && order_supported(f, false);
 }
 
 // cov_out != nullptr: stop after CalculateCovMat and copy Sigma (p x p) there.
@@ -374,6 +402,7 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
     size_t next_ev = 5;
     std::vector<cudaEvent_t> pev;   // per-iteration pair-phase events (opts.timing)
     long long launches = 0;
+    bool order_kernel = false;
     int status = LINGAM_OK;
     do {
         if (cudaEventRecord(ev[0], st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
@@ -402,19 +431,27 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
             cudaEventRecord(ev[4], st);
             break;
         }
-        const int grid = iteration_grid(f, nsm);
+        if (use_order_kernel(f, o)) {
+            for (int it = 0; it < iters; ++it)
+                if (inject_fault("iteration", it)) status = LINGAM_ECUDA;
+            if (status != LINGAM_OK) break;
+            order_kernel = true;
+            if (launch_order(f, iters, nsm, st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
+            ++launches;
+        }
+        const int grid = order_kernel ? 1 : iteration_grid(f, nsm);
         if (grid < 1) {
             status = LINGAM_ECUDA;
             break;
         }
         // opts.timing: one event before the first launch and one after each, so launch it
         // is timed between events it and it + 1 (consecutive launches share an event)
-        if (o.timing) {
+        if (o.timing && !order_kernel) {
             const cudaEvent_t e0 = ev[next_ev++];
             pev.push_back(e0);
             cudaEventRecord(e0, st);
         }
-        for (int it = 0; it < iters && status == LINGAM_OK; ++it) {
+        for (int it = 0; it < iters && status == LINGAM_OK && !order_kernel; ++it) {
             cudaEvent_t e1 = nullptr;
             if (o.timing) {
                 e1 = ev[next_ev++];
@@ -470,6 +507,11 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
                     tp += ms;
                     if (rep->t_pair_iter_ms && k < size_t(p)) rep->t_pair_iter_ms[k] = ms;
                 }
+            if (order_kernel && o.timing) {   // one launch: its time, and the iterations' by the device's timer
+                if (cudaEventElapsedTime(&ms, ev[2], ev[3]) == cudaSuccess) tp = ms;
+                if (rep->t_pair_iter_ms)
+                    cudaMemcpyAsync(rep->t_pair_iter_ms, f.prev, size_t(iters) * 8, cudaMemcpyDefault, st);
+            }
             rep->t_pair_ms = tp;
             rep->kernel_launches = launches;
             rep->t_compute_ms = o.timing ? double(ch.phase_ns[0]) * 1e-6 : 0.0;
@@ -531,7 +573,7 @@ struct BatchItem {
 };
 
 struct BatchLayout {
-    size_t off_fits, off_ctls, off_bctl, off_src, off_rowoff, off_stage_order, off_stage_B, off_idx, off_xsrc;
+    size_t off_fits, off_ctls, off_bctl, off_src, off_rowoff, off_assign, off_queue, off_qhead, off_stage_order, off_stage_B, off_idx, off_xsrc;
     size_t header, total;
     std::vector<size_t> region;
 };
@@ -555,6 +597,12 @@ static BatchLayout make_batch_layout(int count, const long long* p, const long l
     B.off_bctl = take(sizeof(Ctl));
     B.off_src = take(size_t(count) * sizeof(SrcDesc));
     B.off_rowoff = take(size_t(count + 1) * sizeof(int));
+    // the ordering kernel's groups: per launch of up to kBatchLaunchMax problems one entry per CTA and
+    // the queue's head; the queued problems
+    const size_t launches = size_t(count + kBatchLaunchMax - 1) / kBatchLaunchMax;
+    B.off_assign = take(launches * kOrderSlots * sizeof(int4));
+    B.off_queue = take(size_t(count) * sizeof(int));
+    B.off_qhead = take(launches * sizeof(unsigned));
     B.off_stage_order = take(sum_p * sizeof(int));
     B.off_stage_B = take(sum_pp * sizeof(double));
     B.off_idx = take(idx_bytes);
@@ -663,10 +711,15 @@ static ForkStreams* fork_streams(int dev) {
     return found->second.ok ? &found->second : nullptr;
 }
 
+// The ordering kernel's grid and queue length of each launch of a batch.
+struct BatchGroups {
+    std::vector<int> grid, nqueue;
+};
+
 // The device work of a batch, enqueued on st.
 static cudaError_t enqueue_batch(char* ws, const BatchLayout& BL, const std::vector<Fit>& fits,
-                                 const std::vector<Layout>& Ls, const lingam_opts& o, int rows, bool with_B,
-                                 bool gather, int nsm, cudaStream_t st) {
+                                 const std::vector<Layout>& Ls, const lingam_opts& o, const BatchGroups* groups, int rows,
+                                 bool with_B, bool gather, int nsm, cudaStream_t st) {
     const int count = int(fits.size());
     const Fit* fits_dev = reinterpret_cast<const Fit*>(ws + BL.off_fits);
     cudaError_t e = launch_standardize_batch(fits_dev, reinterpret_cast<const SrcDesc*>(ws + BL.off_src),
@@ -718,6 +771,15 @@ static cudaError_t enqueue_batch(char* ws, const BatchLayout& BL, const std::vec
         const int cnt = std::min(kBatchLaunchMax, count - c0);
         int maxp = 0;
         for (int k = c0; k < c0 + cnt; ++k) maxp = std::max(maxp, fits[size_t(k)].p);
+        if (groups) {
+            const size_t l = size_t(c0 / kBatchLaunchMax);
+            e = launch_order_batch(fits_dev + c0, o.precision,
+                                   reinterpret_cast<const int4*>(ws + BL.off_assign) + l * kOrderSlots, groups->grid[l],
+                                   reinterpret_cast<const int*>(ws + BL.off_queue) + c0, groups->nqueue[l],
+                                   reinterpret_cast<unsigned*>(ws + BL.off_qhead) + l, bctl, st);
+            if (e != cudaSuccess) return e;
+            continue;
+        }
         e = launch_batch(fits_dev + c0, cnt, maxp, o.precision, fits[0].tile_rows, fits[0].tile_cols, bctl, nsm, st);
         if (e != cudaSuccess) return e;
     }
@@ -808,9 +870,20 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
     };
     // the pair-tile shape of the whole batch: the caller's, else the batch autotuner's for the
     // largest p and n (the FP64 path: 32 x 32)
-    const TileShape ts = batch_tile_shape(o, *std::max_element(P.begin(), P.end()), *std::max_element(N.begin(), N.end()));
+    const long long maxp = *std::max_element(P.begin(), P.end()), maxn = *std::max_element(N.begin(), N.end());
+    TileShape ts = batch_tile_shape(o, maxp, maxn);
+    // 1 x 1, a size the autotuner never measured, and the FP64 path without an explicit shape: the
+    // ordering kernel, where it takes every problem of the call
+    const bool untuned = o.tile_i == 0 && o.tile_j == 0 && !autotune_batch_measured(maxp, maxn);
+    bool order_kernel = o.reuse && (o.precision == LINGAM_MIXED ? ts.rows == 1 || untuned : o.tile_i <= 1 && o.tile_j <= 1);
+    for (int k = 0; k < count && order_kernel; ++k) {
+        const Layout L = make_layout(P[size_t(k)], N[size_t(k)], o.precision, o.input_dtype);
+        order_kernel = order_supported(make_fit(ws, L, int(P[size_t(k)]), int(N[size_t(k)]), o, false), true);
+    }
+    if (!order_kernel && ts.rows == 1) ts = TileShape{64, 16};
     mix(ts.rows);
     mix(ts.cols);
+    mix(order_kernel ? 1 : 0);
     for (int k = 0; k < count; ++k) {
         BatchItem& it = items[size_t(k)];
         char* base = ws + BL.region[size_t(k)];
@@ -820,6 +893,7 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
         f.ctl = reinterpret_cast<Ctl*>(ws + BL.off_ctls) + k;
         f.tile_rows = ts.rows;
         f.tile_cols = ts.cols;
+        f.split_n = 0;
         f.narrow = 0;   // the batch kernel runs every wave on the call's tile shape
         fits[size_t(k)] = f;
         SrcDesc sd;
@@ -847,6 +921,19 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
         mix(it.rep && it.rep->scores ? 1 : 0);
     }
     std::memcpy(H.data() + BL.off_rowoff + size_t(count) * sizeof(int), &rows, sizeof(int));
+    BatchGroups groups;
+    if (order_kernel) {
+        std::vector<int4> assign;
+        std::vector<int> queue;
+        for (int c0 = 0, l = 0; c0 < count; c0 += kBatchLaunchMax, ++l) {
+            order_batch_plan(fits.data() + c0, std::min(kBatchLaunchMax, count - c0), nsm, assign, queue);
+            std::memcpy(H.data() + BL.off_assign + size_t(l) * kOrderSlots * sizeof(int4), assign.data(), assign.size() * sizeof(int4));
+            if (!queue.empty())
+                std::memcpy(H.data() + BL.off_queue + size_t(c0) * sizeof(int), queue.data(), queue.size() * sizeof(int));
+            groups.grid.push_back(int(assign.size()));
+            groups.nqueue.push_back(int(queue.size()));
+        }
+    }
     std::memcpy(H.data() + BL.off_bctl, &c0, sizeof(Ctl));
     // the tables at the head of the header (the staging and bootstrap areas follow them)
     CKB(cudaMemcpyAsync(ws, H.data(), BL.off_stage_order, cudaMemcpyHostToDevice, st));
@@ -882,7 +969,7 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
     } else if (capture) {
         cudaGraph_t graph = nullptr;
         bool ok = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-        const cudaError_t eq = ok ? enqueue_batch(ws, BL, fits, Ls, o, rows, with_B, gather, nsm, st) : cudaErrorUnknown;
+        const cudaError_t eq = ok ? enqueue_batch(ws, BL, fits, Ls, o, order_kernel ? &groups : nullptr, rows, with_B, gather, nsm, st) : cudaErrorUnknown;
         if (ok) ok = cudaStreamEndCapture(st, &graph) == cudaSuccess && eq == cudaSuccess;
         if (ok) ok = cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess;
         if (graph) cudaGraphDestroy(graph);
@@ -901,10 +988,10 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
             }
             CKB(cudaGraphLaunch(exec, st));
         } else {
-            CKB(enqueue_batch(ws, BL, fits, Ls, o, rows, with_B, gather, nsm, st));
+            CKB(enqueue_batch(ws, BL, fits, Ls, o, order_kernel ? &groups : nullptr, rows, with_B, gather, nsm, st));
         }
     } else {
-        CKB(enqueue_batch(ws, BL, fits, Ls, o, rows, with_B, gather, nsm, st));
+        CKB(enqueue_batch(ws, BL, fits, Ls, o, order_kernel ? &groups : nullptr, rows, with_B, gather, nsm, st));
     }
     CKB(cudaStreamSynchronize(st));
 
