@@ -183,7 +183,9 @@ struct Fit {
     double* sigalt;      // [p x p] the other copy of the covariance (upper triangle)
     void* rec;           // sums of the current wave, per segment, row and column (8-byte values)
     unsigned long long rec_bytes;
+    int unit;            // samples of a warp's unit of work: 1024 or 512 (FP32), 256 (FP64)
     void* rowtab;        // [p] rows of the current wave (RowEnt)
+    int* gcount;         // [kOrderSlots] workers of a row group done with the wave
     double* dscale[2];   // [p] by variable, two copies: the normalised row is the residual times this
 };
 

@@ -49,10 +49,15 @@
 namespace lingam {
 
 constexpr int kMaxCols = 16;     // columns of a wave at most (four quads)
-// Samples of a block: FP32 32 per lane, one lg2 per residual; FP64 8 per lane (a block against four
-// columns then takes about 25 us of a SM's FP64 pipe, so that small fits still spread over the GPU).
+// A unit of a warp's work is 1024 or 512 samples on the FP32 path (32 or 16 per lane, one lg2 per
+// residual; Fit::unit: 512 for single fits of less than 4 M samples in all, whose waves keep few warps
+// busy), 256 samples on the FP64 path, of one row against quad() columns: four on the FP32 path (the
+// row's reads serve four pairs), one on the FP64 path, where a warp alone has only its SM quarter's
+// FP64 unit.  max_unit: what the shared memory is sized for.
 template <class T>
-__host__ __device__ constexpr int blk() { return sizeof(T) == 4 ? 1024 : 256; }
+__host__ __device__ constexpr int max_unit() { return sizeof(T) == 4 ? 1024 : 256; }
+template <class T>
+__host__ __device__ constexpr int quad() { return sizeof(T) == 4 ? 4 : 1; }
 constexpr int kRowBatch = 32;    // rows of a worker between two CTA barriers
 constexpr int kDedicated = 8;    // groups of this many CTAs or more have a controller that does not work
 
@@ -88,20 +93,19 @@ __device__ __forceinline__ RowEnt load_row(const RowEnt* t) {
 }
 
 // The wave word: sequence number (bits 51-63), done (50), removal (49), killers (48), columns
-// (42-46), rows (24-41), segments (0-15).
-__device__ __forceinline__ unsigned long long pack_order_wave(unsigned seq, int done, int removal, int kill, int ncol,
-                                                              int nrow, int nseg) {
-    return (static_cast<unsigned long long>(seq & 0x1fffu) << 51) | (static_cast<unsigned long long>(done) << 50) |
-           (static_cast<unsigned long long>(removal) << 49) | (static_cast<unsigned long long>(kill) << 48) |
-           (static_cast<unsigned long long>(ncol) << 42) | (static_cast<unsigned long long>(nrow) << 24) |
-           static_cast<unsigned long long>(nseg);
-}
+// (43-47), rows (30-42), the root to remove (16-29), segments (0-15).
 struct OrderWave {
-    int done, removal, kill, ncol, nrow, nseg;
+    int done, removal, kill, ncol, nrow, nseg, root;
 };
+__device__ __forceinline__ unsigned long long pack_order_wave(unsigned seq, const OrderWave& w) {
+    return (static_cast<unsigned long long>(seq & 0x1fffu) << 51) | (static_cast<unsigned long long>(w.done) << 50) |
+           (static_cast<unsigned long long>(w.removal) << 49) | (static_cast<unsigned long long>(w.kill) << 48) |
+           (static_cast<unsigned long long>(w.ncol) << 43) | (static_cast<unsigned long long>(w.nrow) << 30) |
+           (static_cast<unsigned long long>(w.root & 0x3fff) << 16) | static_cast<unsigned long long>(w.nseg);
+}
 __device__ __forceinline__ OrderWave unpack_order_wave(unsigned long long w) {
-    return {int((w >> 50) & 1), int((w >> 49) & 1), int((w >> 48) & 1), int((w >> 42) & 31), int((w >> 24) & 0x3ffff),
-            int(w & 0xffff)};
+    return {int((w >> 50) & 1), int((w >> 49) & 1), int((w >> 48) & 1), int((w >> 43) & 31), int((w >> 30) & 0x1fff),
+            int(w & 0xffff), int((w >> 16) & 0x3fff)};
 }
 
 // ------------------------------------------------------------------ sums
@@ -230,13 +234,13 @@ __device__ __forceinline__ void acc_self(AccD& a, double2 x, const double* tab) 
     acc_one(a, x.x, tab);
     acc_one(a, x.y, tab);
 }
-// Closes a warp's block: per residual i the lanes' centred log-cosh sum and their sum of u e^{-u^2/2}
+// Closes a warp's unit: per residual i the lanes' centred log-cosh sum and their sum of u e^{-u^2/2}
 // (FP32: of u' = kScale u), totals 2 i and 2 i + 1 in lane order (lane_value<2 N>).  off is the offset
 // of 32 samples and part the lane's share of them; its low mantissa bits are zero (var_offset), so
 // that the product is exact.  FP32: one lg2 per residual and lane.  FP64: the lanes' products are
 // multiplied first (at most 2^256 for 8 samples a lane) and each log is taken once per warp.
 template <int N>
-__device__ __forceinline__ float close_block(const Acc2 (&a)[N], const float (&off)[N], float part) {
+__device__ __forceinline__ float close_unit(const Acc2 (&a)[N], const float (&off)[N], float part) {
     float v[2 * N];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
@@ -246,7 +250,7 @@ __device__ __forceinline__ float close_block(const Acc2 (&a)[N], const float (&o
     return lane_totals<2 * N>(v);
 }
 template <int N>
-__device__ __forceinline__ double close_block(const AccD (&a)[N], const double (&off)[N], double part) {
+__device__ __forceinline__ double close_unit(const AccD (&a)[N], const double (&off)[N], double part) {
     double v[2 * N], pr[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
@@ -278,55 +282,51 @@ __device__ __forceinline__ double pair_scale(double om, double) { return 1.0 / s
 __device__ __forceinline__ float pair_offset(float off, float) { return off; }
 __device__ __forceinline__ double pair_offset(float, double) { return -double(kSub) * (kLn2 + kBeta); }
 
-// One block of one row against four columns: the 16 sums (per pair the row's residual's two, then
-// the column's two) in lane order.  m of the SPB steps of 32 V's; xg the old row at this lane, rs
-// the staged root, cs the staged columns (cstr elements apart), all at this lane's first sample.
-// The row's next two steps are loaded while two are evaluated.
-template <class T, class V>
-__device__ __forceinline__ T quad_block(const V* __restrict__ xg, const V* rs, const T* cs, int cstr, int m, T c, T inv,
-                                        const T* sc, T off_r, const T* offc, T part, const double* tab) {
-    typename AccOf<T>::Acc acc[8];
-    T s[4], sr[4];
+// One unit of one row against Q columns: the 4 Q sums (per pair the row's residual's two, then the
+// column's two) in lane order.  m steps of 32 V's; xg the old row at this lane, rs the staged root,
+// cs the staged columns (cstr elements apart), all at this lane's first sample.  The row is loaded two
+// steps ahead.  (One copy of the step's code: the kernel's size counts, every wave runs through most
+// of it once.)
+template <class T, class V, int Q>
+__device__ __forceinline__ T quad_unit(const V* __restrict__ xg, const V* rs, const T* cs, int cstr, int m, T c, T inv,
+                                       const T* sc, T off_r, const T* offc, T part, const double* tab) {
+    typename AccOf<T>::Acc acc[2 * Q];
+    T s[Q], sr[Q];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < Q; ++q) {
         s[q] = sc[2 * q];
         sr[q] = sc[2 * q + 1];
         acc_start(acc[2 * q]);
         acc_start(acc[2 * q + 1]);
     }
-    auto step = [&](V a, int k) {
-        const V u = reduce_root(a, rs[32 * k], c, inv);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const V w = *(reinterpret_cast<const V*>(cs + q * cstr) + 32 * k);
-            acc_pair(acc[2 * q], acc[2 * q + 1], u, w, s[q], sr[q], tab);
-        }
-    };
     V n0 = __ldcg(xg), n1 = n0;
     if (m > 1) n1 = __ldcg(xg + 32);
 #pragma unroll 1
-    for (int k = 0; k < m; k += 2) {
-        const V a0 = n0, a1 = n1;
-        if (k + 2 < m) n0 = __ldcg(xg + 32 * (k + 2));
-        if (k + 3 < m) n1 = __ldcg(xg + 32 * (k + 3));
-        step(a0, k);
-        if (k + 1 < m) step(a1, k + 1);
-    }
-    T off[8];
+    for (int k = 0; k < m; ++k) {
+        const V u = reduce_root(n0, rs[32 * k], c, inv);
+        n0 = n1;
+        if (k + 2 < m) n1 = __ldcg(xg + 32 * (k + 2));
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < Q; ++q) {
+            const V w = *(reinterpret_cast<const V*>(cs + q * cstr) + 32 * k);
+            acc_pair(acc[2 * q], acc[2 * q + 1], u, w, s[q], sr[q], tab);
+        }
+    }
+    T off[2 * Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
         off[2 * q] = off_r;
         off[2 * q + 1] = offc[q];
     }
-    return close_block<8>(acc, off, part);
+    return close_unit<2 * Q>(acc, off, part);
 }
 
-// One block of one row on its own: the row without the root is written to its new copy with its
+// One unit of one row on its own: the row without the root is written to its new copy with its
 // moments, and compared with its killer.  Eight sums: the killer pair's four, the row's two, 0, 0.
 template <class T, class V>
-__device__ __forceinline__ T single_block(const V* __restrict__ xg, const V* __restrict__ kg, const V* rs,
-                                          V* __restrict__ out, int m, T c, T inv, T kc, T kinv, T s, T sr, T off_r,
-                                          T off_k, T part, const double* tab) {
+__device__ __forceinline__ T own_unit(const V* __restrict__ xg, const V* __restrict__ kg, const V* rs, V* __restrict__ out,
+                                      int m, T c, T inv, T kc, T kinv, T s, T sr, T off_r, T off_k, T part,
+                                      const double* tab) {
     typename AccOf<T>::Acc acc[4];   // the row's and the killer's residual, the row, nothing
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc_start(acc[q]);
@@ -336,30 +336,28 @@ __device__ __forceinline__ T single_block(const V* __restrict__ xg, const V* __r
         k0 = __ldcg(kg);
         if (m > 1) k1 = __ldcg(kg + 32);
     }
-    auto step = [&](V a, V b, int k) {
-        const V r = rs[32 * k];
-        const V u = reduce_root(a, r, c, inv);
+#pragma unroll 1
+    for (int k = 0; k < m; ++k) {
+        const V r = rs[32 * k], u = reduce_root(n0, r, c, inv), y = k0;
+        n0 = n1;
+        k0 = k1;
+        if (k + 2 < m) {
+            n1 = __ldcg(xg + 32 * (k + 2));
+            if (kg) k1 = __ldcg(kg + 32 * (k + 2));
+        }
         out[32 * k] = u;
         acc_self(acc[2], u, tab);
-        if (kg) acc_pair(acc[0], acc[1], u, reduce_root(b, r, kc, kinv), s, sr, tab);
-    };
-#pragma unroll 1
-    for (int k = 0; k < m; k += 2) {
-        const V a0 = n0, a1 = n1, b0 = k0, b1 = k1;
-        if (k + 2 < m) {
-            n0 = __ldcg(xg + 32 * (k + 2));
-            if (kg) k0 = __ldcg(kg + 32 * (k + 2));
-        }
-        if (k + 3 < m) {
-            n1 = __ldcg(xg + 32 * (k + 3));
-            if (kg) k1 = __ldcg(kg + 32 * (k + 3));
-        }
-        step(a0, b0, k);
-        if (k + 1 < m) step(a1, b1, k + 1);
+        if (kg) acc_pair(acc[0], acc[1], u, reduce_root(y, r, kc, kinv), s, sr, tab);
     }
     const T off[4] = {off_r, off_k, off_r, T(0)};
-    return close_block<4>(acc, off, part);
+    return close_unit<4>(acc, off, part);
 }
+
+// 16 bytes from global to shared memory through L2, asynchronously.
+__device__ __forceinline__ void copy16_async(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(unsigned(__cvta_generic_to_shared(dst))), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // ------------------------------------------------------------------ the group and its memory
 struct Group {
@@ -371,43 +369,74 @@ struct Group {
 };
 
 // Controller state per variable slot (shared memory).
-constexpr size_t kSlotBytes = 16 + 8 + 4 * 11;
+constexpr size_t kSlotBytes = 16 + 8 + 4 * 10;
 // A worker's tables before the staged rows: the batch's rows and the columns, the pairs'
 // coefficients, the warps' sums, and the rows' and columns' coefficients and offsets.
 template <class T>
-__host__ __device__ constexpr size_t order_fixed_bytes(int nw) {
+__host__ __device__ constexpr int unit_slots() { return sizeof(T) == 4 ? 192 : 384; }   // units of a batch of rows
+template <class T>
+__host__ __device__ constexpr int slot_sums() { return 4 * quad<T>() > 8 ? 4 * quad<T>() : 8; }
+template <class T>
+__host__ __device__ constexpr size_t order_fixed_bytes() {
     return size_t(kRowBatch + kMaxCols) * sizeof(RowEnt) + size_t(kRowBatch) * (kMaxCols + 1) * 2 * sizeof(T) +
-           (size_t(kRowBatch) * (kMaxCols / 4 + 1) + nw) * 16 * 8 +
-           size_t(2 * kRowBatch + kMaxCols) * 3 * sizeof(double) +                       // S[root][v], D, new D
+           size_t(unit_slots<T>()) * slot_sums<T>() * sizeof(T) +
+           size_t(2 * kRowBatch + kMaxCols) * 2 * sizeof(double) +                       // S[root][v], new D
            (size_t(kRowBatch) * 6 + size_t(kMaxCols) * 4) * sizeof(T);
 }
-// Columns a wave may have with a work area of `cap` bytes and nrow rows: one block of the root and
+// Columns a wave may have with a work area of `cap` bytes and nrow rows: one unit of the root and
 // of the columns must fit beside the fixed tables, and the controller's I table (one T per row and
 // column or killer) into ctl_cap bytes.
 template <class T>
-__host__ __device__ inline int order_max_cols(size_t cap, int nw, int nrow, size_t ctl_cap) {
+__host__ __device__ inline int order_max_cols(unsigned cap, int nrow, unsigned ctl_cap) {
     for (int c = kMaxCols; c >= 4; c -= 4)
-        if (order_fixed_bytes<T>(nw) + size_t(c + 1) * blk<T>() * sizeof(T) <= cap && size_t(c + 1) * nrow * sizeof(T) <= ctl_cap)
+        if (unsigned(order_fixed_bytes<T>()) + unsigned((c + 1) * max_unit<T>()) * sizeof(T) <= cap &&
+            unsigned((c + 1) * nrow) * sizeof(T) <= ctl_cap)
             return c;
     return 0;
 }
 __host__ __device__ inline size_t order_state_bytes(int p) { return (size_t(p) * kSlotBytes + 127) / 128 * 128; }
 
-// Estimated SM clocks of a wave with nseg segments of the sample axis.  A worker evaluates its rows'
-// pairs at about 6 pair-samples a clock (FP64: one in 14 clocks), stages its columns at about 40
-// bytes a clock, and the controller reads every segment's sums (32 bytes a pair) at about 30.
+// Units of a staged pass of a worker with `us` units of the sample axis: as few passes as the work area
+// of `cap` bytes allows, of equal length.
 template <class T>
-__device__ __forceinline__ float seg_cost(int nseg, int nrow, int ncol, int W, int nblk, int extra) {
+__host__ __device__ inline int most_units(int ncol, int unit, unsigned cap) {
+    const int q = quad<T>(), nq = (ncol + q - 1) / q;
+    const int room = int((cap - unsigned(order_fixed_bytes<T>())) / (unsigned((nq * q + 1) * unit) * unsigned(sizeof(T))));
+    const int slots = unit_slots<T>() / (nq + 1);   // one row's units at least
+    return room < slots ? room : slots;
+}
+template <class T>
+__host__ __device__ inline int pass_units(int us, int ncol, int unit, unsigned cap) {
+    const int most = most_units<T>(ncol, unit, cap);
+    if (us <= most) return us;
+    const int passes = (us + most - 1) / most;
+    return (us + passes - 1) / passes;
+}
+// a / b for 0 <= a < 2^16, 0 < b (the quotient in FP32 is off by less than half of 1 / b).
+__device__ __forceinline__ int small_div(int a, int b) { return int(__fdividef(float(a) + 0.5f, float(b))); }
+
+// Estimated SM clocks of a wave with nseg segments of the sample axis.  A worker evaluates its rows'
+// pairs at about 5 pair-samples a clock (FP64: one in 14 clocks), stages its columns at about 40
+// bytes a clock in passes of about 12,000 clocks of their own, and several segments cost an exchange
+// between a row group's workers.
+template <class T>
+__device__ __forceinline__ float seg_cost(int nseg, int nrow, int ncol, int W, int nw, int nunit, int unit, int pass_most,
+                                          int extra) {
     constexpr bool f32 = sizeof(T) == 4;
-    const int groups = W / nseg;
-    const int rows = (nrow + groups - 1) / groups, blks = (nblk + nseg - 1) / nseg;
-    const int quads = (ncol + 3) / 4;
-    const float unit = (f32 ? 4.f / 6.f : 4.f * 14.f) * blk<T>();   // a block against four columns, at the SM's rate
-    const float lone = f32 ? 6.f * unit : unit;                    // and by one warp alone
-    const float work = fmaxf(float(rows) * blks * (quads * unit + extra * 0.5f * unit), lone);
-    const float stage = float(blks) * (ncol + 1) * (blk<T>() * sizeof(T) / 40.f);
-    const float merge = float(nseg) * nrow * (ncol + extra) * (32.f / 30.f);
-    return work + stage + merge;
+    const float groups = floorf(__fdividef(float(W) + 0.5f, float(nseg)));
+    const float rows = ceilf(__fdividef(float(nrow) - 0.5f, groups)), us = ceilf(__fdividef(float(nunit) - 0.5f, float(nseg)));
+    const int cols = (ncol + quad<T>() - 1) / quad<T>() * quad<T>();
+    const float one = (f32 ? 1.f / 5.f : 14.f) * unit;             // a unit of one pair, at the SM's rate
+    const int q = quad<T>();
+    // the warps' rounds of units, each a warp's unit at a sixteenth of that rate (a quarter at most)
+    const float nu = rows * us * (cols / q + extra), rounds = ceilf(__fdividef(nu, float(nw)));
+    const float conc = fminf(nu, float(nw));
+    const float work = fmaxf(rows * us * (float(cols) + extra * 2.f) * one, rounds * q * one * fmaxf(conc, 4.f));
+    const float stage = us * (ncol + 1) * (unit * sizeof(T) / 40.f);
+    const float passes = ceilf(__fdividef(us - 0.5f, float(pass_most))) * 12000.f;
+    // the segments' sums: added by the last worker of each row group
+    const float merge = nseg > 1 ? 4500.f + rows * (ncol + extra) * nseg * 0.3f : 0.f;
+    return work + stage + passes + merge;
 }
 
 // ------------------------------------------------------------------ a worker's part of a wave
@@ -433,50 +462,59 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
                                          const double* __restrict__ dold, double* __restrict__ dnew) {
     using V = typename OrderTraits<T>::V;
     using Sum = typename OrderTraits<T>::Sum;
-    constexpr int VN = OrderTraits<T>::VN, NW = NT / 32, STEP = 32 * VN, SPB = blk<T>() / STEP;
+    constexpr int VN = OrderTraits<T>::VN, NW = NT / 32, STEP = 32 * VN, Q = quad<T>();
+    constexpr int SLOT = slot_sums<T>();
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int p = f.p, ld = f.ld, nst = ld / STEP, nblk = (nst + SPB - 1) / SPB;
-    const int ncol = wv.ncol, nrow = wv.nrow, nseg = wv.nseg, nq = (ncol + 3) / 4;
+    const int p = f.p, ld = f.ld, unit = f.unit, spu = unit / STEP, nst = ld / STEP, nun = (nst + spu - 1) / spu;
+    const int ncol = wv.ncol, nrow = wv.nrow, nseg = wv.nseg, nq = (ncol + Q - 1) / Q;
     const bool rm = wv.removal != 0;
-    const int has_k = wv.removal;             // the rows' own blocks (new copy, moments, killer)
-    const int ntypes = nq + has_k, RECN = 16 * nq + 8 * has_k, np = ncol + has_k;
+    const int has_k = wv.removal;             // the rows' own units (new copy, moments, killer)
+    const int ntypes = nq + has_k, RECN = 4 * Q * nq + 8 * has_k, np = ncol + has_k;
     const RowEnt* tab = static_cast<const RowEnt*>(f.rowtab);
+    // the wave's sums: per segment (several segments or passes), then the totals of every row
     Sum* rec = static_cast<Sum*>(f.rec);
+    T* tot_out = reinterpret_cast<T*>(rec + size_t(nseg) * nrow * RECN);
     // shared memory
     unsigned char* work = smem_order + g.work;
     RowEnt* s_row = reinterpret_cast<RowEnt*>(work);
     RowEnt* s_col = s_row + kRowBatch;
     T* s_sc = reinterpret_cast<T*>(s_col + kMaxCols);                       // [row][kMaxCols + 1][2]
-    Sum* s_f = reinterpret_cast<Sum*>(s_sc + kRowBatch * (kMaxCols + 1) * 2);
+    T* s_f = s_sc + kRowBatch * (kMaxCols + 1) * 2;                           // [unit][SLOT]
     // per item (row j: j; its killer: kRowBatch + j; column c: 2 kRowBatch + c): S[root][v], new D
-    double* s_sr = reinterpret_cast<double*>(s_f + (size_t(kRowBatch) * (kMaxCols / 4 + 1) + NW) * 16);
+    double* s_sr = reinterpret_cast<double*>(s_f + unit_slots<T>() * SLOT);
     double* s_dn = s_sr + 2 * kRowBatch + kMaxCols;
-    T* s_rc = reinterpret_cast<T*>(s_dn + 2 * (2 * kRowBatch + kMaxCols));   // [row][4]: rho, inv, killer's
+    T* s_rc = reinterpret_cast<T*>(s_dn + 2 * kRowBatch + kMaxCols);         // [row][4]: rho, inv, killer's
     T* s_cc = s_rc + kRowBatch * 4;                                         // [column][2]: rho, inv
     T* s_offr = s_cc + kMaxCols * 2;                                        // [row][2]: offset, killer's
     T* s_offc = s_offr + kRowBatch * 2;                                     // [column]
-    T* s_root = reinterpret_cast<T*>(work + order_fixed_bytes<T>(NW));
+    T* s_root = reinterpret_cast<T*>(work + order_fixed_bytes<T>());
     const double* etab = reinterpret_cast<const double*>(smem_order + g.tab);
-    const int bp = min(nblk, int((g.cap - order_fixed_bytes<T>(NW)) / (size_t(4 * nq + 1) * blk<T>() * sizeof(T))));
-    const int cstr = bp * blk<T>();
+    const int ngr = small_div(g.W, nseg), grp = small_div(g.wk, nseg), seg = g.wk - grp * nseg;
+    const int b0 = nseg == 1 ? 0 : seg * nun / nseg, b1 = nseg == 1 ? nun : (seg + 1) * nun / nseg;
+    const int nr = grp < ngr && grp < nrow ? small_div(nrow - 1 - grp, ngr) + 1 : 0;
+    const int bp = pass_units<T>(b1 - b0, ncol, unit, g.cap);
+    const int cstr = bp * unit;
     T* s_cols = s_root + cstr;
 
-    const int ngr = g.W / nseg, grp = g.wk / nseg, seg = g.wk - grp * nseg;
-    const int b0 = seg * nblk / nseg, b1 = (seg + 1) * nblk / nseg;
-    const int nr = grp < ngr && grp < nrow ? (nrow - 1 - grp) / ngr + 1 : 0;
-    const int root = rm ? __ldcg(&f.ctl->rm_root) : -1;
+    const int root = wv.root;
     const double droot = rm ? __ldcg(dold + root) : 0.0;
-    const V* xroot = reinterpret_cast<const V*>(xold + size_t(rm ? root : 0) * ld);
-    for (int bs = b0; bs < b1 && nr > 0; bs += bp) {
+
+    if (nr == 0) return;
+
+#pragma unroll 1
+    for (int bs = b0; bs < b1; bs += bp) {
         const int nb = min(bp, b1 - bs);
-        for (int r0 = 0; r0 < nr; r0 += kRowBatch) {
-            const int nrb = min(kRowBatch, nr - r0);
+        const int rbatch = min(kRowBatch, small_div(unit_slots<T>(), ntypes * nb));   // rows whose units have slots
+#pragma unroll 1
+        for (int r0 = 0; r0 < nr; r0 += rbatch) {
+            const int nrb = min(rbatch, nr - r0);
+            const bool stage = r0 == 0;
             if (tid < nrb) {
                 const RowEnt e = load_row(tab + grp + (r0 + tid) * ngr);
                 s_row[tid] = e;
                 s_offr[2 * tid] = pair_offset(e.off, T());
                 s_offr[2 * tid + 1] = pair_offset(e.koff, T());
-            } else if (tid >= 64 && tid < 64 + kMaxCols && r0 == 0 && bs == b0) {
+            } else if (tid >= 64 && tid < 64 + kMaxCols && stage && bs == b0) {
                 const int c = tid - 64;
                 RowEnt e = {-1, 0.f, -1, 0.f};
                 if (c < ncol) e = load_row(tab + c);
@@ -484,16 +522,20 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
                 s_offc[c] = pair_offset(e.off, T());
             }
             __syncthreads();   // the tables are there; the previous batch's sums were read
-            // everything that depends on the tables alone is loaded before the coefficients are
-            // formed: this thread's covariance elements and its first samples of root and columns
-            const int base = bs * SPB * 32, nv = min(nb * SPB, nst - bs * SPB) * 32;
-            const bool stage = r0 == 0;
-            V pr = zero_of(V()), px[4];
-            if (stage && tid < nv) {
-                if (rm) pr = __ldcg(xroot + base + tid);
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    if (q < ncol) px[q] = __ldcg(reinterpret_cast<const V*>(xold + size_t(s_col[q].var) * ld) + base + tid);
+            // everything that depends on the tables alone is in flight before the coefficients are
+            // formed: the segment of the root and of the columns, and the covariance's elements
+            const int base = bs * spu * 32, nv = min(nb * spu, nst - bs * spu) * 32;
+            if (stage) {
+#pragma unroll 1
+                for (int t = tid; t < nv; t += NT) {
+                    V* dst = reinterpret_cast<V*>(s_root) + t;
+                    if (rm) copy16_async(dst, reinterpret_cast<const V*>(xold + size_t(root) * ld) + base + t);
+                    else *dst = zero_of(V());
+#pragma unroll 1
+                    for (int c = 0; c < ncol; ++c)
+                        copy16_async(reinterpret_cast<V*>(s_cols + c * cstr) + t,
+                                     reinterpret_cast<const V*>(xold + size_t(s_col[c].var) * ld) + base + t);
+                }
             }
             // the pairs: row j against column c (c == ncol: its killer)
             constexpr int PU = (kRowBatch * (kMaxCols + 1) + NT - 1) / NT;
@@ -501,30 +543,60 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
             int pu[PU];   // the pair's row and item, or -1
 #pragma unroll
             for (int q = 0; q < PU; ++q) {
-                const int u = tid + q * NT, j = u / np, c = u - j * np, e = grp + (r0 + j) * ngr;
+                const int u = tid + q * NT;
                 pu[q] = -1;
                 if (u < nrb * np) {
+                    const int j = small_div(u, np), c = u - j * np, e = grp + (r0 + j) * ngr;
                     const bool kill = c == ncol;
                     const int vi = s_row[j].var, vj = kill ? s_row[j].kvar : s_col[c].var;
                     if (vj >= 0 && (kill || (f.reuse ? e >= ncol || c < e : e != c)) &&
                         LINGAM_INBOUNDS(f.ctl, vi >= 0 && vi < p && vj < p)) {
                         pu[q] = j | (kill ? kMaxCols : c) << 8;
-                        pc[q] = __ldcg(sold + size_t(min(vi, vj)) * p + max(vi, vj));
+                        pc[q] = __ldcg(sold + min(vi, vj) * p + max(vi, vj));
                     }
                 }
             }
+            // UpdateCovMat (Eq. CovUpdate) on S, FP64, upper triangle by variable index, into the other
+            // copy: S[w][j] - S[w][root] S[j][root] / S[root][root] for the batch's rows w and every j > w
+            // (of a removed j the element is never read again), in chunks of 32 elements a warp; the
+            // segments' workers share a row's chunks.  Four of a warp's chunks are in flight, the first here.
+            const int nch = (p + 31) >> 5, mych = small_div(nch + nseg - 1 - seg, nseg);   // chunks seg, seg + nseg, ...
+            int ci = small_div(wid, mych > 0 ? mych : 1), cc = wid - ci * mych;
+            const bool cov = rm && bs == b0 && mych > 0;
+            int cat[4], crow[4];
+            double ca[4], cb[4];
+            auto load_chunks = [&]() {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    cat[q] = -1;
+                    if (cov && ci < nrb) {
+                        const int w = s_row[ci].var, j = (seg + cc * nseg) * 32 + lane;
+                        crow[q] = ci;
+                        if (j > w && j < p) {
+                            cat[q] = w * p + j;   // (p <= 4096)
+                            ca[q] = __ldcg(sold + cat[q]);
+                            cb[q] = __ldcg(sold + min(j, root) * p + max(j, root));
+                        }
+                        cc += NW;
+                        while (cc >= mych) {
+                            cc -= mych;
+                            ++ci;
+                        }
+                    } else {
+                        crow[q] = -1;
+                    }
+                }
+            };
+            load_chunks();
             // the rows', killers' and columns' removal coefficients (FP64)
-            if (tid < 2 * kRowBatch + kMaxCols) {
-                const int k = tid;
-                int v = -1;
-                if (k < kRowBatch) v = k < nrb ? s_row[k].var : -1;
-                else if (k < 2 * kRowBatch) v = k - kRowBatch < nrb && has_k ? s_row[k - kRowBatch].kvar : -1;
-                else v = s_col[k - 2 * kRowBatch].var;
+            if (tid < 2 * nrb + ncol) {
+                const int k = tid < nrb ? tid : tid < 2 * nrb ? kRowBatch + tid - nrb : 2 * kRowBatch + tid - 2 * nrb;
+                const int v = k < kRowBatch ? s_row[k].var : k < 2 * kRowBatch ? s_row[k - kRowBatch].kvar : s_col[k - 2 * kRowBatch].var;
                 double sr = 0.0, d = 0.0, rho = 0.0, inv = 1.0;
                 if (v >= 0) {
                     d = __ldcg(dold + v);
                     if (rm) {
-                        sr = __ldcg(sold + size_t(min(v, root)) * p + max(v, root));
+                        sr = __ldcg(sold + min(v, root) * p + max(v, root));
                         rho = sr * (d * droot);
                         double om = fma(-rho, rho, 1.0);
                         if (!(om > degenerate_om(sizeof(T) == 4))) {
@@ -563,142 +635,100 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
                     sc[0] = s;
                     sc[1] = s * T(rho);
                 }
+            while (crow[0] >= 0) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (cat[q] >= 0) snew[cat[q]] = fma(-s_sr[crow[q]] * dr2, cb[q], ca[q]);
+                load_chunks();
+            }
             if (stage) {
-                // the segment of the root and of the columns, without the root
-                for (int t = tid; t < nv; t += NT) {
-                    const bool first = t == tid;
-                    const V r = first ? pr : rm ? __ldcg(xroot + base + t) : zero_of(V());
-                    reinterpret_cast<V*>(s_root)[t] = r;
+                // the columns without the root (each thread the vectors it copied)
+                copy_wait();
+                if (rm) {
 #pragma unroll 1
-                    for (int c0 = 0; c0 < ncol; c0 += 4) {
-                        V x[4];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            if (first && c0 == 0) x[q] = px[q];
-                            else if (c0 + q < ncol)
-                                x[q] = __ldcg(reinterpret_cast<const V*>(xold + size_t(s_col[c0 + q].var) * ld) + base + t);
+                    for (int t = tid; t < nv; t += NT) {
+                        const V r = reinterpret_cast<const V*>(s_root)[t];
+#pragma unroll 1
+                        for (int c = 0; c < ncol; ++c) {
+                            V* x = reinterpret_cast<V*>(s_cols + c * cstr) + t;
+                            *x = reduce_root(*x, r, s_cc[2 * c], s_cc[2 * c + 1]);
                         }
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            if (c0 + q < ncol)
-                                reinterpret_cast<V*>(s_cols + size_t(c0 + q) * cstr)[t] =
-                                    reduce_root(x[q], r, s_cc[2 * (c0 + q)], s_cc[2 * (c0 + q) + 1]);
                     }
                 }
             }
             __syncthreads();
-            // the blocks of all rows, in the order (row, quad or own, block), spread over the
-            // warps by cost (a quad 4, an own block 2)
-            const int qcost = 4 * nq * nb, rcost = qcost + 2 * has_k * nb, total = nrb * rcost;
-            {
-                const int lo = wid * total / NW, hi = (wid + 1) * total / NW;
-                int j = lo / rcost, u;
-                {
-                    const int rem = lo - j * rcost;
-                    u = rem <= qcost ? (rem + 3) / 4 : nq * nb + (rem - qcost + 1) / 2;
-                    if (u >= ntypes * nb) {
-                        u = 0;
-                        ++j;
-                    }
+            // the units of all rows, first those against columns (row, quad, unit of the segment), then
+            // the rows' own, dealt out to the warps in turn; each leaves its sums in a slot
+            const int nQ = nrb * nq * nb, nU = nQ + nrb * has_k * nb;
+            for (int i = wid; i < nU; i += NW) {
+                const bool own = i >= nQ;
+                const int g2 = small_div(own ? i - nQ : i, nb), b = (own ? i - nQ : i) - g2 * nb;   // (row, quad) or row
+                const int j = own ? g2 : small_div(g2, nq), t = own ? 0 : g2 - j * nq;
+                const int st0 = (bs + b) * spu, m = min(spu, nst - st0);
+                const T part = T(m) * (T(VN) / T(kSub));   // a lane's samples, of 32
+                const T c = s_rc[4 * j], inv = s_rc[4 * j + 1], off_r = s_offr[2 * j];
+                const V* xg = reinterpret_cast<const V*>(xold + size_t(s_row[j].var) * ld) + st0 * 32 + lane;
+                const V* rs = reinterpret_cast<const V*>(s_root) + b * spu * 32 + lane;
+                if (!own) {
+                    const T* cs = s_cols + (Q * t) * cstr + (b * spu * 32 + lane) * VN;
+                    const T tot = quad_unit<T, V, Q>(xg, rs, cs, cstr, m, c, inv, s_sc + (j * (kMaxCols + 1) + Q * t) * 2,
+                                                     off_r, s_offc + Q * t, part, etab);
+                    if ((lane & (32 / (4 * Q) - 1)) == 0) s_f[i * SLOT + lane_value<4 * Q>()] = tot;
+                } else {
+                    const int kv = s_row[j].kvar;
+                    const V* kg = kv >= 0 ? reinterpret_cast<const V*>(xold + size_t(kv) * ld) + st0 * 32 + lane : nullptr;
+                    V* out = reinterpret_cast<V*>(xnew + size_t(s_row[j].var) * ld) + st0 * 32 + lane;
+                    const T* sk = s_sc + (j * (kMaxCols + 1) + kMaxCols) * 2;
+                    const T tot = own_unit<T, V>(xg, kg, rs, out, m, c, inv, s_rc[4 * j + 2], s_rc[4 * j + 3], sk[0], sk[1],
+                                                 off_r, s_offr[2 * j + 1], part, etab);
+                    if ((lane & 3) == 0) s_f[i * SLOT + lane_value<8>()] = tot;
                 }
-                int gcur = -1;
-                Sum acc = sum_of(T(0));
-                auto flush = [&]() {
-                    if (gcur < 0) return;
-                    const bool own = gcur % ntypes == nq;
-                    const int idx = own ? lane_value<8>() : lane_value<16>();
-                    if ((lane & (own ? 3 : 1)) == 0) s_f[(gcur + wid) * 16 + idx] = acc;
-                };
-                while (j < nrb) {
-                    const int start = j * rcost + (u < nq * nb ? 4 * u : qcost + 2 * (u - nq * nb));
-                    if (start >= hi) break;
-                    const int t = u / nb, b = u - t * nb;
-                    const int gi = j * ntypes + t;
-                    if (gi != gcur) {
-                        flush();
-                        gcur = gi;
-                        acc = sum_of(T(0));
-                    }
-                    const int st0 = (bs + b) * SPB, m = min(SPB, nst - st0);
-                    const T part = T(m) * T(1.0 / (SPB == 8 ? 8 : 16));   // of 32 samples a lane
-                    const RowEnt ri = s_row[j];
-                    const T c = s_rc[4 * j], inv = s_rc[4 * j + 1], off_r = s_offr[2 * j];
-                    const V* xg = reinterpret_cast<const V*>(xold + size_t(ri.var) * ld) + st0 * 32 + lane;
-                    const V* rs = reinterpret_cast<const V*>(s_root) + b * SPB * 32 + lane;
-                    T tot;
-                    if (t < nq) {
-                        const T* cs = s_cols + (4 * t) * cstr + (b * SPB * 32 + lane) * VN;
-                        tot = quad_block<T, V>(xg, rs, cs, cstr, m, c, inv, s_sc + (j * (kMaxCols + 1) + 4 * t) * 2,
-                                                    off_r, s_offc + 4 * t, part, etab);
-                    } else {
-                        const V* kg = ri.kvar >= 0
-                                          ? reinterpret_cast<const V*>(xold + size_t(ri.kvar) * ld) + st0 * 32 + lane
-                                          : nullptr;
-                        V* out = reinterpret_cast<V*>(xnew + size_t(ri.var) * ld) + st0 * 32 + lane;
-                        const T* sk = s_sc + (j * (kMaxCols + 1) + kMaxCols) * 2;
-                        tot = single_block<T, V>(xg, kg, rs, out, m, c, inv, s_rc[4 * j + 2], s_rc[4 * j + 3], sk[0],
-                                                      sk[1], off_r, s_offr[2 * j + 1], part, etab);
-                    }
-                    acc = sum_add(acc, sum_of(tot));
-                    if (++u == ntypes * nb) {
-                        u = 0;
-                        ++j;
-                    }
-                }
-                flush();
             }
             __syncthreads();
-            // the warps' sums of each (row, quad or own) in warp order, to the wave's records
+            // the units' sums of each (row, quad or own) in order, to the wave's records
             for (int x = tid; x < nrb * RECN; x += NT) {
-                const int j = x / RECN, v = x - j * RECN;
-                const int t = min(v >> 4, nq), val = v - 16 * t;
-                const int step = t < nq ? 4 : 2;
-                const int s0 = j * rcost + (t < nq ? 4 * t * nb : qcost), s1 = s0 + step * (nb - 1);
-                const int w0 = ((s0 + 1) * NW + total - 1) / total - 1, w1 = ((s1 + 1) * NW + total - 1) / total - 1;
-                const int gi = j * ntypes + t;
-                Sum s = s_f[(gi + w0) * 16 + val];
-                for (int w = w0 + 1; w <= w1; ++w) {
-                    // (a warp whose share of the costs holds no block's start has no sum)
-                    const int lo = w * total / NW, hi = (w + 1) * total / NW;
-                    const int first = s0 + (lo - s0 + step - 1) / step * step;
-                    if (first < hi) s = sum_add(s, s_f[(gi + w) * 16 + val]);
-                }
+                const int j = small_div(x, RECN), v = x - j * RECN;
+                const int t = min(v / (4 * Q), nq), val = v - 4 * Q * t;
+                const T* src = s_f + ((t < nq ? (j * nq + t) * nb : nQ + j * nb)) * SLOT + val;
+                Sum s = sum_of(src[0]);
+                for (int b = 1; b < nb; ++b) s = sum_add(s, sum_of(src[b * SLOT]));
                 const int e = grp + (r0 + j) * ngr;
                 const size_t at = (size_t(seg) * nrow + e) * RECN + v;
-                if (LINGAM_INBOUNDS(f.ctl, (at + 1) * sizeof(Sum) <= f.rec_bytes))
-                    rec[at] = bs == b0 ? s : sum_add(rec[at], s);
+                if (LINGAM_INBOUNDS(f.ctl, (at + 1) * sizeof(Sum) <= f.rec_bytes)) {
+                    if (bs != b0) s = sum_add(rec[at], s);
+                    if (nseg > 1 || bs + bp < b1) rec[at] = s;
+                    else tot_out[e * RECN + v] = sum_val(s);
+                }
             }
         }
     }
-    // UpdateCovMat (Eq. CovUpdate) on S, FP64, upper triangle by variable index, into the other copy:
-    // S[w][j] - S[w][root] S[j][root] / S[root][root] for this worker's rows w of the remaining
-    // variables and every j > w (of a removed j the element is never read again).  Eight elements of a
-    // thread in flight.
-    if (rm) {
-        const double dr2 = droot * droot;
-        const int mine = g.wk < nrow ? (nrow - 1 - g.wk) / g.W + 1 : 0;
-        constexpr int CB = 8;
-        for (int i0 = 0; i0 < mine * p; i0 += CB * NT) {
-            int at_w[CB], at_j[CB];
+    // several segments: the last of a row group's workers to get here adds them
+    if (nseg > 1) {
+        __shared__ int s_last;
+        int* count = f.gcount + grp;
+        __syncthreads();
+        if (tid == 0) {
+            s_last = atom_add_acq_rel(count, 1) == nseg - 1;
+            if (s_last) *count = 0;   // for the next wave
+        }
+        __syncthreads();
+        if (!s_last) return;
+        for (int x = tid; x < nr * RECN; x += NT) {
+            const int j = x < 0x10000 ? small_div(x, RECN) : x / RECN, v = x - j * RECN, e = grp + j * ngr;
+            const Sum* src = rec + size_t(e) * RECN + v;
+            const size_t stride = size_t(nrow) * RECN;
+            Sum s = Sum();
+            int k = 0;
+            for (; k + 8 <= nseg; k += 8) {
+                Sum y[8];
 #pragma unroll
-            for (int q = 0; q < CB; ++q) {
-                const int i = i0 + q * NT + tid, row = i / p;
-                at_j[q] = i - row * p;
-                at_w[q] = row < mine ? __ldcg(&tab[g.wk + row * g.W].var) : p;
+                for (int q = 0; q < 8; ++q) y[q] = __ldcg(src + (k + q) * stride);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) s = sum_add(s, y[q]);
             }
-            double a[CB], b[CB], c[CB];
-#pragma unroll
-            for (int q = 0; q < CB; ++q) {
-                const int w = at_w[q], j = at_j[q];
-                if (j > w) {
-                    a[q] = __ldcg(sold + size_t(w) * p + j);
-                    b[q] = __ldcg(sold + size_t(min(w, root)) * p + max(w, root));
-                    c[q] = __ldcg(sold + size_t(min(j, root)) * p + max(j, root));
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < CB; ++q)
-                if (at_j[q] > at_w[q]) snew[size_t(at_w[q]) * p + at_j[q]] = fma(-b[q] * dr2, c[q], a[q]);
+#pragma unroll 2
+            for (; k < nseg; ++k) s = sum_add(s, __ldcg(src + k * stride));
+            tot_out[e * RECN + v] = sum_val(s);
         }
     }
 }
@@ -740,27 +770,46 @@ __device__ __forceinline__ unsigned key_bits(float x) {
 }
 constexpr unsigned kNoKey = 0xffffffffu;
 
+// What the controller keeps between waves, the same for all its threads.
+struct CtlState {
+    int r, a, it, cmax, want, bestv;
+    long long best;   // key of the iteration's lowest complete score
+    double gamma;
+    OrderWave wave;   // the next wave
+};
 struct OrderShared {
+    CtlState st;
     unsigned long long word;
-    int ok, nseg, npick, root;
-    int qnext;
+    int ok, nseg, npick, qnext;
     long long col[kMaxCols];      // the wave's complete scores (keys)
     unsigned ckey[16 * kMaxCols];
-    int cslot[16 * kMaxCols];
-    int pick[kMaxCols];
+    int cvar[16 * kMaxCols];
     long long lred[16];
     int ired[16], nkill[16];
-    long long rootpt;
+    // to be reported once the next wave is published
+    int rep_ncol, rep_nrow, rep_nw, rep_it, rep_root, rep_bestv;
+    long long rep_best, rep_rootpt;
 };
 
-// Four sums of one record, and their sum over the segments first, first + step, ... (four segments'
-// loads in flight).
-__device__ __forceinline__ void load4(float2 (&v)[4], const float2* p) {
-    const float4 a = __ldcg(reinterpret_cast<const float4*>(p)), b = __ldcg(reinterpret_cast<const float4*>(p) + 1);
-    v[0] = make_float2(a.x, a.y);
-    v[1] = make_float2(a.z, a.w);
-    v[2] = make_float2(b.x, b.y);
-    v[3] = make_float2(b.z, b.w);
+// Barrier of the controller's first `nt` threads (a multiple of 32), and with an "or" over them.
+__device__ __forceinline__ void part_bar(int nt) { asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory"); }
+__device__ __forceinline__ int part_or(int nt, int v) {
+    int out;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\tbar.red.or.pred q, 1, %2, p;\n\tselp.s32 %0, 1, 0, q;\n\t}"
+        : "=r"(out)
+        : "r"(v), "r"(nt)
+        : "memory");
+    return out;
+}
+
+// Four totals of a record.
+__device__ __forceinline__ void load4(float (&v)[4], const float* p) {
+    const float4 a = __ldcg(reinterpret_cast<const float4*>(p));
+    v[0] = a.x;
+    v[1] = a.y;
+    v[2] = a.z;
+    v[3] = a.w;
 }
 __device__ __forceinline__ void load4(double (&v)[4], const double* p) {
     const double2 a = __ldcg(reinterpret_cast<const double2*>(p)), b = __ldcg(reinterpret_cast<const double2*>(p) + 1);
@@ -768,27 +817,6 @@ __device__ __forceinline__ void load4(double (&v)[4], const double* p) {
     v[1] = a.y;
     v[2] = b.x;
     v[3] = b.y;
-}
-template <class Sum>
-__device__ __forceinline__ void sum_segments(Sum (&s)[4], const Sum* p, size_t stride, int nseg, int first, int step) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) s[k] = Sum();
-    int i = first;
-    for (; i + 3 * step < nseg; i += 4 * step) {
-        Sum v[4][4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) load4(v[q], p + size_t(i + q * step) * stride);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) s[k] = sum_add(s[k], v[q][k]);
-    }
-    for (; i < nseg; i += step) {
-        Sum v[4];
-        load4(v, p + size_t(i) * stride);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) s[k] = sum_add(s[k], v[k]);
-    }
 }
 
 // The 32-sample offset of a variable from its 2 (m - beta).
@@ -798,12 +826,14 @@ __device__ __forceinline__ float stat_offset(float y) {
 
 // Slots 0 .. r - 1 hold the remaining variables: first those that were columns in this iteration's
 // earlier waves (a of them), then the current wave's columns, then the others; so the current
-// wave's rows are the slots a .. r - 1.  Every thread holds the same r, a, it, best, ...
+// wave's rows are the slots a .. r - 1.  Only the first nt threads take part once the pairs' measures
+// are formed (two slots a thread, four warps at least): the steps are chains of short dependent
+// operations, which idle warps would only slow down.
 template <class T, int NT>
 struct Controller {
     using Sum = typename OrderTraits<T>::Sum;
     static constexpr bool f32 = std::is_same<T, float>::value;
-    static constexpr int NW = NT / 32;
+    static constexpr int NW = NT / 32, Q = quad<T>();
     const Fit& f;
     const Group& g;
     OrderShared& sh;
@@ -813,7 +843,6 @@ struct Controller {
     float* kc;        // the killer pair's contribution of this iteration
     float* kv0;       // the two largest known contributions, and their partners
     float* kv1;
-    float* key;       // the next iteration's candidate order
     int* keval;       // the killer that was compared (-1: none)
     int* kp0;
     int* kp1;
@@ -822,15 +851,15 @@ struct Controller {
     int* fl;          // kNoRoot
     int* row;         // candidate keys of a selection
     T* I;             // the wave's pair measures
-    size_t icap;
-    int r, a, it, iters, cmax, want;
+    unsigned icap;
+    int iters;
     bool gmode, prunes;
-    long long best;   // key of the iteration's lowest complete score
-    int bestv;
-    long long pairs;
-    double gamma;
+    int r, a, it, nt;
+    // thread 0: counters
+    int waves = 0;
+    long long pairs = 0, total = 0, gsteps = 0;
 
-    __device__ __forceinline__ Controller(const Fit& f_, const Group& g_, OrderShared& sh_, size_t smem_bytes, int iters_)
+    __device__ __forceinline__ Controller(const Fit& f_, const Group& g_, OrderShared& sh_, unsigned smem_bytes, int iters_)
         : f(f_), g(g_), sh(sh_) {
         const int p = f.p;
         st = reinterpret_cast<float4*>(smem_order);
@@ -838,72 +867,71 @@ struct Controller {
         kc = reinterpret_cast<float*>(part + p);
         kv0 = kc + p;
         kv1 = kv0 + p;
-        key = kv1 + p;
-        keval = reinterpret_cast<int*>(key + p);
+        keval = reinterpret_cast<int*>(kv1 + p);
         kp0 = keval + p;
         kp1 = kp0 + p;
         var = kp1 + p;
         slot = var + p;
         fl = slot + p;
         row = fl + p;
-        const size_t state = order_state_bytes(p);
+        const unsigned state = unsigned(order_state_bytes(p));
         I = reinterpret_cast<T*>(smem_order + state);
         icap = smem_bytes - state;
         iters = iters_;
         prunes = f.prune && f.reuse;
         gmode = f.gamma0 > 0.0 && prunes;
-        want = kMaxCols;
-        cmax = order_max_cols<T>(g.cap, NW, p, icap);
         r = p;
         a = it = 0;
-        new_iteration();
+        nt = NT;
     }
-    __device__ __forceinline__ void new_iteration() {
-        best = kMaxScore;
-        bestv = -1;
-        pairs = 0;
-        gamma = f.gamma0;
-    }
+    __device__ __forceinline__ int max_cols(int nrow) const { return order_max_cols<T>(g.cap, nrow, icap); }
+    __device__ __forceinline__ void bar() const { part_bar(nt); }
 
     // The slot of a wave's row (without pair reuse the rows are all variables, the columns first).
     __device__ __forceinline__ int row_slot(int e) const { return a + e < r ? a + e : a + e - r; }
-    // Exchanges two slots (one warp; a lane per array).
-    __device__ __forceinline__ void swap_slots(int x, int y) {
-        if (x == y) return;
-        const int lane = threadIdx.x & 31;
-        const int vx = var[x], vy = var[y];
-        __syncwarp();
-        if (lane == 0) {
+    // Exchanges two slots, array `what` of the ten (the 4-byte arrays kc .. var, and fl, lie one after
+    // another); the variables' slots are not updated.
+    __device__ __forceinline__ void swap_part(int what, int x, int y) {
+        if (what == 0) {
             const float4 t = st[x];
             st[x] = st[y];
             st[y] = t;
-        } else if (lane == 1) {
+        } else if (what == 1) {
             const Sum t = part[x];
             part[x] = part[y];
             part[y] = t;
-        } else if (lane < 11) {   // the 4-byte arrays kc .. var but slot, and fl, lie one after another
-            int* q = reinterpret_cast<int*>(kc) + size_t(lane < 10 ? lane - 2 : 9) * f.p;
+        } else {
+            int* q = reinterpret_cast<int*>(kc) + (what < 9 ? what - 2 : 8) * f.p;
             const int t = q[x];
             q[x] = q[y];
             q[y] = t;
-        } else if (lane == 11) {
-            slot[vx] = y;
-        } else if (lane == 12) {
-            slot[vy] = x;
         }
+    }
+    // Exchanges two slots (one warp).
+    __device__ __forceinline__ void swap_slots(int x, int y) {
+        if (x == y) return;
+        const int lane = threadIdx.x & 31;
+        if (lane < 10) swap_part(lane, x, y);
+        __syncwarp();
+        if (lane < 2) slot[var[lane ? y : x]] = lane ? y : x;
         __syncwarp();
     }
 
     // The `n` slots of [lo, hi) of lowest key (row[k]: the key's bits, kNoKey not a candidate), lowest
     // first, to the positions lo, lo + 1, ...; sh.npick of them.  Each warp takes its lowest by warp
-    // minima, the first warp the lowest of those.  All threads.
-    __device__ __forceinline__ void select_lowest(int lo, int hi, int n) {
+    // minima, the first warp the lowest of those.  drop >= 0: that slot leaves first (to position hi;
+    // not a candidate).  Ends with a barrier.
+    __device__ __forceinline__ void select_lowest(int lo, int hi, int n, int drop) {
         const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-        __syncthreads();
-        for (int i = 0; i < n; ++i) {
+        const int end = drop >= 0 ? hi + 1 : hi;
+        const int sw = end - lo <= 256 ? 1 : nt >> 5;   // selecting warps
+#pragma unroll 1
+#pragma unroll 1
+        for (int i = 0; i < n && wid < sw; ++i) {
             unsigned b = kNoKey;
             int at = -1;
-            for (int k = lo + tid; k < hi; k += NT) {
+#pragma unroll 1
+            for (int k = lo + tid; k < end; k += 32 * sw) {
                 const unsigned v = unsigned(row[k]);
                 if (v < b) {
                     b = v;
@@ -912,6 +940,7 @@ struct Controller {
             }
             const unsigned m = __reduce_min_sync(0xffffffffu, b);
             if (m == kNoKey) {
+#pragma unroll 1
                 for (int q = i + lane; q < n; q += 32) sh.ckey[wid * kMaxCols + q] = kNoKey;
                 break;
             }
@@ -919,34 +948,69 @@ struct Controller {
             if (lane == src) {
                 row[at] = int(kNoKey);
                 sh.ckey[wid * kMaxCols + i] = m;
-                sh.cslot[wid * kMaxCols + i] = var[at];
+                sh.cvar[wid * kMaxCols + i] = var[at];
             }
             __syncwarp();
         }
-        __syncthreads();
+        if (sw > 1) bar();
         if (wid == 0) {
-            int pos = 0, got = 0;
-            for (; got < n; ++got) {   // lane w walks the ascending list of warp w
-                const unsigned v = lane < NW && pos < n ? sh.ckey[lane * kMaxCols + pos] : kNoKey;
+            if (drop >= 0) swap_slots(drop, hi);
+            int pos = 0, got = 0, pick = 0;   // lane i: the i-th pick's slot
+#pragma unroll 1
+            for (; got < n; ++got) {          // lane w walks the ascending list of warp w
+                const unsigned v = lane < sw && pos < n ? sh.ckey[lane * kMaxCols + pos] : kNoKey;
                 const unsigned m = __reduce_min_sync(0xffffffffu, v);
                 if (m == kNoKey) break;
                 const int src = __ffs(__ballot_sync(0xffffffffu, v == m)) - 1;
-                int c = lane == src ? sh.cslot[lane * kMaxCols + pos] : 0;
+                int c = lane == src ? sh.cvar[lane * kMaxCols + pos] : 0;
                 if (lane == src) ++pos;
                 c = __shfl_sync(0xffffffffu, c, src);
-                swap_slots(lo + got, slot[c]);
+                if (lane == got) pick = slot[c];
+            }
+            // the picks behind the first `got` slots change places with the slots among those that
+            // were not picked: exchanges of different pairs of slots, three at a time
+            const bool mine = lane < got, front = mine && pick < lo + got;
+            const unsigned infront = __reduce_or_sync(0xffffffffu, front ? 1u << (pick - lo) : 0u);
+            const unsigned back = __ballot_sync(0xffffffffu, mine && !front);
+            unsigned holes = ((1u << got) - 1u) & ~infront;
+            const int rank = __popc(back & ((1u << lane) - 1u));
+            int hole = 0;   // lane of a back pick: its place
+#pragma unroll 1
+            for (int i = 0; i <= rank && holes; ++i) {
+                hole = __ffs(holes) - 1;
+                holes &= holes - 1u;
+            }
+            const int group = lane < 30 ? lane / 10 : 3, what = lane - 10 * group;
+#pragma unroll 1
+            for (unsigned left = back; left;) {
+                int src = -1;
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    if (left) {
+                        if (group == q) src = __ffs(left) - 1;
+                        left &= left - 1u;
+                    }
+                const int x = __shfl_sync(0xffffffffu, lo + hole, src & 31), y = __shfl_sync(0xffffffffu, pick, src & 31);
+                if (src >= 0) swap_part(what, x, y);
+            }
+            __syncwarp();
+            if (mine && !front) {
+                slot[var[lo + hole]] = lo + hole;
+                slot[var[pick]] = pick;
             }
             if (lane == 0) sh.npick = got;
         }
-        __syncthreads();
+        bar();
     }
 
-    // The wave's rows (and the segments, by the last warp).
-    __device__ __forceinline__ void write_wave(bool removal, bool kill, int ncol, OrderWave& wv) {
-        const int tid = threadIdx.x, nrow = f.reuse ? r - a : r;
+    // The wave's rows, and (last of the warps) its segments.  Nothing of it is read before the CTA's
+    // next barrier.
+    __device__ __forceinline__ void write_wave(bool removal, bool kill, int ncol, int root) {
+        const int tid = threadIdx.x, nrow = f.reuse ? r - a : r, has_k = removal ? 1 : 0;
         RowEnt* tab = static_cast<RowEnt*>(f.rowtab);
-        if (tid < NT - 32) {
-            for (int i = tid; i < nrow; i += NT - 32) {
+        if (tid < nt - 32) {
+#pragma unroll 1
+            for (int i = tid; i < nrow; i += nt - 32) {
                 const int k = row_slot(i);
                 RowEnt e = {var[k], st[k].w, -1, 0.f};
                 if (kill) {
@@ -967,16 +1031,18 @@ struct Controller {
                 if (LINGAM_INBOUNDS(f.ctl, i < f.p && e.var < f.p)) tab[i] = e;
             }
         } else {
-            const int lane = tid & 31, has_k = removal ? 1 : 0;
-            const int nblk = (f.ld + blk<T>() - 1) / blk<T>();
-            const unsigned recb = (16 * ((ncol + 3) / 4) + 8 * has_k) * 8u * unsigned(nrow);
-            const int room = int(min(f.rec_bytes, 0xffffffffull)) < 0 ? int(0xffffffffu / recb) : int(unsigned(f.rec_bytes) / recb);
-            int most = min(min(nblk, g.W), room);
+            const int lane = tid & 31;
+            const int unit = f.unit, nun = (f.ld + unit - 1) / unit, cols = (ncol + Q - 1) / Q * Q;
+            const int pm = most_units<T>(ncol, unit, g.cap);
+            const unsigned recb = unsigned(4 * cols + 8 * has_k) * 8u * unsigned(nrow);
+            const unsigned room = unsigned(min(f.rec_bytes, 0xffffffffull)) / recb - 1u;   // (the totals behind them)
+            int most = min(min(nun, g.W), int(min(room, 0x7fffffffu)));
             if (f.split_n > 0) most = min(most, f.split_n);
             float b = INFINITY;
             int at = 1;
+#pragma unroll 1
             for (int n = 1 + lane; n <= most; n += 32) {
-                const float c = seg_cost<T>(n, nrow, ncol, g.W, nblk, has_k);
+                const float c = seg_cost<T>(n, nrow, ncol, g.W, NW, nun, unit, pm, has_k);
                 if (c < b) {
                     b = c;
                     at = n;
@@ -984,14 +1050,13 @@ struct Controller {
             }
             const unsigned m = __reduce_min_sync(0xffffffffu, __float_as_uint(b));
             at = __reduce_min_sync(0xffffffffu, __float_as_uint(b) == m ? at : 0x7fffffff);
-            if (lane == 0) sh.nseg = at;
+            if (lane == 0) sh.st.wave = OrderWave{0, has_k, kill ? 1 : 0, ncol, nrow, at, root};
         }
-        __syncthreads();
-        wv = OrderWave{0, removal ? 1 : 0, kill ? 1 : 0, ncol, nrow, sh.nseg};
     }
 
-    // Iteration 0: every variable, most non-Gaussian first, nothing known of the pairs.
-    __device__ __forceinline__ bool start() {
+    // Iteration 0: every variable, most non-Gaussian first, nothing known of the pairs (all threads).
+    __device__ __forceinline__ void start() {
+#pragma unroll 1
         for (int v = threadIdx.x; v < f.p; v += NT) {
             var[v] = v;
             slot[v] = v;
@@ -1006,13 +1071,36 @@ struct Controller {
                 st[v] = make_float4(0.f, 0.f, 0.f, 0.f);
                 *reinterpret_cast<double*>(&st[v]) = h;
             }
-            key[v] = float(h);
+            row[v] = int(fl[v] ? kNoKey : key_bits(float(h)));
             f.dscale[0][v] = 1.0;
         }
+        for (int k = threadIdx.x; k < kOrderSlots; k += NT) f.gcount[k] = 0;
+        if (threadIdx.x == 0) sh.rep_nw = 0;
+        const int cm = max_cols(r);
+        new_iteration(cm, kMaxCols);
         __syncthreads();
-        if (r > 1) return true;
-        last_variable();
-        return false;
+        next_wave(0, -1, false, 0);
+        if (r > 1) {
+            next_wave(first_cols(cm, kMaxCols), -1, false, 0);
+        } else {
+            last_variable();
+            done();
+        }
+    }
+    __device__ __forceinline__ void new_iteration(int cmax, int want) {
+        if (threadIdx.x == 0) {
+            sh.st.r = r;
+            sh.st.a = 0;
+            sh.st.it = it;
+            sh.st.cmax = cmax;
+            sh.st.want = want;
+            sh.st.best = kMaxScore;
+            sh.st.bestv = -1;
+            sh.st.gamma = f.gamma0;
+        }
+    }
+    __device__ __forceinline__ void done() {
+        if (threadIdx.x == 0) sh.st.wave = OrderWave{1, 0, 0, 0, 0, 0, 0};
     }
 
     // Algorithm 2: a single remaining variable is the root.
@@ -1024,18 +1112,32 @@ struct Controller {
             f.rep_pairs[it] = 0;
         }
         if (f.want_scores)
-            for (int v = threadIdx.x; v < f.p; v += NT) f.rep_scores[size_t(it) * f.p + v] = v == var[0] ? 0.0 : NAN;
+#pragma unroll 1
+            for (int v = threadIdx.x; v < f.p; v += nt) f.rep_scores[size_t(it) * f.p + v] = v == var[0] ? 0.0 : NAN;
     }
 
-    // The first wave of iteration it: columns of lowest key, killers of the others.
-    __device__ __forceinline__ void plan(bool removal, OrderWave& wv) {
-        if (f.want_scores)
-            for (int v = threadIdx.x; v < f.p; v += NT) f.rep_scores[size_t(it) * f.p + v] = NAN;
-        for (int k = threadIdx.x; k < r; k += NT) row[k] = int((fl[k] & kNoRoot) ? kNoKey : key_bits(key[k]));
-        int c = min(want, cmax);
-        if (r - c <= 2 && r <= cmax) c = r;   // one or two rows left over: columns as well
-        select_lowest(0, r, min(c, r));
-        write_wave(removal, removal && prunes && !gmode, sh.npick, wv);
+    // What the next wave is, for make_wave.  drop: the slot of the root that leaves, or -1.
+    int nx_n, nx_drop, nx_removal, nx_root;
+    __device__ __forceinline__ void next_wave(int n, int drop, bool removal, int root) {
+        nx_n = n;
+        nx_drop = drop;
+        nx_removal = removal;
+        nx_root = root;
+    }
+    // The next wave: columns of lowest key (row[] holds the keys); in the first wave of an iteration
+    // killers of the others.
+    __device__ __forceinline__ void make_wave() {
+        if (nx_n == 0 || int(threadIdx.x) >= nt) return;
+        if (f.want_scores && a == 0)
+#pragma unroll 1
+            for (int v = threadIdx.x; v < f.p; v += nt) f.rep_scores[size_t(it) * f.p + v] = NAN;
+        select_lowest(a, r, nx_n, nx_drop);
+        write_wave(nx_removal, nx_removal && prunes && !gmode, sh.npick, nx_root);
+    }
+    // Columns of an iteration's first wave.
+    __device__ __forceinline__ int first_cols(int cmax, int want) const {
+        const int c = min(want, cmax);
+        return r - c <= 2 && r <= cmax ? r : min(c, r);   // one or two rows left over: columns as well
     }
 
     // The score so far, or more where the killer's pair is not part of it yet.
@@ -1047,10 +1149,10 @@ struct Controller {
     }
 
     // One pair's measure from its four sums: row slot k against slot j.
-    __device__ __forceinline__ T measure(const Sum (&v)[4], int k, int j) const {
+    __device__ __forceinline__ T measure(const T (&v)[4], int k, int j) const {
         T x;
         if constexpr (f32) {
-            x = pair_measure_f(sum_val(v[0]), sum_val(v[1]), sum_val(v[2]), sum_val(v[3]), st[k], st[j], __frcp_rn(float(f.n)));
+            x = pair_measure_f(v[0], v[1], v[2], v[3], st[k], st[j], __frcp_rn(float(f.n)));
         } else {
             const double pad = double(f.ld - f.n) * kBeta;
             const double ha = hterm_inv(v[0] + pad, v[1], f.inv_n), hb = hterm_inv(v[2] + pad, v[3], f.inv_n);
@@ -1061,80 +1163,83 @@ struct Controller {
     }
 
     // After a wave: scores, threshold, and the next wave (or the root and the next iteration's
-    // first wave).  wv: the wave, then the next one (done: the fit is over).
-    __device__ __forceinline__ void finish_wave(OrderWave& wv) {
+    // first wave), into sh.st.
+    __device__ __forceinline__ void finish_wave(const OrderWave& wv) {
         const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-        const int ncol = wv.ncol, nrow = wv.nrow, nseg = wv.nseg, nq = (ncol + 3) / 4, has_k = wv.removal;
-        const int RECN = 16 * nq + 8 * has_k, np = ncol + has_k;
-        const Sum* rec = static_cast<const Sum*>(f.rec);
-        const size_t stride = size_t(nrow) * RECN;
-        const int split = nseg >= 8 ? 8 : 1;   // lanes of one sum over the segments
-        const int sl = tid & (split - 1);
-        // 1. the sums of this thread's first pair are loaded while the rows' own statistics (removal:
-        //    of the new rows) are formed.  Pairs: row e against column c, and its killer (c = ncol)
-        const int units = nrow * np;
-        auto pair_of_unit = [&](int u, int& e, int& c, int& kj) {
-            e = u / np;
-            c = u - e * np;
-            kj = -1;
-            if (u >= units) return;
-            if (c < ncol) {
-                if (f.reuse ? e >= ncol || c < e : e != c) kj = a + c;
-            } else {
-                const int kv = keval[a + e];
-                if (kv >= 0) kj = slot[kv];
-            }
-        };
-        int e0, c0, kj0;
-        pair_of_unit(tid / split, e0, c0, kj0);
-        Sum v0[4] = {Sum(), Sum(), Sum(), Sum()};
-        if (kj0 >= 0) sum_segments<Sum>(v0, rec + size_t(e0) * RECN + (c0 < ncol ? 4 * c0 : 16 * nq), stride, nseg, sl, split);
-        if (has_k) {
-            for (int u0 = 0; u0 < nrow * split; u0 += NT) {
-                const int e = (u0 + tid) / split;
-                Sum v[4] = {Sum(), Sum(), Sum(), Sum()};
-                if (e < nrow) sum_segments<Sum>(v, rec + size_t(e) * RECN + 16 * nq + 4, stride, nseg, sl, split);
-                for (int o = split >> 1; o > 0; o >>= 1) {
-                    v[0] = sum_add(v[0], shfl_xor_sum(v[0], o));
-                    v[1] = sum_add(v[1], shfl_xor_sum(v[1], o));
+        const int ncol = wv.ncol, nrow = wv.nrow, nseg = wv.nseg, nq = (ncol + Q - 1) / Q, has_k = wv.removal;
+        const int RECN = 4 * Q * nq + 8 * has_k, np = ncol + has_k, own = 4 * Q * nq;
+        r = sh.st.r;
+        a = sh.st.a;
+        it = sh.st.it;
+        next_wave(0, -1, false, 0);
+        const int nw = min(NW, max(4, (r + 63) >> 6));
+        nt = 32 * nw;
+        const T* tot = reinterpret_cast<const T*>(static_cast<const Sum*>(f.rec) + size_t(nseg) * nrow * RECN);
+        // 1. the rows' own statistics (removal: of the new rows) and I of every pair.  Units: the rows'
+        //    statistics first, then row e against column c or its killer (c = ncol); a thread has four
+        //    units' totals in flight.
+        const int stats = has_k ? nrow : 0, units = stats + nrow * np;
+        for (int u0 = 0; u0 < units; u0 += 4 * NT) {
+            T v[4][4];
+            int kj[4], es[4];   // the partner's slot (-1: nothing to do), the row
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int u = u0 + q * NT + tid;
+                kj[q] = -1;
+                if (u0 + q * NT < units) {   // (the same for every thread)
+                    int at = 0;
+                    es[q] = u;
+                    if (u < stats) {
+                        kj[q] = 0;
+                        at = u * RECN + own + 4;
+                    } else if (u < units) {
+                        const int e = small_div(u - stats, np), c = u - stats - e * np;
+                        es[q] = e;
+                        at = e * RECN + (c < ncol ? 4 * c : own);
+                        if (c < ncol) {
+                            if (f.reuse ? e >= ncol || c < e : e != c) kj[q] = a + c;
+                        } else {
+                            const int kv = keval[a + e];
+                            if (kv >= 0) kj[q] = slot[kv];
+                        }
+                    }
+                    if (kj[q] >= 0) load4(v[q], tot + at);
                 }
-                if (e < nrow && sl == 0) {
-                    const int k = a + e;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int u = u0 + q * NT + tid;
+                if (u0 + q * NT < stats && u < stats) {
+                    const int k = a + u;
                     if constexpr (f32) {
                         // T is centred by the old offset -32 (ln 2 + m0) over the padded row
                         const float inv_n = __frcp_rn(float(f.n));
-                        const float Ts = sum_val(v[0]), off = st[k].w;
+                        const float Ts = v[q][0], off = st[k].w;
                         const float m0 = -off * (1.f / kSub) - float(kLn2);
                         const float y = 2.f * ((m0 - float(kBeta)) + fmaf(float(f.ld - f.n), m0, Ts) * inv_n);
-                        st[k] = make_float4(-Ts * inv_n, y, sum_val(v[1]) * (kInvScale * inv_n), off);
+                        st[k] = make_float4(-Ts * inv_n, y, v[q][1] * (kInvScale * inv_n), off);
                     } else {
-                        *reinterpret_cast<double*>(&st[k]) =
-                            hterm_inv(sum_val(v[0]) + double(f.ld - f.n) * kBeta, sum_val(v[1]), f.inv_n);
+                        *reinterpret_cast<double*>(&st[k]) = hterm_inv(v[q][0] + double(f.ld - f.n) * kBeta, v[q][1], f.inv_n);
                     }
                 }
             }
-            __syncthreads();
-        }
-        // 2. I of every pair
-        for (int u0 = 0; u0 < units * split; u0 += NT) {
-            int e = e0, c = c0, kj = kj0;
-            const int u = (u0 + tid) / split;
-            if (u0 > 0) {
-                pair_of_unit(u, e, c, kj);
-                if (kj >= 0)
-                    sum_segments<Sum>(v0, rec + size_t(e) * RECN + (c < ncol ? 4 * c : 16 * nq), stride, nseg, sl, split);
-            }
-            for (int o = split >> 1; o > 0; o >>= 1) {
+            if (u0 < stats && u0 + 4 * NT >= stats) __syncthreads();   // the statistics are there
 #pragma unroll
-                for (int k = 0; k < 4; ++k) v0[k] = sum_add(v0[k], shfl_xor_sum(v0[k], o));
+            for (int q = 0; q < 4; ++q) {
+                const int u = u0 + q * NT + tid;
+                if (u0 + q * NT < units && u >= stats && u < units)
+                    I[u - stats] = kj[q] >= 0 ? measure(v[q], row_slot(es[q]), kj[q]) : T(0);
             }
-            if (u < units && sl == 0) I[u] = kj >= 0 ? measure(v0, row_slot(e), kj) : T(0);
         }
         __syncthreads();
+        if (tid >= nt) return;
+        long long best = sh.st.best;
+        int bestv = sh.st.bestv;
         // 3. rows: contributions min(0, I)^2 of the columns, of the killer, and the killers to come
         int nk = 0;   // pairs besides the columns' (distinct ones: a pair may be both's killer, and a
                       // later wave may compare a killer pair again)
-        for (int e = tid; e < nrow && f.reuse; e += NT) {
+#pragma unroll 1
+        for (int e = tid; e < nrow && f.reuse; e += nt) {
             const int k = a + e, ke = keval[k];
             if (ke >= 0) {
                 const int sk = slot[ke];
@@ -1153,6 +1258,7 @@ struct Controller {
                 w0 = m * m;   // keval is kp0
                 kc[k] = w0;
             }
+#pragma unroll 1
             for (int c = 0; c < cm; ++c) {
                 const T m = Ir[c] < T(0) ? Ir[c] : T(0);
                 add_square(acc, m);
@@ -1192,12 +1298,14 @@ struct Controller {
         }
         nk = __reduce_add_sync(0xffffffffu, nk);
         if (lane == 0) sh.nkill[wid] = nk;
-        __syncthreads();
+        bar();
         // 4. columns: max(0, I)^2 over the rows below them, a warp per column
-        for (int c = wid; c < ncol; c += NW) {
+#pragma unroll 1
+        for (int c = wid; c < ncol; c += nw) {
             Sum acc = Sum();
             unsigned top = 0;
             int tope = -1;
+#pragma unroll 1
             for (int e = (f.reuse ? c + 1 : 0) + lane; e < nrow; e += 32) {
                 const T x = I[e * np + c];   // (0 for the column itself)
                 const T m = x > T(0) ? x : T(0);
@@ -1230,8 +1338,9 @@ struct Controller {
                 }
             }
         }
-        __syncthreads();
+        bar();
         // 5. lowest complete score of the iteration (lowest variable index on ties); every thread
+#pragma unroll 1
         for (int c = 0; c < ncol; ++c) {
             const long long kk = sh.col[c];
             const int vc = var[a + c];
@@ -1240,29 +1349,36 @@ struct Controller {
                 bestv = vc;
             }
         }
-        pairs += f.reuse ? (long long)ncol * (ncol - 1) / 2 + (long long)ncol * (nrow - ncol) : (long long)ncol * (nrow - 1);
-        for (int w = 0; w < NW; ++w) pairs += sh.nkill[w];
-        ++waves;
         const int an = a + ncol;   // columned so far
         // 6. threshold: the live candidates of the others
+        double gamma = gmode ? sh.st.gamma : 0.0;
         int live;
+#pragma unroll 1
         for (int pass = 0;; ++pass) {
             const long long thr = gmode ? score_key(sum_from(gamma)) : best;
             int n = 0;
-            for (int k = an + tid; k < r; k += NT) {
+#pragma unroll 1
+            for (int k = an + tid; k < r; k += nt) {
                 const Sum lb = gmode ? part[k] : lower_bound(k, an);
                 const bool on = !(fl[k] & kNoRoot) && !(prunes && score_key(lb) > thr);
                 n += on ? 1 : 0;
                 row[k] = int(on ? key_bits(score_float(lb)) : kNoKey);
             }
-            live = __syncthreads_or(n);
+            live = part_or(nt, n);
             // the paper's schedule: nothing can go on and nothing finished at or below gamma: raise
             // gamma by factors gamma_c until the lowest score that may be the root's is at or below it
             if (!gmode || live || best <= thr || pass > 0) break;
             long long km = best;
-            for (int k = an + tid; k < r; k += NT)
+#pragma unroll 1
+            for (int k = an + tid; k < r; k += nt)
                 if (!(fl[k] & kNoRoot)) km = min(km, score_key(part[k]));
-            km = block_min(km);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) km = min(km, __shfl_xor_sync(0xffffffffu, km, o));
+            if (lane == 0) sh.lred[wid] = km;
+            bar();
+#pragma unroll 1
+            for (int w = 0; w < nw; ++w) km = min(km, sh.lred[w]);
+            bar();
             const double target = score_out(score_of_key(km, Sum()));
             int n2 = 0;
             while (gamma < target && n2 < 4096) {   // gamma_c > 1 and target finite: a few steps
@@ -1272,11 +1388,22 @@ struct Controller {
             if (!(score_key(sum_from(gamma)) >= km)) gamma = target;
             gsteps += n2;
         }
+        if (tid == 0) {
+            sh.rep_ncol = ncol;
+            sh.rep_nrow = nrow;
+            sh.rep_nw = nw;
+            sh.rep_it = -1;
+        }
         if (live) {
             a = an;
-            cmax = order_max_cols<T>(g.cap, NW, f.reuse ? r - a : r, icap);
-            select_lowest(a, r, min(cmax, r - a));
-            write_wave(false, false, sh.npick, wv);
+            const int nr2 = f.reuse ? r - a : r, cm = max_cols(nr2);
+            if (tid == 0) {
+                sh.st.a = a;
+                sh.st.best = best;
+                sh.st.bestv = bestv;
+                sh.st.gamma = gamma;
+            }
+            next_wave(min(cm, r - a), -1, false, 0);
             return;
         }
         // 7. the root, its margin, and the next iteration's candidate order
@@ -1284,8 +1411,10 @@ struct Controller {
         const int rs = slot[root];
         long long second = kMaxScore;
         int need = 0;
-        for (int k = tid; k < r; k += NT) {
-            const Sum lb = k < an ? part[k] : lower_bound(k, an);
+#pragma unroll 1
+        for (int k = tid; k < r; k += nt) {
+            const Sum pk = part[k];
+            const Sum lb = k < an ? pk : lower_bound(k, an);
             const int v = var[k];
             if (v != bestv && !(fl[k] & kNoRoot)) second = min(second, score_key(lb));
             // a column whose strongest pair alone would not have excluded it
@@ -1299,8 +1428,7 @@ struct Controller {
             } else if (rs >= an && keval[k] == root) {
                 ctr = kc[k];
             }
-            key[k] = fmaxf(score_float(lb) - ctr, 0.f);
-            if (k == rs) sh.rootpt = score_key(part[k]);
+            if (k == rs) sh.rep_rootpt = score_key(pk);
             if (kp0[k] == root) {
                 kp0[k] = kp1[k];
                 kv0[k] = kv1[k];
@@ -1315,55 +1443,70 @@ struct Controller {
                 f.anc_cnt[v] = left;
                 if (left == 0) fl[k] &= ~kNoRoot;
             }
+            row[k] = int(k == rs || (fl[k] & kNoRoot) ? kNoKey : key_bits(fmaxf(score_float(lb) - ctr, 0.f)));
             if constexpr (f32) st[k].w = stat_offset(st[k].y);
-            if (k >= an) part[k] = Sum();   // (the columns' are read below)
+            part[k] = Sum();
         }
-        {
-            // the lowest other score and the count, one barrier for both
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) second = min(second, __shfl_xor_sync(0xffffffffu, second, o));
-            need = __reduce_add_sync(0xffffffffu, need);
-            if (lane == 0) {
-                sh.lred[wid] = second;
-                sh.ired[wid] = need;
-            }
-            __syncthreads();
-            need = 0;
-            for (int w = 0; w < NW; ++w) need += sh.ired[w];
-            for (int k = tid; k < an; k += NT) part[k] = Sum();
+        for (int o = 16; o > 0; o >>= 1) second = min(second, __shfl_xor_sync(0xffffffffu, second, o));
+        need = __reduce_add_sync(0xffffffffu, need);
+        if (lane == 0) {
+            sh.lred[wid] = second;
+            sh.ired[wid] = need;
         }
         if (tid == 0) {
-            for (int w = 0; w < NW; ++w) second = min(second, sh.lred[w]);
-            f.order[it] = root;
-            const double bs = score_out(score_of_key(best, Sum()));
-            f.rep_root_score[it] = root == bestv ? bs : score_out(score_of_key(sh.rootpt, Sum()));
-            f.rep_margin[it] = (second == kMaxScore ? double(INFINITY) : score_out(score_of_key(second, Sum()))) - bs;
-            f.rep_pairs[it] = pairs;
-            f.ctl->rm_root = root;
+            sh.rep_it = it;
+            sh.rep_root = root;
+            sh.rep_bestv = bestv;
+            sh.rep_best = best;
         }
-        total += pairs;
+        bar();
         ++it;
         if (it >= iters) {
-            wv.done = 1;
+            done();
             return;
         }
-        if (tid < 32) swap_slots(rs, r - 1);   // the root leaves
-        __syncthreads();
+        need = 0;
+#pragma unroll 1
+        for (int w = 0; w < nw; ++w) need += sh.ired[w];
         r -= 1;
         a = 0;
-        new_iteration();
+        const int cmax = max_cols(r), want = prunes && !gmode ? (need + 4) / 4 * 4 : kMaxCols;
+        new_iteration(cmax, want);
         if (r == 1) {
+            if (tid < 32) swap_slots(rs, 1);
+            bar();
             last_variable();
-            wv.done = 1;
+            done();
             return;
         }
-        cmax = order_max_cols<T>(g.cap, NW, r, icap);
-        want = prunes && !gmode ? (need + 4) / 4 * 4 : kMaxCols;
-        plan(true, wv);
+        next_wave(first_cols(cmax, want), rs, true, root);
     }
 
-    int waves = 0;
-    long long total = 0, gsteps = 0;
+    // Thread 0, once the next wave is published: the finished wave's counts, and the finished
+    // iteration's results.
+    __device__ __forceinline__ void report() {
+        if (sh.rep_nw == 0) return;
+        const int ncol = sh.rep_ncol, nrow = sh.rep_nrow;
+        pairs += f.reuse ? (long long)ncol * (ncol - 1) / 2 + (long long)ncol * (nrow - ncol) : (long long)ncol * (nrow - 1);
+#pragma unroll 1
+        for (int w = 0; w < sh.rep_nw; ++w) pairs += sh.nkill[w];
+        ++waves;
+        const int i = sh.rep_it;
+        if (i >= 0) {
+            long long second = kMaxScore;
+#pragma unroll 1
+            for (int w = 0; w < sh.rep_nw; ++w) second = min(second, sh.lred[w]);
+            const double bs = score_out(score_of_key(sh.rep_best, Sum()));
+            f.order[i] = sh.rep_root;
+            f.rep_root_score[i] = sh.rep_root == sh.rep_bestv ? bs : score_out(score_of_key(sh.rep_rootpt, Sum()));
+            f.rep_margin[i] = (second == kMaxScore ? double(INFINITY) : score_out(score_of_key(second, Sum()))) - bs;
+            f.rep_pairs[i] = pairs;
+            total += pairs;
+            pairs = 0;
+        }
+        sh.rep_nw = 0;
+    }
 
     __device__ __forceinline__ static Sum sum_from(double x) {
         if constexpr (f32) {
@@ -1372,17 +1515,6 @@ struct Controller {
         } else {
             return x;
         }
-    }
-    __device__ __forceinline__ long long block_min(long long v) {
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-        __syncthreads();
-        if (lane == 0) sh.lred[wid] = v;
-        __syncthreads();
-        for (int w = 0; w < NW; ++w) v = min(v, sh.lred[w]);
-        __syncthreads();
-        return v;
     }
 };
 
@@ -1459,9 +1591,7 @@ __device__ __forceinline__ bool run_problem(const Fit& f, Ctl* top, int rank, in
         for (unsigned seq = 1;; ++seq) {
             OrderWave wv;
             if (!wait_order_wave(f.ctl, top, seq, tmo, sh, wv)) return false;
-            if (wv.done) {
-                return true;
-            }
+            if (wv.done) return true;
             worker_wave<T, NT>(f, wv, g, xb[cur], xb[cur ^ 1], sb[cur], sb[cur ^ 1], f.dscale[cur], f.dscale[cur ^ 1]);
             if (wv.removal) cur ^= 1;
             __syncthreads();
@@ -1470,24 +1600,40 @@ __device__ __forceinline__ bool run_problem(const Fit& f, Ctl* top, int rank, in
     }
     // the controller
     Controller<T, NT> c(f, g, sh, smem_bytes, iters);
-    OrderWave wv{1, 0, 0, 0, 0, 0};
-    if (threadIdx.x == 0) sh.ok = *reinterpret_cast<volatile int*>(&f.ctl->status) == 0;
+    if (threadIdx.x == 0) {
+        sh.ok = *reinterpret_cast<volatile int*>(&f.ctl->status) == 0;
+        sh.rep_nw = 0;
+    }
     __syncthreads();
-    if (sh.ok != 0 && c.start()) c.plan(false, wv);
+    c.next_wave(0, -1, false, 0);
+    if (sh.ok != 0) c.start();
+    else c.done();
     const bool timed = f.timing && threadIdx.x == 0;
     unsigned long long tit = timed ? global_ns() : 0, tph = tit;
     unsigned arrivals = 0;
+    int bad = 0;
     for (unsigned seq = 1;; ++seq) {
-        __syncthreads();   // the row table is written
-        if (threadIdx.x == 0 && size > 1)
-            st_release64(&f.ctl->wave_word, pack_order_wave(seq, wv.done, wv.removal, wv.kill, wv.ncol, wv.nrow, wv.nseg));
-        if (wv.done) break;
-        if (timed) {
-            const unsigned long long t = global_ns();
-            f.ctl->phase_ns[1] += t - tph;
-            tph = t;
+        c.make_wave();
+        bad = __syncthreads_or(bad);   // the row table and the next wave are written
+        OrderWave wv = sh.st.wave;
+        if (bad) wv = OrderWave{1, 0, 0, 0, 0, 0, 0};
+        if (threadIdx.x == 0) {
+            if (size > 1) st_release64(&f.ctl->wave_word, pack_order_wave(seq, wv));
+            const int before = sh.rep_nw ? sh.rep_it : -1;
+            c.report();
+            if (timed) {
+                const unsigned long long t = global_ns();
+                f.ctl->phase_ns[1] += t - tph;
+                tph = t;
+                if (before >= 0) {
+                    f.prev[before] = double(t - tit) * 1e-6;
+                    tit = t;
+                }
+            }
         }
+        if (wv.done) break;
         if (!dedicated) {
+            __syncthreads();   // (thread 0 has reported; the worker's tables overlay the I table)
             worker_wave<T, NT>(f, wv, g, xb[cur], xb[cur ^ 1], sb[cur], sb[cur ^ 1], f.dscale[cur], f.dscale[cur ^ 1]);
             __syncthreads();
         }
@@ -1499,18 +1645,10 @@ __device__ __forceinline__ bool run_problem(const Fit& f, Ctl* top, int rank, in
             f.ctl->phase_ns[0] += t - tph;
             tph = t;
         }
-        // a failure recorded by a worker ends the fit (the others of a batch go on); read now, looked
+        // a failure recorded by a worker ends the fit (the others of a batch go on): read now, looked
         // at after the wave's work
-        int bad = 0;
         if (threadIdx.x == 0) bad = *reinterpret_cast<volatile int*>(&f.ctl->status);
-        const int before = c.it;
         c.finish_wave(wv);
-        if (__syncthreads_or(bad)) wv = OrderWave{1, 0, 0, 0, 0, 0};
-        if (timed && c.it != before) {
-            const unsigned long long t = global_ns();
-            f.prev[before] = double(t - tit) * 1e-6;
-            tit = t;
-        }
     }
     if (threadIdx.x == 0) {
         f.ctl->waves = c.waves;
@@ -1568,20 +1706,20 @@ constexpr size_t kOrderSmem256 = 108 * 1024;
 
 // Largest p whose controller state and I table (four columns) fit.
 template <class T>
-static bool order_fits_smem(long long p, size_t smem, bool dedicated, int nw) {
+static bool order_fits_smem(long long p, size_t smem, bool dedicated) {
     const size_t state = order_state_bytes(int(p));
     if (state >= smem) return false;
-    return order_max_cols<T>(smem - (dedicated ? 0 : state), nw, int(p), smem - state) >= 4;
+    return order_max_cols<T>(unsigned(smem - (dedicated ? 0 : state)), int(p), unsigned(smem - state)) >= 4;
 }
 
 bool order_supported(const Fit& f, bool batch) {
     const bool f32 = f.precision == LINGAM_MIXED;
     if (f.p > 4096 || f.ld / 256 > 0xffff) return false;
-    if (f.rec_bytes < size_t(f.p) * (16 * (kMaxCols / 4) + 8) * 8) return false;   // one segment of a full wave
+    if (f.rec_bytes < 2 * size_t(f.p) * (4 * kMaxCols + 8) * 8) return false;   // one segment of a full wave
     const size_t smem = (batch ? kOrderSmem256 : kOrderSmem512) - (f32 ? 0 : kExpTab * sizeof(double));
     // (a single fit's group is below kDedicated CTAs only when p is small)
-    return f32 ? order_fits_smem<float>(f.p, smem, !batch && f.p >= 64, batch ? 8 : 16)
-               : order_fits_smem<double>(f.p, smem, !batch && f.p >= 64, batch ? 8 : 16);
+    return f32 ? order_fits_smem<float>(f.p, smem, !batch && f.p >= 64)
+               : order_fits_smem<double>(f.p, smem, !batch && f.p >= 64);
 }
 
 template <class T, int NT>
@@ -1604,13 +1742,12 @@ static cudaError_t launch_order_t(const Fit& f, int iters, const Fit* fits, cons
     return cudaLaunchKernelEx(&cfg, k_order<T, NT>, f, iters, fits, assign, queue, nqueue, qhead, top, smem);
 }
 
-// CTAs of a single fit: enough for four warps' blocks each (a row against a quad, and the row's own;
-// FP64: for one block) in the first wave, the whole GPU at most.
+// CTAs of a single fit: enough for four warps' units each in the first removal's wave (a row against
+// four columns, and the row's own), the whole GPU at most.
 int order_grid(const Fit& f, int nsm) {
     const bool f32 = f.precision == LINGAM_MIXED;
-    const int b = f32 ? blk<float>() : blk<double>();
-    const long long units = (long long)f.p * ((f.ld + b - 1) / b) * 2;
-    return int(std::max(1ll, std::min((long long)nsm, 1 + (f32 ? (units + 3) / 4 : units))));
+    const long long units = (long long)f.p * ((f.ld + f.unit - 1) / f.unit) * (f32 ? 2 : 5);
+    return int(std::max(1ll, std::min((long long)nsm, 1 + (units + 3) / 4)));
 }
 
 cudaError_t launch_order(const Fit& f, int iters, int nsm, cudaStream_t st) {

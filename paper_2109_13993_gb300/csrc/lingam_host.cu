@@ -278,14 +278,17 @@ static Fit make_fit(char* base, const Layout& L, int p, int n, const lingam_opts
     f.bout = reinterpret_cast<double*>(base + L.off_bout);
     f.ctl = reinterpret_cast<Ctl*>(base + L.off_ctl);
     // the ordering kernel's buffers lie over what it does not use: see make_layout; the row table
-    // and the rows' scales (32 bytes a variable) over the I buffer (at least 256)
+    // and the rows' scales (32 bytes a variable) and the groups'
+    // counters over the I buffer (8 KB per 32 variables)
     f.rec = f.partials;
     f.rec_bytes = L.alt_in_xin ? L.partial_bytes : L.partial_bytes / 2 / kAlign * kAlign;
     f.xalt = L.alt_in_xin ? base + L.off_xin : base + L.off_partials + f.rec_bytes;
     f.sigalt = f.cmat;
+    f.unit = o.precision == LINGAM_MIXED ? (size_t(p) * size_t(L.ld) < (size_t(4) << 20) ? 512 : 1024) : 256;
     f.rowtab = f.ibuf;
     f.dscale[0] = reinterpret_cast<double*>(static_cast<char*>(f.ibuf) + size_t(p) * 16);
     f.dscale[1] = f.dscale[0] + p;
+    f.gcount = reinterpret_cast<int*>(f.dscale[1] + p);
     f.maxtiles = L.maxtiles;
     f.maxsplit = L.maxsplit;
     f.nslots = L.nslots;
@@ -894,6 +897,7 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
         f.tile_rows = ts.rows;
         f.tile_cols = ts.cols;
         f.split_n = 0;
+        if (o.precision == LINGAM_MIXED) f.unit = 1024;   // many problems: the warps are busy
         f.narrow = 0;   // the batch kernel runs every wave on the call's tile shape
         fits[size_t(k)] = f;
         SrcDesc sd;
