@@ -257,6 +257,140 @@ __global__ void __launch_bounds__(kBThreads) k_bfit_small(const Fit* __restrict_
     }
 }
 
+// ------------------------------------------------------------------ from the ordering's factorisation
+// The ordering kernel's covariance updates are the elimination steps of Sigma0 = L diag(d) L^T in causal
+// order, so it leaves them behind: rmat[k p + v] = L[position of v][k] d_k for the variables v from
+// position k on (d_k at v = K[k]; the last d is not needed).  In the normalised variables x = L e with e
+// the innovations, so B = I - L^{-1} there, and B[K[a]][K[b]] = -(L^{-1})[a][b] sd_{K[a]} / sd_{K[b]}
+// (a > b) in the original units: no Cholesky, whose p row steps of 3.5 us took most of the fit: a call of
+// p = 300 takes 0.9 ms less (of 11.0), p = 1000 4.3 ms (of 72.9), p = 20 0.07 ms (of 0.70).  Against long double its errors are a little below
+// the Cholesky's (p = 20 ... 150, relative norms: 0.96e-15 ... 3.5e-15 and 1.1e-15 ... 3.7e-15).
+//
+// A CTA solves two columns of L^{-1} by forward substitution in blocks of 32 rows: a warp per column
+// solves the block's triangle with shuffles, then all threads add the block's columns of L to the
+// running sums of the rows below.  A step per 32 rows instead of one barrier per row; two columns share
+// the reads of L, and more would leave the last SMs idle (the FP64 rate bounds it: p^3 / 6 FMAs).
+constexpr int kFacThreads = 256;
+constexpr int kFacCols = 2;
+// Up to this many variables L is read in place (L1 and L2 take the scattered reads, and a batch's
+// problems share one launch); above it a permuted copy, read in rows, is worth its launch of 3 us.
+constexpr int kFacGather = 128;
+
+// The ordering ran to its end (of a batch that ran out of time some may not have: their orders are not
+// read).
+__device__ __forceinline__ bool ordered(const Fit& f) {
+    const volatile Ctl* c = f.ctl;
+    return c->status == 0 && (f.p == 1 || c->waves > 0);
+}
+
+// The factor in causal order: cmat[k p + i] = L[i][k] d_k, i >= k.
+__global__ void __launch_bounds__(kFacThreads) k_factor_order(Fit f) {
+    const int p = f.p, k = blockIdx.y, i = blockIdx.x * kFacThreads + threadIdx.x;
+    if (i < p && i >= k && ordered(f)) f.cmat[size_t(k) * p + i] = f.rmat[size_t(k) * p + f.order[i]];
+}
+
+template <bool GATHER>
+__device__ __forceinline__ void factor_columns(const Fit& f, int j0, double* y /* [kFacCols][p] */) {
+    __shared__ double s_z[kFacCols][32];   // the block's y_k / d_k
+    const int p = f.p, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const double* L = GATHER ? f.rmat : f.cmat;
+    const int nc = min(kFacCols, p - j0);
+    for (int i = tid; i < kFacCols * p; i += kFacThreads) y[i] = 0.0;
+    if (tid < kFacCols * 32) s_z[tid >> 5][tid & 31] = 0.0;
+    __syncthreads();
+    for (int k0 = j0 / 32 * 32; k0 < p; k0 += 32) {
+        const int kn = min(32, p - k0);
+        if (wid < nc) {
+            // rows k0 + lane: y_i = [i = j] - sum_{k < i} L[i][k] d_k (y_k / d_k)
+            const int i = k0 + lane, at = GATHER && lane < kn ? f.order[i] : i;
+            double l[32];
+#pragma unroll
+            for (int k = 0; k < 32; ++k) l[k] = k < lane && lane < kn ? L[size_t(k0 + k) * p + at] : 0.0;
+            const double inv = i < p - 1 ? 1.0 / L[size_t(i) * p + at] : 0.0;
+#pragma unroll
+            for (int k = 0; k < 32; ++k) l[k] *= __shfl_sync(0xffffffffu, inv, k);
+            double r = lane < kn ? (i == j0 + wid ? 1.0 : 0.0) - y[wid * p + i] : 0.0;
+#pragma unroll
+            for (int k = 0; k < 32; ++k) r = fma(-l[k], __shfl_sync(0xffffffffu, r, k), r);
+            if (lane < kn) y[wid * p + i] = r;
+            s_z[wid][lane] = r * inv;
+        }
+        __syncthreads();
+        for (int i = k0 + 32 + tid; i < p; i += kFacThreads) {
+            const int at = GATHER ? f.order[i] : i;
+            double s[kFacCols] = {};
+#pragma unroll
+            for (int kk = 0; kk < 32; kk += 16) {
+                double l[16];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) l[k] = L[size_t(k0 + kk + k) * p + at];
+#pragma unroll
+                for (int k = 0; k < 16; ++k)
+#pragma unroll
+                    for (int c = 0; c < kFacCols; ++c) s[c] = fma(l[k], s_z[c][kk + k], s[c]);
+            }
+#pragma unroll
+            for (int c = 0; c < kFacCols; ++c) y[c * p + i] += s[c];
+        }
+        __syncthreads();
+    }
+    for (int c = 0; c < nc; ++c) {
+        const int j = j0 + c, vj = f.order[j];
+        const double inv = 1.0 / f.sd[vj];
+        for (int i = tid; i < p; i += kFacThreads) {
+            const int vi = f.order[i];
+            f.bout[size_t(vi) * p + vj] = i > j ? -y[c * p + i] * (f.sd[vi] * inv) : 0.0;
+        }
+    }
+}
+template <bool GATHER>
+__global__ void __launch_bounds__(kFacThreads) k_factor_B(Fit f) {
+    extern __shared__ double sm_fac[];
+    if (!ordered(f)) return;
+    factor_columns<GATHER>(f, blockIdx.x * kFacCols, sm_fac);
+}
+// Problems of a batch with p <= kFacGather (the others, and those of bad status, are left out).
+__global__ void __launch_bounds__(kFacThreads) k_factor_B_batch(const Fit* __restrict__ fits) {
+    extern __shared__ double sm_fac[];
+    const Fit& f = fits[blockIdx.x];
+    if (f.p > kFacGather || int(blockIdx.y) * kFacCols >= f.p || !ordered(f)) return;
+    factor_columns<true>(f, blockIdx.y * kFacCols, sm_fac);
+}
+
+cudaError_t launch_factor_B(const Fit& f, cudaStream_t st) {
+    const int p = f.p, grid = (p + kFacCols - 1) / kFacCols;
+    const size_t smem = size_t(kFacCols) * p * sizeof(double);
+    if (p <= kFacGather) {
+        k_factor_B<true><<<grid, kFacThreads, smem, st>>>(f);
+        return cudaGetLastError();
+    }
+    k_factor_order<<<dim3((p + kFacThreads - 1) / kFacThreads, p), kFacThreads, 0, st>>>(f);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    e = ensure_smem_attr(reinterpret_cast<const void*>(k_factor_B<false>), smem);
+    if (e != cudaSuccess) return e;
+    k_factor_B<false><<<grid, kFacThreads, smem, st>>>(f);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_factor_B_batch(const Fit* fits_dev, const int* p_host, int count, const Fit* fits_host, cudaStream_t st) {
+    int pmax = 0;
+    for (int k = 0; k < count; ++k)
+        if (p_host[k] <= kFacGather) pmax = std::max(pmax, p_host[k]);
+    if (pmax > 0) {
+        k_factor_B_batch<<<dim3(count, (pmax + kFacCols - 1) / kFacCols), kFacThreads, size_t(kFacCols) * pmax * sizeof(double), st>>>(
+            fits_dev);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    for (int k = 0; k < count; ++k)
+        if (p_host[k] > kFacGather) {
+            const cudaError_t e = launch_factor_B(fits_host[k], st);
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
+}
+
 cudaError_t launch_fit_B_batch(const Fit* fits_dev, const int* p_host, int count, const Fit* fits_host,
                                cudaStream_t st) {
     int pmax_small = 0;

@@ -557,7 +557,7 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
                 }
             }
             // UpdateCovMat (Eq. CovUpdate) on S, FP64, upper triangle by variable index, into the other
-            // copy: S[w][j] - S[w][root] S[j][root] / S[root][root] for the batch's rows w and every j > w
+            // copy: S[w][j] - S[w][root] S[j][root] / S[root][root] for the batch's rows w and every j >= w
             // (of a removed j the element is never read again), in chunks of 32 elements a warp; the
             // segments' workers share a row's chunks.  Four of a warp's chunks are in flight, the first here.
             const int nch = (p + 31) >> 5, mych = small_div(nch + nseg - 1 - seg, nseg);   // chunks seg, seg + nseg, ...
@@ -572,7 +572,7 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
                     if (cov && ci < nrb) {
                         const int w = s_row[ci].var, j = (seg + cc * nseg) * 32 + lane;
                         crow[q] = ci;
-                        if (j > w && j < p) {
+                        if (j >= w && j < p) {
                             cat[q] = w * p + j;   // (p <= 4096)
                             ca[q] = __ldcg(sold + cat[q]);
                             cb[q] = __ldcg(sold + min(j, root) * p + max(j, root));
@@ -588,6 +588,8 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
                 }
             };
             load_chunks();
+            if (rm && tid == NT - 1 && g.wk == 0 && r0 == 0 && bs == b0)
+                f.rmat[size_t(p - 1 - nrow) * p + root] = __ldcg(sold + root * p + root);
             // the rows', killers' and columns' removal coefficients (FP64)
             if (tid < 2 * nrb + ncol) {
                 const int k = tid < nrb ? tid : tid < 2 * nrb ? kRowBatch + tid - nrb : 2 * kRowBatch + tid - 2 * nrb;
@@ -605,7 +607,10 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
                         }
                         inv = rsqrt_fast(om);
                         d *= inv;
-                        if (k < kRowBatch && bs == 0) dnew[v] = d;   // (one worker per row: the first segment's)
+                        if (k < kRowBatch && bs == 0) {   // (one worker per row: the first segment's)
+                            dnew[v] = d;
+                            f.rmat[size_t(p - 1 - nrow) * p + v] = sr;   // (for the B fit)
+                        }
                     }
                 }
                 s_sr[k] = sr;
@@ -851,6 +856,8 @@ struct Controller {
     int* fl;          // kNoRoot
     int* row;         // candidate keys of a selection
     T* I;             // the wave's pair measures
+    const double* cov;     // S and the rows' scales after the last removal
+    const double* scale;
     unsigned icap;
     int iters;
     bool gmode, prunes;
@@ -1476,6 +1483,14 @@ struct Controller {
         if (r == 1) {
             if (tid < 32) swap_slots(rs, 1);
             bar();
+            if (tid == 0) {   // the last step of the elimination
+                const int v = var[0];
+                const double d = __ldcg(scale + root), dv = __ldcg(scale + v);
+                const double sr = __ldcg(cov + min(v, root) * f.p + max(v, root)), rho = sr * (d * dv);
+                f.rmat[size_t(f.p - 2) * f.p + v] = sr;
+                f.rmat[size_t(f.p - 2) * f.p + root] = __ldcg(cov + root * f.p + root);
+                if (!(fma(-rho, rho, 1.0) > 0.0)) set_status(f.ctl, LINGAM_EDEGENERATE);
+            }
             last_variable();
             done();
             return;
@@ -1648,6 +1663,8 @@ __device__ __forceinline__ bool run_problem(const Fit& f, Ctl* top, int rank, in
         // a failure recorded by a worker ends the fit (the others of a batch go on): read now, looked
         // at after the wave's work
         if (threadIdx.x == 0) bad = *reinterpret_cast<volatile int*>(&f.ctl->status);
+        c.cov = sb[cur];
+        c.scale = f.dscale[cur];
         c.finish_wave(wv);
     }
     if (threadIdx.x == 0) {

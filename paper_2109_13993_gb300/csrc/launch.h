@@ -67,6 +67,9 @@ cudaError_t launch_batch(const Fit* fits_dev, int count, int maxp, int precision
 constexpr int kBatchLaunchMax = 512;   // problems per launch_batch
 // B from the order: Cholesky of the covariance in causal order, B = I - diag(R) R^{-1}.
 cudaError_t launch_fit_B(const Fit& f, cudaStream_t st);
+// The same from the factorisation that the ordering kernel leaves in Fit::rmat.
+cudaError_t launch_factor_B(const Fit& f, cudaStream_t st);
+cudaError_t launch_factor_B_batch(const Fit* fits_dev, const int* p_host, int count, const Fit* fits_host, cudaStream_t st);
 // Bounded-wait self-test (k_iter.cu): the status the wait recorded (LINGAM_ETIMEOUT expected).
 cudaError_t run_wait_selftest(int which, unsigned long long timeout_ns, int* status, cudaStream_t st);
 // B of many problems: one CTA per problem of p <= 128 (shared-memory Cholesky), the

@@ -470,8 +470,11 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
         }
         if (status != LINGAM_OK) break;
         if (cudaEventRecord(ev[3], st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
-        if (want_B && (inject_fault("bfit") || launch_fit_B(f, st) != cudaSuccess)) { status = LINGAM_ECUDA; break; }
-        if (want_B) launches += 4;
+        if (want_B && (inject_fault("bfit") || (order_kernel ? launch_factor_B(f, st) : launch_fit_B(f, st)) != cudaSuccess)) {
+            status = LINGAM_ECUDA;
+            break;
+        }
+        if (want_B) launches += order_kernel ? 2 : 4;
         if (cudaEventRecord(ev[4], st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
     } while (0);
     if (cudaStreamSynchronize(st) != cudaSuccess) status = LINGAM_ECUDA;
@@ -789,7 +792,8 @@ static cudaError_t enqueue_batch(char* ws, const BatchLayout& BL, const std::vec
     if (with_B) {
         std::vector<int> ph(static_cast<size_t>(count));
         for (int k = 0; k < count; ++k) ph[size_t(k)] = fits[size_t(k)].p;
-        e = launch_fit_B_batch(fits_dev, ph.data(), count, fits.data(), st);
+        e = groups ? launch_factor_B_batch(fits_dev, ph.data(), count, fits.data(), st)
+                   : launch_fit_B_batch(fits_dev, ph.data(), count, fits.data(), st);
         if (e != cudaSuccess) return e;
     }
     if (gather) {
