@@ -390,7 +390,7 @@ template <class T>
 __host__ __device__ inline int order_max_cols(unsigned cap, int nrow, unsigned ctl_cap) {
     for (int c = kMaxCols; c >= 4; c -= 4)
         if (unsigned(order_fixed_bytes<T>()) + unsigned((c + 1) * max_unit<T>()) * sizeof(T) <= cap &&
-            unsigned((c + 1) * nrow) * sizeof(T) <= ctl_cap)
+            unsigned((c + 1) | 1) * nrow * sizeof(T) <= ctl_cap)
             return c;
     return 0;
 }
@@ -455,6 +455,62 @@ __device__ __forceinline__ double rsqrt_fast(double x) {
 struct Removal {
     double rho, inv;
 };
+
+// Four totals of a record.
+__device__ __forceinline__ void load4(float (&v)[4], const float* p) {
+    const float4 a = __ldcg(reinterpret_cast<const float4*>(p));
+    v[0] = a.x;
+    v[1] = a.y;
+    v[2] = a.z;
+    v[3] = a.w;
+}
+__device__ __forceinline__ void load4(double (&v)[4], const double* p) {
+    const double2 a = __ldcg(reinterpret_cast<const double2*>(p)), b = __ldcg(reinterpret_cast<const double2*>(p) + 1);
+    v[0] = a.x;
+    v[1] = a.y;
+    v[2] = b.x;
+    v[3] = b.y;
+}
+
+// A pair's measure from its four sums and the two variables' statistics.
+__device__ __forceinline__ float measure_of(const Fit& f, const float (&v)[4], float4 si, float4 sj) {
+    return pair_measure_f(v[0], v[1], v[2], v[3], si, sj, __frcp_rn(float(f.n)));
+}
+__device__ __forceinline__ double measure_of(const Fit& f, const double (&v)[4], double hi, double hj) {
+    const double pad = double(f.ld - f.n) * kBeta;
+    return (hj - hi) + (hterm_inv(v[0] + pad, v[1], f.inv_n) - hterm_inv(v[2] + pad, v[3], f.inv_n));
+}
+// The statistics of the rows of a wave without a removal, in the order of its table.
+__device__ __forceinline__ float4* row_stats(const Fit& f, float) { return f.vstat; }
+__device__ __forceinline__ double* row_stats(const Fit& f, double) { return f.hx; }
+// The pitch of such a wave's measures.
+__device__ __forceinline__ int measure_pitch(int ncol) { return (ncol + 3) & ~3; }
+
+// Total t of row e: sum v of its record; four consecutive lanes have a pair's.  A removal's are left as
+// they are (its new statistics are not known to every worker).  Otherwise they are pair (e, column
+// v / 4)'s, and its measure is left: a quarter of what the controller would read, and no work of its own
+// per pair (16 columns: 8,400 -> 3,600 clocks with 300 rows, 36,000 -> 12,000 with 565).
+template <class T>
+__device__ __forceinline__ void close_total(const Fit& f, const OrderWave& wv, T* tot, T t, int e, int v) {
+    if (wv.removal) {
+        constexpr int Q = quad<T>();
+        tot[e * (4 * Q * ((wv.ncol + Q - 1) / Q) + 8) + v] = t;
+    } else {
+        const int lane = threadIdx.x & 31, c = v >> 2;
+        T m[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) m[i] = __shfl_sync(0xfu << (lane & 28), t, (lane & 28) + i);
+        if ((v & 3) == 0 && c < wv.ncol) {
+            T x = T(0);
+            if (f.reuse ? e >= wv.ncol || c < e : e != c) {
+                const auto* st = row_stats(f, T());
+                x = measure_of(f, m, __ldcg(st + e), __ldcg(st + c));
+                if (!isfinite(x)) set_status(f.ctl, LINGAM_EDEGENERATE);
+            }
+            tot[e * measure_pitch(wv.ncol) + c] = x;
+        }
+    }
+}
 
 template <class T, int NT>
 __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const Group g, const T* __restrict__ xold,
@@ -702,7 +758,7 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
                 if (LINGAM_INBOUNDS(f.ctl, (at + 1) * sizeof(Sum) <= f.rec_bytes)) {
                     if (bs != b0) s = sum_add(rec[at], s);
                     if (nseg > 1 || bs + bp < b1) rec[at] = s;
-                    else tot_out[e * RECN + v] = sum_val(s);
+                    else close_total(f, wv, tot_out, sum_val(s), e, v);
                 }
             }
         }
@@ -733,7 +789,7 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
             }
 #pragma unroll 2
             for (; k < nseg; ++k) s = sum_add(s, __ldcg(src + k * stride));
-            tot_out[e * RECN + v] = sum_val(s);
+            close_total(f, wv, tot_out, sum_val(s), e, v);
         }
     }
 }
@@ -785,10 +841,11 @@ struct CtlState {
 struct OrderShared {
     CtlState st;
     unsigned long long word;
-    int ok, nseg, npick, qnext;
+    int ok, nseg, npick, nswap, qnext;
     long long col[kMaxCols];      // the wave's complete scores (keys)
-    unsigned ckey[16 * kMaxCols];
-    int cvar[16 * kMaxCols];
+    unsigned ckey[16 * kMaxCols];   // select_lowest: the warps' keys and slots, the exchanges
+    int cslot[16 * kMaxCols];
+    int xhole[kMaxCols], xback[kMaxCols];
     long long lred[16];
     int ired[16], nkill[16];
     // to be reported once the next wave is published
@@ -806,22 +863,6 @@ __device__ __forceinline__ int part_or(int nt, int v) {
         : "r"(v), "r"(nt)
         : "memory");
     return out;
-}
-
-// Four totals of a record.
-__device__ __forceinline__ void load4(float (&v)[4], const float* p) {
-    const float4 a = __ldcg(reinterpret_cast<const float4*>(p));
-    v[0] = a.x;
-    v[1] = a.y;
-    v[2] = a.z;
-    v[3] = a.w;
-}
-__device__ __forceinline__ void load4(double (&v)[4], const double* p) {
-    const double2 a = __ldcg(reinterpret_cast<const double2*>(p)), b = __ldcg(reinterpret_cast<const double2*>(p) + 1);
-    v[0] = a.x;
-    v[1] = a.y;
-    v[2] = b.x;
-    v[3] = b.y;
 }
 
 // The 32-sample offset of a variable from its 2 (m - beta).
@@ -924,88 +965,103 @@ struct Controller {
         __syncwarp();
     }
 
-    // The `n` slots of [lo, hi) of lowest key (row[k]: the key's bits, kNoKey not a candidate), lowest
-    // first, to the positions lo, lo + 1, ...; sh.npick of them.  Each warp takes its lowest by warp
-    // minima, the first warp the lowest of those.  drop >= 0: that slot leaves first (to position hi;
-    // not a candidate).  Ends with a barrier.
+    // The `n` slots of [lo, hi) of lowest key (row[k]: the key's bits, kNoKey not a candidate) to the
+    // positions lo, lo + 1, ...; sh.npick of them.  The keys are in registers, a warp takes its lowest
+    // one after another by warp minima, and with several selecting warps the first takes the lowest of
+    // their lists.  drop >= 0: that slot leaves first (to position hi; not a candidate).  Ends with a
+    // barrier.
     __device__ __forceinline__ void select_lowest(int lo, int hi, int n, int drop) {
+        constexpr int KPT = 8;   // keys a lane; p <= 32 KPT NT / 32
         const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
         const int end = drop >= 0 ? hi + 1 : hi;
-        const int sw = end - lo <= 256 ? 1 : nt >> 5;   // selecting warps
-#pragma unroll 1
-#pragma unroll 1
-        for (int i = 0; i < n && wid < sw; ++i) {
-            unsigned b = kNoKey;
+        const int sw = end - lo <= 32 * KPT ? 1 : nt >> 5;   // selecting warps
+        int got = 0, pick = 0;   // lane i of the first warp: the i-th pick's slot
+        if (wid == 1 && drop >= 0) swap_slots(drop, hi);   // (no key changes place)
+        if (wid < sw) {
+            unsigned key[KPT], b = kNoKey;   // the lane's keys, the lowest and its slot
             int at = -1;
-#pragma unroll 1
-            for (int k = lo + tid; k < end; k += 32 * sw) {
-                const unsigned v = unsigned(row[k]);
-                if (v < b) {
-                    b = v;
+#pragma unroll
+            for (int q = 0; q < KPT; ++q) {
+                const int k = lo + tid + q * 32 * sw;
+                key[q] = k < end ? unsigned(row[k]) : kNoKey;
+                if (key[q] < b) {
+                    b = key[q];
                     at = k;
                 }
             }
-            const unsigned m = __reduce_min_sync(0xffffffffu, b);
-            if (m == kNoKey) {
 #pragma unroll 1
-                for (int q = i + lane; q < n; q += 32) sh.ckey[wid * kMaxCols + q] = kNoKey;
-                break;
-            }
-            const int src = __ffs(__ballot_sync(0xffffffffu, b == m)) - 1;
-            if (lane == src) {
-                row[at] = int(kNoKey);
-                sh.ckey[wid * kMaxCols + i] = m;
-                sh.cvar[wid * kMaxCols + i] = var[at];
-            }
-            __syncwarp();
-        }
-        if (sw > 1) bar();
-        if (wid == 0) {
-            if (drop >= 0) swap_slots(drop, hi);
-            int pos = 0, got = 0, pick = 0;   // lane i: the i-th pick's slot
-#pragma unroll 1
-            for (; got < n; ++got) {          // lane w walks the ascending list of warp w
-                const unsigned v = lane < sw && pos < n ? sh.ckey[lane * kMaxCols + pos] : kNoKey;
-                const unsigned m = __reduce_min_sync(0xffffffffu, v);
+            for (; got < n; ++got) {
+                const unsigned m = __reduce_min_sync(0xffffffffu, b);
                 if (m == kNoKey) break;
-                const int src = __ffs(__ballot_sync(0xffffffffu, v == m)) - 1;
-                int c = lane == src ? sh.cvar[lane * kMaxCols + pos] : 0;
-                if (lane == src) ++pos;
-                c = __shfl_sync(0xffffffffu, c, src);
-                if (lane == got) pick = slot[c];
+                const int src = __ffs(__ballot_sync(0xffffffffu, b == m)) - 1;
+                const int k = __shfl_sync(0xffffffffu, at, src);
+                if (lane == got) {
+                    pick = k;
+                    sh.ckey[wid * kMaxCols + lane] = m;
+                }
+                if (lane == src) {
+                    b = kNoKey;
+#pragma unroll
+                    for (int q = 0; q < KPT; ++q) {
+                        const int kq = lo + tid + q * 32 * sw;
+                        if (kq == k) key[q] = kNoKey;
+                        if (key[q] < b) {
+                            b = key[q];
+                            at = kq;
+                        }
+                    }
+                }
             }
+            if (sw > 1) {
+                if (lane < got) sh.cslot[wid * kMaxCols + lane] = pick;
+                else if (lane < n) sh.ckey[wid * kMaxCols + lane] = kNoKey;
+            }
+        }
+        if (sw > 1) {
+            bar();
+            if (wid == 0) {
+                int pos = 0;   // lane w walks the ascending list of warp w
+                unsigned b = lane < sw ? sh.ckey[lane * kMaxCols] : kNoKey;
+#pragma unroll 1
+                for (got = 0; got < n; ++got) {
+                    const unsigned m = __reduce_min_sync(0xffffffffu, b);
+                    if (m == kNoKey) break;
+                    const int src = __ffs(__ballot_sync(0xffffffffu, b == m)) - 1;
+                    const int from = __shfl_sync(0xffffffffu, pos, src);
+                    if (lane == got) pick = src * kMaxCols + from;
+                    if (lane == src) {
+                        ++pos;
+                        b = pos < n ? sh.ckey[lane * kMaxCols + pos] : kNoKey;
+                    }
+                }
+                if (lane < got) pick = sh.cslot[pick];
+            }
+        }
+        if (wid == 0) {
             // the picks behind the first `got` slots change places with the slots among those that
-            // were not picked: exchanges of different pairs of slots, three at a time
+            // were not picked (as many)
+            if (pick == hi && drop >= 0) pick = drop;
             const bool mine = lane < got, front = mine && pick < lo + got;
             const unsigned infront = __reduce_or_sync(0xffffffffu, front ? 1u << (pick - lo) : 0u);
-            const unsigned back = __ballot_sync(0xffffffffu, mine && !front);
-            unsigned holes = ((1u << got) - 1u) & ~infront;
-            const int rank = __popc(back & ((1u << lane) - 1u));
-            int hole = 0;   // lane of a back pick: its place
+            const unsigned back = __ballot_sync(0xffffffffu, mine && !front), lt = (1u << lane) - 1u;
+            const unsigned holes = (got < 32 ? (1u << got) - 1u : 0xffffffffu) & ~infront;
+            if (holes >> lane & 1u) sh.xhole[__popc(holes & lt)] = lo + lane;
+            if (mine && !front) sh.xback[__popc(back & lt)] = pick;
+            if (lane == 0) {
+                sh.npick = got;
+                sh.nswap = __popc(back);
+            }
+        }
+        bar();
+        const int ns = sh.nswap;
 #pragma unroll 1
-            for (int i = 0; i <= rank && holes; ++i) {
-                hole = __ffs(holes) - 1;
-                holes &= holes - 1u;
+        for (int u = tid; u < 10 * ns; u += nt) {
+            const int i = small_div(u, 10), what = u - 10 * i, x = sh.xhole[i], y = sh.xback[i];
+            swap_part(what, x, y);
+            if (what == 8) {   // var
+                slot[var[x]] = x;
+                slot[var[y]] = y;
             }
-            const int group = lane < 30 ? lane / 10 : 3, what = lane - 10 * group;
-#pragma unroll 1
-            for (unsigned left = back; left;) {
-                int src = -1;
-#pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    if (left) {
-                        if (group == q) src = __ffs(left) - 1;
-                        left &= left - 1u;
-                    }
-                const int x = __shfl_sync(0xffffffffu, lo + hole, src & 31), y = __shfl_sync(0xffffffffu, pick, src & 31);
-                if (src >= 0) swap_part(what, x, y);
-            }
-            __syncwarp();
-            if (mine && !front) {
-                slot[var[lo + hole]] = lo + hole;
-                slot[var[pick]] = pick;
-            }
-            if (lane == 0) sh.npick = got;
         }
         bar();
     }
@@ -1035,7 +1091,13 @@ struct Controller {
                     keval[k] = -1;
                 }
                 if (a == 0) kc[k] = 0.f;
-                if (LINGAM_INBOUNDS(f.ctl, i < f.p && e.var < f.p)) tab[i] = e;
+                if (LINGAM_INBOUNDS(f.ctl, i < f.p && e.var < f.p)) {
+                    tab[i] = e;
+                    if (!removal) {
+                        if constexpr (f32) f.vstat[i] = st[k];
+                        else f.hx[i] = *reinterpret_cast<const double*>(&st[k]);
+                    }
+                }
             }
         } else {
             const int lane = tid & 31;
@@ -1158,13 +1220,8 @@ struct Controller {
     // One pair's measure from its four sums: row slot k against slot j.
     __device__ __forceinline__ T measure(const T (&v)[4], int k, int j) const {
         T x;
-        if constexpr (f32) {
-            x = pair_measure_f(v[0], v[1], v[2], v[3], st[k], st[j], __frcp_rn(float(f.n)));
-        } else {
-            const double pad = double(f.ld - f.n) * kBeta;
-            const double ha = hterm_inv(v[0] + pad, v[1], f.inv_n), hb = hterm_inv(v[2] + pad, v[3], f.inv_n);
-            x = (*reinterpret_cast<const double*>(&st[j]) - *reinterpret_cast<const double*>(&st[k])) + (ha - hb);
-        }
+        if constexpr (f32) x = measure_of(f, v, st[k], st[j]);
+        else x = measure_of(f, v, *reinterpret_cast<const double*>(&st[k]), *reinterpret_cast<const double*>(&st[j]));
         if (!isfinite(x)) set_status(f.ctl, LINGAM_EDEGENERATE);
         return x;
     }
@@ -1174,18 +1231,39 @@ struct Controller {
     __device__ __forceinline__ void finish_wave(const OrderWave& wv) {
         const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
         const int ncol = wv.ncol, nrow = wv.nrow, nseg = wv.nseg, nq = (ncol + Q - 1) / Q, has_k = wv.removal;
-        const int RECN = 4 * Q * nq + 8 * has_k, np = ncol + has_k, own = 4 * Q * nq;
+        const int RECN = 4 * Q * nq + 8 * has_k, np = ncol + has_k, own = 4 * Q * nq, ip = np | 1;   // (ip: I's pitch)
         r = sh.st.r;
         a = sh.st.a;
         it = sh.st.it;
         next_wave(0, -1, false, 0);
-        const int nw = min(NW, max(4, (r + 63) >> 6));
+        const int nw = min(NW, max(4, ncol > 8 ? (r + 31) >> 5 : (r + 63) >> 6));
         nt = 32 * nw;
         const T* tot = reinterpret_cast<const T*>(static_cast<const Sum*>(f.rec) + size_t(nseg) * nrow * RECN);
         // 1. the rows' own statistics (removal: of the new rows) and I of every pair.  Units: the rows'
         //    statistics first, then row e against column c or its killer (c = ncol); a thread has four
-        //    units' totals in flight.
-        const int stats = has_k ? nrow : 0, units = stats + nrow * np;
+        //    units' totals in flight.  Without a removal the workers have left the measures.
+        const int stats = has_k ? nrow : 0, units = has_k ? stats + nrow * np : 0;
+        if (!has_k) {
+            const int w4 = measure_pitch(ncol) / 4, n4 = nrow * w4;
+#pragma unroll 1
+            for (int u0 = 0; u0 < n4; u0 += 4 * NT) {
+                T v[4][4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (u0 + q * NT + tid < n4) load4(v[q], tot + 4 * (u0 + q * NT + tid));
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int u = u0 + q * NT + tid;
+                    if (u < n4) {
+                        const int e = small_div(u, w4), c = 4 * (u - e * w4);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (c + i < ncol) I[e * ip + c + i] = v[q][i];
+                    }
+                }
+            }
+        }
+#pragma unroll 1
         for (int u0 = 0; u0 < units; u0 += 4 * NT) {
             T v[4][4];
             int kj[4], es[4];   // the partner's slot (-1: nothing to do), the row
@@ -1235,7 +1313,7 @@ struct Controller {
             for (int q = 0; q < 4; ++q) {
                 const int u = u0 + q * NT + tid;
                 if (u0 + q * NT < units && u >= stats && u < units)
-                    I[u - stats] = kj[q] >= 0 ? measure(v[q], row_slot(es[q]), kj[q]) : T(0);
+                    I[u - stats + es[q] * (ip - np)] = kj[q] >= 0 ? measure(v[q], row_slot(es[q]), kj[q]) : T(0);
             }
         }
         __syncthreads();
@@ -1253,7 +1331,7 @@ struct Controller {
                 if (keval[sk] != var[k] || var[k] < ke)
                     nk += has_k ? 1 : (sk >= a && (k < a + ncol || sk < a + ncol)) ? -1 : 0;
             }
-            const T* Ir = I + e * np;
+            const T* Ir = I + e * ip;
             const int cm = min(e, ncol);
             Sum acc = Sum();
             float top = 0.f;
@@ -1314,7 +1392,7 @@ struct Controller {
             int tope = -1;
 #pragma unroll 1
             for (int e = (f.reuse ? c + 1 : 0) + lane; e < nrow; e += 32) {
-                const T x = I[e * np + c];   // (0 for the column itself)
+                const T x = I[e * ip + c];   // (0 for the column itself)
                 const T m = x > T(0) ? x : T(0);
                 add_square(acc, m);
                 const float ctr = float(m) * float(m);
@@ -1430,7 +1508,7 @@ struct Controller {
             float ctr = 0.f;
             if (rs >= a && rs < an && k >= a && k != rs) {
                 const int c = rs - a, e = k - a;
-                const float x = e > c ? fminf(float(I[e * np + c]), 0.f) : fmaxf(float(I[c * np + e]), 0.f);
+                const float x = e > c ? fminf(float(I[e * ip + c]), 0.f) : fmaxf(float(I[c * ip + e]), 0.f);
                 ctr = x * x;
             } else if (rs >= an && keval[k] == root) {
                 ctr = kc[k];
