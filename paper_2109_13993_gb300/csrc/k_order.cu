@@ -49,11 +49,10 @@
 namespace lingam {
 
 constexpr int kMaxCols = 16;     // columns of a wave at most (four quads)
-// A unit of a warp's work is 1024 or 512 samples on the FP32 path (32 or 16 per lane, one lg2 per
-// residual; Fit::unit: 512 for single fits of less than 4 M samples in all, whose waves keep few warps
-// busy), 256 samples on the FP64 path, of one row against quad() columns: four on the FP32 path (the
-// row's reads serve four pairs), one on the FP64 path, where a warp alone has only its SM quarter's
-// FP64 unit.  max_unit: what the shared memory is sized for.
+// A unit of a warp's work is 1024 samples or less (Fit::unit) on the FP32 path (up to 32 per lane, one
+// lg2 per residual), 256 or less on the FP64 path, of one row against quad() columns: four on the FP32
+// path (the row's reads serve four pairs), one on the FP64 path, where a warp alone has only its SM
+// quarter's FP64 unit.  max_unit: what the shared memory is sized for.
 template <class T>
 __host__ __device__ constexpr int max_unit() { return sizeof(T) == 4 ? 1024 : 256; }
 template <class T>
@@ -1556,7 +1555,10 @@ struct Controller {
         for (int w = 0; w < nw; ++w) need += sh.ired[w];
         r -= 1;
         a = 0;
-        const int cmax = max_cols(r), want = prunes && !gmode ? (need + 4) / 4 * 4 : kMaxCols;
+        // As many columns as this iteration would have needed, had it known its strongest pairs: whole
+        // quads with one to spare on the FP32 path (a column of a started quad is free), no more on the
+        // FP64 path (65 x 2001: 4.0 ms, one or two to spare 4.3 and 4.9, quads 5.3).
+        const int cmax = max_cols(r), want = !prunes || gmode ? kMaxCols : f32 ? (need + 4) / 4 * 4 : max(need, 1);
         new_iteration(cmax, want);
         if (r == 1) {
             if (tid < 32) swap_slots(rs, 1);

@@ -213,6 +213,17 @@ static EventPool* event_pool(int dev) {
     return &pools[dev];
 }
 
+// Samples of the ordering kernel's units of a problem of `samples` (rows x padded length; a batch's:
+// any number).  Small problems have few units for the chip's warps, each as long as its steps' latencies
+// (and an FP64 warp alone has less than half its quarter's FP64 rate); large ones save the units' sums.
+// Ordering, ms: mixed 20 x 2000 0.405 (512), 0.397 (256), 50 x 2000 1.073 and 1.059, 100 x 10000 2.63 and
+// 2.70, 300 x 5000 8.95 (1024) and 8.88 (512), 50 x 100000 2.03 and 2.08; FP64 20 x 2000 1.07 (256),
+// 0.88 (128), 0.83 (64), 30 x 2000 1.55, 1.35, 1.33, 65 x 2001 4.28, 4.04, 4.31, 100 x 3000 17.4, 18.1, 20.4.
+static int order_unit(int precision, size_t samples) {
+    if (precision == LINGAM_MIXED) return samples < (size_t(1) << 18) ? 256 : samples < (size_t(4) << 20) ? 512 : 1024;
+    return samples < (size_t(1) << 16) ? 64 : samples < (size_t(1) << 18) ? 128 : 256;
+}
+
 // The device view of one problem laid out in `base` (a workspace region of layout L).
 // Narrow waves: waves of <= 16 columns and at least this many rows run on 128 x 16 tiles
 // (LINGAM_NARROW=<rows> overrides the default; 0 turns them off, a switch for measuring them).
@@ -284,7 +295,7 @@ static Fit make_fit(char* base, const Layout& L, int p, int n, const lingam_opts
     f.rec_bytes = L.alt_in_xin ? L.partial_bytes : L.partial_bytes / 2 / kAlign * kAlign;
     f.xalt = L.alt_in_xin ? base + L.off_xin : base + L.off_partials + f.rec_bytes;
     f.sigalt = f.cmat;
-    f.unit = o.precision == LINGAM_MIXED ? (size_t(p) * size_t(L.ld) < (size_t(4) << 20) ? 512 : 1024) : 256;
+    f.unit = order_unit(o.precision, size_t(p) * size_t(L.ld));
     f.rowtab = f.ibuf;
     f.dscale[0] = reinterpret_cast<double*>(static_cast<char*>(f.ibuf) + size_t(p) * 16);
     f.dscale[1] = f.dscale[0] + p;
@@ -325,9 +336,16 @@ static bool check_prior(const signed char* prior, int p, std::vector<int>& anc) 
 }
 
 // Single fits run the ordering kernel (k_order.cu) unless an option asks for the tile kernels
-// (an explicit tile shape, LINGAM_NARROW) or the problem is too large for it.
+// (an explicit tile shape, LINGAM_NARROW) or the problem is too large for it.  Without the killer pairs
+// (no pruning, no pair reuse, the paper's threshold schedule) most columns are computed, and the tile
+// kernels' waves of 32 columns win on the mixed path from about 150 variables on: unpruned, ordering
+// kernel against tile kernels, p 100 11.3 and 13.3 ms, p 150 21.7 and 22.7, p 300 93.6 and 80.6; with
+// the schedule from 10^-3 9.2 and 11.4, 17.0 and 18.2, 72.9 and 58.6.
+constexpr int kOrderFullP = 160;
 static bool use_order_kernel(const Fit& f, const lingam_opts& o) {
-    return o.tile_i == 0 && o.tile_j == 0 && !narrow_set() && order_supported(f, false);
+    const bool killers = o.prune && o.reuse && !(o.gamma0 > 0.0);
+    return o.tile_i == 0 && o.tile_j == 0 && !narrow_set() &&
+           (killers || o.precision != LINGAM_MIXED || f.p <= kOrderFullP) && order_supported(f, false);
 }
 
 // cov_out != nullptr: stop after CalculateCovMat and copy Sigma (p x p) there.
@@ -901,7 +919,7 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
         f.tile_rows = ts.rows;
         f.tile_cols = ts.cols;
         f.split_n = 0;
-        if (o.precision == LINGAM_MIXED) f.unit = 1024;   // many problems: the warps are busy
+        f.unit = order_unit(o.precision, ~size_t(0));   // many problems: the warps are busy
         f.narrow = 0;   // the batch kernel runs every wave on the call's tile shape
         fits[size_t(k)] = f;
         SrcDesc sd;
