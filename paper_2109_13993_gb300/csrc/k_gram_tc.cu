@@ -3,29 +3,33 @@
 //
 // Error-free splitting (the scheme of Ozaki, Ogita, Oishi and Rump, 2012):
 // each row i is scaled by a power of two 2^-e_i so that |y| < 1, and
-// y 2^7 = D0 + 2^-7 D1 + 2^-14 T with D0, D1 integers (|D0| <= 128,
-// |D1| <= 64) and T the TF32 rounding of the remaining tail (|T| <= 64); all
-// three are exact TF32 operands.  Then
-//   x_i x_j 2^(14 - e_i - e_j) = D0D0 + 2^-7 (D0D1 + D1D0)
-//                              + 2^-14 (D0T + TD0 + D1D1) + 2^-21 (D1T + TD1) + O(2^-28 TT),
+// y 2^7 = D0 + 2^-8 D1 + 2^-16 T with D0, D1 integers (|D0|, |D1| <= 128) and T
+// the remaining tail (|T| <= 128) rounded to FP16's eleven bits; all three are
+// FP16 operands (kind::f16 runs at twice the rate of kind::tf32, whose operands
+// hold the same eleven bits, and moves half the bytes: the covariance of
+// p = 1000, n = 10000 0.183 -> 0.124 ms on the device).  Then
+//   x_i x_j 2^(14 - e_i - e_j) = D0D0 + 2^-8 (D0D1 + D1D0)
+//                              + 2^-16 (D0T + TD0 + D1D1) + 2^-24 (D1T + TD1) + O(2^-32 TT),
 // and the four levels accumulate in four tensor-memory accumulators (the
 // whole 512-column TMEM).  The products of the first two levels are integers
-// of at most 2^14, so their FP32 sums stay exact for 512 samples whatever the
-// rounding of the tensor core's adder; the last two levels carry weights of
-// 2^-14 and 2^-21, so their FP32 rounding is negligible.  Every 512 samples
+// of at most 2^14, one a sample in the first and two in the second, so their
+// FP32 sums stay exact (at most 2^24) for 512 samples whatever the rounding of
+// the tensor core's adder; the last two levels carry weights of 2^-16 and
+// 2^-24, so their FP32 rounding is negligible.  Every 512 samples
 // the accumulators are drained into float-float sums in registers.  The
 // split of the sample axis over CTAs is summed in FP64 by a second kernel,
 // which also applies 2^(e_i + e_j - 14) / (n - 1).
 //
-// Per CTA (320 threads): warp 8 streams the six 128 x 32 operand blocks of a
+// Per CTA (320 threads): warp 8 streams the six 128 x 64 operand blocks of a
 // k-step (D0, D1, T of the row tile and of the column tile) into a two-stage
 // shared-memory ring with 2-D TMA loads (128-byte swizzle); warp 9 issues the
-// tcgen05.mma instructions (kind::tf32, M = N = 128, K = 8) that read the ring
+// tcgen05.mma instructions (kind::f16, M = N = 128, K = 16) that read the ring
 // through shared-memory matrix descriptors, and commits each stage back to
 // the producer; warps 0-7 drain the accumulators (warp w reads TMEM lanes
 // 32 (w mod 4) ... and columns 64 (w / 4) ... of each level).  All waits are
 // bounded by the fit's timeout.
 #include <cuda.h>
+#include <cuda_fp16.h>
 
 #include "common.cuh"
 #include "launch.h"
@@ -34,12 +38,12 @@
 namespace lingam {
 
 constexpr int kGM = 128;                          // tile rows = tile columns
-constexpr int kGKB = 32;                          // samples per k-step (128 bytes of FP32)
+constexpr int kGKB = 64;                          // samples per k-step (128 bytes of FP16)
 constexpr int kGStagesTC = 2;
 constexpr int kGOps = 6;                          // operand blocks per stage
-constexpr uint32_t kGBlockBytes = kGM * kGKB * 4;  // one 128 x 32 operand block, 16 KB
+constexpr uint32_t kGBlockBytes = kGM * kGKB * 2;  // one 128 x 64 operand block, 16 KB
 constexpr uint32_t kGStageBytes = kGOps * kGBlockBytes;
-constexpr int kGDrain = 16;                       // k-steps (512 samples) per accumulation group
+constexpr int kGDrain = 8;                        // k-steps (512 samples) per accumulation group
 constexpr int kGDrainWarps = 8;
 constexpr int kGThreads = 32 * (kGDrainWarps + 2);
 constexpr uint32_t kGTmemCols = 4 * kGM;          // four level accumulators
@@ -62,13 +66,13 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {  
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
-// D[tmem] (+)= A[desc] * B[desc]^T, both K-major, TF32 inputs, FP32 accumulator.
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+// D[tmem] (+)= A[desc] * B[desc]^T, both K-major, FP16 inputs, FP32 accumulator.
+__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
@@ -114,9 +118,8 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t smem_addr) {
     d |= uint64_t(2) << 61;                       // 128-byte swizzle
     return d;
 }
-// Instruction descriptor: D FP32, A and B TF32, both K-major, M = N = 128.
-constexpr uint32_t kIdescTF32 = (1u << 4) | (2u << 7) | (2u << 10) | (uint32_t(kGM >> 3) << 17) |
-                                (uint32_t(kGM >> 4) << 24);
+// Instruction descriptor: D FP32, A and B FP16 (format 0), both K-major, M = N = 128.
+constexpr uint32_t kIdescF16 = (1u << 4) | (uint32_t(kGM >> 3) << 17) | (uint32_t(kGM >> 4) << 24);
 
 __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Ctl* ctl, unsigned long long tmo) {
     return mbar_wait_bounded(bar, parity, ctl, tmo);
@@ -131,10 +134,18 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 
 // ------------------------------------------------------------------ digits of the normalised rows
 // One CTA per row: e = the exponent of max_t |x_t| (so |x 2^-e| < 1), then the
-// digits D0, D1 and the TF32 tail T of y 2^7 = x 2^(7-e), written as FP32.
+// digits D0, D1 and the tail T of y 2^7 = x 2^(7-e) in FP16 (tails below 2^-14 are
+// subnormal there: off by 2^-25 at most, against 2^-5 for the largest).
 constexpr int kDigitThreads = 256;
-__global__ void __launch_bounds__(kDigitThreads) k_digits(const float* __restrict__ x, float* __restrict__ d0,
-                                                        float* __restrict__ d1, float* __restrict__ tt,
+__device__ __forceinline__ void put_half4(__half* dst, const float (&v)[4]) {
+    const __half2 a = __floats2half2_rn(v[0], v[1]), b = __floats2half2_rn(v[2], v[3]);
+    uint2 w;
+    w.x = *reinterpret_cast<const unsigned*>(&a);
+    w.y = *reinterpret_cast<const unsigned*>(&b);
+    *reinterpret_cast<uint2*>(dst) = w;
+}
+__global__ void __launch_bounds__(kDigitThreads) k_digits(const float* __restrict__ x, __half* __restrict__ d0,
+                                                        __half* __restrict__ d1, __half* __restrict__ tt,
                                                         int* __restrict__ expo, int ld) {
     __shared__ float red[kDigitThreads / 32];
     const size_t row = size_t(blockIdx.x) * ld;
@@ -153,16 +164,22 @@ __global__ void __launch_bounds__(kDigitThreads) k_digits(const float* __restric
     int e = 0;
     frexpf(m, &e);   // m = f 2^e, f in [0.5, 1) (e = 0 for m = 0)
     if (threadIdx.x == 0) expo[blockIdx.x] = e;
-    for (int t = threadIdx.x; t < ld; t += kDigitThreads) {
-        const float y = ldexpf(x[row + t], 7 - e);   // exact: a power-of-two scaling
-        const float a = rintf(y);
-        const float r0 = ldexpf(y - a, 7);            // y - a is exact, |y - a| <= 1/2
-        const float b = rintf(r0);
-        const float r1 = ldexpf(r0 - b, 7);
-        const float c = __uint_as_float((__float_as_uint(r1) + 0x1000u) & 0xFFFFE000u);   // TF32 rounding
-        d0[row + t] = a;
-        d1[row + t] = b;
-        tt[row + t] = c;
+    const float up = ldexpf(1.f, 7 - e);   // (e >= -126: finite)
+    for (int t = threadIdx.x * 4; t < ld; t += kDigitThreads * 4) {
+        const float4 v = *reinterpret_cast<const float4*>(x + row + t);
+        const float y[4] = {v.x, v.y, v.z, v.w};
+        float q[3][4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float z = y[k] * up;                // exact: a power-of-two scaling
+            q[0][k] = rintf(z);
+            const float r0 = (z - q[0][k]) * 256.f;   // the difference is exact, at most 1/2
+            q[1][k] = rintf(r0);
+            q[2][k] = (r0 - q[1][k]) * 256.f;
+        }
+        put_half4(d0 + row + t, q[0]);
+        put_half4(d1 + row + t, q[1]);
+        put_half4(tt + row + t, q[2]);
     }
 }
 
@@ -237,7 +254,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
                 tc_fence_after();
                 const uint32_t base = smem_u32(smem + size_t(s) * kGStageBytes);
 #pragma unroll
-                for (int j = 0; j < kGKB / 8; ++j) {   // K = 8 TF32 values = 32 bytes per instruction
+                for (int j = 0; j < kGKB / 16; ++j) {   // K = 16 FP16 values = 32 bytes per instruction
                     const uint64_t a0 = sw128_desc(base + 0 * kGBlockBytes + 32 * j);
                     const uint64_t a1 = sw128_desc(base + 1 * kGBlockBytes + 32 * j);
                     const uint64_t at = sw128_desc(base + 2 * kGBlockBytes + 32 * j);
@@ -245,14 +262,14 @@ __global__ void __launch_bounds__(kGThreads, 1)
                     const uint64_t b1 = sw128_desc(base + 4 * kGBlockBytes + 32 * j);
                     const uint64_t bt = sw128_desc(base + 5 * kGBlockBytes + 32 * j);
                     const uint32_t acc = (first && j == 0) ? 0u : 1u;
-                    mma_tf32(tmem + 0 * kGM, a0, b0, kIdescTF32, acc);   // level 0
-                    mma_tf32(tmem + 1 * kGM, a0, b1, kIdescTF32, acc);   // level 1
-                    mma_tf32(tmem + 1 * kGM, a1, b0, kIdescTF32, 1);
-                    mma_tf32(tmem + 2 * kGM, a0, bt, kIdescTF32, acc);   // level 2
-                    mma_tf32(tmem + 2 * kGM, at, b0, kIdescTF32, 1);
-                    mma_tf32(tmem + 2 * kGM, a1, b1, kIdescTF32, 1);
-                    mma_tf32(tmem + 3 * kGM, a1, bt, kIdescTF32, acc);   // level 3
-                    mma_tf32(tmem + 3 * kGM, at, b1, kIdescTF32, 1);
+                    mma_f16(tmem + 0 * kGM, a0, b0, kIdescF16, acc);   // level 0
+                    mma_f16(tmem + 1 * kGM, a0, b1, kIdescF16, acc);   // level 1
+                    mma_f16(tmem + 1 * kGM, a1, b0, kIdescF16, 1);
+                    mma_f16(tmem + 2 * kGM, a0, bt, kIdescF16, acc);   // level 2
+                    mma_f16(tmem + 2 * kGM, at, b0, kIdescF16, 1);
+                    mma_f16(tmem + 2 * kGM, a1, b1, kIdescF16, 1);
+                    mma_f16(tmem + 3 * kGM, a1, bt, kIdescF16, acc);   // level 3
+                    mma_f16(tmem + 3 * kGM, at, b1, kIdescF16, 1);
                 }
                 mma_commit(&empty[s]);   // stage s may be refilled once these MMAs are done
                 if ((k % kGDrain) == kGDrain - 1 || k == nkb - 1) mma_commit(&tfull);
@@ -278,7 +295,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     float hi, lo, s, e;
-                    two_sum(v0[q], __fmul_rn(v1[q], 0x1p-7f), hi, lo);   // exact integers: exact sum
+                    two_sum(v0[q], __fmul_rn(v1[q], 0x1p-8f), hi, lo);   // exact integers: exact sum
                     two_sum(S[c0 + q], hi, s, e);
                     S[c0 + q] = s;
                     E[c0 + q] = __fadd_rn(E[c0 + q], __fadd_rn(e, lo));
@@ -286,7 +303,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
                 tmem_ld8x2(taddr + 2 * kGM + c0, taddr + 3 * kGM + c0, v0, v1);
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
-                    E[c0 + q] = __fadd_rn(E[c0 + q], __fmaf_rn(v1[q], 0x1p-21f, __fmul_rn(v0[q], 0x1p-14f)));
+                    E[c0 + q] = __fadd_rn(E[c0 + q], __fmaf_rn(v1[q], 0x1p-24f, __fmul_rn(v0[q], 0x1p-16f)));
             }
             tc_fence_before();
             __syncwarp();
@@ -310,45 +327,58 @@ __global__ void __launch_bounds__(kGThreads, 1)
 }
 
 // Sum the split partial tiles in split order (FP64), scale by 2^(e_i + e_j - 14) / (n - 1),
-// write Sigma and Sigma0 (both triangles) with a unit diagonal.
-__global__ void k_gram_tc_reduce(Fit f, const float2* __restrict__ partial, const int* __restrict__ expo, int nt,
-                                 int nsplit) {
-    const int tile = blockIdx.y;
+// write Sigma and Sigma0 (both triangles) with a unit diagonal.  A CTA takes an 8 x 8 part of a
+// tile, an element a thread, and writes its transpose out of shared memory, whole sectors as well.
+// Small parts, because the splits' sums (up to 32, in FP64) of a small p would sit on few SMs'
+// FP64 units: p = 100 with 32 splits 33 us in parts of 8 rows x 128, 43 us in 32 x 32, 8 us so.
+constexpr int kRPart = 8;
+__global__ void __launch_bounds__(kRPart* kRPart)
+    k_gram_tc_reduce(Fit f, const float2* __restrict__ partial, const int* __restrict__ expo, int nt, int nsplit) {
+    __shared__ double s_v[kRPart][kRPart + 1];
+    const int tile = blockIdx.y, part = blockIdx.x;   // part: kGM / kRPart squared of a tile
     int bi = 0, rem = tile;
     while (rem >= nt - bi) {
         rem -= nt - bi;
         ++bi;
     }
     const int bj = bi + rem;
-    const size_t ntri = size_t(nt) * (nt + 1) / 2;
+    const int r0 = part / (kGM / kRPart) * kRPart, c0 = part % (kGM / kRPart) * kRPart, i0 = bi * kGM + r0, j0 = bj * kGM + c0;
+    const int p = f.p, tx = threadIdx.x % kRPart, ty = threadIdx.x / kRPart;
+    if (i0 >= p || j0 >= p || i0 > j0) return;   // (the same for the whole CTA)
+    const size_t step = size_t(nt) * (nt + 1) / 2 * kGM * kGM;
     const double inv = 1.0 / double(f.n - 1);
-    const int p = f.p;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < kGM * kGM; e += gridDim.x * blockDim.x) {
-        const int r = e / kGM, c = e % kGM;
-        const int i = bi * kGM + r, j = bj * kGM + c;
-        if (i >= p || j >= p || i > j) continue;
-        // split order; eight loads in flight at a time
-        double s = 0.0;
-        int sp = 0;
-        for (; sp + 8 <= nsplit; sp += 8) {
-            float2 v[8];
+    {
+        const int i = i0 + ty, j = j0 + tx;
+        if (i < p && j < p && i <= j) {
+            const float2* src = partial + (size_t(tile) * kGM + r0 + ty) * kGM + c0 + tx;
+            // split order; eight loads in flight at a time
+            double s = 0.0;
+            int sp = 0;
+            for (; sp + 8 <= nsplit; sp += 8) {
+                float2 v[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = partial[((size_t(sp + q) * ntri + tile) * kGM + r) * kGM + c];
+                for (int q = 0; q < 8; ++q) v[q] = src[size_t(sp + q) * step];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) s += double(v[q].x) + double(v[q].y);
+                for (int q = 0; q < 8; ++q) s += double(v[q].x) + double(v[q].y);
+            }
+            for (; sp < nsplit; ++sp) {
+                const float2 v = src[size_t(sp) * step];
+                s += double(v.x) + double(v.y);
+            }
+            const double v = i == j ? 1.0 : ldexp(s, expo[i] + expo[j] - 14) * inv;
+            s_v[ty][tx] = v;
+            f.sig[size_t(i) * p + j] = v;
+            f.sig0[size_t(i) * p + j] = v;
+            f.sigf[size_t(i) * p + j] = sig_pair_f(v);
         }
-        for (; sp < nsplit; ++sp) {
-            const float2 v = partial[((size_t(sp) * ntri + tile) * kGM + r) * kGM + c];
-            s += double(v.x) + double(v.y);
-        }
-        const double v = (i == j) ? 1.0 : ldexp(s, expo[i] + expo[j] - 14) * inv;
-        f.sig[size_t(i) * p + j] = v;
+    }
+    __syncthreads();
+    const int i = i0 + tx, j = j0 + ty;
+    if (i < p && j < p && i < j) {
+        const double v = s_v[tx][ty];
         f.sig[size_t(j) * p + i] = v;
-        f.sig0[size_t(i) * p + j] = v;
         f.sig0[size_t(j) * p + i] = v;
-        const float2 vf = sig_pair_f(v);
-        f.sigf[size_t(i) * p + j] = vf;
-        f.sigf[size_t(j) * p + i] = vf;
+        f.sigf[size_t(j) * p + i] = sig_pair_f(v);
     }
 }
 
@@ -376,6 +406,7 @@ size_t gram_tc_partial_bytes(long long p, int ld) {
     return size_t(g.nsplit) * size_t(g.ntri) * kGM * kGM * sizeof(float2);
 }
 
+// Half of it is used: the sizes that the entry points state (and refuse) are those of FP32 planes.
 size_t gram_tc_digit_bytes(long long p, int ld) {
     return 3 * size_t(p) * size_t(ld) * sizeof(float) + size_t(p) * sizeof(int);
 }
@@ -401,25 +432,25 @@ static EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// 2-D map over a p x ld FP32 matrix (row stride ld), boxes of 32 samples x 128 rows,
+// 2-D map over a p x ld FP16 matrix (row stride ld), boxes of 64 samples x 128 rows,
 // 128-byte swizzle, rows beyond p read as zero.
 static bool make_map(CUtensorMap* map, void* base, int p, int ld) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     const cuuint64_t dims[2] = {cuuint64_t(ld), cuuint64_t(p)};
-    const cuuint64_t strides[1] = {cuuint64_t(ld) * sizeof(float)};
+    const cuuint64_t strides[1] = {cuuint64_t(ld) * sizeof(__half)};
     const cuuint32_t box[2] = {cuuint32_t(kGKB), cuuint32_t(kGM)};
     const cuuint32_t estr[2] = {1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 cudaError_t launch_gram_tc(const Fit& f, void* digits, void* partial, cudaStream_t st) {
     const size_t plane = size_t(f.p) * f.ld;
-    float* d0 = static_cast<float*>(digits);
-    float* d1 = d0 + plane;
-    float* tt = d1 + plane;
+    __half* d0 = static_cast<__half*>(digits);
+    __half* d1 = d0 + plane;
+    __half* tt = d1 + plane;
     int* expo = reinterpret_cast<int*>(tt + plane);
     k_digits<<<f.p, kDigitThreads, 0, st>>>(static_cast<const float*>(f.xt), d0, d1, tt, expo, f.ld);
     cudaError_t e = cudaGetLastError();
@@ -435,7 +466,7 @@ cudaError_t launch_gram_tc(const Fit& f, void* digits, void* partial, cudaStream
                                                                          g.kb_total, g.nsplit, f.ctl);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_gram_tc_reduce<<<dim3(16, g.ntri), 256, 0, st>>>(f, part, expo, g.nt, g.nsplit);
+    k_gram_tc_reduce<<<dim3((kGM / kRPart) * (kGM / kRPart), g.ntri), kRPart * kRPart, 0, st>>>(f, part, expo, g.nt, g.nsplit);
     return cudaGetLastError();
 }
 
