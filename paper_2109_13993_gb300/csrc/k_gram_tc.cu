@@ -3,19 +3,19 @@
 //
 // Error-free splitting (the scheme of Ozaki, Ogita, Oishi and Rump, 2012):
 // each row i is scaled by a power of two 2^-e_i so that |y| < 1, and
-// y 2^7 = D0 + 2^-8 D1 + 2^-16 T with D0, D1 integers (|D0|, |D1| <= 128) and T
-// the remaining tail (|T| <= 128) rounded to FP16's eleven bits; all three are
-// FP16 operands (kind::f16 runs at twice the rate of kind::tf32, whose operands
-// hold the same eleven bits, and moves half the bytes: the covariance of
-// p = 1000, n = 10000 0.183 -> 0.124 ms on the device).  Then
-//   x_i x_j 2^(14 - e_i - e_j) = D0D0 + 2^-8 (D0D1 + D1D0)
-//                              + 2^-16 (D0T + TD0 + D1D1) + 2^-24 (D1T + TD1) + O(2^-32 TT),
+// y 2^7 = D0 + 2^-7 D1 + 2^-14 T with D0, D1 integers (|D0| <= 128,
+// |D1| <= 64) and T the remaining tail (|T| <= 64) rounded to FP16's eleven
+// bits; all three are FP16 operands (kind::f16 runs at twice the rate of
+// kind::tf32, whose operands hold the same eleven bits, and moves half the
+// bytes: the covariance of p = 1000, n = 10000 0.183 -> 0.124 ms on the device,
+// its error the same, 9.5e-9 of its norm).  Then
+//   x_i x_j 2^(14 - e_i - e_j) = D0D0 + 2^-7 (D0D1 + D1D0)
+//                              + 2^-14 (D0T + TD0 + D1D1) + 2^-21 (D1T + TD1) + O(2^-28 TT),
 // and the four levels accumulate in four tensor-memory accumulators (the
 // whole 512-column TMEM).  The products of the first two levels are integers
-// of at most 2^14, one a sample in the first and two in the second, so their
-// FP32 sums stay exact (at most 2^24) for 512 samples whatever the rounding of
-// the tensor core's adder; the last two levels carry weights of 2^-16 and
-// 2^-24, so their FP32 rounding is negligible.  Every 512 samples
+// of at most 2^14, so their FP32 sums stay exact for 512 samples whatever the
+// rounding of the tensor core's adder; the last two levels carry weights of
+// 2^-14 and 2^-21, so their FP32 rounding is negligible.  Every 512 samples
 // the accumulators are drained into float-float sums in registers.  The
 // split of the sample axis over CTAs is summed in FP64 by a second kernel,
 // which also applies 2^(e_i + e_j - 14) / (n - 1).
@@ -30,6 +30,8 @@
 // bounded by the fit's timeout.
 #include <cuda.h>
 #include <cuda_fp16.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "launch.h"
@@ -135,7 +137,7 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // ------------------------------------------------------------------ digits of the normalised rows
 // One CTA per row: e = the exponent of max_t |x_t| (so |x 2^-e| < 1), then the
 // digits D0, D1 and the tail T of y 2^7 = x 2^(7-e) in FP16 (tails below 2^-14 are
-// subnormal there: off by 2^-25 at most, against 2^-5 for the largest).
+// subnormal there: off by 2^-25 at most, against 2^-6 for the largest).
 constexpr int kDigitThreads = 256;
 __device__ __forceinline__ void put_half4(__half* dst, const float (&v)[4]) {
     const __half2 a = __floats2half2_rn(v[0], v[1]), b = __floats2half2_rn(v[2], v[3]);
@@ -173,9 +175,9 @@ __global__ void __launch_bounds__(kDigitThreads) k_digits(const float* __restric
         for (int k = 0; k < 4; ++k) {
             const float z = y[k] * up;                // exact: a power-of-two scaling
             q[0][k] = rintf(z);
-            const float r0 = (z - q[0][k]) * 256.f;   // the difference is exact, at most 1/2
+            const float r0 = (z - q[0][k]) * 128.f;   // the difference is exact, at most 1/2
             q[1][k] = rintf(r0);
-            q[2][k] = (r0 - q[1][k]) * 256.f;
+            q[2][k] = (r0 - q[1][k]) * 128.f;
         }
         put_half4(d0 + row + t, q[0]);
         put_half4(d1 + row + t, q[1]);
@@ -295,7 +297,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     float hi, lo, s, e;
-                    two_sum(v0[q], __fmul_rn(v1[q], 0x1p-8f), hi, lo);   // exact integers: exact sum
+                    two_sum(v0[q], __fmul_rn(v1[q], 0x1p-7f), hi, lo);   // exact integers: exact sum
                     two_sum(S[c0 + q], hi, s, e);
                     S[c0 + q] = s;
                     E[c0 + q] = __fadd_rn(E[c0 + q], __fadd_rn(e, lo));
@@ -303,7 +305,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
                 tmem_ld8x2(taddr + 2 * kGM + c0, taddr + 3 * kGM + c0, v0, v1);
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
-                    E[c0 + q] = __fadd_rn(E[c0 + q], __fmaf_rn(v1[q], 0x1p-24f, __fmul_rn(v0[q], 0x1p-16f)));
+                    E[c0 + q] = __fadd_rn(E[c0 + q], __fmaf_rn(v1[q], 0x1p-21f, __fmul_rn(v0[q], 0x1p-14f)));
             }
             tc_fence_before();
             __syncwarp();
@@ -388,11 +390,11 @@ __global__ void __launch_bounds__(kRPart* kRPart)
 struct GramTcPlan {
     int nt, ntri, kb_total, kb_per_split, nsplit;
 };
-static GramTcPlan gram_tc_plan(long long p, int ld) {
+static GramTcPlan gram_tc_plan(long long p, int ld, int step = kGKB) {
     GramTcPlan g;
     g.nt = int((p + kGM - 1) / kGM);
     g.ntri = g.nt * (g.nt + 1) / 2;
-    g.kb_total = ld / kGKB;
+    g.kb_total = ld / step;
     int want = 152 / g.ntri;
     want = want < 1 ? 1 : (want > 32 ? 32 : want);
     if (want > g.kb_total) want = g.kb_total;
@@ -401,9 +403,11 @@ static GramTcPlan gram_tc_plan(long long p, int ld) {
     return g;
 }
 
+// Of k-steps of 32 samples, never fewer splits than of kGKB: like the digits' bytes, the sizes that the
+// entry points state.
 size_t gram_tc_partial_bytes(long long p, int ld) {
-    const GramTcPlan g = gram_tc_plan(p, ld);
-    return size_t(g.nsplit) * size_t(g.ntri) * kGM * kGM * sizeof(float2);
+    const GramTcPlan g = gram_tc_plan(p, ld), h = gram_tc_plan(p, ld, 32);
+    return size_t(std::max(g.nsplit, h.nsplit)) * size_t(g.ntri) * kGM * kGM * sizeof(float2);
 }
 
 // Half of it is used: the sizes that the entry points state (and refuse) are those of FP32 planes.
