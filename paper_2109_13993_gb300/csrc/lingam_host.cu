@@ -10,6 +10,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <tuple>
 #include <utility>
@@ -87,7 +88,13 @@ static Layout make_layout(long long p, long long n, int precision, int input_dty
         return at;
     };
     const size_t P = size_t(p), PP = size_t(p) * size_t(p);
+    // the results lie one after another: control block, order, report rows, B (one copy takes them out)
     L.off_ctl = take(sizeof(Ctl));
+    L.off_order = take(P * 4);
+    L.off_rs = take(P * 8);
+    L.off_rm = take(P * 8);
+    L.off_rp = take(P * 8);
+    L.off_bout = take(PP * 8);
     // the host-input copy is dead once the rows are normalised; the mixed path's
     // tensor-core Gram reuses it for the digit planes of its operands
     const size_t split_bytes = precision == LINGAM_MIXED ? gram_tc_digit_bytes(p, L.ld) : 0;
@@ -121,7 +128,6 @@ static Layout make_layout(long long p, long long n, int precision, int input_dty
     L.off_sigma_alt = take(P * 4);
     L.off_rows = take(P * 4);
     L.off_cols = take(kTJ * 4);
-    L.off_order = take(P * 4);
     L.off_forced = take(P * 4);
     L.off_prior = take(with_prior ? PP : 0);
     L.off_anc = take(with_prior ? P * 4 : 0);
@@ -132,14 +138,10 @@ static Layout make_layout(long long p, long long n, int precision, int input_dty
     L.off_invroot = take(P * 8);
     L.off_tilecnt = take(size_t(L.maxtiles) * 4);
     L.off_ibuf = take(size_t(L.maxtiles) * 64 * kTJ * L.esz);
-    L.off_rs = take(P * 8);
-    L.off_rm = take(P * 8);
-    L.off_rp = take(P * 8);
     L.off_rsc = take(PP * 8);
     L.off_cmat = take(PP * 8);
     L.off_rmat = take(PP * 8);
     L.off_rinv = take(PP * 8);
-    L.off_bout = take(PP * 8);
     L.total = o;
     return L;
 }
@@ -187,9 +189,25 @@ static bool is_device_ptr(const void* ptr) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Touches the pages of a result buffer in ordinary host memory, contents unchanged, while the device
+// works: a fresh array's pages are mapped on first touch, 0.14 ms for 8 MB.
+static void touch_pages(void* dst, size_t bytes) {
+    cudaPointerAttributes a;
+    if (!dst || bytes < (size_t(64) << 10)) return;
+    if (cudaPointerGetAttributes(&a, dst) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    if (a.type != cudaMemoryTypeUnregistered) return;
+    volatile char* c = static_cast<char*>(dst);
+    for (size_t o = 0; o < bytes; o += 4096) c[o] = c[o];
+    c[bytes - 1] = c[bytes - 1];
+}
+
 // CUDA events of the calls made by one host thread on one device: created on first need,
 // reused by every later call (each call synchronises its stream before it returns, so no
 // event is still pending when the next call records it), destroyed when the thread ends.
+constexpr size_t kStageBytes = size_t(256) << 10;
 struct EventPool {
     std::vector<cudaEvent_t> ev;
     bool reserve(size_t k) {
@@ -203,8 +221,29 @@ struct EventPool {
         }
         return true;
     }
+    // Pinned memory for the call's results, at most kStageBytes (nullptr: more, or none to be had).
+    char* stage = nullptr;
+    size_t stage_bytes = 0;
+    char* staging(size_t bytes) {
+        if (bytes > kStageBytes) return nullptr;
+        if (bytes > stage_bytes) {
+            if (stage) cudaFreeHost(stage);
+            stage = nullptr;
+            stage_bytes = 0;
+            const size_t want = std::min(kStageBytes, std::max(bytes, size_t(16) << 10));
+            void* q = nullptr;
+            if (cudaHostAlloc(&q, want, cudaHostAllocDefault) == cudaSuccess) {
+                stage = static_cast<char*>(q);
+                stage_bytes = want;
+            } else {
+                cudaGetLastError();
+            }
+        }
+        return stage;
+    }
     ~EventPool() {
         for (cudaEvent_t e : ev) cudaEventDestroy(e);
+        if (stage) cudaFreeHost(stage);
         cudaGetLastError();
     }
 };
@@ -394,7 +433,12 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
     const double tmo = o.timeout_s > 0 ? o.timeout_s : 10.0;
     c0.timeout_ns = (unsigned long long)(tmo * 1e9);
     c0.root = -1;
-    CK(cudaMemcpyAsync(f.ctl, &c0, sizeof(c0), cudaMemcpyHostToDevice, st));
+    // the results' initial values: the control block, -1 for iterations not run, zeros
+    const size_t res_bytes = L.off_rp + size_t(p) * 8;
+    std::vector<char> init(res_bytes, 0);
+    std::memcpy(init.data() + L.off_ctl, &c0, sizeof(c0));
+    std::memset(init.data() + L.off_order, 0xff, size_t(p) * 4);
+    CK(cudaMemcpyAsync(base, init.data(), res_bytes, cudaMemcpyHostToDevice, st));
     CK(cudaMemsetAsync(f.tile_cnt, 0, size_t(L.maxtiles) * 4, st));
     if (o.forced_order)
         CK(cudaMemcpyAsync(base + L.off_forced, o.forced_order, size_t(p) * 4, cudaMemcpyHostToDevice, st));
@@ -410,10 +454,6 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
         xdev = base + L.off_xin;
     }
 
-    CK(cudaMemsetAsync(f.order, 0xff, size_t(p) * 4, st));   // -1 for iterations not run
-    CK(cudaMemsetAsync(f.rep_pairs, 0, size_t(p) * 8, st));
-    CK(cudaMemsetAsync(f.rep_root_score, 0, size_t(p) * 8, st));
-    CK(cudaMemsetAsync(f.rep_margin, 0, size_t(p) * 8, st));
     const int iters = (o.max_iters > 0 && o.max_iters < p) ? o.max_iters : p;
     const bool want_B = B != nullptr && iters == p;
     // the call's events come from this host thread's pool (created once, reused by every call)
@@ -495,11 +535,25 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
         if (want_B) launches += order_kernel ? 2 : 4;
         if (cudaEventRecord(ev[4], st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
     } while (0);
+    // The results in one copy behind the kernels, B with them where it is small (one copy of pageable
+    // memory after another took 11 us each, 70 us of a fit of 20 x 2000)
+    const size_t b_bytes = size_t(p) * p * 8;
+    const bool staged_B = want_B && !cov_out && b_bytes <= (size_t(64) << 10);
+    const size_t out_bytes = cov_out ? sizeof(Ctl) : staged_B ? L.off_bout + b_bytes : res_bytes;
+    std::vector<char> pageable;
+    char* out = pool->staging(out_bytes);
+    if (!out) {
+        pageable.resize(out_bytes);
+        out = pageable.data();
+    }
+    if (status == LINGAM_OK && cudaMemcpyAsync(out, base, out_bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess) status = LINGAM_ECUDA;
+    if (status == LINGAM_OK) touch_pages(cov_out ? static_cast<void*>(cov_out) : want_B ? B : nullptr, b_bytes);
     if (cudaStreamSynchronize(st) != cudaSuccess) status = LINGAM_ECUDA;
     Ctl ch;
+    std::memset(&ch, 0, sizeof(ch));
     if (status == LINGAM_OK) {
-        if (cudaMemcpy(&ch, f.ctl, sizeof(ch), cudaMemcpyDeviceToHost) != cudaSuccess) status = LINGAM_ECUDA;
-        else if (ch.status != 0) status = ch.status;
+        std::memcpy(&ch, out + L.off_ctl, sizeof(ch));
+        if (ch.status != 0) status = ch.status;
     }
     if (status == LINGAM_OK && cov_out) {
         if (cudaMemcpy(cov_out, f.sig, size_t(p) * p * 8, cudaMemcpyDefault) != cudaSuccess) status = LINGAM_ECUDA;
@@ -510,15 +564,23 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
             rep->kernel_launches = launches;
         }
     } else if (status == LINGAM_OK) {
-        // outputs (cudaMemcpyDefault: host or device destinations)
-        if (cudaMemcpyAsync(order, f.order, size_t(p) * 4, cudaMemcpyDefault, st) != cudaSuccess) status = LINGAM_ECUDA;
-        if (want_B && cudaMemcpyAsync(B, f.bout, size_t(p) * p * 8, cudaMemcpyDefault, st) != cudaSuccess)
-            status = LINGAM_ECUDA;
+        // outputs (host or device destinations)
+        bool pending = false;
+        const auto give = [&](void* dst, size_t off, size_t bytes, bool staged) {
+            if (staged && !is_device_ptr(dst)) {
+                std::memcpy(dst, out + off, bytes);
+                return true;
+            }
+            pending = true;
+            return cudaMemcpyAsync(dst, base + off, bytes, cudaMemcpyDefault, st) == cudaSuccess;
+        };
+        if (!give(order, L.off_order, size_t(p) * 4, true)) status = LINGAM_ECUDA;
+        if (want_B && !give(B, L.off_bout, b_bytes, staged_B)) status = LINGAM_ECUDA;
         if (rep) {
-            if (rep->root_score) cudaMemcpyAsync(rep->root_score, f.rep_root_score, size_t(p) * 8, cudaMemcpyDefault, st);
-            if (rep->margin_lb) cudaMemcpyAsync(rep->margin_lb, f.rep_margin, size_t(p) * 8, cudaMemcpyDefault, st);
-            if (rep->pairs_evaluated)
-                cudaMemcpyAsync(rep->pairs_evaluated, f.rep_pairs, size_t(p) * 8, cudaMemcpyDefault, st);
+            if (rep->root_score) give(rep->root_score, L.off_rs, size_t(p) * 8, true);
+            if (rep->margin_lb) give(rep->margin_lb, L.off_rm, size_t(p) * 8, true);
+            if (rep->pairs_evaluated) give(rep->pairs_evaluated, L.off_rp, size_t(p) * 8, true);
+            pending = pending || rep->scores || (order_kernel && o.timing);
             if (rep->scores) cudaMemcpyAsync(rep->scores, f.rep_scores, size_t(p) * p * 8, cudaMemcpyDefault, st);
             float ms = 0.f;
             rep->t_standardize_ms = cudaEventElapsedTime(&ms, ev[0], ev[1]) == cudaSuccess ? ms : -1.0;
@@ -547,19 +609,18 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
             rep->empty_col_pairs = ch.empty_col_pairs;
             rep->pad_row_pairs = ch.pad_row_pairs;
         }
-        if (cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess) status = LINGAM_ECUDA;
+        if ((pending && cudaStreamSynchronize(st) != cudaSuccess) || cudaGetLastError() != cudaSuccess) status = LINGAM_ECUDA;
         if (rep && status == LINGAM_OK) {
-            std::vector<long long> pe(static_cast<size_t>(p));
-            if (cudaMemcpy(pe.data(), f.rep_pairs, size_t(p) * 8, cudaMemcpyDeviceToHost) == cudaSuccess) {
-                long long tot = 0, unp = 0;
-                for (int k = 0; k < iters; ++k) {
-                    tot += pe[size_t(k)];
-                    const long long r = p - k;
-                    unp += o.reuse ? r * (r - 1) / 2 : r * (r - 1);
-                }
-                rep->pairs_total = tot;
-                rep->pairs_unpruned = unp;
+            long long tot = 0, unp = 0;
+            for (int k = 0; k < iters; ++k) {
+                long long e;
+                std::memcpy(&e, out + L.off_rp + size_t(k) * 8, 8);
+                tot += e;
+                const long long r = p - k;
+                unp += o.reuse ? r * (r - 1) / 2 : r * (r - 1);
             }
+            rep->pairs_total = tot;
+            rep->pairs_unpruned = unp;
         }
     }
     if (log_level() >= 1) {
@@ -1019,6 +1080,19 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
     } else {
         CKB(enqueue_batch(ws, BL, fits, Ls, o, order_kernel ? &groups : nullptr, rows, with_B, gather, nsm, st));
     }
+    // while the device works: the results' host memory.  B goes straight to the caller's array where
+    // the problems' lie one after another (a bootstrap's do) and every fit succeeded.
+    size_t sp = 0, spp = 0;
+    bool adjacent = gather && with_B;
+    for (int k = 0; k < count; ++k) {
+        adjacent = adjacent && items[size_t(k)].B == items[0].B + spp;
+        sp += size_t(P[size_t(k)]);
+        spp += size_t(P[size_t(k)]) * size_t(P[size_t(k)]);
+    }
+    std::vector<int> sorder(gather ? sp : 0);
+    std::unique_ptr<double[]> sB;
+    if (gather && with_B && !adjacent) sB.reset(new double[spp]);
+    if (gather && with_B) touch_pages(adjacent ? items[0].B : sB.get(), spp * sizeof(double));
     CKB(cudaStreamSynchronize(st));
 
     // statuses and outputs
@@ -1026,19 +1100,13 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
     Ctl bc;
     CKB(cudaMemcpy(ctls.data(), ws + BL.off_ctls, size_t(count) * sizeof(Ctl), cudaMemcpyDeviceToHost));
     CKB(cudaMemcpy(&bc, ws + BL.off_bctl, sizeof(Ctl), cudaMemcpyDeviceToHost));
-    std::vector<int> sorder;
-    std::vector<double> sB;
+    bool all_ok = bc.status == 0;
+    for (int k = 0; k < count; ++k) all_ok = all_ok && ctls[size_t(k)].status == 0;
     if (gather) {
-        size_t sp = 0, spp = 0;
-        for (int k = 0; k < count; ++k) {
-            sp += size_t(P[size_t(k)]);
-            spp += size_t(P[size_t(k)]) * size_t(P[size_t(k)]);
-        }
-        sorder.resize(sp);
         CKB(cudaMemcpy(sorder.data(), ws + BL.off_stage_order, sp * sizeof(int), cudaMemcpyDeviceToHost));
         if (with_B) {
-            sB.resize(spp);
-            CKB(cudaMemcpy(sB.data(), ws + BL.off_stage_B, spp * sizeof(double), cudaMemcpyDeviceToHost));
+            if (adjacent && !all_ok) sB.reset(new double[spp]);
+            CKB(cudaMemcpy(sB ? sB.get() : items[0].B, ws + BL.off_stage_B, spp * sizeof(double), cudaMemcpyDeviceToHost));
         }
     }
     int first = LINGAM_OK;
@@ -1051,7 +1119,7 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
         if (stk == LINGAM_OK) {
             if (gather) {
                 std::memcpy(it.order, sorder.data() + po, pk * sizeof(int));
-                if (with_B) std::memcpy(it.B, sB.data() + pb, pk * pk * sizeof(double));
+                if (with_B && sB) std::memcpy(it.B, sB.get() + pb, pk * pk * sizeof(double));
             } else {
                 if (cudaMemcpy(it.order, f.order, pk * sizeof(int), cudaMemcpyDefault) != cudaSuccess) stk = LINGAM_ECUDA;
                 if (with_B && cudaMemcpy(it.B, f.bout, pk * pk * sizeof(double), cudaMemcpyDefault) != cudaSuccess)
