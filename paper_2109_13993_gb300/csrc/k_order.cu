@@ -19,8 +19,8 @@
 // Pairs evaluated, of all pairs: p = 300, n = 5000 graphs with one causal order 82 % -> 6 %, p = 1000,
 // n = 10^4 79 % -> 1.7 %, random graphs of in-degree 3 at p = 300 31 % -> 19 %, with 1.0-1.7 waves per
 // iteration instead of 1.4-8.9.  Whole fits against the tile kernels with a barrier per phase:
-// p = 1000, n = 10^4 1145 -> 100 ms, p = 300, n = 5000 56 -> 14 ms, p = 20, n = 2000 1.23 -> 0.91 ms;
-// FP64 p = 65, n = 2001 74 -> 7.4 ms.
+// p = 1000, n = 10^4 1145 -> 66 ms (a random graph 589 -> 567), p = 300, n = 5000 56 -> 9.2 ms,
+// p = 100, n = 10^4 11.1 -> 2.8, p = 20, n = 2000 1.23 -> 0.51 ms; FP64 p = 65, n = 2001 72 -> 4.3 ms.
 //
 // One hand-over per wave.  The first wave of an iteration removes the previous root on the way:
 // a worker reads the old rows, forms (x_w - Sigma[w,root] x_root) / sqrt(1 - Sigma[w,root]^2) of
@@ -28,14 +28,22 @@
 // owns to the other of two copies; the pair coefficients come from the old covariance the same
 // way, and the covariance downdate itself (Eq. CovUpdate, FP64, upper triangle) goes to its other
 // copy.  So no barrier separates removal and comparison: the workers arrive once per wave, the
-// controller merges, decides and publishes the next wave in one word.
+// controller merges, decides and publishes the next wave in one word.  The removed root's column of
+// the covariance stays behind in Fit::rmat, the factorisation that the B fit solves with.
 //
 // Work split of a wave: nseg segments of the sample axis times W / nseg row groups; a worker
 // stages its segment of the columns (and of the root) in shared memory and streams its rows from
-// L2.  A warp takes blocks of samples of one row against four columns (lanes across the
-// samples, coalesced), closes a block with one lg2 per residual and lane, adds the lanes in a
-// fixed tree and the blocks in float-float, so that a sum does not depend on how the blocks were
-// spread over warps and CTAs (beyond 2^-48).
+// L2.  A warp takes a unit of samples of one row against four columns (one on the FP64 path; lanes
+// across the samples, coalesced), closes it with one lg2 per residual and lane and adds the lanes in a
+// fixed tree; the units and segments are added in order in float-float (the last worker of a row
+// group to arrive adds the segments), so that a sum does not depend on how the units were spread over
+// warps and CTAs (beyond 2^-48).
+//
+// What bounds it.  Small fits: the chain of a wave, about 60,000 clocks of which the two flags take
+// 2,000-2,800 each (a word written by one SM and read by another costs 1,100-1,500), the row table 4,500,
+// coefficients 6,000, staging 3,000, the units 6,000-12,000, the controller 15,000.  Large ones: the
+// units, at 60 % of the exponentials' rate with four warps a quarter (1024 samples of a row against
+// four columns 13,700 clocks; 8,200 at 32 ex2 a clock and SM), and a row's own unit at 40 %.
 #include <algorithm>
 #include <queue>
 #include <type_traits>
@@ -551,6 +559,8 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
     const int cstr = bp * unit;
     T* s_cols = s_root + cstr;
 
+    __shared__ int s_next;   // units taken from the batch, beyond a warp's first
+
     const int root = wv.root;
     const double droot = rm ? __ldcg(dold + root) : 0.0;
 
@@ -701,6 +711,7 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
                     if (cat[q] >= 0) snew[cat[q]] = fma(-s_sr[crow[q]] * dr2, cb[q], ca[q]);
                 load_chunks();
             }
+            if (tid == 0) s_next = 0;
             if (stage) {
                 // the columns without the root (each thread the vectors it copied)
                 copy_wait();
@@ -718,9 +729,16 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
             }
             __syncthreads();
             // the units of all rows, first those against columns (row, quad, unit of the segment), then
-            // the rows' own, dealt out to the warps in turn; each leaves its sums in a slot
+            // the rows' own (the short ones last); each leaves its sums in a slot.  Dealt out to the warps in
+            // turn, in a batch's CTAs, whose warps have many each, taken by the next warp that is free (64
+            // uneven datasets 10.24 -> 9.92 ms; single fits gain and lose less than 1%, and the FP64 quarters
+            // are loaded evenly only in turn).
             const int nQ = nrb * nq * nb, nU = nQ + nrb * has_k * nb;
-            for (int i = wid; i < nU; i += NW) {
+            const auto next_unit = [&](int i) {
+                if constexpr (sizeof(T) == 8 || NT == 512) return i + NW;
+                else return NW + __shfl_sync(0xffffffffu, lane == 0 ? atomicAdd(&s_next, 1) : 0, 0);
+            };
+            for (int i = wid; i < nU; i = next_unit(i)) {
                 const bool own = i >= nQ;
                 const int g2 = small_div(own ? i - nQ : i, nb), b = (own ? i - nQ : i) - g2 * nb;   // (row, quad) or row
                 const int j = own ? g2 : small_div(g2, nq), t = own ? 0 : g2 - j * nq;
