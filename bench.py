@@ -43,9 +43,10 @@ L2_FLUSH_BYTES = 256 << 20
 # Pair kernel SFU roofline: per pair-sample 4 ex2 (32 per SM per clock on sm_103a)
 # plus 2 lg2 per 32 samples (16 per SM per clock).
 SFU_CLK_PER_PAIR_SAMPLE = 4.0 / 32.0 + (2.0 / 32.0) / 16.0
-# DRAM bytes (read + write) per launch of the iteration kernel, from an ncu capture of
-# the current kernel version (profiles/); None until the current version is captured.
-ITER_TRAFFIC_BYTES = 71.6e6   # ncu dram__bytes_read.sum + dram__bytes_write.sum, iteration 2 (55.1 + 16.5 MB)
+# DRAM bytes (read + write) of the ordering kernel's launch, from an ncu capture of the current
+# kernel version; None until the current version is captured (a capture of the full-size launch
+# takes several passes over a kernel of half a second).
+ITER_TRAFFIC_BYTES = None
 
 
 def unpruned_pair_samples(p: int, n: int) -> float:
@@ -508,8 +509,8 @@ def run_ours(args, rank: int, world: int):
             pairs.append(res.pairs_total)
             launches.append(res.kernel_launches)
     clocks = clk.summary()
-    # a separate pass with the library's instrumentation on: the iteration kernel's launch
-    # times (CUDA events on the launching stream, one after each launch) for the roofline,
+    # a separate pass with the library's instrumentation on: the ordering kernel's launch
+    # time (CUDA events on the launching stream) for the roofline,
     # and CTA 0's phase timers
     pair_ms, phases = [], []
     for _ in range(max(1, min(args.steps, 3))):
@@ -552,18 +553,18 @@ def run_ours(args, rank: int, world: int):
     traffic = ITER_TRAFFIC_BYTES if (p, n) == (P_DEFAULT, N_DEFAULT) else None
     roofline = {"bound": "alu", "achieved": achieved / 1e9, "peak": peak / 1e9, "unit": "Gpair-samples/s",
                 "frac": achieved / peak, "traffic": traffic,
-                "traffic_basis": "ncu dram__bytes_read+write of one launch (iteration 2 of a fit, cold caches)",
-                "kernel": "k_iteration<float>",
-                "timing_basis": "separate instrumented pass (one CUDA event after each launch); the timed steps run "
-                                "without instrumentation",
+                "traffic_basis": "not captured for the current kernel",
+                "kernel": "k_order<float, 512>",
+                "timing_basis": "separate instrumented pass (CUDA events around the ordering's one launch); the timed "
+                                "steps run without instrumentation",
                 "peak_basis": f"SFU: 4 ex2 + 1/16 lg2 per pair-sample, {nsm} SMs x 32 ex2/clk at sm_max {sm_max:.0f} MHz"}
     # the same work over the pair-compute phases of the waves alone (device timer; the rest
-    # of each launch is merging, wave finalisation, removal and grid barriers)
+    # of the launch is the controller's: scores, threshold and the next wave)
     ph = np.mean(np.array(phases), axis=0)
     comp = float(np.mean(pairs)) * n / (float(np.mean([x[0] for x in phases])) / 1000.0)
     roofline["compute_phase"] = {"achieved": comp / 1e9, "frac": comp / peak,
                                  "ms_per_step": {"pair_compute": ph[0], "merge_finalize": ph[1], "removal": ph[2]}}
-    # the pair tiles' own efficiency: useful pairs over the pairs the waves' tiles computed
+    # useful pairs over the pairs that the waves computed
     roofline["waves_per_step"] = int(rt.waves)
     roofline["tile_pairs_per_step"] = int(rt.tile_pairs)
     roofline["useful_fraction_of_tile_pairs"] = float(rt.pairs_total) / max(1, int(rt.tile_pairs))

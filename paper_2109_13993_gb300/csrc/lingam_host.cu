@@ -157,7 +157,7 @@ static bool valid_opts(const lingam_opts& o) {
     return (o.precision == LINGAM_MIXED || o.precision == LINGAM_FP64) &&
            (o.input_dtype == LINGAM_F32 || o.input_dtype == LINGAM_F64) && (o.prune == 0 || o.prune == 1) &&
            (o.reuse == 0 || o.reuse == 1) && o.split_n >= 0 &&
-           ((o.tile_i == 1 && o.tile_j == 1) ||   // the batch kernel's pair-per-warp mode
+           ((o.tile_i == 1 && o.tile_j == 1) ||   // batches: the ordering kernel
             ((o.tile_i == 0 || o.tile_i == 32 || o.tile_i == 64) && (o.tile_j == 0 || o.tile_j == 16 || o.tile_j == 32))) &&
            std::isfinite(o.gamma0) && o.gamma0 >= 0.0 &&
            (o.gamma0 == 0.0 || (o.prune == 1 && o.reuse == 1 && std::isfinite(o.gamma_c) && o.gamma_c > 1.0));
@@ -174,8 +174,8 @@ static TileShape batch_tile_shape(const lingam_opts& o, long long maxp, long lon
     return t;
 }
 
-// Single fits run 64 x 32, 32 x 32 or 64 x 16 tiles (32 x 16 tiles and the pair-per-warp
-// mode, 1 x 1, are batch shapes).
+// Single fits run 64 x 32, 32 x 32 or 64 x 16 tiles (32 x 16 tiles and 1 x 1,
+// the ordering kernel, are batch shapes).
 static bool single_fit_shape(const lingam_opts& o) {
     return !(o.tile_i == 32 && o.tile_j == 16) && !(o.tile_i == 1 && o.tile_j == 1);
 }

@@ -333,7 +333,7 @@ def autotune(X, stream=None, workspace=None):
 
 def autotune_batch(Xs, stream=None, workspace=None):
     """lingam_autotune_batch on a list of datasets: times lingam_fit_batch with 64x32, 32x32,
-    64x16 and 32x16 pair tiles and the pair-per-warp mode (1x1), records the fastest for the
+    64x16 and 32x16 pair tiles and the ordering kernel (1x1), records the fastest for the
     bucket of the largest p and n;
     returns ((rows, cols), {shape: ms})."""
     L = load()

@@ -1,0 +1,92 @@
+"""The ordering kernel, its factor-based B fit and the covariance kernels at the sizes where their splits
+change: units and the last, partial one (128 / 64 samples a step), rows of a worker (32), columns
+(4 ... 16), the controller's warps, in-place and permuted factors (128 variables), the line between
+ordering and tile kernels (160), queued problems of a batch (more than 304), tiles and parts of the
+covariance (128, 8; 32 on the FP64 path)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2109_13993_gb300 import lingam, synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    from paper_2109_13993_gb300 import build
+    build.build()
+    lingam.load()
+    oracle.build()
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+
+
+def _data(p, n, seed):
+    return synth.lingam_dataset(p, n, min(1.0, 3.0 / max(p - 1, 1)), seed).X
+
+
+def _dev(X, dtype):
+    return torch.tensor(np.ascontiguousarray(X), dtype=dtype, device="cuda")
+
+
+SIZES = [(1, 9), (2, 5), (3, 40), (4, 63), (5, 64), (9, 65), (16, 127), (17, 128), (18, 129), (33, 257), (34, 1023),
+         (40, 1025), (65, 300)]
+
+
+@pytest.mark.parametrize("p,n", SIZES)
+@pytest.mark.parametrize("prune", [True, False])
+def test_fp64_fit_matches_oracle(p, n, prune):
+    # FP64 throughout: 1e-10 relative on scores and B, as for the whole FP64 path
+    X = _data(p, n, 100 * p + n)
+    o_order, o_B, o_S = oracle.fit(X)
+    f = lingam.fit(_dev(X, torch.float64), precision="fp64", prune=prune)
+    assert np.array_equal(f.order, o_order)
+    want = np.array([o_S[k, o_order[k]] for k in range(p)])
+    assert np.all(np.abs(f.root_score - want) <= 1e-10 * np.abs(want) + 1e-14)
+    assert np.abs(f.B - o_B).max() <= 1e-10 * max(1.0, np.abs(o_B).max())
+
+
+@pytest.mark.parametrize("p,n", SIZES + [(127, 500), (128, 500), (129, 500), (160, 640), (161, 640)])
+def test_mixed_scores_and_pruned_roots(p, n):
+    # every score within the mixed path's 1e-4 of the oracle; the killer pairs change no root's score:
+    # equal up to the FP32 rounding of I (2e-6 sqrt(m S) <= 2e-8 at these scores)
+    X = _data(p, n, 100 * p + n).astype(np.float32)
+    o_order, o_B, o_S = oracle.fit(X.astype(np.float64))
+    full = lingam.fit(_dev(X, torch.float32), prune=False, forced_order=o_order, want_scores=True)
+    m = ~np.isnan(o_S)
+    assert np.array_equal(m, ~np.isnan(full.scores))
+    assert np.abs(full.scores[m] - o_S[m]).max() <= 1e-4
+    assert np.abs(full.B - o_B).max() <= 1e-4 * max(1.0, np.abs(o_B).max())
+    pruned = lingam.fit(_dev(X, torch.float32), forced_order=o_order)
+    assert np.allclose(pruned.root_score, full.root_score, rtol=1e-4, atol=2e-8)
+    assert np.abs(pruned.B - full.B).max() <= 1e-12 * max(1.0, np.abs(o_B).max())
+
+
+def test_batch_with_queued_problems_matches_oracle():
+    # more problems than CTA slots, of 2 ... 13 variables, one large enough for a group of its own
+    Xs = [_data(2 + k % 12, 40 + 17 * (k % 23), 7000 + k) for k in range(330)] + [_data(60, 3001, 8000)]
+    got = lingam.fit_batch([_dev(X, torch.float64) for X in Xs], precision="fp64")
+    assert got.status == lingam.LINGAM_OK
+    for X, order, B in zip(Xs, got.orders, got.Bs):
+        o_order, o_B, _ = oracle.fit(X, want_scores=False)
+        assert np.array_equal(order, o_order)
+        assert np.abs(B - o_B).max() <= 1e-10 * max(1.0, np.abs(o_B).max())
+
+
+@pytest.mark.parametrize("p", [1, 7, 8, 9, 31, 32, 33, 127, 128, 129, 136])
+@pytest.mark.parametrize("n", [3, 64, 65, 511, 577])
+def test_covariance_at_tile_and_part_edges(p, n):
+    X = np.random.default_rng(1000 * p + n).standard_normal((p, n))
+    X32 = X.astype(np.float32)
+    ref = oracle.covariance(X32.astype(np.float64))
+    got = lingam.covariance(_dev(X32, torch.float32))[0]
+    # rows rounded to FP32 (2^-24 relative), their tails off by 2^-27 of 2^e <= 2 max |x| and the tails'
+    # product, 2^-30 of 2^(e_i + e_j), left out; max |x| <= sqrt(n - 1), sums by the Cauchy-Schwarz inequality
+    tol = 2 * (2.0**-24 + 2.0**-26 * np.sqrt(n - 1)) + 2.0**-28 * (n - 1)
+    assert np.abs(got - ref).max() <= tol
+    ref = oracle.covariance(X)
+    got = lingam.covariance(_dev(X, torch.float64), precision="fp64")[0]
+    # the rows' means, deviations and products in FP64: n roundings of 2^-53 on sums of at most n - 1
+    assert np.abs(got - ref).max() <= 8 * n * 2.0**-53
