@@ -1872,10 +1872,10 @@ cudaError_t launch_order(const Fit& f, int iters, int nsm, cudaStream_t st) {
 }
 
 // Clocks (estimate) of a problem on g CTAs of 256 threads: 3 pair-samples a clock and CTA (FP64:
-// 1/40 of that), about 7 pairs per row and iteration, and the hand-over of a wave.
+// 1/40 of that), about 7 pairs per row and iteration (unpruned: all), and the hand-over of a wave.
 static double batch_clocks(const Fit& f, int g) {
     const double p = f.p, rate = f.precision == LINGAM_MIXED ? 3.0 : 0.075;
-    const double work = 3.5 * p * p * f.ld / rate;
+    const double work = (f.prune ? 3.5 * p * p : p * p * p / 6.0) * f.ld / rate;
     const int W = g >= kDedicated ? g - 1 : g;
     return work / W + p * (g > 1 ? 16000.0 : 8000.0);
 }

@@ -375,14 +375,15 @@ static bool check_prior(const signed char* prior, int p, std::vector<int>& anc) 
 }
 
 // Single fits run the ordering kernel (k_order.cu) unless an option asks for the tile kernels
-// (an explicit tile shape, LINGAM_NARROW) or the problem is too large for it.  Without the killer pairs
-// (no pruning, no pair reuse, the paper's threshold schedule) most columns are computed, and the tile
-// kernels' waves of 32 columns win on the mixed path from about 150 variables on: unpruned, ordering
-// kernel against tile kernels, p 100 11.3 and 13.3 ms, p 150 21.7 and 22.7, p 300 93.6 and 80.6; with
-// the schedule from 10^-3 9.2 and 11.4, 17.0 and 18.2, 72.9 and 58.6.
+// (an explicit tile shape, LINGAM_NARROW) or the problem is too large for it.  Without pruning or pair
+// reuse there are no killer pairs, all columns are computed, and the tile kernels' waves of 32 columns
+// win on the mixed path from about 150 variables on: unpruned, ordering kernel against tile kernels,
+// p 100 11.3 and 13.3 ms, p 150 21.7 and 22.7, p 300 93.6 and 80.6.  (The paper's threshold schedule has
+// none either, but its roots and scores are those of the default run to the last rounding only in the
+// same kernel: 100 x 10000 from 10^-3 11.4 -> 9.2 ms, 300 x 5000 58.6 -> 72.9.)
 constexpr int kOrderFullP = 160;
 static bool use_order_kernel(const Fit& f, const lingam_opts& o) {
-    const bool killers = o.prune && o.reuse && !(o.gamma0 > 0.0);
+    const bool killers = o.prune && o.reuse;
     return o.tile_i == 0 && o.tile_j == 0 && !narrow_set() &&
            (killers || o.precision != LINGAM_MIXED || f.p <= kOrderFullP) && order_supported(f, false);
 }
@@ -961,7 +962,9 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
     // 1 x 1, a size the autotuner never measured, and the FP64 path without an explicit shape: the
     // ordering kernel, where it takes every problem of the call
     const bool untuned = o.tile_i == 0 && o.tile_j == 0 && !autotune_batch_measured(maxp, maxn);
-    bool order_kernel = o.reuse && (o.precision == LINGAM_MIXED ? ts.rows == 1 || untuned : o.tile_i <= 1 && o.tile_j <= 1);
+    // (unpruned sets of more than kOrderFullP variables: tiles, as for single fits)
+    bool order_kernel = o.reuse && (o.precision == LINGAM_MIXED ? ts.rows == 1 || (untuned && (o.prune || maxp <= kOrderFullP))
+                                                                : o.tile_i <= 1 && o.tile_j <= 1);
     for (int k = 0; k < count && order_kernel; ++k) {
         const Layout L = make_layout(P[size_t(k)], N[size_t(k)], o.precision, o.input_dtype);
         order_kernel = order_supported(make_fit(ws, L, int(P[size_t(k)]), int(N[size_t(k)]), o, false), true);
