@@ -81,7 +81,8 @@ typedef struct {
     int prune;               /* 1 = threshold pruning (Sec. III-B), 0 = compare every pair */
     int reuse;               /* 1 = one evaluation per unordered pair (Sec. III-A), 0 = every ordered pair */
     int tile_i, tile_j;      /* both 0 (default): single fits run the ordering kernel (no tiles; p up to
-                                about 2000), batch calls as lingam_fit_batch says.  Else the pair-tile
+                                about 2000; on the mixed path without pruning or reuse
+                                up to 160), batch calls as lingam_fit_batch says.  Else the pair-tile
                                 shape of the tile kernels on the mixed path, rows x columns: 64 x 32,
                                 32 x 32 or 64 x 16, and for batch calls only 32 x 16, and 1 x 1 (the
                                 ordering kernel) (a zero in one takes 64 rows or 32 columns).  The FP64

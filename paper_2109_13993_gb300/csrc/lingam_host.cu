@@ -207,7 +207,6 @@ static void touch_pages(void* dst, size_t bytes) {
 // CUDA events of the calls made by one host thread on one device: created on first need,
 // reused by every later call (each call synchronises its stream before it returns, so no
 // event is still pending when the next call records it), destroyed when the thread ends.
-constexpr size_t kStageBytes = size_t(256) << 10;
 struct EventPool {
     std::vector<cudaEvent_t> ev;
     bool reserve(size_t k) {
@@ -221,29 +220,8 @@ struct EventPool {
         }
         return true;
     }
-    // Pinned memory for the call's results, at most kStageBytes (nullptr: more, or none to be had).
-    char* stage = nullptr;
-    size_t stage_bytes = 0;
-    char* staging(size_t bytes) {
-        if (bytes > kStageBytes) return nullptr;
-        if (bytes > stage_bytes) {
-            if (stage) cudaFreeHost(stage);
-            stage = nullptr;
-            stage_bytes = 0;
-            const size_t want = std::min(kStageBytes, std::max(bytes, size_t(16) << 10));
-            void* q = nullptr;
-            if (cudaHostAlloc(&q, want, cudaHostAllocDefault) == cudaSuccess) {
-                stage = static_cast<char*>(q);
-                stage_bytes = want;
-            } else {
-                cudaGetLastError();
-            }
-        }
-        return stage;
-    }
     ~EventPool() {
         for (cudaEvent_t e : ev) cudaEventDestroy(e);
-        if (stage) cudaFreeHost(stage);
         cudaGetLastError();
     }
 };
@@ -541,19 +519,16 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
     const size_t b_bytes = size_t(p) * p * 8;
     const bool staged_B = want_B && !cov_out && b_bytes <= (size_t(64) << 10);
     const size_t out_bytes = cov_out ? sizeof(Ctl) : staged_B ? L.off_bout + b_bytes : res_bytes;
-    std::vector<char> pageable;
-    char* out = pool->staging(out_bytes);
-    if (!out) {
-        pageable.resize(out_bytes);
-        out = pageable.data();
+    std::vector<char> out(out_bytes);
+    if (status == LINGAM_OK) {
+        touch_pages(cov_out ? static_cast<void*>(cov_out) : want_B ? B : nullptr, b_bytes);
+        if (cudaMemcpyAsync(out.data(), base, out_bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess) status = LINGAM_ECUDA;
     }
-    if (status == LINGAM_OK && cudaMemcpyAsync(out, base, out_bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess) status = LINGAM_ECUDA;
-    if (status == LINGAM_OK) touch_pages(cov_out ? static_cast<void*>(cov_out) : want_B ? B : nullptr, b_bytes);
     if (cudaStreamSynchronize(st) != cudaSuccess) status = LINGAM_ECUDA;
     Ctl ch;
     std::memset(&ch, 0, sizeof(ch));
     if (status == LINGAM_OK) {
-        std::memcpy(&ch, out + L.off_ctl, sizeof(ch));
+        std::memcpy(&ch, out.data() + L.off_ctl, sizeof(ch));
         if (ch.status != 0) status = ch.status;
     }
     if (status == LINGAM_OK && cov_out) {
@@ -569,7 +544,7 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
         bool pending = false;
         const auto give = [&](void* dst, size_t off, size_t bytes, bool staged) {
             if (staged && !is_device_ptr(dst)) {
-                std::memcpy(dst, out + off, bytes);
+                std::memcpy(dst, out.data() + off, bytes);
                 return true;
             }
             pending = true;
@@ -615,7 +590,7 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
             long long tot = 0, unp = 0;
             for (int k = 0; k < iters; ++k) {
                 long long e;
-                std::memcpy(&e, out + L.off_rp + size_t(k) * 8, 8);
+                std::memcpy(&e, out.data() + L.off_rp + size_t(k) * 8, 8);
                 tot += e;
                 const long long r = p - k;
                 unp += o.reuse ? r * (r - 1) / 2 : r * (r - 1);
