@@ -841,6 +841,10 @@ __device__ __forceinline__ void add_square(float2& s, float m) {
 }
 __device__ __forceinline__ void add_square(double& s, double m) { s = fma(m, m, s); }
 
+// As a float, rounded towards zero.
+__device__ __forceinline__ float toward_zero(float x) { return x; }
+__device__ __forceinline__ float toward_zero(double x) { return __double2float_rz(x); }
+
 // Order-preserving bits of a float.
 __device__ __forceinline__ unsigned key_bits(float x) {
     const unsigned b = __float_as_uint(x);
@@ -903,7 +907,7 @@ struct Controller {
     // per slot
     float4* st;       // {corr, 2 (m - beta), g, offset} (FP32), or {H(x) - H(nu)} as a double (FP64)
     Sum* part;        // score so far; complete for columns
-    float* kc;        // the killer pair's contribution of this iteration
+    float* kc;        // the killer pair's contribution of this iteration, rounded down
     float* kv0;       // the two largest known contributions, and their partners
     float* kv1;
     int* keval;       // the killer that was compared (-1: none)
@@ -1355,9 +1359,9 @@ struct Controller {
             int topc = -1;
             int p0 = kp0[k], p1 = kp1[k];
             float w0 = kv0[k], w1 = kv1[k];
-            if (has_k && ke >= 0) {
-                const float m = fminf(float(Ir[ncol]), 0.f);
-                w0 = m * m;   // keval is kp0
+            if (has_k && ke >= 0) {   // (keval is kp0)
+                const float m = toward_zero(Ir[ncol] < T(0) ? Ir[ncol] : T(0));
+                w0 = __fmul_rz(m, m);   // part of a lower bound: never more than the pair contributes
                 kc[k] = w0;
             }
 #pragma unroll 1

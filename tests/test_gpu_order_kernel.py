@@ -66,6 +66,37 @@ def test_mixed_scores_and_pruned_roots(p, n):
     assert np.abs(pruned.B - full.B).max() <= 1e-12 * max(1.0, np.abs(o_B).max())
 
 
+def _near_tie(seed, weight):
+    """Six variables whose second iteration ends in a near tie: weight moves the scores, in steps far
+    below their gap."""
+    p, n = 6, 300
+    X = np.stack([synth.noise(synth.Stream(seed, v), (synth.NOISE_LAPLACE, synth.NOISE_UNIFORM)[v % 2], n)
+                  for v in range(p)])
+    W = np.tril(2 * synth.Stream(seed, 9).uniform(p * p).reshape(p, p) - 1, -1)
+    W[5, 4] = weight
+    for i in range(p):
+        X[i] += W[i, :i] @ X[:i]
+    return X
+
+
+@pytest.mark.parametrize("seed,weight", [(187, 0.299236631094986), (327, -0.5675924855453444),
+                                         (358, -0.4380522633860032), (1345, 0.04396862919510971),
+                                         (1399, -0.6748515948032312)])
+def test_fp64_pruning_is_exact_at_a_near_tie(seed, weight):
+    # the lowest score lies 3e-8 below the next and comes from a single pair, whose square rounded to the
+    # nearest FP32 value is above the next score: as a killer's share it has to be rounded down (seed 327
+    # is one where it is the killer's)
+    X = _near_tie(seed, weight)
+    o_order, _, o_S = oracle.fit(X)
+    low, second = np.sort(o_S[1][~np.isnan(o_S[1])])[:2]
+    assert 1e-8 < (second - low) / low < 1e-7
+    full = lingam.fit(_dev(X, torch.float64), precision="fp64", prune=False)
+    pruned = lingam.fit(_dev(X, torch.float64), precision="fp64")
+    assert np.array_equal(full.order, o_order)
+    assert np.array_equal(pruned.order, o_order)
+    assert 0.0 <= pruned.margin_lb[1] <= (second - low) * (1 + 1e-3)   # (scores to 1e-10: 3e-3 of the gap at most)
+
+
 def test_batch_with_queued_problems_matches_oracle():
     # more problems than CTA slots, of 2 ... 13 variables, one large enough for a group of its own
     Xs = [_data(2 + k % 12, 40 + 17 * (k % 23), 7000 + k) for k in range(330)] + [_data(60, 3001, 8000)]
