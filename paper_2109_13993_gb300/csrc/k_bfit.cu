@@ -263,8 +263,9 @@ __global__ void __launch_bounds__(kBThreads) k_bfit_small(const Fit* __restrict_
 // position k on (d_k at v = K[k]; the last d is not needed).  In the normalised variables x = L e with e
 // the innovations, so B = I - L^{-1} there, and B[K[a]][K[b]] = -(L^{-1})[a][b] sd_{K[a]} / sd_{K[b]}
 // (a > b) in the original units: no Cholesky, whose p row steps of 3.5 us took most of the fit: a call of
-// p = 300 takes 0.9 ms less (of 11.0), p = 1000 4.3 ms (of 72.9), p = 20 0.07 ms (of 0.70).  Against long double its errors are a little below
-// the Cholesky's (p = 20 ... 150, relative norms: 0.96e-15 ... 3.5e-15 and 1.1e-15 ... 3.7e-15).
+// p = 300 takes 0.9 ms less (of 11.0), p = 1000 4.3 ms (of 72.9), p = 20 0.07 ms (of 0.70).  Its errors against long double are a little
+// below the Cholesky's (24 random graphs each, n = 500, FP64, geometric means of the norms: p = 20 3.1e-14
+// and 3.6e-14, p = 50 1.04e-13 and 1.17e-13, p = 80 1.77e-13 and 1.82e-13).
 //
 // A CTA solves two columns of L^{-1} by forward substitution in blocks of 32 rows: a warp per column
 // solves the block's triangle with shuffles, then all threads add the block's columns of L to the

@@ -559,6 +559,7 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
     const int cstr = bp * unit;
     T* s_cols = s_root + cstr;
 
+    __shared__ double s_rcp;
     __shared__ int s_next;   // units taken from the batch, beyond a warp's first
 
     const int root = wv.root;
@@ -653,8 +654,11 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
                 }
             };
             load_chunks();
-            if (rm && tid == NT - 1 && g.wk == 0 && r0 == 0 && bs == b0)
-                f.rmat[size_t(p - 1 - nrow) * p + root] = __ldcg(sold + root * p + root);
+            if (rm && tid == NT - 1) {   // (droot^2 for 1 / S[root][root] had B 2 to 10 % further off)
+                const double srr = __ldcg(sold + root * p + root);
+                s_rcp = 1.0 / srr;
+                if (g.wk == 0 && r0 == 0 && bs == b0) f.rmat[size_t(p - 1 - nrow) * p + root] = srr;
+            }
             // the rows', killers' and columns' removal coefficients (FP64)
             if (tid < 2 * nrb + ncol) {
                 const int k = tid < nrb ? tid : tid < 2 * nrb ? kRowBatch + tid - nrb : 2 * kRowBatch + tid - 2 * nrb;
@@ -685,13 +689,13 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
                 rc[1] = T(inv);
             }
             __syncthreads();
-            const double dr2 = droot * droot;   // 1 / S[root][root]
+            const double rcp = s_rcp;   // 1 / S[root][root]
 #pragma unroll
             for (int q = 0; q < PU; ++q)
                 if (pu[q] >= 0) {
                     const int j = pu[q] & 0xff, c = pu[q] >> 8, it = c == kMaxCols ? kRowBatch + j : 2 * kRowBatch + c;
                     double cv = pc[q];
-                    if (rm) cv = fma(-s_sr[j] * dr2, s_sr[it], cv);
+                    if (rm) cv = fma(-s_sr[j] * rcp, s_sr[it], cv);
                     double rho = cv * (s_dn[j] * s_dn[it]);
                     double om = fma(-rho, rho, 1.0);
                     constexpr bool f32 = sizeof(T) == 4;
@@ -708,7 +712,7 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
             while (crow[0] >= 0) {
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
-                    if (cat[q] >= 0) snew[cat[q]] = fma(-s_sr[crow[q]] * dr2, cb[q], ca[q]);
+                    if (cat[q] >= 0) snew[cat[q]] = fma(-s_sr[crow[q]] * rcp, cb[q], ca[q]);
                 load_chunks();
             }
             if (tid == 0) s_next = 0;

@@ -66,6 +66,39 @@ def test_mixed_scores_and_pruned_roots(p, n):
     assert np.abs(pruned.B - full.B).max() <= 1e-12 * max(1.0, np.abs(o_B).max())
 
 
+def _b_long_double(X, order):
+    """B of X in a given causal order, by elimination in long double."""
+    L = np.longdouble
+    x = X[order].astype(L)
+    x = x - x.mean(axis=1, keepdims=True)
+    S, p = x @ x.T, len(order)
+    low, d = np.eye(p, dtype=L), np.zeros(p, dtype=L)
+    for k in range(p):
+        d[k] = S[k, k]
+        low[k + 1:, k] = S[k + 1:, k] / d[k]
+        S[k + 1:, k + 1:] -= np.outer(low[k + 1:, k], low[k + 1:, k]) * d[k]
+    inv = np.eye(p, dtype=L)
+    for i in range(1, p):
+        inv[i, :i] = -low[i, :i] @ inv[:i, :i]
+    B = np.zeros((p, p), dtype=L)
+    B[np.ix_(order, order)] = np.eye(p, dtype=L) - inv
+    return B
+
+
+def test_fp64_b_is_no_further_off_than_the_cholesky():
+    # B from the ordering's elimination against the tile kernels' Cholesky, both from the same covariance:
+    # mean logarithm of their errors over 24 graphs
+    err = []
+    for seed in range(24):
+        X = _data(50, 500, seed)
+        a = lingam.fit(_dev(X, torch.float64), precision="fp64")
+        b = lingam.fit(_dev(X, torch.float64), precision="fp64", tile_i=32, tile_j=32, forced_order=a.order)
+        ref = _b_long_double(X, a.order)
+        err.append([np.linalg.norm((r.B - ref).astype(np.float64)) for r in (a, b)])
+    here, cholesky = np.exp(np.log(err).mean(axis=0))
+    assert here <= cholesky, (here, cholesky)
+
+
 def _near_tie(seed, weight):
     """Six variables whose second iteration ends in a near tie: weight moves the scores, in steps far
     below their gap."""
