@@ -1791,7 +1791,10 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2)
             const int* __restrict__ queue, int nqueue, unsigned* qhead, Ctl* top, unsigned smem_bytes) {
     __shared__ OrderShared sh;
     __shared__ Fit s_fit;
-    if (*reinterpret_cast<volatile int*>(&top->status) != 0) return;
+    // A group's CTAs leave together, when its controller says so: a single fit's status may be set by a CTA
+    // that started earlier, so it is only the controller that reads it.  (A batch's: whoever sets the flag
+    // has given up, and so does every CTA that waits.)
+    if (fits && *reinterpret_cast<volatile int*>(&top->abort) != 0) return;
     if constexpr (sizeof(T) == 8) {   // the exponentials' table, behind everything else
         smem_bytes -= kExpTab * sizeof(double);
         double* tab = reinterpret_cast<double*>(smem_order + smem_bytes);

@@ -60,6 +60,31 @@ def test_injected_host_fault_is_reported_and_the_next_call_succeeds(step, monkey
     assert np.array_equal(again.order, ref.order) and np.array_equal(again.B, ref.B)
 
 
+@pytest.mark.parametrize("kw", [{}, {"precision": "fp64"}])
+def test_degenerate_fit_ends_at_once_while_another_stream_works(kw):
+    """A collinear pair is met by whichever CTA compares it first; CTAs that start later, here because
+    copies of another stream take part of the GPU, must still take part until all leave together:
+    the status comes at once, not after a wait of timeout_s."""
+    d = synth.lingam_dataset(40, 3000, 0.1, seed=13)
+    X = d.X.copy()
+    X[31] = 2.0 * X[3]
+    dt = torch.float64 if kw.get("precision") == "fp64" else torch.float32
+    Xd = torch.tensor(X, dtype=dt, device="cuda")
+    a = torch.empty(64 << 20, dtype=torch.float32, device="cuda")
+    b = torch.empty_like(a)
+    side = torch.cuda.Stream()
+    for _ in range(5):
+        with torch.cuda.stream(side):
+            for _ in range(40):
+                b.copy_(a)
+        t0 = time.perf_counter()
+        with pytest.raises(lingam.LingamError) as e:
+            lingam.fit(Xd, timeout_s=4.0, **kw)
+        assert e.value.status == lingam.LINGAM_EDEGENERATE
+        assert time.perf_counter() - t0 < 3.0
+    torch.cuda.synchronize()
+
+
 def test_call_log_on_stderr():
     """LINGAM_LOG=1: one line per call on stderr with the sizes and the status."""
     import subprocess
