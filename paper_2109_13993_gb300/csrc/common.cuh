@@ -81,7 +81,7 @@ struct Ctl {
     // published wave (wave words continue across the iterations of a fit)
     int rm_r, rm_root;
     unsigned seq0;
-    int pad3;
+    int stop;            // the status after the iteration's last wave, for the next launch
     // the paper's threshold schedule (Fit::gamma0 > 0): the current threshold, reset to gamma0
     // at each iteration's plan, and the number of times it was raised over the fit
     double gamma;

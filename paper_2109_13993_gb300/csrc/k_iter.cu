@@ -1598,6 +1598,8 @@ __device__ __noinline__ void iteration_tail(const Fit& f, int it, IterShared& sh
     const int fc = int(gridDim.x) - 1;
     if (int(blockIdx.x) == fc) {
         plan_phase<Cfg::CONS, Cfg::TI, Cfg::TJ>(f, it + 1, smem_dyn, sh.red, f.sigma_alt);
+        // (every CTA is through with its pairs)
+        if (threadIdx.x == 0) f.ctl->stop = *reinterpret_cast<volatile int*>(&f.ctl->status);
     } else {
         volatile Ctl* vc = f.ctl;
         const int r = vc->rm_r, root = vc->rm_root, vb = int(blockIdx.x), vG = int(gridDim.x) - 1;
@@ -1687,9 +1689,9 @@ __global__ void __launch_bounds__(Cfg::CONS, Cfg::MINB) k_iteration(Fit f, int i
     uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + ring_or_sort);
     uint64_t* empty = full + kStages;
     volatile Ctl* vc = ctl;
-    // A failure recorded before this launch: every CTA reads it before the first
-    // barrier, so all of them leave together.
-    if (vc->status != 0) return;
+    // A failure recorded before this launch: all CTAs leave together.  (The status itself may be set by a
+    // CTA of this launch that is already comparing pairs, except in iteration 0, which starts with a barrier.)
+    if (vc->abort != 0 || (it == 0 ? vc->status : vc->stop) != 0) return;
     const unsigned long long tmo = vc->timeout_ns;
     if (threadIdx.x == 0) {
         for (int s = 0; s < Cfg::STAGES; ++s) {

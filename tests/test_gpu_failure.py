@@ -60,7 +60,8 @@ def test_injected_host_fault_is_reported_and_the_next_call_succeeds(step, monkey
     assert np.array_equal(again.order, ref.order) and np.array_equal(again.B, ref.B)
 
 
-@pytest.mark.parametrize("kw", [{}, {"precision": "fp64"}])
+@pytest.mark.parametrize("kw", [{}, {"tile_i": 64, "tile_j": 32}, {"precision": "fp64"},
+                                {"precision": "fp64", "tile_i": 32, "tile_j": 32}])
 def test_degenerate_fit_ends_at_once_while_another_stream_works(kw):
     """A collinear pair is met by whichever CTA compares it first; CTAs that start later, here because
     copies of another stream take part of the GPU, must still take part until all leave together:
