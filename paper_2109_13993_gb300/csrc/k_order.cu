@@ -1204,6 +1204,7 @@ struct Controller {
             f.rep_root_score[it] = 0.0;
             f.rep_margin[it] = INFINITY;
             f.rep_pairs[it] = 0;
+            if (f.timing) f.prev[it] = 0.0;   // no wave, so no time of its own
         }
         if (f.want_scores)
 #pragma unroll 1

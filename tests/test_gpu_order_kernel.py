@@ -130,6 +130,19 @@ def test_fp64_pruning_is_exact_at_a_near_tie(seed, weight):
     assert 0.0 <= pruned.margin_lb[1] <= (second - low) * (1 + 1e-3)   # (scores to 1e-10: 3e-3 of the gap at most)
 
 
+@pytest.mark.parametrize("p,max_iters", [(1, 0), (2, 0), (20, 0), (20, 7)])
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_iteration_times_do_not_hold_what_the_workspace_held(p, max_iters, precision):
+    X = _dev(_data(p, 700, 50 + p), torch.float64)
+    ws = lingam.alloc_workspace(lingam.workspace_size(p, 700, precision, np.float64))
+    ws.fill_(0xff)   # NaN as doubles
+    r = lingam.fit(X, precision=precision, timing=True, max_iters=max_iters, workspace=ws)
+    t = r.t_pair_iter_ms
+    assert np.all(np.isfinite(t)) and np.all(t >= 0.0)
+    assert t.sum() <= r.times_ms["pair"]
+    assert np.all(t[:(max_iters or p - 1)] > 0.0)
+
+
 def test_batch_with_queued_problems_matches_oracle():
     # more problems than CTA slots, of 2 ... 13 variables, one large enough for a group of its own
     Xs = [_data(2 + k % 12, 40 + 17 * (k % 23), 7000 + k) for k in range(330)] + [_data(60, 3001, 8000)]
