@@ -358,9 +358,10 @@ __global__ void __launch_bounds__(kFacThreads) k_factor_B_batch(const Fit* __res
     factor_columns<true>(f, blockIdx.y * kFacCols, sm_fac);
 }
 
-cudaError_t launch_factor_B(const Fit& f, cudaStream_t st) {
+cudaError_t launch_factor_B(const Fit& f, cudaStream_t st, long long* launches) {
     const int p = f.p, grid = (p + kFacCols - 1) / kFacCols;
     const size_t smem = size_t(kFacCols) * p * sizeof(double);
+    if (launches) *launches += p <= kFacGather ? 1 : 2;
     if (p <= kFacGather) {
         k_factor_B<true><<<grid, kFacThreads, smem, st>>>(f);
         return cudaGetLastError();
@@ -386,7 +387,7 @@ cudaError_t launch_factor_B_batch(const Fit* fits_dev, const int* p_host, int co
     }
     for (int k = 0; k < count; ++k)
         if (p_host[k] > kFacGather) {
-            const cudaError_t e = launch_factor_B(fits_host[k], st);
+            const cudaError_t e = launch_factor_B(fits_host[k], st, nullptr);
             if (e != cudaSuccess) return e;
         }
     return cudaSuccess;

@@ -107,13 +107,14 @@ __global__ void __launch_bounds__(256) k_gram_reduce(Fit f, const double* __rest
 
 // (the partial tiles take at most 608 x 8 KB, or nothing: they fit the FP64 path's partial-moment
 // region, at least 64 KB per tile of 32 variables and 32 samples, up to 320 of them)
-cudaError_t launch_gram(const Fit& f, size_t partial_bytes, cudaStream_t st) {
+cudaError_t launch_gram(const Fit& f, size_t partial_bytes, cudaStream_t st, long long* launches) {
     const int nt = (f.p + kGT - 1) / kGT, ntri = nt * (nt + 1) / 2;
     const int room = int(std::min<size_t>(partial_bytes / (size_t(ntri) * kGT * kGT * sizeof(double)), 1 << 20));
     const int nsplit = std::max(1, std::min(std::min(kGSplitCtas / ntri, f.ld / kGK), room));
     double* partial = static_cast<double*>(f.partials);
     k_gram<<<ntri * nsplit, 256, 0, st>>>(f, partial, nt, nsplit);
     cudaError_t e = cudaGetLastError();
+    if (launches) *launches += nsplit > 1 ? 2 : 1;
     if (e != cudaSuccess || nsplit == 1) return e;
     k_gram_reduce<<<dim3(ntri, kGT * kGT / 256), 256, 0, st>>>(f, partial, nt, nsplit);
     return cudaGetLastError();

@@ -21,8 +21,8 @@ cudaError_t launch_standardize(const Fit& f, const void* x, int input_dtype, cud
 cudaError_t launch_standardize_batch(const Fit* fits, const SrcDesc* src, const int* rowoff, int count, int rows,
                                      int precision, int input_dtype, cudaStream_t st);
 // FP64 path: Sigma = Xn Xn^T / (n-1) of the normalised rows (CalculateCovMat, Algorithm 3); sig0 = sig.
-// partial_bytes: what f.partials holds.
-cudaError_t launch_gram(const Fit& f, size_t partial_bytes, cudaStream_t st);
+// partial_bytes: what f.partials holds.  launches: NULL, or increased by the kernels launched (here and below).
+cudaError_t launch_gram(const Fit& f, size_t partial_bytes, cudaStream_t st, long long* launches);
 // The same product on the tensor cores (mixed path): the rows are split into exact
 // TF32 digits (three p x ld float planes and p exponents in `digits`), tcgen05 MMAs
 // over 128 x 128 tiles of the upper triangle with the sample axis split over CTAs,
@@ -68,7 +68,7 @@ constexpr int kBatchLaunchMax = 512;   // problems per launch_batch
 // B from the order: Cholesky of the covariance in causal order, B = I - diag(R) R^{-1}.
 cudaError_t launch_fit_B(const Fit& f, cudaStream_t st);
 // The same from the factorisation that the ordering kernel leaves in Fit::rmat.
-cudaError_t launch_factor_B(const Fit& f, cudaStream_t st);
+cudaError_t launch_factor_B(const Fit& f, cudaStream_t st, long long* launches);
 cudaError_t launch_factor_B_batch(const Fit* fits_dev, const int* p_host, int count, const Fit* fits_host, cudaStream_t st);
 // Bounded-wait self-test (k_iter.cu): the status the wait recorded (LINGAM_ETIMEOUT expected).
 cudaError_t run_wait_selftest(int which, unsigned long long timeout_ns, int* status, cudaStream_t st);

@@ -460,10 +460,10 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
                 status = LINGAM_ECUDA;
                 break;
             }
-            launches += 4;
+            launches += 4;   // (the rows' kernel among them)
         } else {
-            if (launch_gram(f, L.partial_bytes, st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
-            launches += 2;
+            ++launches;
+            if (launch_gram(f, L.partial_bytes, st, &launches) != cudaSuccess) { status = LINGAM_ECUDA; break; }
         }
         if (cudaEventRecord(ev[2], st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
         if (cov_out) {
@@ -507,11 +507,11 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
         }
         if (status != LINGAM_OK) break;
         if (cudaEventRecord(ev[3], st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
-        if (want_B && (inject_fault("bfit") || (order_kernel ? launch_factor_B(f, st) : launch_fit_B(f, st)) != cudaSuccess)) {
+        if (want_B && (inject_fault("bfit") || (order_kernel ? launch_factor_B(f, st, &launches) : launch_fit_B(f, st)) != cudaSuccess)) {
             status = LINGAM_ECUDA;
             break;
         }
-        if (want_B) launches += order_kernel ? 2 : 4;
+        if (want_B && !order_kernel) launches += 4;
         if (cudaEventRecord(ev[4], st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
     } while (0);
     // The results in one copy behind the kernels, B with them where it is small (one copy of pageable
@@ -818,7 +818,7 @@ static cudaError_t enqueue_batch(char* ws, const BatchLayout& BL, const std::vec
         cudaStream_t sk = nfork > 0 ? fs->s[j++ % nfork] : st;
         e = o.precision == LINGAM_MIXED
                 ? launch_gram_tc(fits[size_t(k)], ws + BL.region[size_t(k)] + Ls[size_t(k)].off_xin, fits[size_t(k)].partials, sk)
-                : launch_gram(fits[size_t(k)], Ls[size_t(k)].partial_bytes, sk);
+                : launch_gram(fits[size_t(k)], Ls[size_t(k)].partial_bytes, sk, nullptr);
     }
     for (int i = 0; i < nfork; ++i) {
         const cudaError_t ej = cudaEventRecord(fs->join[i], fs->s[i]) == cudaSuccess

@@ -130,6 +130,21 @@ def test_fp64_pruning_is_exact_at_a_near_tie(seed, weight):
     assert 0.0 <= pruned.margin_lb[1] <= (second - low) * (1 + 1e-3)   # (scores to 1e-10: 3e-3 of the gap at most)
 
 
+@pytest.mark.parametrize("p,precision,gram,factor", [(20, "mixed", 3, 1), (128, "mixed", 3, 1), (129, "mixed", 3, 2),
+                                                     (20, "fp64", 2, 1), (129, "fp64", 2, 2), (800, "fp64", 1, 0)])
+def test_kernel_launches_reported(p, precision, gram, factor):
+    # the rows, the covariance (FP64: without splits of the samples from 25 x 25 tiles of 32 on, one kernel),
+    # the ordering, B (above 128 variables from a permuted copy)
+    X = _dev(_data(min(p, 200), 900, 60 + p), torch.float64)
+    if factor:
+        r = lingam.fit(X[:p], precision=precision)
+        assert r.kernel_launches == 1 + gram + 1 + factor
+        assert lingam.fit(X[:p], precision=precision, want_B=False).kernel_launches == 1 + gram + 1
+    else:
+        X = torch.randn(p, 900, dtype=torch.float64, device="cuda")
+    assert lingam.covariance(X[:p], precision=precision)[1]["kernel_launches"] == 1 + gram
+
+
 @pytest.mark.parametrize("p,max_iters", [(1, 0), (2, 0), (20, 0), (20, 7)])
 @pytest.mark.parametrize("precision", ["mixed", "fp64"])
 def test_iteration_times_do_not_hold_what_the_workspace_held(p, max_iters, precision):
