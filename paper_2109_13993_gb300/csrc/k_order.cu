@@ -1227,7 +1227,7 @@ struct Controller {
 #pragma unroll 1
             for (int v = threadIdx.x; v < f.p; v += nt) f.rep_scores[size_t(it) * f.p + v] = NAN;
         select_lowest(a, r, nx_n, nx_drop);
-        write_wave(nx_removal, nx_removal && prunes && !gmode, sh.npick, nx_root);
+        write_wave(nx_removal, nx_removal && prunes, sh.npick, nx_root);
     }
     // Columns of an iteration's first wave.
     __device__ __forceinline__ int first_cols(int cmax, int want) const {
@@ -1464,25 +1464,27 @@ struct Controller {
         // 6. threshold: the live candidates of the others
         double gamma = gmode ? sh.st.gamma : 0.0;
         int live;
+        long long thr;
 #pragma unroll 1
         for (int pass = 0;; ++pass) {
-            const long long thr = gmode ? score_key(sum_from(gamma)) : best;
+            thr = gmode ? score_key(sum_from(gamma)) : best;
             int n = 0;
 #pragma unroll 1
             for (int k = an + tid; k < r; k += nt) {
-                const Sum lb = gmode ? part[k] : lower_bound(k, an);
+                const Sum lb = lower_bound(k, an);
                 const bool on = !(fl[k] & kNoRoot) && !(prunes && score_key(lb) > thr);
                 n += on ? 1 : 0;
                 row[k] = int(on ? key_bits(score_float(lb)) : kNoKey);
             }
             live = part_or(nt, n);
             // the paper's schedule: nothing can go on and nothing finished at or below gamma: raise
-            // gamma by factors gamma_c until the lowest score that may be the root's is at or below it
+            // gamma by factors gamma_c until the lowest bound of a score that may be the root's is at or
+            // below it
             if (!gmode || live || best <= thr || pass > 0) break;
             long long km = best;
 #pragma unroll 1
             for (int k = an + tid; k < r; k += nt)
-                if (!(fl[k] & kNoRoot)) km = min(km, score_key(part[k]));
+                if (!(fl[k] & kNoRoot)) km = min(km, score_key(lower_bound(k, an)));
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) km = min(km, __shfl_xor_sync(0xffffffffu, km, o));
             if (lane == 0) sh.lred[wid] = km;
@@ -1529,7 +1531,7 @@ struct Controller {
             const int v = var[k];
             if (v != bestv && !(fl[k] & kNoRoot)) second = min(second, score_key(lb));
             // a column whose strongest pair alone would not have excluded it
-            if (k < an && score_key(sum_of(T(kv0[k]))) <= best) ++need;
+            if (k < an && score_key(sum_of(T(kv0[k]))) <= thr) ++need;
             // without the root's contribution, where this iteration's last wave compared the two
             float ctr = 0.f;
             if (rs >= a && rs < an && k >= a && k != rs) {
@@ -1585,7 +1587,7 @@ struct Controller {
         // As many columns as this iteration would have needed, had it known its strongest pairs: whole
         // quads with one to spare on the FP32 path (a column of a started quad is free), no more on the
         // FP64 path (65 x 2001: 4.0 ms, one or two to spare 4.3 and 4.9, quads 5.3).
-        const int cmax = max_cols(r), want = !prunes || gmode ? kMaxCols : f32 ? (need + 4) / 4 * 4 : max(need, 1);
+        const int cmax = max_cols(r), want = !prunes ? kMaxCols : f32 ? (need + 4) / 4 * 4 : max(need, 1);
         new_iteration(cmax, want);
         if (r == 1) {
             if (tid < 32) swap_slots(rs, 1);

@@ -357,8 +357,7 @@ static bool check_prior(const signed char* prior, int p, std::vector<int>& anc) 
 // reuse there are no killer pairs, all columns are computed, and the tile kernels' waves of 32 columns
 // win on the mixed path from about 150 variables on: unpruned, ordering kernel against tile kernels,
 // p 100 11.3 and 13.3 ms, p 150 21.7 and 22.7, p 300 93.6 and 80.6.  (The paper's threshold schedule has
-// none either, but its roots and scores are those of the default run to the last rounding only in the
-// same kernel: 100 x 10000 from 10^-3 11.4 -> 9.2 ms, 300 x 5000 58.6 -> 72.9.)
+// them: random graphs, 300 x 5000 from a low start 60.6 -> 35.4 ms, from a high one 38.6 -> 35.6.)
 constexpr int kOrderFullP = 160;
 static bool use_order_kernel(const Fit& f, const lingam_opts& o) {
     const bool killers = o.prune && o.reuse;

@@ -158,6 +158,23 @@ def test_iteration_times_do_not_hold_what_the_workspace_held(p, max_iters, preci
     assert np.all(t[:(max_iters or p - 1)] > 0.0)
 
 
+@pytest.mark.parametrize("p,n", [(50, 2000), (150, 2000), (161, 700)])
+@pytest.mark.parametrize("start", ["low", "high"])
+def test_threshold_schedule_compares_no_more_pairs_than_the_tile_kernels(p, n, start):
+    # the killer pairs bound the scores under the paper's threshold schedule too; the roots are the same
+    X = _dev(_data(p, n, 1), torch.float32)
+    ref = lingam.fit(X)
+    rs = ref.root_score[ref.root_score > 0]
+    gamma0 = float(1e-3 * rs.min() if start == "low" else 10.0 * rs.max())
+    here = lingam.fit(X, gamma0=gamma0, forced_order=ref.order)
+    tiles = lingam.fit(X, gamma0=gamma0, forced_order=ref.order, tile_i=64, tile_j=32)
+    assert here.pairs_total < tiles.pairs_total
+    assert (here.threshold_updates > 0) == (tiles.threshold_updates > 0) == (start == "low")
+    assert np.allclose(here.root_score, ref.root_score, rtol=1e-6, atol=1e-9)
+    free = lingam.fit(X, gamma0=gamma0)
+    assert np.array_equal(free.order, ref.order)
+
+
 def test_batch_with_queued_problems_matches_oracle():
     # more problems than CTA slots, of 2 ... 13 variables, one large enough for a group of its own
     Xs = [_data(2 + k % 12, 40 + 17 * (k % 23), 7000 + k) for k in range(330)] + [_data(60, 3001, 8000)]
