@@ -354,15 +354,18 @@ static bool check_prior(const signed char* prior, int p, std::vector<int>& anc) 
 
 // Single fits run the ordering kernel (k_order.cu) unless an option asks for the tile kernels
 // (an explicit tile shape, LINGAM_NARROW) or the problem is too large for it.  Without pruning or pair
-// reuse there are no killer pairs, all columns are computed, and the tile kernels' waves of 32 columns
-// win on the mixed path from about 150 variables on: unpruned, ordering kernel against tile kernels,
-// p 100 11.3 and 13.3 ms, p 150 21.7 and 22.7, p 300 93.6 and 80.6.  (The paper's threshold schedule has
-// them: random graphs, 300 x 5000 from a low start 60.6 -> 35.4 ms, from a high one 38.6 -> 35.6.)
-constexpr int kOrderFullP = 160;
+// reuse there are no killer pairs, all columns are computed, and on the mixed path the tile kernels'
+// waves of 32 columns win from about 100 variables on, later where the rows are long.  Unpruned, tile
+// kernels' time over the ordering kernel's, n = 300, 1000, 5000, 20000: p 64 1.10 1.15 1.33 1.48, p 80 1.04
+// 1.09 1.28 1.40, p 100 0.95 1.00 1.18 1.26, p 130 0.87 0.92 1.10 1.13, p 150 0.84 0.89 1.05 1.08 (without
+// reuse p 130 0.91 0.97 1.11 1.00, p 150 0.88 0.94 1.02 0.97).
+static bool order_wins_unpruned(long long p, long long n, bool reuse) {
+    return p <= 80 || (p <= (reuse ? 150 : 130) && n >= 24 * p);
+}
 static bool use_order_kernel(const Fit& f, const lingam_opts& o) {
     const bool killers = o.prune && o.reuse;
     return o.tile_i == 0 && o.tile_j == 0 && !narrow_set() &&
-           (killers || o.precision != LINGAM_MIXED || f.p <= kOrderFullP) && order_supported(f, false);
+           (killers || o.precision != LINGAM_MIXED || order_wins_unpruned(f.p, f.n, o.reuse != 0)) && order_supported(f, false);
 }
 
 // cov_out != nullptr: stop after CalculateCovMat and copy Sigma (p x p) there.
@@ -936,8 +939,8 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
     // 1 x 1, a size the autotuner never measured, and the FP64 path without an explicit shape: the
     // ordering kernel, where it takes every problem of the call
     const bool untuned = o.tile_i == 0 && o.tile_j == 0 && !autotune_batch_measured(maxp, maxn);
-    // (unpruned sets of more than kOrderFullP variables: tiles, as for single fits)
-    bool order_kernel = o.reuse && (o.precision == LINGAM_MIXED ? ts.rows == 1 || (untuned && (o.prune || maxp <= kOrderFullP))
+    // (unpruned sets of more than 160 variables: tiles, as for single fits)
+    bool order_kernel = o.reuse && (o.precision == LINGAM_MIXED ? ts.rows == 1 || (untuned && (o.prune || maxp <= 160))
                                                                 : o.tile_i <= 1 && o.tile_j <= 1);
     for (int k = 0; k < count && order_kernel; ++k) {
         const Layout L = make_layout(P[size_t(k)], N[size_t(k)], o.precision, o.input_dtype);

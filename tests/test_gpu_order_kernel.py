@@ -48,7 +48,8 @@ def test_fp64_fit_matches_oracle(p, n, prune):
     assert np.abs(f.B - o_B).max() <= 1e-10 * max(1.0, np.abs(o_B).max())
 
 
-@pytest.mark.parametrize("p,n", SIZES + [(127, 500), (128, 500), (129, 500), (160, 640), (161, 640)])
+@pytest.mark.parametrize("p,n", SIZES + [(80, 500), (81, 500), (100, 2399), (100, 2400), (127, 500), (128, 500), (129, 500),
+                                         (150, 3600), (151, 3700), (160, 640), (161, 640)])
 def test_mixed_scores_and_pruned_roots(p, n):
     # every score within the mixed path's 1e-4 of the oracle; the killer pairs change no root's score.
     # Equal up to the FP32 rounding of I, 1e-6 absolute: S = sum of m squares I_j^2 moves by at most
