@@ -2220,6 +2220,250 @@ __global__ void __launch_bounds__(Cfg::CONS, Cfg::MINB) k_batch(const Fit* __res
     }
 }
 
+// ------------------------------------------------------------------ batches: one pair per warp
+// The pair mode of the batch kernel, for many small problems: a wave's needed pairs (its
+// columns against each other and against the other rows, Sec. III-A) are enumerated and each
+// is evaluated whole by one warp, so no pair slot of a tile is computed in vain.
+// The per-sample arithmetic, the group closing and the pair measure are the tile path's; the
+// lanes' group sums are added in a tree.  Each problem's pair measures go to its I buffer; one CTA per
+// problem then sums its rows' and columns' contributions in a fixed order and runs the wave
+// finalisation.  Waves have up to kPairTJ columns; a wave has one nominal "tile" of kPairTI
+// rows (the finalisation's column parts: part 0 holds the sums, the others stay zero).
+constexpr int kPairTJ = 16;
+constexpr int kPairTI = 1024;
+constexpr int kPairThr = 256;
+
+// Unordered pair q of a wave with ncol columns and nrow rows (columns first): column c of
+// row slot e, for c < ncol <= e (the columns against the other rows), then c < e < ncol
+// (the columns' own triangle).
+__device__ __forceinline__ void pair_of(long long q, int ncol, int nrow, int& e, int& c) {
+    const int qq = int(q);   // below ncol * nrow <= kPairTJ * 16384
+    const int cross = ncol * (nrow - ncol);
+    if (qq < cross) {
+        const int k = qq / ncol;
+        e = ncol + k;
+        c = qq - k * ncol;
+    } else {
+        const int t = qq - cross;   // triangle index: e (e - 1) / 2 + c, c < e < ncol <= kPairTJ
+        int ee = 1;
+        while ((ee + 1) * ee / 2 <= t) ++ee;
+        e = ee;
+        c = t - ee * (ee - 1) / 2;
+    }
+}
+__device__ __forceinline__ long long wave_pairs(int ncol, int nrow) {
+    return (long long)ncol * (ncol - 1) / 2 + (long long)ncol * (nrow - ncol);
+}
+
+// Closes one 32-sample group of both directions into the lane's sums (the tile path's group
+// closing: one lg2 of the product, the centring offset .w of each variable).
+__device__ __forceinline__ void close_group(const Acc2& aa, const Acc2& ab, float4 si, float4 sj, float& Da,
+                                            float& Ga, float& Db, float& Gb) {
+    Da += fmaf(float(kLn2), lg2_approx(aa.P.x * aa.P.y), fmaf(aa.A.x + aa.A.y, kInvScale / -kC3, si.w));
+    Ga += aa.G.x + aa.G.y;
+    Db += fmaf(float(kLn2), lg2_approx(ab.P.x * ab.P.y), fmaf(ab.A.x + ab.A.y, kInvScale / -kC3, sj.w));
+    Gb += ab.G.x + ab.G.y;
+}
+
+// One pair (row variable vi, column variable vj) by a whole warp; the measure I to every lane.
+// A 32-sample group of a lane is any 32 of the row's samples (the centring offset is per group
+// and the padding samples are zero), so the reads are coalesced: in each block of 1024
+// samples lane l takes the four samples 4l .. 4l + 3 of each 128-sample chunk, eight chunks
+// making its group.  The rows' last ld mod 1024 samples (a multiple of 128) are closed as
+// whole 32-sample groups, one per lane.
+__device__ __forceinline__ float pair_by_warp(const Fit& f, int vi, int vj, bool& degenerate) {
+    const int lane = threadIdx.x & 31;
+    const int p = f.p, ld = f.ld;
+    float2 ro = __ldcg(f.sigf + size_t(vi) * p + vj);
+    degenerate = !(ro.y > float(degenerate_om(true)));
+    if (degenerate) ro = make_float2(0.f, 1.f);
+    const float sc = kScale / sqrtf(ro.y);
+    const float2 s2 = make_float2(sc, sc), sr2 = make_float2(-sc * ro.x, -sc * ro.x);
+    const float4 si = __ldcg(f.vstat + vi), sj = __ldcg(f.vstat + vj);
+    const float* xi = static_cast<const float*>(f.xt) + size_t(vi) * ld;
+    const float* xj = static_cast<const float*>(f.xt) + size_t(vj) * ld;
+    float Da = 0.f, Ga = 0.f, Db = 0.f, Gb = 0.f;
+    const int nblk = ld >> 10;
+    for (int b = 0; b < nblk; ++b) {
+        const float4* ri = reinterpret_cast<const float4*>(xi + (size_t(b) << 10)) + lane;
+        const float4* rj = reinterpret_cast<const float4*>(xj + (size_t(b) << 10)) + lane;
+        float4 a4[8], b4[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            a4[k] = ri[32 * k];
+            b4[k] = rj[32 * k];
+        }
+        Acc2 aa, ab;
+        acc_init(aa);
+        acc_init(ab);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) acc_pair4(aa, ab, a4[k], b4[k], s2, sr2);
+        close_group(aa, ab, si, sj, Da, Ga, Db, Gb);
+    }
+    const int g = (nblk << 5) + lane;   // tail: one contiguous group per lane
+    if (g < ld / kSub) {
+        const float4* ri = reinterpret_cast<const float4*>(xi + size_t(g) * kSub);
+        const float4* rj = reinterpret_cast<const float4*>(xj + size_t(g) * kSub);
+        Acc2 aa, ab;
+        acc_init(aa);
+        acc_init(ab);
+#pragma unroll 4
+        for (int k = 0; k < kSub / 4; ++k) acc_pair4(aa, ab, ri[k], rj[k], s2, sr2);
+        close_group(aa, ab, si, sj, Da, Ga, Db, Gb);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        Da += __shfl_xor_sync(0xffffffffu, Da, o);
+        Ga += __shfl_xor_sync(0xffffffffu, Ga, o);
+        Db += __shfl_xor_sync(0xffffffffu, Db, o);
+        Gb += __shfl_xor_sync(0xffffffffu, Gb, o);
+    }
+    return pair_measure_f(Da, Ga, Db, Gb, si, sj, __frcp_rn(float(f.n)));
+}
+
+// One problem's wave after its pairs: the rows' contributions sum_c min(0, I)^2 (a thread per
+// row) and the columns' sum_e max(0, I)^2 (a warp per column, lanes over the rows, then a
+// tree), float-float in a fixed order, into the buffers the finalisation reads.
+template <int NTH>
+__device__ void pairs_merge(const Fit& f, const Wave& wv) {
+    const int ncol = wv.ncol, nrow = wv.nrow, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const float* I = static_cast<const float*>(f.ibuf);
+    for (int e = tid; e < nrow; e += NTH) {
+        FF acc;
+        const int cmax = e < ncol ? e : ncol;   // the pairs of row slot e
+        for (int c = 0; c < cmax; ++c) acc.add_sq(fminf(I[size_t(e) * kPairTJ + c], 0.f));
+        f.rowsum[e] = acc.value();
+    }
+    constexpr int PARTS = NTH / 64;
+    const int nparts = wv.ntiles * PARTS;
+    for (int c = wid; c < kPairTJ; c += NTH / 32) {
+        FF acc;
+        if (c < ncol)
+            for (int e = c + 1 + lane; e < nrow; e += 32) acc.add_sq(fmaxf(I[size_t(e) * kPairTJ + c], 0.f));
+        float2 v = make_float2(acc.hi, acc.lo);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float2 w = make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+            v = ff_add(v, w);
+        }
+        for (int at = lane; at < nparts; at += 32) {
+            const float2 ff = at == 0 ? v : make_float2(0.f, 0.f);
+            f.colsum[size_t(at) * kPairTJ + c] = *reinterpret_cast<const double*>(&ff);
+        }
+    }
+}
+
+// Every needed pair of every problem's wave, one warp per pair, into the problems' I
+// buffers.  Out of line, so that the sample loop's registers are allocated apart from the
+// rest of the kernel.
+__device__ __noinline__ void pairs_compute(const Fit* __restrict__ fits, int count, const BatchShared& bs,
+                                           long long ptot) {
+    constexpr int NW = kPairThr / 32;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (long long g = (long long)blockIdx.x * NW + wid; g < ptot; g += (long long)gridDim.x * NW) {
+        const int d = last_le(bs.uoff, count, g);
+        const Fit& f = fits[d];
+        const Wave wv = bs.wave[d];
+        int e, c;
+        pair_of(g - bs.uoff[d], wv.ncol, wv.nrow, e, c);
+        bool degenerate;
+        const float I = pair_by_warp(f, ld2(f.rows + e), ld2(f.cols + c), degenerate);
+        if (lane == 0) {
+            if (degenerate || !isfinite(I)) set_status(f.ctl, LINGAM_EDEGENERATE);
+            static_cast<float*>(f.ibuf)[size_t(e) * kPairTJ + c] = I;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kPairThr, 2) k_batch_pairs(const Fit* __restrict__ fits, int count, int maxp,
+                                                             Ctl* bctl) {
+    unsigned char* smem_raw = smem_dyn;
+    __shared__ IterShared sh;
+    __shared__ BatchShared bs;
+    volatile Ctl* vb = bctl;
+    if (vb->status != 0) return;
+    const unsigned long long tmo = vb->timeout_ns;
+    for (int it = 0; it < maxp; ++it) {
+        batch_active(fits, count, it, 0, bs);
+        for (int d = blockIdx.x; d < count; d += gridDim.x)
+            if (bs.act[d]) plan_phase<kPairThr, kPairTI, kPairTJ, 2048>(fits[d], it, smem_raw, sh.red, fits[d].sigma);
+        if (!grid_sync(bctl, tmo)) return;
+        for (;;) {
+            // the wave of every problem whose iteration is not done, and its pairs' offsets
+            // (a wave may have no pair left to evaluate, one column whose partners were all
+            // columns before: it is still finalised)
+            long long pbase = 0, nact = 0;
+            for (int base = 0; base < count; base += kPairThr) {
+                const int d = base + int(threadIdx.x);
+                long long q = 0, a = 0;
+                if (d < count) {
+                    const Fit& f = fits[d];
+                    volatile Ctl* c = f.ctl;
+                    Wave w = {0, 0, 0};
+                    if (it < f.p && !c->done && c->status == 0) {
+                        w = {c->ntiles, c->ncol, c->nrow};
+                        q = wave_pairs(w.ncol, w.nrow);
+                        a = 1;
+                    }
+                    bs.wave[d] = w;
+                    bs.act[d] = (unsigned char)a;
+                }
+                long long tq, ta;
+                const long long eq = block_excl_scan<kPairThr>(q, sh.lred, &tq);
+                block_excl_scan<kPairThr>(a, sh.lred, &ta);
+                if (d < count) bs.uoff[d] = pbase + eq;
+                pbase += tq;
+                nact += ta;
+            }
+            if (threadIdx.x == 0) bs.uoff[count] = pbase;
+            __syncthreads();
+            const long long ptot = bs.uoff[count];
+            if (nact == 0) break;
+            pairs_compute(fits, count, bs, ptot);   // every needed pair of every problem
+            if (!grid_sync(bctl, tmo)) return;
+            // each problem's sums and finalisation, one CTA per problem
+            for (int d = blockIdx.x; d < count; d += gridDim.x) {
+                if (!bs.act[d]) continue;
+                pairs_merge<kPairThr>(fits[d], bs.wave[d]);
+                __syncthreads();   // the sums precede the finalisation's reads (same CTA)
+                wave_finalize<kPairThr, kPairTI, kPairTJ>(fits[d], bs.wave[d], it, sh.red, 0u);
+                __syncthreads();
+            }
+            if (!grid_sync(bctl, tmo)) return;
+        }
+        // UpdateData and UpdateCovMat of every problem that took a root (the tile path's)
+        batch_active(fits, count, it, 1, bs);
+        int rtot;
+        long long etot;
+        batch_removal_layout<kPairThr>(fits, count, bs, sh, rtot, etot);
+        batch_remove_data<CfgF16>(fits, count, bs, rtot);
+        batch_remove_cov<CfgF16>(fits, count, bs, etot);
+        if (!grid_sync(bctl, tmo)) return;
+    }
+}
+
+static cudaError_t launch_batch_pairs(const Fit* fits_dev, int count, int maxp, Ctl* bctl, int nsm, cudaStream_t st) {
+    const size_t smem = size_t(2048) * sizeof(unsigned long long);   // the candidate sort
+    cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(k_batch_pairs), smem);
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_pairs, kPairThr, smem);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    cudaLaunchConfig_t cfg = {};
+    const int grid = nsm * (per_sm < 2 ? per_sm : 2);
+    cfg.gridDim = dim3(grid < kMaxGrid ? grid : kMaxGrid);
+    cfg.blockDim = dim3(kPairThr);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_batch_pairs, fits_dev, count, maxp, bctl);
+}
+
 // ------------------------------------------------------------------ host side
 template <class Cfg>
 static int grid_for(int nsm) {
@@ -2287,6 +2531,7 @@ cudaError_t launch_batch(const Fit* fits_dev, int count, int maxp, int precision
     if (tile_rows == 64 && tile_cols == 16) return launch_batch_cfg<CfgF16>(fits_dev, count, maxp, bctl, nsm, st);
     if (tile_rows == 32 && tile_cols == 32) return launch_batch_cfg<CfgF32>(fits_dev, count, maxp, bctl, nsm, st);
     if (tile_rows == 32 && tile_cols == 16) return launch_batch_cfg<CfgB>(fits_dev, count, maxp, bctl, nsm, st);
+    if (tile_rows == 1 && tile_cols == 1) return launch_batch_pairs(fits_dev, count, maxp, bctl, nsm, st);
     return cudaErrorInvalidValue;
 }
 

@@ -362,6 +362,19 @@ static bool check_prior(const signed char* prior, int p, std::vector<int>& anc) 
 static bool order_wins_unpruned(long long p, long long n, bool reuse) {
     return p <= 80 || (p <= (reuse ? 150 : 130) && n >= 24 * p);
 }
+// Unpruned batches on the mixed path, against pairs by warps (up to 128 variables by default), whose
+// throughput is higher: no columns are staged.  The ordering kernel wins where the rows are short (a
+// pair's warp has little to do), and where the problems do not fill the GPU: groups of CTAs then share
+// one.  `samples`: of all rows.  Pairs' time over the ordering kernel's, one problem, 16 and 256 (or 64):
+// 30 x 1000 1.15 1.21 1.08, 50 x 300 1.17 1.25 1.79, 50 x 2000 1.08 1.03 0.83, 100 x 300 0.97 1.26 2.13,
+// 100 x 1000 0.86 0.98 1.08, 100 x 2000 0.86 0.89 0.85, 100 x 10000 1.37 0.71; 64 uneven sets 0.79.
+// 32 x 32 tiles' time (beyond 128 variables): 150 x 300 0.97 0.97 1.21, 150 x 1000 1.15 1.11 1.31,
+// 150 x 5000 1.52 1.07.
+static bool order_wins_unpruned_batch(long long maxp, long long maxn, int count, long long samples, TileShape other) {
+    if (other.rows != 1) return maxp <= 160 && (maxn > 512 || count >= 32);
+    return (maxn <= 512 && (maxp <= 64 || count >= 4)) || (maxp <= 64 && (maxn <= 1024 || samples < 4000000)) ||
+           (maxn >= 8000 && samples < 4000000);
+}
 static bool use_order_kernel(const Fit& f, const lingam_opts& o) {
     const bool killers = o.prune && o.reuse;
     return o.tile_i == 0 && o.tile_j == 0 && !narrow_set() &&
@@ -937,16 +950,18 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
     const long long maxp = *std::max_element(P.begin(), P.end()), maxn = *std::max_element(N.begin(), N.end());
     TileShape ts = batch_tile_shape(o, maxp, maxn);
     // 1 x 1, a size the autotuner never measured, and the FP64 path without an explicit shape: the
-    // ordering kernel, where it takes every problem of the call
+    // ordering kernel, where it takes every problem of the call and, without pruning, where it wins;
+    // else pairs by warps (1 x 1) or tiles
     const bool untuned = o.tile_i == 0 && o.tile_j == 0 && !autotune_batch_measured(maxp, maxn);
-    // (unpruned sets of more than 160 variables: tiles, as for single fits)
-    bool order_kernel = o.reuse && (o.precision == LINGAM_MIXED ? ts.rows == 1 || (untuned && (o.prune || maxp <= 160))
-                                                                : o.tile_i <= 1 && o.tile_j <= 1);
+    long long samples = 0;
+    for (int k = 0; k < count; ++k) samples += P[size_t(k)] * N[size_t(k)];
+    bool order_kernel = o.reuse && (o.precision == LINGAM_MIXED
+                                        ? (ts.rows == 1 || untuned) && (o.prune || order_wins_unpruned_batch(maxp, maxn, count, samples, ts))
+                                        : o.tile_i <= 1 && o.tile_j <= 1);
     for (int k = 0; k < count && order_kernel; ++k) {
         const Layout L = make_layout(P[size_t(k)], N[size_t(k)], o.precision, o.input_dtype);
         order_kernel = order_supported(make_fit(ws, L, int(P[size_t(k)]), int(N[size_t(k)]), o, false), true);
     }
-    if (!order_kernel && ts.rows == 1) ts = TileShape{64, 16};
     mix(ts.rows);
     mix(ts.cols);
     mix(order_kernel ? 1 : 0);

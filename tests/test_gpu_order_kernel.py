@@ -176,6 +176,24 @@ def test_threshold_schedule_compares_no_more_pairs_than_the_tile_kernels(p, n, s
     assert np.array_equal(free.order, ref.order)
 
 
+@pytest.mark.parametrize("sizes", [[(64, 600)] * 2, [(65, 600)] * 2, [(40, 1025)] * 3, [(70, 512)] * 3, [(70, 512)] * 4,
+                                   [(70, 513)] * 4, [(20, 8000)] * 2, [(70, 8000)], [(70, 7999)], [(128, 700), (3, 40)],
+                                   [(129, 513), (9, 100)], [(129, 512), (9, 100)], [(161, 600), (9, 100)], [(1, 9), (2, 5)]])
+@pytest.mark.parametrize("tile", [0, 1])
+def test_unpruned_batches_on_either_side_of_the_routes(sizes, tile):
+    # ordering kernel, pairs by warps and tiles: scores of every variable against FP64, B against the single
+    # fit's.  1e-4 is the mixed path's stated tolerance
+    Xs = [_data(p, n, 9000 + 10 * k + p).astype(np.float32) for k, (p, n) in enumerate(sizes)]
+    got = lingam.fit_batch([_dev(X, torch.float32) for X in Xs], prune=False, want_scores=True, tile_i=tile, tile_j=tile)
+    assert got.status == lingam.LINGAM_OK
+    for X, order, B, S in zip(Xs, got.orders, got.Bs, got.scores):
+        ref = lingam.fit(_dev(X, torch.float64), precision="fp64", prune=False, forced_order=order, want_scores=True)
+        m = ~np.isnan(ref.scores)
+        assert np.array_equal(m, ~np.isnan(S))
+        assert np.abs(S[m] - ref.scores[m]).max() <= 1e-4
+        assert np.abs(B - ref.B).max() <= 1e-4 * max(1.0, np.abs(ref.B).max())
+
+
 def test_batch_with_queued_problems_matches_oracle():
     # more problems than CTA slots, of 2 ... 13 variables, one large enough for a group of its own
     Xs = [_data(2 + k % 12, 40 + 17 * (k % 23), 7000 + k) for k in range(330)] + [_data(60, 3001, 8000)]
