@@ -121,6 +121,7 @@ struct Fit {
     int has_forced;      // forced order given
     int want_scores;     // fill the per-iteration score matrix
     int timing;          // accumulate the phase times in Ctl::phase_ns
+    int first_it;        // tile kernels: their first iteration (0 unless the ordering kernel has handed over)
     void* xt;            // p x ld normalised data (float or double)
     double* mu;          // [p] row means
     double* sd;          // [p] row standard deviations (divisor n-1)
@@ -184,6 +185,7 @@ struct Fit {
     void* rec;           // sums of the current wave, per segment, row and column (8-byte values)
     unsigned long long rec_bytes;
     int unit;            // samples of a warp's unit of work: 1024 or 512 (FP32), 256 (FP64)
+    int handover;        // it may leave the rest of the fit to the tile kernels (Ctl::it then says from where)
     void* rowtab;        // [p] rows of the current wave (RowEnt)
     int* gcount;         // [kOrderSlots] workers of a row group done with the wave
     double* dscale[2];   // [p] by variable, two copies: the normalised row is the residual times this

@@ -277,11 +277,11 @@ constexpr int kFacCols = 2;
 // problems share one launch); above it a permuted copy, read in rows, is worth its launch of 3 us.
 constexpr int kFacGather = 128;
 
-// The ordering ran to its end (of a batch that ran out of time some may not have: their orders are not
+// The ordering ran to its end (a single fit's may have been handed over to the tile kernels; of a batch that ran out of time some may not have: their orders are not
 // read).
 __device__ __forceinline__ bool ordered(const Fit& f) {
     const volatile Ctl* c = f.ctl;
-    return c->status == 0 && (f.p == 1 || c->waves > 0);
+    return c->status == 0 && c->it == 0 && (f.p == 1 || c->waves > 0);
 }
 
 // The factor in causal order: cmat[k p + i] = L[i][k] d_k, i >= k.

@@ -1690,8 +1690,8 @@ __global__ void __launch_bounds__(Cfg::CONS, Cfg::MINB) k_iteration(Fit f, int i
     uint64_t* empty = full + kStages;
     volatile Ctl* vc = ctl;
     // A failure recorded before this launch: all CTAs leave together.  (The status itself may be set by a
-    // CTA of this launch that is already comparing pairs, except in iteration 0, which starts with a barrier.)
-    if (vc->abort != 0 || (it == 0 ? vc->status : vc->stop) != 0) return;
+    // CTA of this launch that is already comparing pairs, except in the first one, which starts with a barrier.)
+    if (vc->abort != 0 || (it == f.first_it ? vc->status : vc->stop) != 0) return;
     const unsigned long long tmo = vc->timeout_ns;
     if (threadIdx.x == 0) {
         for (int s = 0; s < Cfg::STAGES; ++s) {
@@ -1703,9 +1703,9 @@ __global__ void __launch_bounds__(Cfg::CONS, Cfg::MINB) k_iteration(Fit f, int i
     }
     __syncthreads();
 
-    // Iteration 0 is planned here; every later one was planned by the previous launch, during
+    // The first iteration is planned here; every later one was planned by the previous launch, during
     // its removal (the candidate order in f.sigma, the first wave in the control block).
-    if (it == 0) {
+    if (it == f.first_it) {
         if (blockIdx.x == 0) plan_phase<Cfg::CONS, Cfg::TI, Cfg::TJ>(f, it, smem_raw, sh.red, f.sigma);
         if (!grid_sync(ctl, tmo)) return;
     }

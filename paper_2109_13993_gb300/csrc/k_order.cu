@@ -66,6 +66,14 @@ __host__ __device__ constexpr int max_unit() { return sizeof(T) == 4 ? 1024 : 25
 template <class T>
 __host__ __device__ constexpr int quad() { return sizeof(T) == 4 ? 4 : 1; }
 constexpr int kRowBatch = 32;    // rows of a worker between two CTA barriers
+// A single fit on the mixed path is left to the tile kernels once kHandIters iterations in a row (after the
+// first) took kHandCols columns or more: killer pairs do not help there, and 32-column waves are cheaper.
+// The time of the rest of a fit, tile kernels over this one, by the columns an iteration takes: pure noise
+// 300 x 500 0.94 at 165 columns, 300 x 5000 0.98 at 176, 500 x 1000 0.78 at 310 and 1.00 at 133, 1000 x 4000
+// 0.67 at 681 and 0.96 at 193; random graphs 1000 x 1300 0.97 at 178 and 1.01 at 157, 1000 x 10000 0.98 at
+// 207 and 1.01 at 181, 2000 x 2300 0.70 at 375.
+constexpr int kHandCols = 176;
+constexpr int kHandIters = 4;
 constexpr int kDedicated = 8;    // groups of this many CTAs or more have a controller that does not work
 
 extern __shared__ __align__(128) unsigned char smem_order[];
@@ -875,6 +883,8 @@ struct OrderShared {
     int ired[16], nkill[16];
     // to be reported once the next wave is published
     int rep_ncol, rep_nrow, rep_nw, rep_it, rep_root, rep_bestv;
+    int wide;     // iterations in a row that took kHandCols columns or more
+    int raised;   // the threshold schedule has raised its threshold in this fit
     long long rep_best, rep_rootpt;
 };
 
@@ -1243,6 +1253,22 @@ struct Controller {
         return lb;
     }
 
+    // Iteration `it` goes to the tile kernels, which start it anew: this wave has removed the last root from
+    // the rows and the covariance, and its statistics are the new rows'.  By variable: what is left in U, the
+    // statistics, and the scores so far (the candidates' order); see k_hand_over.
+    __device__ __forceinline__ void hand_over(int an) {
+#pragma unroll 1
+        for (int k = threadIdx.x; k < f.p; k += nt) {
+            const int v = var[k];
+            f.flags[v] = k < r ? kAlive : 0;
+            if (k < r) {
+                f.vstat[v] = st[k];
+                f.hx[v] = score_out(k < an ? part[k] : lower_bound(k, an));
+            }
+        }
+        if (threadIdx.x == 0) f.ctl->it = it;
+    }
+
     // One pair's measure from its four sums: row slot k against slot j.
     __device__ __forceinline__ T measure(const T (&v)[4], int k, int j) const {
         T x;
@@ -1500,6 +1526,7 @@ struct Controller {
             }
             if (!(score_key(sum_from(gamma)) >= km)) gamma = target;
             gsteps += n2;
+            if (tid == 0 && n2 > 0) sh.raised = 1;
         }
         if (tid == 0) {
             sh.rep_ncol = ncol;
@@ -1508,6 +1535,13 @@ struct Controller {
             sh.rep_it = -1;
         }
         if (live) {
+            // (the schedule's raises cost the tile kernels more: random 1000 x 2000 from a low start 387 ms
+            // here, 668 there)
+            if (f32 && has_k && f.handover && sh.wide >= kHandIters && sh.raised == 0) {
+                hand_over(an);
+                done();
+                return;
+            }
             a = an;
             const int nr2 = f.reuse ? r - a : r, cm = max_cols(nr2);
             if (tid == 0) {
@@ -1568,6 +1602,7 @@ struct Controller {
             sh.ired[wid] = need;
         }
         if (tid == 0) {
+            sh.wide = it > 0 && an >= kHandCols ? sh.wide + 1 : 0;
             sh.rep_it = it;
             sh.rep_root = root;
             sh.rep_bestv = bestv;
@@ -1726,7 +1761,7 @@ __device__ __forceinline__ bool run_problem(const Fit& f, Ctl* top, int rank, in
     Controller<T, NT> c(f, g, sh, smem_bytes, iters);
     if (threadIdx.x == 0) {
         sh.ok = *reinterpret_cast<volatile int*>(&f.ctl->status) == 0;
-        sh.rep_nw = 0;
+        sh.rep_nw = sh.wide = sh.raised = 0;
     }
     __syncthreads();
     c.next_wave(0, -1, false, 0);
@@ -1827,6 +1862,44 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2)
         rank = 0;
         size = 1;
     }
+}
+
+// ------------------------------------------------------------------ to the tile kernels
+// One CTA per variable left in U (f.flags): its row into f.xt, its covariances with the later variables,
+// normalised, into both triangles of f.sig and f.sigf, its statistics by its own mean, and its sort key.
+// cur: the copies that hold the current rows, covariance and scales.  Runs once, about 0.1 ms at p = 1000.
+constexpr int kHandThreads = 256;
+__global__ void __launch_bounds__(kHandThreads) k_hand_over(Fit f, int cur) {
+    const int p = f.p, ld = f.ld, v = blockIdx.x, tid = threadIdx.x;
+    if (!(f.flags[v] & kAlive)) return;
+    const double* S = cur ? f.sigalt : f.sig;   // (in place when it is f.sig: each element is read here alone)
+    const double* D = f.dscale[cur];
+    if (cur) {
+        const float4* src = reinterpret_cast<const float4*>(static_cast<const float*>(f.xalt) + size_t(v) * ld);
+        float4* dst = reinterpret_cast<float4*>(static_cast<float*>(f.xt) + size_t(v) * ld);
+        for (int t = tid; t < ld / 4; t += kHandThreads) dst[t] = src[t];
+    }
+    const double dv = D[v];
+    for (int j = v + tid; j < p; j += kHandThreads) {
+        if (!(f.flags[j] & kAlive)) continue;
+        const double c = j == v ? 1.0 : S[size_t(v) * p + j] * (dv * D[j]);
+        const float2 cf = sig_pair_f(c);
+        f.sig[size_t(v) * p + j] = c;
+        f.sig[size_t(j) * p + v] = c;
+        f.sigf[size_t(v) * p + j] = cf;
+        f.sigf[size_t(j) * p + v] = cf;
+    }
+    if (tid == 0) {
+        // the row's sum centred by the offset -32 (ln 2 + m0) over the padded row is -corr n
+        const float4 s = f.vstat[v];
+        const double m0 = -double(s.w) / kSub - kLn2, m = (double(ld) * m0 - double(s.x) * f.n) * f.inv_n;
+        f.vstat[v] = var_stats_inv((m - kBeta) * f.n, double(s.z) * f.n, f.n, ld, f.inv_n);
+        f.prev[v] = f.hx[v];
+    }
+}
+cudaError_t launch_hand_over(const Fit& f, int it, cudaStream_t st) {
+    k_hand_over<<<f.p, kHandThreads, 0, st>>>(f, it & 1);   // (a removal per iteration, each into the other copy)
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ host side

@@ -50,6 +50,9 @@ int iteration_grid(const Fit& f, int nsm);
 // SM, p up to about 1200).
 bool order_supported(const Fit& f, bool batch);
 int order_grid(const Fit& f, int nsm);
+// Behind an ordering kernel that stopped at iteration `it` (Ctl::it > 0, Fit::handover): rows, covariance
+// and statistics of the remaining variables as the tile kernels keep them.
+cudaError_t launch_hand_over(const Fit& f, int it, cudaStream_t st);
 cudaError_t launch_order(const Fit& f, int iters, int nsm, cudaStream_t st);
 // Batches: the CTAs' first problems (assign, one entry per CTA of the grid) and the queue of the
 // others, planned on the host; then the launch of the table.

@@ -413,6 +413,7 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
     f.prior = with_prior ? reinterpret_cast<const signed char*>(base + L.off_prior) : nullptr;
     f.anc_cnt = with_prior ? reinterpret_cast<int*>(base + L.off_anc) : nullptr;
     f.timing = o.timing ? 1 : 0;
+    f.handover = o.precision == LINGAM_MIXED && o.prune && o.reuse;
 
 #define CK(call)                                  \
     do {                                          \
@@ -459,6 +460,33 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
     long long launches = 0;
     bool order_kernel = false;
     int status = LINGAM_OK;
+    // the tile kernels' iterations from `first` on
+    const auto run_tiles = [&](int first) {
+        const int grid = iteration_grid(f, nsm);
+        if (grid < 1) return false;
+        // opts.timing: one event before the first launch and one after each, so that a launch is timed
+        // between two consecutive events
+        if (o.timing) {
+            const cudaEvent_t e0 = ev[next_ev++];
+            pev.push_back(e0);
+            cudaEventRecord(e0, st);
+        }
+        for (int it = first; it < iters; ++it) {
+            // the candidate orders alternate between the two lists: iteration it reads the
+            // one the previous launch planned and plans the next into the other
+            Fit fi = f;
+            fi.first_it = first;
+            if ((it - first) & 1) std::swap(fi.sigma, fi.sigma_alt);
+            if (inject_fault("iteration", it) || launch_iteration(fi, it, grid, st) != cudaSuccess) return false;
+            ++launches;
+            if (o.timing) {
+                const cudaEvent_t e1 = ev[next_ev++];
+                pev.push_back(e1);
+                cudaEventRecord(e1, st);
+            }
+        }
+        return true;
+    };
     do {
         if (cudaEventRecord(ev[0], st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
         if (inject_fault("standardize") || launch_standardize(f, xdev, o.input_dtype, st) != cudaSuccess) {
@@ -494,32 +522,7 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
             if (launch_order(f, iters, nsm, st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
             ++launches;
         }
-        const int grid = order_kernel ? 1 : iteration_grid(f, nsm);
-        if (grid < 1) {
-            status = LINGAM_ECUDA;
-            break;
-        }
-        // opts.timing: one event before the first launch and one after each, so launch it
-        // is timed between events it and it + 1 (consecutive launches share an event)
-        if (o.timing && !order_kernel) {
-            const cudaEvent_t e0 = ev[next_ev++];
-            pev.push_back(e0);
-            cudaEventRecord(e0, st);
-        }
-        for (int it = 0; it < iters && status == LINGAM_OK && !order_kernel; ++it) {
-            cudaEvent_t e1 = nullptr;
-            if (o.timing) {
-                e1 = ev[next_ev++];
-                pev.push_back(e1);
-            }
-            // the candidate orders alternate between the two lists: iteration it reads the
-            // one the previous launch planned and plans the next into the other
-            Fit fi = f;
-            if (it & 1) std::swap(fi.sigma, fi.sigma_alt);
-            if (inject_fault("iteration", it) || launch_iteration(fi, it, grid, st) != cudaSuccess) status = LINGAM_ECUDA;
-            ++launches;
-            if (o.timing) cudaEventRecord(e1, st);
-        }
+        if (!order_kernel && !run_tiles(0)) status = LINGAM_ECUDA;
         if (status != LINGAM_OK) break;
         if (cudaEventRecord(ev[3], st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
         if (want_B && (inject_fault("bfit") || (order_kernel ? launch_factor_B(f, st, &launches) : launch_fit_B(f, st)) != cudaSuccess)) {
@@ -545,6 +548,42 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
     if (status == LINGAM_OK) {
         std::memcpy(&ch, out.data() + L.off_ctl, sizeof(ch));
         if (ch.status != 0) status = ch.status;
+    }
+    // the ordering kernel has left the iterations from ch.it on to the tile kernels
+    const int handed = status == LINGAM_OK && order_kernel ? ch.it : 0;
+    double order_ms = 0.0;           // opts.timing: the ordering kernel's launch and its iterations
+    std::vector<double> order_iter_ms;
+    if (handed > 0) {
+        do {
+            if (o.timing) {
+                float ms = 0.f;
+                if (cudaEventElapsedTime(&ms, ev[2], ev[3]) == cudaSuccess) order_ms = ms;
+                order_iter_ms.resize(size_t(handed));
+                if (cudaMemcpy(order_iter_ms.data(), f.prev, size_t(handed) * 8, cudaMemcpyDeviceToHost) != cudaSuccess) {
+                    status = LINGAM_ECUDA;
+                    break;
+                }
+            }
+            if (launch_hand_over(f, handed, st) != cudaSuccess) { status = LINGAM_ECUDA; break; }
+            ++launches;
+            ch.bar_count = 0;   // as when a fit starts
+            ch.wave_word = 0;
+            ch.seq0 = 0;
+            ch.done = 0;
+            if (cudaMemcpyAsync(f.ctl, &ch, sizeof(ch), cudaMemcpyHostToDevice, st) != cudaSuccess || !run_tiles(handed) ||
+                cudaEventRecord(ev[3], st) != cudaSuccess || (want_B && launch_fit_B(f, st) != cudaSuccess) ||
+                cudaEventRecord(ev[4], st) != cudaSuccess) {
+                status = LINGAM_ECUDA;
+                break;
+            }
+            if (want_B) launches += 4;
+            if (cudaMemcpyAsync(out.data(), base, out_bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess) status = LINGAM_ECUDA;
+        } while (0);
+        if (cudaStreamSynchronize(st) != cudaSuccess) status = LINGAM_ECUDA;
+        if (status == LINGAM_OK) {
+            std::memcpy(&ch, out.data() + L.off_ctl, sizeof(ch));
+            if (ch.status != 0) status = ch.status;
+        }
     }
     if (status == LINGAM_OK && cov_out) {
         if (cudaMemcpy(cov_out, f.sig, size_t(p) * p * 8, cudaMemcpyDefault) != cudaSuccess) status = LINGAM_ECUDA;
@@ -582,9 +621,12 @@ static int fit_one(const void* X, long long p_, long long n_, int* order, double
             for (size_t k = 0; k + 1 < pev.size(); ++k)
                 if (cudaEventElapsedTime(&ms, pev[k], pev[k + 1]) == cudaSuccess) {
                     tp += ms;
-                    if (rep->t_pair_iter_ms && k < size_t(p)) rep->t_pair_iter_ms[k] = ms;
+                    if (rep->t_pair_iter_ms && k < size_t(p)) rep->t_pair_iter_ms[size_t(handed) + k] = ms;
                 }
-            if (order_kernel && o.timing) {   // one launch: its time, and the iterations' by the device's timer
+            if (handed > 0 && o.timing) {
+                tp += order_ms;
+                if (rep->t_pair_iter_ms) std::memcpy(rep->t_pair_iter_ms, order_iter_ms.data(), size_t(handed) * 8);
+            } else if (order_kernel && o.timing) {   // one launch: its time, and the iterations' by the device's timer
                 if (cudaEventElapsedTime(&ms, ev[2], ev[3]) == cudaSuccess) tp = ms;
                 if (rep->t_pair_iter_ms)
                     cudaMemcpyAsync(rep->t_pair_iter_ms, f.prev, size_t(iters) * 8, cudaMemcpyDefault, st);

@@ -3,6 +3,8 @@ change: units and the last, partial one (128 / 64 samples a step), rows of a wor
 (4 ... 16), the controller's warps, in-place and permuted factors (128 variables), the line between
 ordering and tile kernels (160), queued problems of a batch (more than 304), tiles and parts of the
 covariance (128, 8; 32 on the FP64 path)."""
+import functools
+
 import numpy as np
 import pytest
 
@@ -192,6 +194,71 @@ def test_unpruned_batches_on_either_side_of_the_routes(sizes, tile):
         assert np.array_equal(m, ~np.isnan(S))
         assert np.abs(S[m] - ref.scores[m]).max() <= 1e-4
         assert np.abs(B - ref.B).max() <= 1e-4 * max(1.0, np.abs(ref.B).max())
+
+
+def _common_causes(p, n, causes, seed):
+    """Independent variables but for `causes` of them, each a parent of all the others."""
+    e = np.random.default_rng(seed).laplace(size=(p, n))
+    for c in range(causes):
+        e[c + 1:] += 0.8 * e[c]
+    return e.astype(np.float32)
+
+
+@functools.lru_cache(maxsize=None)
+def _common_causes_fp64(p, n, causes, seed):
+    X = _common_causes(p, n, causes, seed)
+    return X, lingam.fit(_dev(X, torch.float64), precision="fp64", prune=False, want_scores=True)
+
+
+def _handed_over_at(res, p, want_B=True):
+    """Iteration from which tile kernels ran: rows, covariance (3), ordering, the step between, an iteration
+    each, B's two kernels tried before and four after."""
+    return p - (res.kernel_launches - 6 - (6 if want_B else 0))
+
+
+@pytest.mark.parametrize("kw", [{}, {"gamma0": 1.0}, {"prior": True}, {"timing": True}, {"split_n": 2}])
+def test_hand_over_to_the_tile_kernels(kw):
+    # many independent variables: no killer pairs to speak of.  Scores along FP64's order within the mixed
+    # path's 1e-4 before and behind the iteration, at even and odd ones (the rows lie in either copy)
+    p, n, at = 400, 640, set()
+    for causes in (0, 1, 2, 5):
+        X, full = _common_causes_fp64(p, n, causes, 70 + causes)
+        opts = dict(kw)
+        if opts.pop("prior", None):
+            opts["prior"] = np.zeros((p, p), dtype=np.int8)
+            opts["prior"][full.order[200], full.order[0]] = opts["prior"][full.order[-1], full.order[100]] = 1
+        got = lingam.fit(_dev(X, torch.float32), forced_order=full.order, want_scores=True, **opts)
+        it0 = _handed_over_at(got, p)
+        assert 5 <= it0 < 30
+        at.add(it0 % 2)
+        m = ~np.isnan(got.scores)
+        assert np.abs(got.scores[m] - full.scores[m]).max() <= 1e-4
+        assert m[:-1].sum(axis=1).min() >= 2
+        if "gamma0" not in kw:
+            # a variable left out is not the root: its score is above the lowest complete one
+            low = np.where(m, got.scores, np.inf).min(axis=1)
+            out = ~m & ~np.isnan(full.scores)
+            if "prior" not in kw:
+                assert np.all(np.where(out, full.scores, np.inf).min(axis=1) >= low - 1e-6)
+        assert np.abs(got.root_score - full.root_score).max() <= 1e-6
+        assert np.abs(got.B - full.B).max() <= 1e-4 * max(1.0, np.abs(full.B).max())
+        assert sorted(lingam.fit(_dev(X, torch.float32), **opts).order.tolist()) == list(range(p))
+        if "timing" in kw:
+            t = got.t_pair_iter_ms
+            assert np.all(np.isfinite(t)) and np.all(t[:-1] > 0.0) and t.sum() <= got.times_ms["order"]
+    assert at == ({1} if "gamma0" in kw else {0, 1})   # (nothing is pruned below 1: iteration 5 each time)
+
+
+def test_hand_over_within_a_bounded_number_of_iterations():
+    p, n = 400, 640
+    X = _dev(_common_causes(p, n, 1, 71), torch.float32)
+    ref = lingam.fit(X)
+    it0 = _handed_over_at(ref, p)
+    for iters in (it0 - 1, it0, it0 + 1, it0 + 2):
+        part = lingam.fit(X, max_iters=iters)
+        assert np.array_equal(part.order[:iters], ref.order[:iters]) and np.all(part.order[iters:] == -1)
+        assert np.array_equal(part.root_score[:iters], ref.root_score[:iters])
+        assert part.kernel_launches == 5 + (iters > it0) * (1 + iters - it0)
 
 
 def test_batch_with_queued_problems_matches_oracle():
