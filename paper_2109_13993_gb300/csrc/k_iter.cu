@@ -1679,7 +1679,7 @@ __device__ bool wait_wave(Ctl* ctl, unsigned seq, unsigned long long tmo, Wave& 
 }
 
 template <class Cfg>
-__global__ void __launch_bounds__(Cfg::CONS, Cfg::MINB) k_iteration(Fit f, int it) {
+__global__ void __launch_bounds__(Cfg::CONS, Cfg::MINB) k_iteration(const __grid_constant__ Fit f, int it) {
     unsigned char* smem_raw = smem_dyn;
     __shared__ IterShared sh;
     using T = typename Cfg::T;
@@ -1691,7 +1691,8 @@ __global__ void __launch_bounds__(Cfg::CONS, Cfg::MINB) k_iteration(Fit f, int i
     volatile Ctl* vc = ctl;
     // A failure recorded before this launch: all CTAs leave together.  (The status itself may be set by a
     // CTA of this launch that is already comparing pairs, except in the first one, which starts with a barrier.)
-    if (vc->abort != 0 || (it == f.first_it ? vc->status : vc->stop) != 0) return;
+    const int aborted = vc->abort, failed = *(it == f.first_it ? &vc->status : &vc->stop);   // (both in flight)
+    if (aborted != 0 || failed != 0) return;
     const unsigned long long tmo = vc->timeout_ns;
     if (threadIdx.x == 0) {
         for (int s = 0; s < Cfg::STAGES; ++s) {
