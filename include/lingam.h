@@ -271,10 +271,11 @@ void lingam_autotune_reset(void);
  * record LINGAM_ETIMEOUT in its control block, and the kernel must end normally (the context
  * stays usable).  which = 0: an mbarrier phase that no thread completes (the copy-ring waits
  * of the iteration and batch kernels); 1: the grid barrier with its arrival count started one
- * arrival off, two CTAs (the barrier of the iteration and batch kernels); 2: the wave word of
- * a single fit that nothing publishes; 3: a row flag of the B fit's Cholesky that nothing
- * sets.  The control block and flag are library-owned device variables.  *observed receives
- * the recorded status.  Returns LINGAM_EINVAL for which outside 0..3, timeout_s outside
+ * arrival off, two CTAs (the barrier of the iteration and batch kernels), then the ordering
+ * kernel's wait for its workers' arrivals; 2: the wave word of a single fit that nothing
+ * publishes, the tile kernels' and then the ordering kernel's; 3: a row flag of the B fit's
+ * Cholesky that nothing sets.  Each wait has timeout_s.  The control blocks and flag are library-owned device variables.  *observed receives
+ * the recorded status (of two, the first that is not LINGAM_ETIMEOUT).  Returns LINGAM_EINVAL for which outside 0..3, timeout_s outside
  * (0, 60] or a NULL observed, LINGAM_ECUDA if the launch fails, else LINGAM_OK.  Synchronous
  * on the legacy default stream.
  */

@@ -1864,6 +1864,34 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2)
     }
 }
 
+// ------------------------------------------------------------------ bounded-wait self-test
+// which = 1: the controller's wait for arrivals of workers that are not there; 2: a worker's wait for a
+// wave word that nothing publishes.
+__device__ Ctl g_order_selftest_ctl;
+__global__ void k_order_wait_selftest(int which) {
+    __shared__ OrderShared sh;
+    Ctl* ctl = &g_order_selftest_ctl;
+    const unsigned long long tmo = *reinterpret_cast<volatile unsigned long long*>(&ctl->timeout_ns);
+    OrderWave wv;
+    if (which == 1) wait_arrivals(ctl, ctl, 1u, tmo, sh);
+    else wait_order_wave(ctl, ctl, 1u, tmo, sh, wv);
+}
+cudaError_t run_order_wait_selftest(int which, unsigned long long timeout_ns, int* status, cudaStream_t st) {
+    Ctl h = {};
+    h.timeout_ns = timeout_ns;
+    cudaError_t e = cudaMemcpyToSymbolAsync(g_order_selftest_ctl, &h, sizeof(h), 0, cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return e;
+    k_order_wait_selftest<<<1, 32, 0, st>>>(which);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    e = cudaMemcpyFromSymbolAsync(&h, g_order_selftest_ctl, sizeof(h), 0, cudaMemcpyDeviceToHost, st);
+    if (e != cudaSuccess) return e;
+    e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return e;
+    *status = h.status;
+    return cudaSuccess;
+}
+
 // ------------------------------------------------------------------ to the tile kernels
 // One CTA per variable left in U (f.flags): its row into f.xt, its covariances with the later variables,
 // normalised, into both triangles of f.sig and f.sigf, its statistics by its own mean, and its sort key.

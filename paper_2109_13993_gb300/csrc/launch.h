@@ -74,6 +74,8 @@ cudaError_t launch_fit_B(const Fit& f, cudaStream_t st);
 cudaError_t launch_factor_B(const Fit& f, cudaStream_t st, long long* launches);
 cudaError_t launch_factor_B_batch(const Fit* fits_dev, const int* p_host, int count, const Fit* fits_host, cudaStream_t st);
 // Bounded-wait self-test (k_iter.cu): the status the wait recorded (LINGAM_ETIMEOUT expected).
+// (which 1 and 2 also have a counterpart in the ordering kernel, k_order.cu).
+cudaError_t run_order_wait_selftest(int which, unsigned long long timeout_ns, int* status, cudaStream_t st);
 cudaError_t run_wait_selftest(int which, unsigned long long timeout_ns, int* status, cudaStream_t st);
 // B of many problems: one CTA per problem of p <= 128 (shared-memory Cholesky), the
 // multi-launch fit for larger ones.  p_host and fits_host mirror the device table.

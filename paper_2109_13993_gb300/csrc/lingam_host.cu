@@ -1381,7 +1381,9 @@ int lingam_fit_bootstrap(const void* X, long long p, long long n, int nboot, con
 int lingam_selftest_wait(int which, double timeout_s, int* observed) {
     if (which < 0 || which > 3 || !(timeout_s > 0.0) || timeout_s > 60.0 || !observed) return LINGAM_EINVAL;
     int st = 0;
-    if (run_wait_selftest(which, (unsigned long long)(timeout_s * 1e9), &st, nullptr) != cudaSuccess) {
+    const unsigned long long ns = (unsigned long long)(timeout_s * 1e9);
+    if (run_wait_selftest(which, ns, &st, nullptr) != cudaSuccess ||
+        ((which == 1 || which == 2) && st == LINGAM_ETIMEOUT && run_order_wait_selftest(which, ns, &st, nullptr) != cudaSuccess)) {
         cudaGetLastError();
         return LINGAM_ECUDA;
     }

@@ -372,8 +372,8 @@ def autotune_reset():
 
 def selftest_wait(which: int, timeout_s: float) -> int:
     """lingam_selftest_wait: the status one device-side wait recorded after waiting for an
-    event that never happens (0: mbarrier phase, 1: grid barrier, 2: wave word, 3: the B
-    fit's Cholesky row flag)."""
+    event that never happens (0: mbarrier phase, 1: grid barrier and the ordering
+    kernel's arrivals, 2: wave words of both, 3: the B fit's Cholesky row flag)."""
     obs = ctypes.c_int(0)
     st = load().lingam_selftest_wait(int(which), float(timeout_s), ctypes.byref(obs))
     if st != LINGAM_OK:

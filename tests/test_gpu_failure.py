@@ -1,6 +1,6 @@
 """Failure detection on the GPU without a GPU fault: each kind of device-side wait of the
 library (copy-ring mbarrier and grid barrier of the iteration and batch kernels, wave
-word, the B fit's Cholesky row flag) is made to wait for an event that never happens; it
+word, the ordering kernel's arrivals and wave word, the B fit's Cholesky row flag) is made to wait for an event that never happens; it
 must give up after the timeout, record LINGAM_ETIMEOUT, and let the kernel end, so that
 the context stays usable (a fit and a batch right after it succeed)."""
 import time
@@ -38,6 +38,14 @@ def test_wait_gives_up_with_timeout_status(which):
     assert sorted(r.order.tolist()) == list(range(8))
     rb = lingam.fit_batch([X, X[:5]], precision="mixed")
     assert rb.status == 0 and sorted(rb.orders[0].tolist()) == list(range(8))
+
+
+@pytest.mark.parametrize("which", [1, 2])
+def test_both_waits_of_a_kind_run_out(which):
+    # the tile kernels' and the ordering kernel's (arrivals and wave word), each for its whole limit
+    t0 = time.perf_counter()
+    assert lingam.selftest_wait(which, 0.2) == lingam.LINGAM_ETIMEOUT
+    assert time.perf_counter() - t0 >= 0.4
 
 
 @pytest.mark.parametrize("step", ["standardize", "covariance", "iteration:3", "bfit", "batch"])
