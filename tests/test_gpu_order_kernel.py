@@ -51,7 +51,7 @@ def test_fp64_fit_matches_oracle(p, n, prune):
 
 
 @pytest.mark.parametrize("p,n", SIZES + [(80, 500), (81, 500), (100, 2399), (100, 2400), (127, 500), (128, 500), (129, 500),
-                                         (150, 3600), (151, 3700), (160, 640), (161, 640)])
+                                         (160, 640), (161, 640)])
 def test_mixed_scores_and_pruned_roots(p, n):
     # every score within the mixed path's 1e-4 of the oracle; the killer pairs change no root's score.
     # Equal up to the FP32 rounding of I, 1e-6 absolute: S = sum of m squares I_j^2 moves by at most
@@ -259,6 +259,104 @@ def test_hand_over_within_a_bounded_number_of_iterations():
         assert np.array_equal(part.order[:iters], ref.order[:iters]) and np.all(part.order[iters:] == -1)
         assert np.array_equal(part.root_score[:iters], ref.root_score[:iters])
         assert part.kernel_launches == 5 + (iters > it0) * (1 + iters - it0)
+
+
+# padded samples p x ld (ld a multiple of 128) just below and above the sizes where the units change: 64 and
+# 128 samples at 2^16, 128 and 256 at 2^18 (FP64), 256 and 512 at 2^18, 512 and 1024 at 2^22 (mixed); a last
+# unit that is not full; samples for several staged passes of a worker (split_n = 1); candidates for the
+# several-warp selection (more than 256)
+@pytest.mark.parametrize("p,n,split_n", [(40, 1500, 0), (40, 1601, 0), (64, 3967, 0), (64, 4090, 0), (9, 70001, 1)])
+def test_fp64_units(p, n, split_n):
+    X = _data(p, n, 300 + p)
+    o_order, o_B, o_S = oracle.fit(X)
+    for prune in (True, False):
+        f = lingam.fit(_dev(X, torch.float64), precision="fp64", prune=prune, forced_order=o_order, split_n=split_n)
+        want = np.array([o_S[k, o_order[k]] for k in range(p)])
+        assert np.all(np.abs(f.root_score - want) <= 1e-10 * np.abs(want) + 1e-14)
+        assert np.abs(f.B - o_B).max() <= 1e-10 * max(1.0, np.abs(o_B).max())
+
+
+@pytest.mark.parametrize("p,n,split_n", [(64, 3967, 0), (64, 4090, 0), (41, 102200, 0), (41, 102300, 0), (9, 200001, 1),
+                                         (257, 700, 0), (258, 513, 0), (300, 900, 0)])
+def test_mixed_units_and_selection(p, n, split_n):
+    X = _data(p, n, 300 + p).astype(np.float32)
+    ref = lingam.fit(_dev(X, torch.float64), precision="fp64", prune=False, want_scores=True)
+    got = lingam.fit(_dev(X, torch.float32), forced_order=ref.order, want_scores=True, split_n=split_n)
+    m = ~np.isnan(got.scores)
+    assert not np.any(m & np.isnan(ref.scores))
+    assert np.abs(got.scores[m] - ref.scores[m]).max() <= 1e-4
+    left = p - 1 - np.arange(p)   # (the bound of test_mixed_scores_and_pruned_roots)
+    assert np.all(np.abs(got.root_score - ref.root_score) <= 2e-6 * np.sqrt(left * ref.root_score) + left * 1e-12)
+    assert np.abs(got.B - ref.B).max() <= 1e-4 * max(1.0, np.abs(ref.B).max())
+
+
+def test_mixed_batch_units():
+    # a batch's units of 1024 samples with a last one that is not full
+    Xs = [_data(p, n, 400 + p).astype(np.float32) for p, n in [(20, 5001), (33, 2047), (9, 1025), (50, 3333), (7, 1023)]]
+    got = lingam.fit_batch([_dev(X, torch.float32) for X in Xs], want_scores=True)
+    for X, order, S in zip(Xs, got.orders, got.scores):
+        ref = lingam.fit(_dev(X, torch.float64), precision="fp64", prune=False, forced_order=order, want_scores=True)
+        m = ~np.isnan(S)
+        assert m[:-1].sum(axis=1).min() >= 1
+        assert np.abs(S[m] - ref.scores[m]).max() <= 1e-4
+
+
+def _chain(p, n, seed):
+    X = np.random.default_rng(seed).laplace(size=(p, n))
+    for i in range(1, p):
+        X[i] += 0.7 * X[i - 1]
+    return X[np.random.default_rng(seed + 1).permutation(p)]
+
+
+# the last sizes of 16, 12, 8 and 4 columns a wave and the first ones below (controller state and measures
+# share 220 KB), and the first sizes for the tile kernels
+@pytest.mark.parametrize("p,precision", [(1706, "mixed"), (1707, "mixed"), (1942, "mixed"), (1943, "mixed"), (2252, "mixed"),
+                                         (2253, "mixed"), (2681, "mixed"), (2682, "mixed"), (1116, "fp64"), (1117, "fp64"),
+                                         (1641, "fp64"), (2146, "fp64")])
+def test_largest_single_fits_against_the_tile_kernels(p, precision):
+    X = _dev(_chain(p, 192, p), torch.float32 if precision == "mixed" else torch.float64)
+    kw = dict(precision=precision, max_iters=4, want_scores=True, want_B=False)
+    tiles = lingam.fit(X, tile_i=32, tile_j=32, **kw)
+    order = tiles.order[:4].tolist()
+    forced = np.array(order + sorted(set(range(p)) - set(order)), dtype=np.int32)
+    got = lingam.fit(X, forced_order=forced, **kw)
+    assert got.kernel_launches <= tiles.kernel_launches - (0 if p == 2682 else 3)
+    m = ~np.isnan(got.scores[:4]) & ~np.isnan(tiles.scores[:4])
+    assert m.sum(axis=1).min() >= 1
+    s = tiles.scores[:4][m]
+    bound = 2e-6 * np.sqrt(p * s) + p * 1e-12 if precision == "mixed" else 1e-10 * s + 1e-14
+    assert np.all(np.abs(got.scores[:4][m] - s) <= bound)
+    want = tiles.root_score[:4]
+    assert np.all(np.abs(got.root_score[:4] - want) <= (2e-6 * np.sqrt(p * want) + p * 1e-12 if precision == "mixed" else 1e-10 * want))
+
+
+def test_b_of_a_large_fit():
+    # the permuted factor, two columns of 2100 doubles a CTA
+    p, n = 2100, 8000   # (enough samples that it is not handed over)
+    X = _chain(p, n, 5).astype(np.float32)
+    got = lingam.fit(_dev(X, torch.float32))
+    assert got.kernel_launches == 7
+    x = X[got.order].astype(np.float64)
+    low = np.linalg.cholesky(np.cov(x))
+    want = np.eye(p) - np.diag(low)[:, None] * np.linalg.inv(low)
+    B = got.B[np.ix_(got.order, got.order)]
+    assert np.all(np.triu(B) == 0.0)
+    assert np.abs(B - np.tril(want, -1)).max() <= 1e-4 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("p", [332, 333, 844, 845, 1100, 1101])
+def test_largest_problems_of_a_batch(p):
+    # 16, 12, 8 and 4 columns a wave in 108 KB, and the first size for tiles
+    X = _dev(_chain(p, p + 200, p), torch.float32)
+    small = _dev(_chain(12, 300, 1), torch.float32)
+    got = lingam.fit_batch([X, small], want_report=True)
+    assert got.status == lingam.LINGAM_OK
+    one = lingam.fit(X, forced_order=got.orders[0])
+    left = p - 1 - np.arange(p)
+    s = one.root_score
+    assert np.all(np.abs(got.root_scores[0] - s) <= 4e-6 * np.sqrt(left * s) + left * 4e-12)   # (both rounded)
+    assert np.abs(got.Bs[0] - one.B).max() <= 1e-9 * np.abs(one.B).max()
+    assert np.array_equal(got.orders[1], lingam.fit(small).order)
 
 
 def test_batch_with_queued_problems_matches_oracle():
