@@ -932,13 +932,13 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
         return LINGAM_EINVAL;
     if (!is_device_ptr(workspace) || (reinterpret_cast<uintptr_t>(workspace) % kAlign) != 0) return LINGAM_EINVAL;
     std::vector<long long> P(static_cast<size_t>(count)), N(static_cast<size_t>(count));
-    bool with_B = true, gather = true;
+    bool with_B = false, gather = true;   // (with_B: of any dataset)
     for (int k = 0; k < count; ++k) {
         const BatchItem& it = items[size_t(k)];
         if (!it.X || !it.order || it.p < 1 || it.n < 3 || it.p > kMaxP || it.n > (1ll << 30)) return LINGAM_EINVAL;
         P[size_t(k)] = it.p;
         N[size_t(k)] = it.n;
-        if (!it.B) with_B = false;
+        if (it.B) with_B = true;
         if (is_device_ptr(it.order) || (it.B && is_device_ptr(it.B))) gather = false;
     }
     const size_t esz = o.input_dtype == LINGAM_F32 ? 4 : 8;
@@ -1122,7 +1122,7 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
     size_t sp = 0, spp = 0;
     bool adjacent = gather && with_B;
     for (int k = 0; k < count; ++k) {
-        adjacent = adjacent && items[size_t(k)].B == items[0].B + spp;
+        adjacent = adjacent && items[size_t(k)].B && items[size_t(k)].B == items[0].B + spp;
         sp += size_t(P[size_t(k)]);
         spp += size_t(P[size_t(k)]) * size_t(P[size_t(k)]);
     }
@@ -1156,10 +1156,10 @@ static int fit_many(std::vector<BatchItem>& items, void* workspace, const lingam
         if (stk == LINGAM_OK) {
             if (gather) {
                 std::memcpy(it.order, sorder.data() + po, pk * sizeof(int));
-                if (with_B && sB) std::memcpy(it.B, sB.get() + pb, pk * pk * sizeof(double));
+                if (it.B && sB) std::memcpy(it.B, sB.get() + pb, pk * pk * sizeof(double));
             } else {
                 if (cudaMemcpy(it.order, f.order, pk * sizeof(int), cudaMemcpyDefault) != cudaSuccess) stk = LINGAM_ECUDA;
-                if (with_B && cudaMemcpy(it.B, f.bout, pk * pk * sizeof(double), cudaMemcpyDefault) != cudaSuccess)
+                if (it.B && cudaMemcpy(it.B, f.bout, pk * pk * sizeof(double), cudaMemcpyDefault) != cudaSuccess)
                     stk = LINGAM_ECUDA;
             }
             if (it.rep) {

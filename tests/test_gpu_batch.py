@@ -251,6 +251,34 @@ def test_batch_degenerate_member_does_not_stop_the_others():
         assert _agree_until_unresolved(res.orders[k], single.order, roots, margins) > 0
 
 
+@pytest.mark.parametrize("without", [0, 1, 2])
+def test_batch_with_one_dataset_that_wants_no_B(without):
+    """B[k] == NULL leaves out that dataset's B only."""
+    import ctypes
+    ps, n = [7, 12, 9], 600
+    Xs = [_dev(synth.lingam_dataset(p, n, 0.3, seed=170 + p).X.astype(np.float32)) for p in ps]
+    ref = lingam.fit_batch(Xs)
+    L = lingam.load()
+    o, _ = lingam.make_opts("mixed", np.float32)
+    pa, na = (ctypes.c_longlong * 3)(*ps), (ctypes.c_longlong * 3)(*[n] * 3)
+    ws = lingam.alloc_workspace(int(L.lingam_workspace_size_batch(3, pa, na, ctypes.byref(o))))
+    orders = [np.zeros(p, dtype=np.int32) for p in ps]
+    Bs = [np.full((p, p), np.nan) for p in ps]
+    xp = (ctypes.c_void_p * 3)(*[X.data_ptr() for X in Xs])
+    op = (ctypes.c_void_p * 3)(*[a.ctypes.data for a in orders])
+    bp = (ctypes.c_void_p * 3)(*[None if k == without else Bs[k].ctypes.data for k in range(3)])
+    status = np.full(3, -9, dtype=np.int32)
+    torch.cuda.synchronize()
+    assert L.lingam_fit_batch(3, xp, pa, na, op, bp, ctypes.c_void_p(ws.data_ptr()), ctypes.byref(o),
+                              status.ctypes.data_as(ctypes.POINTER(ctypes.c_int)), None) == lingam.LINGAM_OK
+    for k in range(3):
+        assert np.array_equal(orders[k], ref.orders[k])
+        if k == without:
+            assert np.all(np.isnan(Bs[k]))
+        else:
+            assert np.array_equal(Bs[k], ref.Bs[k])
+
+
 def test_batch_graph_replay_is_identical():
     ds = synth.uneven_batch(5, seed=9)
     Xs = [_dev(d.X[:, :2000].astype(np.float32)) for d in ds]
