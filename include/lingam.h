@@ -80,14 +80,16 @@ typedef struct {
     int input_dtype;         /* element type of X: LINGAM_F32 or LINGAM_F64 */
     int prune;               /* 1 = threshold pruning (Sec. III-B), 0 = compare every pair */
     int reuse;               /* 1 = one evaluation per unordered pair (Sec. III-A), 0 = every ordered pair */
-    int tile_i, tile_j;      /* both 0 (default): single fits run the ordering kernel (no tiles; p up to
-                                about 2000; on the mixed path without pruning or reuse
-                                up to 160), batch calls as lingam_fit_batch says.  Else the pair-tile
+    int tile_i, tile_j;      /* both 0 (default): single fits run the ordering kernel (no tiles) up to
+                                p = 2681 (FP64 path: 2146); on the mixed path without pruning or reuse
+                                up to 80, or up to 150 (130 without reuse) with 24 samples a variable,
+                                and a fit whose iterations keep taking 176 candidates or more is left to
+                                the tile kernels; batch calls as lingam_fit_batch says.  Else the pair-tile
                                 shape of the tile kernels on the mixed path, rows x columns: 64 x 32,
-                                32 x 32 or 64 x 16, and for batch calls only 32 x 16, and 1 x 1 (the
-                                ordering kernel) (a zero in one takes 64 rows or 32 columns).  The FP64
-                                path's tiles are 32 x 32.  Larger problems run the tile kernels with the
-                                autotuner's shape (lingam_tile_rows/_cols, lingam_batch_tile_rows/_cols). */
+                                32 x 32 or 64 x 16, and for batch calls only 32 x 16, and 1 x 1 (no
+                                tiles, see lingam_fit_batch) (a zero in one takes 64 rows or 32 columns).
+                                The FP64 path's tiles are 32 x 32.  Where both are 0 the tile kernels take
+                                the autotuner's shape (lingam_tile_rows/_cols, lingam_batch_tile_rows/_cols). */
     int split_n;             /* single fits: split of the sample axis.  0 (default) = as the kernel
                                 chooses (the ordering kernel the number of segments that takes the
                                 shortest estimated time; the tile kernels spread a wave's (tile, 32-sample
@@ -205,8 +207,8 @@ int lingam_fit(const void* X, long long p, long long n, int* order, double* B, v
  *   Sigma      [p*p] doubles, host or device, row-major; Sigma[i*p + i] = 1 exactly.
  *   report     NULL, or a report whose t_standardize_ms, t_gram_ms and kernel_launches
  *              are filled in (the other fields are left untouched).
- * precision LINGAM_MIXED computes the product on the tensor cores from a TF32 + FP32
- * split of the FP32 rows (FP32 accumulation, FP64 sum of the sample-axis splits);
+ * precision LINGAM_MIXED computes the product on the tensor cores from three FP16
+ * digits of each FP32 value (FP32 accumulation, FP64 sum of the sample-axis splits);
  * LINGAM_FP64 computes it in FP64.  Sigma is written only on LINGAM_OK; rows with zero
  * variance or non-finite values give LINGAM_EDEGENERATE.
  */
@@ -217,7 +219,7 @@ int lingam_covariance(const void* X, long long p, long long n, double* Sigma, vo
  * Pair-tile autotuner (the paper has no counterpart: its GPU design has one tile shape).
  * The tile kernels evaluate pairs in tiles of rows x columns variables: 64 x 32 (512
  * threads), 32 x 32 or 64 x 16 (256 threads, two CTAs per SM).  Single fits with the default
- * options do not use them (lingam_opts.tile_i), larger ones than the ordering kernel takes do.  The columns of a tile are
+ * options use them only where lingam_opts.tile_i says so.  The columns of a tile are
  * the candidates a wave completes, so 16-column tiles prune more finely (fewer pairs, more
  * waves).  Which shape is faster depends on p, n and the data.  The library keeps a
  * process-wide table of the choice per size bucket (ceil(log2 p), ceil(log2 n)); a
@@ -236,17 +238,16 @@ int lingam_covariance(const void* X, long long p, long long n, double* Sigma, vo
  *                       largest problem has maxp variables and maxn samples, when
  *                       opts->tile_i and opts->tile_j are 0.  Batches have a table of their
  *                       own (bucket of the largest p and n); a bucket never measured runs the
- *                       ordering kernel (1 x 1) where it takes every problem of the call (p up to
- *                       about 800), else, and as these functions report it, 1 x 1 when maxp <= 128
+ *                       ordering kernel where it takes every problem of the call (p up to
+ *                       1100), else, and as these functions report it, 1 x 1 when maxp <= 128
  *                       and 32 x 32 tiles beyond.  With opts->reuse = 0, 1 x 1 runs as 64 x 16.
  * lingam_autotune_batch -- measures lingam_fit_batch on the caller's count datasets (as
  *                       lingam_fit_batch with opts on the mixed path, B not fitted) with
  *                       each shape: a warm-up call, the call that captures the graph, and
  *                       the timed third call (host wall time of the synchronous call).
  *                       Batches have two more shapes for many small problems: 32 x 16
- *                       tiles (128 threads, three CTAs per SM, 64-sample chunks), and 1 x 1, the
- *                       ordering kernel (groups of CTAs per problem, none waiting for another's).
- *                       Records the fastest for the bucket of
+ *                       tiles (128 threads, three CTAs per SM, 64-sample chunks), and 1 x 1 (see
+ *                       lingam_fit_batch).  Records the fastest for the bucket of
  *                       the batch's largest p and n, returns it in *tile_rows, *tile_cols,
  *                       and ms[0..4] (if not NULL) receive the times with 64 x 32, 32 x 32,
  *                       64 x 16, 32 x 16 and 1 x 1.  Costs fifteen batch calls; the
@@ -303,10 +304,12 @@ size_t lingam_workspace_size_batch(int count, const long long* p, const long lon
  * run without a graph.  opts->forced_order and opts->prior must be NULL, and
  * opts->max_iters and opts->gamma0 0; opts->split_n is ignored.  Pair tiles: on the
  * mixed path opts->tile_i x opts->tile_j for every problem of the call (64 x 32, 32 x 32,
- * 64 x 16, 32 x 16, or 1 x 1: the ordering kernel, which needs opts->reuse = 1 and p up to
- * about 800 and otherwise runs as 64 x 16), or, with both 0, what the batch autotuner measured
+ * 64 x 16, 32 x 16, or 1 x 1: the ordering kernel, or, for more than 1100 variables and for
+ * unpruned batches that fill the GPU with long rows, each pair by one warp; without
+ * opts->reuse 64 x 16), or, with both 0, what the batch autotuner measured
  * for the largest p and n, else the ordering kernel where it takes the call (see
- * lingam_batch_tile_rows/_cols); on the FP64 path the ordering kernel, else 32 x 32.
+ * lingam_batch_tile_rows/_cols; unpruned up to 160 variables, by the rule of 1 x 1 up to 128);
+ * on the FP64 path the ordering kernel up to 952 variables, else 32 x 32.
  */
 int lingam_fit_batch(int count, const void* const* X, const long long* p, const long long* n, int* const* order,
                      double* const* B, void* workspace, const lingam_opts* opts, int* status,

@@ -52,7 +52,7 @@ constexpr int kNoRoot = 8;     // a known ancestor is still in U (prior knowledg
 // host only after the final stream synchronisation.
 struct Ctl {
     int status;          // first error (lingam_status), 0 = OK
-    int it;              // current iteration
+    int it;              // current iteration (ordering kernel: 0, or the one from which it leaves the fit to the tile kernels)
     int r;               // variables left in U at this iteration
     int root;            // root chosen at this iteration
     int done;            // iteration finished (root chosen)

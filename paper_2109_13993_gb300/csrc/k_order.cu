@@ -16,6 +16,7 @@
 //   - candidates are taken in the order of their last known score without the contribution of
 //     the variable just removed, so that the children of the removed root come first.
 // Neither changes the root: a partial score is a lower bound of the score whatever pairs it holds.
+// Where they leave most pairs to compare, a single fit goes on in the tile kernels (kHandCols).
 // Pairs evaluated, of all pairs: p = 300, n = 5000 graphs with one causal order 82 % -> 6 %, p = 1000,
 // n = 10^4 79 % -> 1.7 %, random graphs of in-degree 3 at p = 300 31 % -> 19 %, with 1.0-1.7 waves per
 // iteration instead of 1.4-8.9.  Whole fits against the tile kernels with a barrier per phase:
@@ -866,7 +867,7 @@ constexpr unsigned kNoKey = 0xffffffffu;
 
 // What the controller keeps between waves, the same for all its threads.
 struct CtlState {
-    int r, a, it, cmax, want, bestv;
+    int r, a, it, bestv;
     long long best;   // key of the iteration's lowest complete score
     double gamma;
     OrderWave wave;   // the next wave
@@ -1181,7 +1182,7 @@ struct Controller {
         for (int k = threadIdx.x; k < kOrderSlots; k += NT) f.gcount[k] = 0;
         if (threadIdx.x == 0) sh.rep_nw = 0;
         const int cm = max_cols(r);
-        new_iteration(cm, kMaxCols);
+        new_iteration();
         __syncthreads();
         next_wave(0, -1, false, 0);
         if (r > 1) {
@@ -1191,13 +1192,11 @@ struct Controller {
             done();
         }
     }
-    __device__ __forceinline__ void new_iteration(int cmax, int want) {
+    __device__ __forceinline__ void new_iteration() {
         if (threadIdx.x == 0) {
             sh.st.r = r;
             sh.st.a = 0;
             sh.st.it = it;
-            sh.st.cmax = cmax;
-            sh.st.want = want;
             sh.st.best = kMaxScore;
             sh.st.bestv = -1;
             sh.st.gamma = f.gamma0;
@@ -1623,7 +1622,7 @@ struct Controller {
         // quads with one to spare on the FP32 path (a column of a started quad is free), no more on the
         // FP64 path (65 x 2001: 4.0 ms, one or two to spare 4.3 and 4.9, quads 5.3).
         const int cmax = max_cols(r), want = !prunes ? kMaxCols : f32 ? (need + 4) / 4 * 4 : max(need, 1);
-        new_iteration(cmax, want);
+        new_iteration();
         if (r == 1) {
             if (tid < 32) swap_slots(rs, 1);
             bar();

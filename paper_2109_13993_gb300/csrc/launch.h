@@ -23,8 +23,8 @@ cudaError_t launch_standardize_batch(const Fit* fits, const SrcDesc* src, const 
 // FP64 path: Sigma = Xn Xn^T / (n-1) of the normalised rows (CalculateCovMat, Algorithm 3); sig0 = sig.
 // partial_bytes: what f.partials holds.  launches: NULL, or increased by the kernels launched (here and below).
 cudaError_t launch_gram(const Fit& f, size_t partial_bytes, cudaStream_t st, long long* launches);
-// The same product on the tensor cores (mixed path): the rows are split into exact
-// TF32 digits (three p x ld float planes and p exponents in `digits`), tcgen05 MMAs
+// The same product on the tensor cores (mixed path): the rows are split into FP16
+// digits (three p x ld half planes and p exponents in `digits`), tcgen05 MMAs
 // over 128 x 128 tiles of the upper triangle with the sample axis split over CTAs,
 // float-float partial tiles in `partial`, summed in FP64 into sig and sig0.
 cudaError_t launch_gram_tc(const Fit& f, void* digits, void* partial, cudaStream_t st);
@@ -45,9 +45,9 @@ cudaError_t launch_iteration(const Fit& f, int it, int grid, cudaStream_t st);
 // Largest co-resident grid of the iteration kernel (one CTA per SM).
 int iteration_grid(const Fit& f, int nsm);
 // The ordering kernel (k_order.cu): all iterations in one persistent cooperative launch, with
-// killer pairs.  order_supported: whether it takes a problem (pair reuse on; the state of its
-// variables in shared memory, p up to about 2300 for a single fit; batch: 256-thread CTAs, two per
-// SM, p up to about 1200).
+// killer pairs.  order_supported: whether it takes a problem: the state of its variables and four
+// columns' measures fit into the controller's shared memory up to p = 2681 (mixed path) and 2146 (FP64) in a
+// single fit, 1100 and 952 in a batch (256-thread CTAs, two per SM).  Without pair reuse it takes single fits.
 bool order_supported(const Fit& f, bool batch);
 int order_grid(const Fit& f, int nsm);
 // Behind an ordering kernel that stopped at iteration `it` (Ctl::it > 0, Fit::handover): rows, covariance
