@@ -466,8 +466,9 @@ __device__ __forceinline__ double rsqrt_fast(double x) {
 }
 
 // The removal's coefficients of variable v: S the covariance of the un-normalised remaining rows and
-// D their scales (row = residual times D, so Sigma[v][w] = S[v][w] D[v] D[w]); with rho = S[v][root]
-// D[v] D[root], the normalised row loses rho times the root's and is scaled by 1 / sqrt(1 - rho^2).
+// D their scales, 1 / sqrt(S[v][v]) (row = residual times D, so Sigma[v][w] = S[v][w] D[v] D[w]); with
+// rho = S[v][root] D[v] D[root], the normalised row loses rho times the root's and is scaled by
+// 1 / sqrt(1 - rho^2) = D_new / D.
 struct Removal {
     double rho, inv;
 };
@@ -677,14 +678,24 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
                     d = __ldcg(dold + v);
                     if (rm) {
                         sr = __ldcg(sold + min(v, root) * p + max(v, root));
+                        const double svv = __ldcg(sold + v * p + v);
                         rho = sr * (d * droot);
                         double om = fma(-rho, rho, 1.0);
                         if (!(om > degenerate_om(sizeof(T) == 4))) {
                             set_status(f.ctl, LINGAM_EDEGENERATE);
                             om = 1.0;
                         }
-                        inv = rsqrt_fast(om);
-                        d *= inv;
+                        // the new scale from the element itself, so that no rounding is carried on from
+                        // iteration to iteration (elements that cancelled to nothing: from the old scale)
+                        const double left = svv * om;
+                        if (left > 1e-30) {
+                            const double dn = rsqrt_fast(left);
+                            inv = dn * (svv * d);
+                            d = dn;
+                        } else {
+                            inv = rsqrt_fast(om);
+                            d *= inv;
+                        }
                         if (k < kRowBatch && bs == 0) {   // (one worker per row: the first segment's)
                             dnew[v] = d;
                             f.rmat[size_t(p - 1 - nrow) * p + v] = sr;   // (for the B fit)
