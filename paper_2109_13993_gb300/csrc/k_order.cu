@@ -686,16 +686,12 @@ __device__ __noinline__ void worker_wave(const Fit& f, const OrderWave wv, const
                             om = 1.0;
                         }
                         // the new scale from the element itself, so that no rounding is carried on from
-                        // iteration to iteration (elements that cancelled to nothing: from the old scale)
-                        const double left = svv * om;
-                        if (left > 1e-30) {
-                            const double dn = rsqrt_fast(left);
-                            inv = dn * (svv * d);
-                            d = dn;
-                        } else {
-                            inv = rsqrt_fast(om);
-                            d *= inv;
-                        }
+                        // iteration to iteration (an element that cancelled to nothing: from the old scale)
+                        const double left = fma(-sr * (droot * droot), sr, svv);
+                        const bool own = left > 1e-30;
+                        const double y = rsqrt_fast(own ? left : om);
+                        inv = own ? y * (svv * d) : y;
+                        d = own ? y : d * y;
                         if (k < kRowBatch && bs == 0) {   // (one worker per row: the first segment's)
                             dnew[v] = d;
                             f.rmat[size_t(p - 1 - nrow) * p + v] = sr;   // (for the B fit)
