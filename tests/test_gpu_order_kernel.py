@@ -1,7 +1,8 @@
 """The ordering kernel, its factor-based B fit and the covariance kernels at the sizes where their splits
 change: units and the last, partial one (128 / 64 samples a step), rows of a worker (32), columns
-(4 ... 16), the controller's warps, in-place and permuted factors (128 variables), the line between
-ordering and tile kernels (160), queued problems of a batch (more than 304), tiles and parts of the
+(4 ... 16), the controller's warps, in-place and permuted factors (128 variables), the lines between
+ordering and tile kernels (unpruned 80 variables or 24 samples a variable; the largest sizes; fits
+that are handed over), queued problems of a batch (more than 304), tiles and parts of the
 covariance (128, 8; 32 on the FP64 path)."""
 import functools
 
